@@ -263,10 +263,11 @@ int lbm_step(lbm_ctx *ctx, long n);
 /* Macroscopic fields of the current state f(t):
  *   flow : rho[N] = sum f (Eq. 24 / step (vi)); u[dim][N] = (sum f e + h a_pre P/2)/rho
  *   D2Q5 : rho[N] receives phi = sum g + h a_pre S/2 (Eqs. 42-43); u unused (may be NULL)
- * with h = 1 if half_forced, else 0 (u^o and phi^o).  Rounding: the sums in a
- * fixed grouping per lattice; j + a_pre P/2 rounded once; u = that times the
- * correctly rounded 1/rho (each product rounded), so u is within two units in
- * the last place of the exact quotient.  Every FP64 readback
+ * with h = 1 if half_forced, else 0 (u^o and phi^o).  Rounding: the sums are
+ * formed in fixed point at the scale of the node's largest population (exactly,
+ * up to 3 to 5 bits below that population's last one) and rounded once, on D2Q5
+ * and outside 2^-523 .. 2^50 in FP64; j + a_pre P/2 rounded once; u = that times
+ * the correctly rounded 1/rho (each product rounded).  Every FP64 readback
  * (lbm_batch_moments, lbm_batch_moments_packed, lbm_batch_step_read) returns
  * these same bits.  where = 0: host pointers (the call synchronises);
  * where = 1: device pointers (asynchronous).

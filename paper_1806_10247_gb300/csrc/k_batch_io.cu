@@ -29,10 +29,7 @@ __device__ __forceinline__ void member_moments(const BatchItem &B, const BatchMo
     } else {
         float d[L::Q];
         load_pulled_dev<L, T>(reinterpret_cast<const T *>(B.buf[p]), g, x, y, z, i, d);
-        double dd[L::Q];
-#pragma unroll
-        for (int a = 0; a < L::Q; a++) dd[a] = (double)d[a];
-        zeroth_first<L>(dd, m0, j);
+        zeroth_first<L>(d, m0, j);
         m0 += B.rho_ref;  // the rest state carries no momentum
     }
     const bool forced = M.half && B.fkind != FK_NONE;

@@ -28,10 +28,7 @@ __device__ __forceinline__ void dev_moments(const T *__restrict__ fin, const Geo
 {
     float d[L::Q];
     load_pulled_dev<L, T>(fin, g, x, y, z, i, d);
-    double dd[L::Q];
-#pragma unroll
-    for (int a = 0; a < L::Q; a++) dd[a] = (double)d[a];
-    zeroth_first<L>(dd, dm0, j);
+    zeroth_first<L>(d, dm0, j);
 }
 
 // Equilibrium populations whose central moments are Eq. 20 (flow; the

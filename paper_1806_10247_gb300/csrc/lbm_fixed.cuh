@@ -1,0 +1,524 @@
+// FP64 steps in fixed point.
+//
+// This GPU issues 1.69 FP64 adds, multiplies or multiply-adds per clock and SM
+// (2.0 conversions between FP64 and integers), but 62 64-bit integer adds and
+// about 5 signed 64 x 64 -> high-64 products, and the two kinds of unit work
+// side by side.  So the step kernels of the FP64 storage convert a node's
+// populations to 64-bit integers at one scale per node, run the moment
+// transforms and the collision on those, and convert the results back.
+//
+// Scale: with E the exponent of the node's largest |f|, X = f 2^(S - E),
+// rounded to nearest even, |X| < 2^(S + 1).  S (FxGrid) leaves the headroom
+// that the sums of the lattice need and keeps S - 52 bits below the last bit
+// of the largest population (3 on D3Q27, 5 on D2Q9): the sums and differences
+// of the transforms are then exact, and a product rounds at 2^-S of the
+// largest population, where an FP64 operation on quantities of the size of rho
+// rounds at 2^-53 of rho.  Mass and momentum are carried without any rounding
+// between the two conversions.  The result is rounded to FP64 once, to nearest
+// even.
+//
+// What the fixed-point form does not take (a population that is not finite, an
+// exponent outside [kEmaxLo, kEmaxHi], |u| >= 1/2, a density far below the
+// largest population, a force as large as the populations, a result that is
+// negative or below 2^-25 of the largest population) is left to the FP64 form:
+// the functions return false and the caller takes that node's FP64 path.
+//
+// Everything here compiles for the host too (tests run it against 64-bit and
+// wider arithmetic on the CPU).
+#pragma once
+
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define FX_HD __host__ __device__ __forceinline__
+#else
+#include <math.h>
+#include <string.h>
+#define FX_HD inline
+#endif
+
+namespace lbmk {
+
+typedef long long i64;
+typedef unsigned long long u64;
+
+// ---- words ------------------------------------------------------------------
+FX_HD u64 fx_bits(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (u64)__double_as_longlong(x);
+#else
+    u64 b;
+    memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+FX_HD double fx_double(u64 b)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((i64)b);
+#else
+    double x;
+    memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+FX_HD unsigned fx_hi(u64 b) { return (unsigned)(b >> 32); }
+
+// High 64 bits of the signed product.
+FX_HD i64 fx_mul(i64 a, i64 b)
+{
+#ifdef __CUDA_ARCH__
+    return __mul64hi(a, b);
+#else
+    return (i64)(((__int128)a * b) >> 64);
+#endif
+}
+// x 2^n for a normal x or 0 (which becomes a value below 2^(n - 1000)): an
+// integer add on the exponent, no FP64 operation.
+FX_HD double fx_ldexp(double x, int n) { return fx_double(fx_bits(x) + ((u64)(unsigned)n << 52)); }
+// Round to nearest even.
+FX_HD i64 fx_round(double x)
+{
+#ifdef __CUDA_ARCH__
+    return __double2ll_rn(x);
+#else
+    return llrint(x);
+#endif
+}
+FX_HD double fx_to_double(i64 x)
+{
+#ifdef __CUDA_ARCH__
+    return __ll2double_rn(x);
+#else
+    return (double)x;
+#endif
+}
+// About 1/x to 2^-22, x > 0.
+FX_HD float fx_rcp_approx(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+
+// ---- scale --------------------------------------------------------------------
+constexpr int kEmaxLo = 500, kEmaxHi = 1073;  // biased exponents the fixed-point forms take (2^-523 .. 2^50)
+
+// S by lattice: after the forward transform the grid is refined by one bit (so
+// that half of a first moment is an integer), and the largest sum formed is the
+// trace of the second moments, at most sum |e|^2 = 54 (D3Q27), 30 (D3Q15), 12
+// (D2Q9) times the largest population: 54 2^(S + 2) < 2^63 and so on.
+template <int Q>
+struct FxGrid;
+template <>
+struct FxGrid<27> {
+    static constexpr int S = 55;
+};
+template <>
+struct FxGrid<15> {
+    static constexpr int S = 56;
+};
+template <>
+struct FxGrid<9> {
+    static constexpr int S = 57;
+};
+template <>
+struct FxGrid<5> {
+    static constexpr int S = 57;
+};
+
+// Biased exponent of the largest |f|.
+template <int Q>
+FX_HD int fx_emax(const double (&f)[Q])
+{
+    unsigned m = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < Q; a++) {
+        const unsigned h = fx_hi(fx_bits(f[a])) & 0x7fffffffu;
+        m = h > m ? h : m;
+    }
+    return (int)(m >> 20);
+}
+FX_HD bool fx_in_range(int emax) { return (unsigned)(emax - kEmaxLo) <= (unsigned)(kEmaxHi - kEmaxLo); }
+
+// Populations at the node's scale; k = S + 1023 - emax.
+template <int Q>
+FX_HD void fx_load(const double (&f)[Q], int k, i64 (&X)[Q])
+{
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < Q; a++) X[a] = fx_round(fx_ldexp(f[a], k));
+}
+
+// X 2^-k, rounded to nearest even; 0 gives 0.
+FX_HD double fx_value(i64 X, int k)
+{
+    const double d = fx_to_double(X);
+    return X == 0 ? 0.0 : fx_ldexp(d, -k);
+}
+
+// The same for 2^32 <= X < 2^62, without an FP64 conversion: shift the leading
+// bit to bit 62, round away the 10 bits below FP64's last one (to nearest
+// even), add the exponent.  `bad` goes negative for any other X.
+FX_HD double fx_value_pos(i64 X, int k, int &bad)
+{
+    const unsigned hi = (unsigned)((u64)X >> 32);
+    bad |= (int)hi - 1;
+#ifdef __CUDA_ARCH__
+    unsigned n;
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(n) : "r"(hi));
+    n -= 1u;
+#else
+    if ((int)hi <= 0) return 0.0;
+    const unsigned n = (unsigned)__builtin_clz(hi) - 1u;
+#endif
+    u64 v = (u64)X << n;
+    v += 0x1ffull + ((v >> 10) & 1ull);
+    v >>= 10;
+    // v = 2^52 .. 2^53: its leading bit adds one to the exponent field
+    return fx_double(v + ((u64)(unsigned)(1023 + 51 + 10 - k - (int)n) << 52));
+}
+
+// ---- force --------------------------------------------------------------------
+// Fixed-point form of a force along one axis at a node, on the refined grid
+// (scale 2^(k + 1)): h1 = F_pre / 4 (half of the pre-collision half force),
+// h2 = (F_pre + F_post) / 4.  h2 enters the momentum of every step, so it is
+// rounded with 8 more bits and a dither from the node's own low bits: a fixed
+// rounding would add up over a steady run.
+struct FxForce {
+    i64 h1, h2;
+};
+// q1 = a_pre / 4, q2 = (a_pre + a_post) / 4, P the shape's value.
+FX_HD bool fx_force(double P, double q1, double q2, int k, int emax, unsigned dither, FxForce &F)
+{
+    const double f1 = q1 * P, f2 = q2 * P;
+    const unsigned m1 = fx_hi(fx_bits(f1)) & 0x7fffffffu, m2 = fx_hi(fx_bits(f2)) & 0x7fffffffu;
+    F.h1 = fx_round(fx_ldexp(f1, k + 1));
+    F.h2 = (fx_round(fx_ldexp(f2, k + 9)) + (i64)(dither & 0xffu)) >> 8;
+    return (int)((m1 > m2 ? m1 : m2) >> 20) <= emax - 6;
+}
+
+// ---- velocity -----------------------------------------------------------------
+// U = j / rho 2^64 for |j| < rho / 2 (refined grid or not: j and rho alike), to
+// a relative 2^-52.  bad < 0 when some |j| is not below rho / 2 or rho is not
+// above 2^52.
+template <int D>
+FX_HD void fx_velocity(i64 rho, const i64 (&j)[3], i64 (&U)[3], int &bad)
+{
+    const int rh = (int)(rho >> 32);
+    bad |= rh - (1 << 20);
+    const double r = fx_ldexp(fx_to_double(rho), -32);
+    const double x = (double)fx_rcp_approx((float)rh);
+    // x (1 + e + e^2) with e = 1 - r x, |e| < 2^-19
+#ifdef __CUDA_ARCH__
+    const double e = fma(-r, x, 1.0);
+    const double p = fma(e, e, e);
+    const double ri = fx_ldexp(fma(x, p, x), 32);
+#else
+    const double e = ::fma(-r, x, 1.0);
+    const double p = ::fma(e, e, e);
+    const double ri = fx_ldexp(::fma(x, p, x), 32);
+#endif
+    const i64 half = (i64)((u64)rho >> 1);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int d = 0; d < D; d++) {
+        // half - |j| > 0 (the shift above is exact up to one unit)
+        bad |= (int)(((half - 1) - (j[d] < 0 ? -j[d] : j[d])) >> 32);
+        U[d] = fx_round(fx_to_double(j[d]) * ri);
+    }
+}
+
+// Constants as fractions of 2^64.
+constexpr i64 kFx3 = 0x5555555555555555ll;   // 1/3
+constexpr i64 kFx6 = 0x2aaaaaaaaaaaaaabll;   // 1/6
+constexpr i64 kFx9 = 0x1c71c71c71c71c72ll;   // 1/9
+constexpr i64 kFx36 = 0x071c71c71c71c71cll;  // 1/36
+constexpr i64 kFx216 = 0x012f684bda12f685ll; // 1/216
+
+// Relaxation factors of a launch: shear (1 - omega_s) 2^63 and bulk
+// (omega_b - 1) 2^63 (D3Q27); D2Q9: (1 - omega_4) 2^62, (1 - omega_5) 2^62 and
+// (omega_3 - 1) 2^62.
+struct FxRates {
+    i64 a, b, c;
+};
+inline i64 fx_fraction(double x, int bits)
+{
+    const double v = x * (double)(1ll << (bits - 1)) * 2.0, top = 9223372036854774784.0;  // 2^63 - 1024
+    return (i64)(v > top ? top : (v < -top ? -top : v));
+}
+inline FxRates fx_rates27(double wb, double ws) { return FxRates{fx_fraction(1.0 - ws, 63), fx_fraction(wb - 1.0, 63), 0}; }
+inline FxRates fx_rates9(double w3, double w4, double w5)
+{
+    return FxRates{fx_fraction(1.0 - w4, 62), fx_fraction(1.0 - w5, 62), fx_fraction(w3 - 1.0, 62)};
+}
+
+// ---- D3Q27 --------------------------------------------------------------------
+// The forward sums of a node's populations (fixed point or any other type), as
+// far as a unit-rates collision and a readback need them.
+template <class V>
+struct FxSums27 {
+    V rho, jx, jy, jz, xx, yy, zz, xy, xz, yz;
+};
+template <class V>
+FX_HD void fx_sums27(const V (&f)[27], FxSums27<V> &s)
+{
+    V a0[9], a1[9], a2[9];  // lines along x: order 0, 1, 2
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int t = 0; t < 9; t++) {
+        const V e = f[3 * t + 2] + f[3 * t];
+        a0[t] = e + f[3 * t + 1];
+        a1[t] = f[3 * t + 2] - f[3 * t];
+        a2[t] = e;
+    }
+    V Y0[3], Y1[3], Y2[3], X0[3], X1[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int c = 0; c < 3; c++) {
+        const V e = a0[3 * c + 2] + a0[3 * c];
+        Y0[c] = e + a0[3 * c + 1];
+        Y1[c] = a0[3 * c + 2] - a0[3 * c];
+        Y2[c] = e;
+        X0[c] = a1[3 * c + 2] + a1[3 * c] + a1[3 * c + 1];
+        X1[c] = a1[3 * c + 2] - a1[3 * c];
+    }
+    s.zz = Y0[2] + Y0[0];
+    s.rho = s.zz + Y0[1];
+    s.jz = Y0[2] - Y0[0];
+    s.jy = Y1[2] + Y1[0] + Y1[1];
+    s.yz = Y1[2] - Y1[0];
+    s.yy = Y2[2] + Y2[0] + Y2[1];
+    s.jx = X0[2] + X0[0] + X0[1];
+    s.xz = X0[2] - X0[0];
+    s.xy = X1[2] + X1[0] + X1[1];
+    s.xx = ((a2[0] + a2[1]) + (a2[2] + a2[3])) + ((a2[4] + a2[5]) + (a2[6] + a2[7])) + a2[8];
+}
+
+// One line of the halved back-shift (k0, k1/2, k2/2 central -> raw); UH = U / 2.
+FX_HD void fx_shift(i64 k0, i64 &k1, i64 &k2, i64 U, i64 UH)
+{
+    const i64 m1 = k1 + fx_mul(k0, UH);
+    k2 += fx_mul(k1 + m1, U);
+    k1 = m1;
+}
+// Lines with known zeros: k1 = k2 = 0 on entry; k0 = k2 = 0.
+FX_HD void fx_shift_k0(i64 k0, i64 &k1, i64 &k2, i64 U, i64 UH)
+{
+    k1 = fx_mul(k0, UH);
+    k2 = fx_mul(k1, U);
+}
+// k2 = 0 on entry.
+FX_HD void fx_shift_k01(i64 k0, i64 &k1, i64 &k2, i64 U, i64 UH)
+{
+    const i64 m1 = k1 + fx_mul(k0, UH);
+    k2 = fx_mul(k1 + m1, U);
+    k1 = m1;
+}
+FX_HD void fx_shift_k1(i64 k1, i64 &k2, i64 U) { k2 = fx_mul(k1 + k1, U); }
+// k1 = 0 on entry.
+FX_HD void fx_shift_k02(i64 k0, i64 &k1, i64 &k2, i64 U, i64 UH)
+{
+    k1 = fx_mul(k0, UH);
+    k2 += fx_mul(k1, U);
+}
+// k1 known (half of a first moment), its central value 0.
+FX_HD void fx_shift_first(i64 k1, i64 &k2, i64 U) { k2 += fx_mul(k1, U); }
+
+FX_HD void fx_back(i64 &m0, i64 &m1, i64 &m2)
+{
+    const i64 a = m2 - m1, b = m2 + m1;
+    m1 = m0 - m2 - m2;
+    m0 = a;
+    m2 = b;
+}
+
+// The D3Q27 collision with omega_3 .. omega_6 = 1 (see k_d3q27.cu collide_w1
+// for the steps): s are the sums on the grid k, force F per axis (axes 1 and 2
+// unused with XO).  m: post-collision populations on the grid k + 1.
+template <bool XO>
+FX_HD void fx_collide27(const FxSums27<i64> &s, const FxForce (&F)[3], const FxRates &w, i64 (&m)[27], int &bad)
+{
+    // halves of the half-forced first moments on the refined grid: j / 2 there is j here
+    const i64 hx = s.jx + F[0].h1, hy = XO ? s.jy : s.jy + F[1].h1, hz = XO ? s.jz : s.jz + F[2].h1;
+    const i64 rho = s.rho + s.rho;
+    const i64 j[3] = {hx + hx, hy + hy, hz + hz};
+    i64 U[3];
+    fx_velocity<3>(rho, j, U, bad);
+    const i64 cxx = s.xx + s.xx - fx_mul(j[0], U[0]), cyy = s.yy + s.yy - fx_mul(j[1], U[1]);
+    const i64 czz = s.zz + s.zz - fx_mul(j[2], U[2]);
+    const i64 cxy = s.xy + s.xy - fx_mul(j[0], U[1]), cxz = s.xz + s.xz - fx_mul(j[0], U[2]);
+    const i64 cyz = s.yz + s.yz - fx_mul(j[1], U[2]);
+    // relaxation: Ts = T + omega_b (rho - T); halved deviatoric parts
+    i64 Ts = rho;
+    if (w.b != 0) {
+        const i64 d = fx_mul(rho - (cxx + cyy + czz), w.b);
+        Ts += d + d;
+    }
+    const i64 D1h = fx_mul(cxx - cyy, w.a), D2h = fx_mul(cxx - czz, w.a);
+    const i64 sxx = fx_mul(Ts, kFx6) + fx_mul(D1h + D2h, kFx3);
+    const i64 wq = w.a >> 1;
+    const i64 e4 = fx_mul(rho, kFx36);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int q = 0; q < 27; q++) m[q] = 0;
+    m[0] = rho;
+    m[1] = hx;
+    m[3] = hy;
+    m[9] = hz;
+    m[2] = sxx;
+    m[6] = sxx - D1h;
+    m[18] = sxx - D2h;
+    m[4] = fx_mul(cxy, wq);
+    m[10] = fx_mul(cxz, wq);
+    m[12] = fx_mul(cyz, wq);
+    m[8] = m[20] = m[24] = e4;
+    m[26] = fx_mul(rho, kFx216);
+    const i64 ux = U[0], uy = U[1], uz = U[2], uhx = ux >> 1, uhy = uy >> 1, uhz = uz >> 1;
+    // along x: (b, c) = (0,0) (1,0) (2,0) (0,1) (1,1) (0,2) (2,2); the other lines are 0
+    fx_shift_first(m[1], m[2], ux);
+    fx_shift_k1(m[4], m[5], ux);
+    fx_shift_k02(m[6], m[7], m[8], ux, uhx);
+    fx_shift_k1(m[10], m[11], ux);
+    fx_shift_k0(m[12], m[13], m[14], ux, uhx);
+    fx_shift_k02(m[18], m[19], m[20], ux, uhx);
+    fx_shift_k02(m[24], m[25], m[26], ux, uhx);
+    // along y, lines (a, c)
+    fx_shift_first(m[3], m[6], uy);
+    fx_shift(m[1], m[4], m[7], uy, uhy);
+    fx_shift(m[2], m[5], m[8], uy, uhy);
+    fx_shift_k1(m[12], m[15], uy);
+    fx_shift_k01(m[10], m[13], m[16], uy, uhy);
+    fx_shift_k01(m[11], m[14], m[17], uy, uhy);
+    fx_shift_k02(m[18], m[21], m[24], uy, uhy);
+    fx_shift_k02(m[19], m[22], m[25], uy, uhy);
+    fx_shift_k02(m[20], m[23], m[26], uy, uhy);
+    // along z, lines (a, b)
+    fx_shift_first(m[9], m[18], uz);
+    fx_shift(m[1], m[10], m[19], uz, uhz);
+    fx_shift(m[2], m[11], m[20], uz, uhz);
+    fx_shift(m[3], m[12], m[21], uz, uhz);
+    fx_shift(m[4], m[13], m[22], uz, uhz);
+    fx_shift(m[5], m[14], m[23], uz, uhz);
+    fx_shift(m[6], m[15], m[24], uz, uhz);
+    fx_shift(m[7], m[16], m[25], uz, uhz);
+    fx_shift(m[8], m[17], m[26], uz, uhz);
+    // post-collision force: m_100 gains F_post / 2, m_120 and m_102 (F_pre +
+    // F_post) / 3, m_122 (F_pre + F_post) 2 / 9; halved per nonzero order
+    m[1] = s.jx + F[0].h2;
+    {
+        const i64 g3 = fx_mul(F[0].h2, kFx3), g9 = fx_mul(F[0].h2, kFx9);
+        m[7] += g3;
+        m[19] += g3;
+        m[25] += g9;
+    }
+    if (!XO) {
+        m[3] = s.jy + F[1].h2;
+        m[9] = s.jz + F[2].h2;
+        const i64 g3 = fx_mul(F[1].h2, kFx3), g9 = fx_mul(F[1].h2, kFx9);
+        m[5] += g3;
+        m[21] += g3;
+        m[23] += g9;
+        const i64 h3 = fx_mul(F[2].h2, kFx3), h9 = fx_mul(F[2].h2, kFx9);
+        m[11] += h3;
+        m[15] += h3;
+        m[17] += h9;
+    }
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int t = 0; t < 9; t++) fx_back(m[t], m[t + 9], m[t + 18]);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int t = 0; t < 9; t++) fx_back(m[t % 3 + 9 * (t / 3)], m[t % 3 + 9 * (t / 3) + 3], m[t % 3 + 9 * (t / 3) + 6]);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int t = 0; t < 9; t++) fx_back(m[3 * t], m[3 * t + 1], m[3 * t + 2]);
+}
+
+// ---- D2Q9 ---------------------------------------------------------------------
+template <class V>
+struct FxSums9 {
+    V rho, jx, jy, xx, yy, xy;
+};
+template <class V>
+FX_HD void fx_sums9(const V (&f)[9], FxSums9<V> &s)
+{
+    const V s0 = f[1] + f[3], d0 = f[1] - f[3];  // row ey = 0
+    const V s1 = f[5] + f[6], d1 = f[5] - f[6];  // row ey = +1
+    const V s2 = f[8] + f[7], d2 = f[8] - f[7];  // row ey = -1
+    const V B0 = f[2] + s1, C0 = f[4] + s2;
+    s.yy = B0 + C0;
+    s.rho = f[0] + s0 + s.yy;
+    s.jx = d0 + d1 + d2;
+    s.jy = B0 - C0;
+    s.xx = s0 + s1 + s2;
+    s.xy = d1 - d2;
+}
+
+// The D2Q9 collision with omega_6 .. omega_8 = 1 (see k_d2q9.cu collide_w1).
+template <bool XO>
+FX_HD void fx_collide9(const FxSums9<i64> &s, const FxForce (&F)[2], const FxRates &w, i64 (&f)[9], int &bad)
+{
+    const i64 hx = s.jx + F[0].h1, hy = XO ? s.jy : s.jy + F[1].h1;
+    const i64 rho = s.rho + s.rho;
+    const i64 j[3] = {hx + hx, hy + hy, 0};
+    i64 U[3];
+    fx_velocity<2>(rho, j, U, bad);
+    const i64 ux = U[0], uy = U[1], uhx = ux >> 1, uhy = uy >> 1;
+    const i64 cxx = s.xx + s.xx - fx_mul(j[0], ux), cyy = s.yy + s.yy - fx_mul(j[1], uy);
+    const i64 cxy = s.xy + s.xy - fx_mul(j[0], uy);
+    // (T + omega_3 (2 rho / 3 - T)) / 4, (1 - omega_4) D / 4, (1 - omega_5) c_xy / 4
+    const i64 r6 = fx_mul(rho, kFx6);
+    i64 Tq = r6;
+    if (w.c != 0) Tq += fx_mul(4 * r6 - (cxx + cyy), w.c);
+    const i64 Dq = fx_mul(cxx - cyy, w.a);
+    i64 m20 = Tq + Dq, m02 = Tq - Dq, m11 = fx_mul(cxy, w.b);
+    i64 m22 = fx_mul(rho, kFx36), m21, m12;
+    // back-shift along x, then along y (halved moments)
+    fx_shift_first(hx, m20, ux);
+    fx_shift_k1(m11, m21, ux);
+    fx_shift_k02(m02, m12, m22, ux, uhx);
+    fx_shift_first(hy, m02, uy);
+    fx_shift(hx, m11, m12, uy, uhy);
+    fx_shift(m20, m21, m22, uy, uhy);
+    // post-collision force: m_10 gains F_post / 2, m_12 (F_pre + F_post) / 3 (halved: / 12)
+    i64 m10 = s.jx + F[0].h2, m01 = hy;
+    m12 += fx_mul(F[0].h2, kFx3);
+    if (!XO) {
+        m01 = s.jy + F[1].h2;
+        m21 += fx_mul(F[1].h2, kFx3);
+    }
+    i64 a0 = rho, b0 = m01, c0 = m02, a1 = m10, b1 = m11, c1 = m12, a2 = m20, b2 = m21, c2 = m22;
+    fx_back(a0, b0, c0);  // x-order 0; e_y = -1, 0, +1
+    fx_back(a1, b1, c1);
+    fx_back(a2, b2, c2);
+    fx_back(a0, a1, a2);  // e_y = -1: e_x = -1, 0, +1
+    fx_back(b0, b1, b2);
+    fx_back(c0, c1, c2);
+    f[0] = b1;
+    f[1] = b2;
+    f[3] = b0;
+    f[2] = c1;
+    f[5] = c2;
+    f[6] = c0;
+    f[4] = a1;
+    f[8] = a2;
+    f[7] = a0;
+}
+
+}  // namespace lbmk

@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 
 #include "lbm_device.cuh"
+#include "lbm_fixed.cuh"
 
 namespace lbmk {
 
@@ -185,86 +186,110 @@ __device__ __forceinline__ void load_pulled_dev(const Planes<T, L::Q> &P, const 
     pull_node<L>(g, x, y, z, i, d, [&](int p, int k) { return Dev<T>::get(P.in[p] + k); });
 }
 
-// Zeroth and first moments of a node's populations (summed in velocity order).
+// Zeroth and first moments of a node's populations in any arithmetic.
+template <class L, class V>
+__device__ __forceinline__ void sum_moments(const V (&f)[L::Q], V &m0, V (&j)[3])
+{
+    if constexpr (L::Q == 27) {
+        FxSums27<V> s;
+        fx_sums27(f, s);
+        m0 = s.rho;
+        j[0] = s.jx;
+        j[1] = s.jy;
+        j[2] = s.jz;
+    } else if constexpr (L::Q == 9) {
+        FxSums9<V> s;
+        fx_sums9(f, s);
+        m0 = s.rho;
+        j[0] = s.jx;
+        j[1] = s.jy;
+        j[2] = V(0);
+    } else {
+        m0 = f[0];
+        j[0] = j[1] = j[2] = V(0);
+#pragma unroll
+        for (int a = 1; a < L::Q; a++) {
+            m0 += f[a];
+            if (L::ex(a) == 1) j[0] += f[a];
+            if (L::ex(a) == -1) j[0] -= f[a];
+            if (L::ey(a) == 1) j[1] += f[a];
+            if (L::ey(a) == -1) j[1] -= f[a];
+            if (L::ez(a) == 1) j[2] += f[a];
+            if (L::ez(a) == -1) j[2] -= f[a];
+        }
+    }
+}
+
+// Zeroth and first moments of a node as every FP64 readback and reduction
+// forms them: summed in fixed point (lbm_fixed.cuh), where the sums are exact,
+// and rounded once; a node outside the fixed-point range is summed in FP64.  The
+// FP64 sums of D3Q27 took 40 clocks of an SM's FP64 unit per node, the 27 + 4
+// conversions take 15.5.  D2Q5's four FP64 adds cost less than six conversions
+// and stay.
 template <class L>
 __device__ __forceinline__ void zeroth_first(const double (&f)[L::Q], double &m0, double (&j)[3])
 {
-    m0 = f[0];
-    j[0] = j[1] = j[2] = 0.0;
+    const int em = fx_emax(f);
+    if (L::Q != 5 && fx_in_range(em)) {
+        const int k = FxGrid<L::Q>::S + 1023 - em;
+        i64 X[L::Q], M, J[3];
+        fx_load(f, k, X);
+        sum_moments<L>(X, M, J);
+        m0 = fx_value(M, k);
 #pragma unroll
-    for (int a = 0; a < L::Q; a++) {
-        if (a > 0) m0 += f[a];
-        if (L::ex(a) == 1) j[0] += f[a];
-        if (L::ex(a) == -1) j[0] -= f[a];
-        if (L::ey(a) == 1) j[1] += f[a];
-        if (L::ey(a) == -1) j[1] -= f[a];
-        if (L::ez(a) == 1) j[2] += f[a];
-        if (L::ez(a) == -1) j[2] -= f[a];
+        for (int d = 0; d < 3; d++) j[d] = d < L::DIM ? fx_value(J[d], k) : 0.0;
+        return;
     }
+    sum_moments<L>(f, m0, j);
 }
 
-// D2Q9: the same sums grouped as the collision groups them (x-moments of the
-// rows e_y = 0, +1, -1 first), so that a step kernel's own rho and j are
-// these bits and a fused readback can store them without summing again.
-template <>
-__device__ __forceinline__ void zeroth_first<LD2Q9>(const double (&f)[9], double &m0, double (&j)[3])
-{
-    const double s0 = f[1] + f[3], s1 = f[5] + f[6], s2 = f[8] + f[7];
-    const double B0 = f[2] + s1, C0 = f[4] + s2;
-    m0 = (f[0] + s0) + (B0 + C0);
-    j[0] = (f[1] - f[3]) + ((f[5] - f[6]) + (f[8] - f[7]));
-    j[1] = B0 - C0;
-    j[2] = 0.0;
-}
-
-// D3Q27: grouped as the factorised collision forms them — the 1D transform
-// (f_+ + f_-) + f_0 and f_+ - f_- along x on every line, then along y, then
-// along z — so that the collision's own rho and j are these bits.
-template <>
-__device__ __forceinline__ void zeroth_first<LD3Q27>(const double (&f)[27], double &m0, double (&j)[3])
-{
-    double Y0[3], Y1[3], XY[3];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        double X0[3], X1[3];
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            const int k = 3 * b + 9 * c;  // velocities (-1, 0, +1) along x at k, k + 1, k + 2
-            X0[b] = (f[k + 2] + f[k]) + f[k + 1];
-            X1[b] = f[k + 2] - f[k];
-        }
-        Y0[c] = (X0[2] + X0[0]) + X0[1];
-        Y1[c] = X0[2] - X0[0];
-        XY[c] = (X1[2] + X1[0]) + X1[1];
-    }
-    m0 = (Y0[2] + Y0[0]) + Y0[1];
-    j[0] = (XY[2] + XY[0]) + XY[1];
-    j[1] = (Y1[2] + Y1[0]) + Y1[1];
-    j[2] = Y0[2] - Y0[0];
-}
-
-// Stores the packed fields of a node: rho (phi for the scalar lattice) at
-// rho[off + i] and u_d = jd_d (1/rho) at u[dim * off + d * N + i], with rinv =
-// the correctly rounded 1/rho (__drcp_rn) and the product rounded on its own.
+// The same sums of FP32 deviations: every value becomes a 24-bit integer
+// shifted to the node's scale (32 bits below the largest deviation's last),
+// without an FP64 conversion per value: converting to FP64 and adding there
+// took 53 clocks of the FP64 unit per D3Q27 node, this takes about 8 of the
+// integer units (moments of a 384^3 FP32 lattice: 9.5 -> 2.0 ms, the memory's
+// time 1.2).
 template <class L>
-__device__ __forceinline__ void put_fields(double m0, const double (&jd)[3], double rinv, int i, int N, long long off,
-                                           double *rho, double *u)
+__device__ __forceinline__ void zeroth_first(const float (&d)[L::Q], double &m0, double (&j)[3])
 {
-    rho[off + i] = m0;
-    if (L::Q == 5) return;
+    unsigned m = 0;
 #pragma unroll
-    for (int d = 0; d < L::DIM; d++) u[L::DIM * off + (long long)d * N + i] = __dmul_rn(jd[d], rinv);
+    for (int a = 0; a < L::Q; a++) m = max(m, __float_as_uint(d[a]) & 0x7fffffffu);
+    const int em = (int)(m >> 23);
+    if (m == 0) {  // a node at the reference state
+        m0 = j[0] = j[1] = j[2] = 0.0;
+        return;
+    }
+    if (em >= 40 && em < 255) {
+        i64 X[L::Q], M, J[3];
+#pragma unroll
+        for (int a = 0; a < L::Q; a++) {
+            const unsigned b = __float_as_uint(d[a]);
+            const int e = (int)((b >> 23) & 0xffu);
+            // a zero or subnormal value lies more than 2^39 below the largest: nothing is left of it
+            const u64 v = (u64)((b & 0x7fffffu) | 0x800000u) << 32 >> min(em - e, 63);
+            const i64 s = (i64)((int)b >> 31);
+            X[a] = ((i64)v ^ s) - s;
+        }
+        sum_moments<L>(X, M, J);
+        const int k = 23 + 32 + 127 - em;  // X = d 2^k
+        m0 = fx_value(M, k);
+#pragma unroll
+        for (int q = 0; q < 3; q++) j[q] = q < L::DIM ? fx_value(J[q], k) : 0.0;
+        return;
+    }
+    double dd[L::Q];
+#pragma unroll
+    for (int a = 0; a < L::Q; a++) dd[a] = (double)d[a];
+    sum_moments<L>(dd, m0, j);
 }
 
 // The packed fields of a node from its zeroth and first moments, as every
 // readback writes them: rho (phi for the scalar lattice) at rho[off + i],
-// velocity component d at u[dim * off + d * N + i]; with `forced` the
-// pre-collision half force / source a_pre P / 2 is included (Eq. 25 / 43).
-// Rounded operation by operation (no contraction), so that every kernel that
-// forms them gives the same bits.  A step kernel that has rho, the half-forced
-// j and 1/rho at hand stores them with put_fields instead: j + (a_pre P)/2
-// rounded once equals fma(0.5, a_pre P, j), and phi + (a_pre/2) P equals
-// phi + (a_pre P)/2 (halving is exact for products in the normal range).
+// velocity component d at u[dim * off + d * N + i] = j_d (1/rho), with 1/rho
+// correctly rounded; with `forced` the pre-collision half force / source
+// a_pre P / 2 is included (Eq. 25 / 43).  Rounded operation by operation (no
+// contraction), so that every kernel that forms them gives the same bits.
 template <class L>
 __device__ __forceinline__ void store_fields(double m0, const double (&j)[3], bool forced, double apre, const FieldDev &F,
                                              int fkind, int x, int y, int z, int i, int N, long long off, double *rho,
@@ -274,11 +299,14 @@ __device__ __forceinline__ void store_fields(double m0, const double (&j)[3], bo
         rho[off + i] = forced ? __dadd_rn(m0, __dmul_rn(0.5, __dmul_rn(apre, field_value(F, fkind, 0, x, y, z, i)))) : m0;
         return;
     }
-    double jd[3] = {0.0, 0.0, 0.0};
+    rho[off + i] = m0;
+    const double rinv = __drcp_rn(m0);
 #pragma unroll
-    for (int d = 0; d < L::DIM; d++)
-        jd[d] = forced ? __dadd_rn(j[d], __dmul_rn(0.5, __dmul_rn(apre, field_value(F, fkind, d, x, y, z, i)))) : j[d];
-    put_fields<L>(m0, jd, __drcp_rn(m0), i, N, off, rho, u);
+    for (int d = 0; d < L::DIM; d++) {
+        const double jd =
+            forced ? __dadd_rn(j[d], __dmul_rn(0.5, __dmul_rn(apre, field_value(F, fkind, d, x, y, z, i)))) : j[d];
+        u[L::DIM * off + (long long)d * N + i] = __dmul_rn(jd, rinv);
+    }
 }
 
 // Copy an object into shared memory cooperatively (word by word); the caller
