@@ -311,10 +311,57 @@ __device__ __forceinline__ void collide_w1(double (&m)[27], const double (&F)[3]
     finish<kZeroW1, XO>(m, ux, uy, uz, F, Fq);
 }
 
+// One node's step in fixed point (unit higher rates): get() pulls the
+// populations, shape(d) gives the force shape's component d, q1 = a_pre / 4 and
+// q2 = (a_pre + a_post) / 4, put(a, f) stores a result.  Returns false for a
+// node that needs the FP64 form (what it has stored is then overwritten).
+template <bool FORCED, bool XO, class Shape, class Put>
+__device__ __forceinline__ bool fixed_step27(const double (&f)[27], const FxRates &w, double q1, double q2, Shape shape,
+                                             Put put)
+{
+    const int em = fx_emax(f);
+    const int k = FxGrid<27>::S + 1023 - em;
+    int bad = fx_in_range(em) ? 0 : -1;
+    FxForce F[3] = {{0, 0}, {0, 0}, {0, 0}};
+    if (FORCED) {
+        const unsigned dither = (unsigned)fx_bits(f[13]);
+#pragma unroll
+        for (int d = 0; d < (XO ? 1 : 3); d++)
+            if (!fx_force(shape(d), q1, q2, k, em, dither >> (8 * d), F[d])) bad = -1;
+    }
+    i64 X[27];
+    fx_load(f, k, X);
+    FxSums27<i64> s;
+    fx_sums27(X, s);
+    fx_collide27<XO>(s, F, w, X, bad);
+#pragma unroll
+    for (int a = 0; a < 27; a++) put(a, fx_value_pos(X[a], k + 1, bad));
+    return bad >= 0;
+}
+
+// The FP64 form of a node's step.
+template <bool W1, bool XO, class Shape>
+__device__ __forceinline__ void double_step27(double (&m)[27], const Rates27 &w, bool forced, double apre, double apost,
+                                              Shape shape)
+{
+    double F[3] = {0.0, 0.0, 0.0}, Fq[3] = {0.0, 0.0, 0.0};
+    if (forced) {
+#pragma unroll
+        for (int d = 0; d < (XO ? 1 : 3); d++) {
+            const double P = shape(d);
+            F[d] = apre * P;
+            Fq[d] = apost * P;
+        }
+    }
+    if (W1) collide_w1<XO>(m, F, Fq, w);
+    else collide<XO>(m, F, Fq, w);
+}
+
 // XO: the force has no y and z components (checked on the host).
 template <int FK, bool W1, bool XO>
 __global__ void __launch_bounds__(kBlock)
-k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double apre, double apost, Rates27 w)
+k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double apre, double apost, Rates27 w,
+       FxRates fx)
 {
     int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
@@ -322,17 +369,14 @@ k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double
     node_xyz(g, i, x, y, z);
     double m[27];
     load_pulled<LD3Q27>(P, g, x, y, z, i, m);
-    double F[3] = {0.0, 0.0, 0.0}, Fq[3] = {0.0, 0.0, 0.0};
-    if (FK != FK_NONE) {
-#pragma unroll
-        for (int d = 0; d < (XO ? 1 : 3); d++) {
-            const double P = field_value(Fd, FK, d, x, y, z, i);
-            F[d] = apre * P;
-            Fq[d] = apost * P;
-        }
+    auto shape = [&](int d) { return field_value(Fd, FK, d, x, y, z, i); };
+    if (W1) {
+        if (fixed_step27<FK != FK_NONE, XO>(m, fx, 0.25 * apre, 0.25 * (apre + apost), shape,
+                                            [&](int a, double v) { P.out[a][i] = v; }))
+            return;
+        load_pulled<LD3Q27>(P, g, x, y, z, i, m);
     }
-    if (W1) collide_w1<XO>(m, F, Fq, w);
-    else collide<XO>(m, F, Fq, w);
+    double_step27<W1, XO>(m, w, FK != FK_NONE, apre, apost, shape);
 #pragma unroll
     for (int a = 0; a < 27; a++) P.out[a][i] = m[a];
 }
@@ -350,22 +394,25 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     node_xyz(g, i, x, y, z);
     double m[27];
     load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
-    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, ap.x);  // fused readback of f(t)'s fields
-    double F[3] = {0.0, 0.0, 0.0}, Fq[3] = {0.0, 0.0, 0.0};
-    if (B.fkind != FK_NONE) {
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            const double P = field_value(B.F, B.fkind, d, x, y, z, i);
-            F[d] = ap.x * P;
-            Fq[d] = ap.y * P;
-        }
-    }
+    // fused readback of f(t)'s fields
+    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, ap.x);
+    const bool forced = B.fkind != FK_NONE;
+    auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
+    auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates27 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
-    if (B.variant == 3) collide_w1<true>(m, F, Fq, w);  // uniform over the member
-    else if (B.variant == 1) collide_w1<false>(m, F, Fq, w);
-    else collide(m, F, Fq, w);
+    if (B.variant == 3) {  // uniform over the member
+        if (fixed_step27<true, true>(m, B.fx, 0.25 * ap.x, 0.25 * (ap.x + ap.y), shape, put)) return;
+        load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
+        double_step27<true, true>(m, w, forced, ap.x, ap.y, shape);
+    } else if (B.variant == 1) {
+        if (fixed_step27<true, false>(m, B.fx, 0.25 * ap.x, 0.25 * (ap.x + ap.y), shape, put)) return;
+        load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
+        double_step27<true, false>(m, w, forced, ap.x, ap.y, shape);
+    } else {
+        double_step27<false, false>(m, w, forced, ap.x, ap.y, shape);
+    }
 #pragma unroll
-    for (int a = 0; a < 27; a++) fout[a * g.Np + i] = m[a];
+    for (int a = 0; a < 27; a++) put(a, m[a]);
 }
 
 template <int TB, int MODE>
@@ -382,6 +429,7 @@ bool high_rates_one(const double *om) { return om[3] == 1.0 && om[4] == 1.0 && o
 void d3q27_batch_coef(const double omega[9], BatchItem &item)
 {
     for (int k = 0; k < 6; k++) item.coef[k] = omega[k + 1];
+    item.fx = fx_rates27(omega[1], omega[2]);
 }
 
 cudaError_t d3q27_batch_step(const BatchLaunch &L, int nblocks, int tile, cudaStream_t s)
@@ -403,20 +451,21 @@ cudaError_t d3q27_step(const LaunchArgs &a)
     const bool w1 = high_rates_one(a.omega);
     const Planes<double, 27> P = make_planes<double, 27>(a.fin, a.fout, a.g.Np);
     const bool xo = force_x_only(a.fkind, a.F, 3);
+    const FxRates fx = fx_rates27(a.omega[1], a.omega[2]);
     switch (a.fkind) {
     case FK_NONE:
-        if (w1) k_step<FK_NONE, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
-        else k_step<FK_NONE, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
+        if (w1) k_step<FK_NONE, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        else k_step<FK_NONE, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
         break;
     case FK_CONST:
-        if (w1 && xo) k_step<FK_CONST, true, true><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
-        else if (w1) k_step<FK_CONST, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
-        else k_step<FK_CONST, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
+        if (w1 && xo) k_step<FK_CONST, true, true><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        else if (w1) k_step<FK_CONST, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        else k_step<FK_CONST, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
         break;
     default:
-        if (w1 && xo) k_step<FK_GENERAL, true, true><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
-        else if (w1) k_step<FK_GENERAL, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
-        else k_step<FK_GENERAL, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w);
+        if (w1 && xo) k_step<FK_GENERAL, true, true><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        else if (w1) k_step<FK_GENERAL, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        else k_step<FK_GENERAL, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
         break;
     }
     return cudaGetLastError();

@@ -187,6 +187,13 @@ FX_HD double fx_value_pos(i64 X, int k, int &bad)
     return fx_double(v + ((u64)(unsigned)(1023 + 51 + 10 - k - (int)n) << 52));
 }
 
+// The same for values of either sign, 2^32 <= |X| < 2^62.
+FX_HD double fx_value_signed(i64 X, int k, int &bad)
+{
+    const i64 s = X >> 63;
+    return fx_double(fx_bits(fx_value_pos((X ^ s) - s, k, bad)) | ((u64)X & 0x8000000000000000ull));
+}
+
 // ---- force --------------------------------------------------------------------
 // Fixed-point form of a force along one axis at a node, on the refined grid
 // (scale 2^(k + 1)): h1 = F_pre / 4 (half of the pre-collision half force),
@@ -196,46 +203,44 @@ FX_HD double fx_value_pos(i64 X, int k, int &bad)
 struct FxForce {
     i64 h1, h2;
 };
-// q1 = a_pre / 4, q2 = (a_pre + a_post) / 4, P the shape's value.
+// q1 = a_pre / 4, q2 = (a_pre + a_post) / 4, P the shape's value.  With q2 = 2
+// q1 (an envelope that does not change over the step) one product and one
+// conversion do.
 FX_HD bool fx_force(double P, double q1, double q2, int k, int emax, unsigned dither, FxForce &F)
 {
-    const double f1 = q1 * P, f2 = q2 * P;
-    const unsigned m1 = fx_hi(fx_bits(f1)) & 0x7fffffffu, m2 = fx_hi(fx_bits(f2)) & 0x7fffffffu;
-    F.h1 = fx_round(fx_ldexp(f1, k + 1));
+    const double f2 = q2 * P;
+    unsigned m = fx_hi(fx_bits(f2)) & 0x7fffffffu;
     F.h2 = (fx_round(fx_ldexp(f2, k + 9)) + (i64)(dither & 0xffu)) >> 8;
-    return (int)((m1 > m2 ? m1 : m2) >> 20) <= emax - 6;
+    if (q2 == q1 + q1) {
+        F.h1 = F.h2 >> 1;
+    } else {
+        const double f1 = q1 * P;
+        const unsigned m1 = fx_hi(fx_bits(f1)) & 0x7fffffffu;
+        m = m1 > m ? m1 : m;
+        F.h1 = fx_round(fx_ldexp(f1, k + 1));
+    }
+    return (int)(m >> 20) <= emax - 6;
 }
 
 // ---- velocity -----------------------------------------------------------------
-// U = j / rho 2^64 for |j| < rho / 2 (refined grid or not: j and rho alike), to
-// a relative 2^-52.  bad < 0 when some |j| is not below rho / 2 or rho is not
-// above 2^52.
-template <int D>
-FX_HD void fx_velocity(i64 rho, const i64 (&j)[3], i64 (&U)[3], int &bad)
+// 2^64 / rho to a relative 2^-52; bad < 0 when rho is not above 2^52.
+FX_HD double fx_reciprocal(i64 rho, int &bad)
 {
     const int rh = (int)(rho >> 32);
     bad |= rh - (1 << 20);
     const double r = fx_ldexp(fx_to_double(rho), -32);
     const double x = (double)fx_rcp_approx((float)rh);
     // x (1 + e + e^2) with e = 1 - r x, |e| < 2^-19
-#ifdef __CUDA_ARCH__
     const double e = fma(-r, x, 1.0);
     const double p = fma(e, e, e);
-    const double ri = fx_ldexp(fma(x, p, x), 32);
-#else
-    const double e = ::fma(-r, x, 1.0);
-    const double p = ::fma(e, e, e);
-    const double ri = fx_ldexp(::fma(x, p, x), 32);
-#endif
-    const i64 half = (i64)((u64)rho >> 1);
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-    for (int d = 0; d < D; d++) {
-        // half - |j| > 0 (the shift above is exact up to one unit)
-        bad |= (int)(((half - 1) - (j[d] < 0 ? -j[d] : j[d])) >> 32);
-        U[d] = fx_round(fx_to_double(j[d]) * ri);
-    }
+    return fx_ldexp(fma(x, p, x), 32);
+}
+// j / rho 2^64 for |j| < rho / 2, ri = 2^64 / rho; bad < 0 for a larger |j|.
+FX_HD i64 fx_ratio(i64 j, i64 rho, double ri, int &bad)
+{
+    // rho / 2 - 1 - |j| >= 0 (the shift is exact up to one unit)
+    bad |= (int)((((rho >> 1) - 1) - (j < 0 ? -j : j)) >> 32);
+    return fx_round(fx_to_double(j) * ri);
 }
 
 // Constants as fractions of 2^64.
@@ -354,8 +359,8 @@ FX_HD void fx_collide27(const FxSums27<i64> &s, const FxForce (&F)[3], const FxR
     const i64 hx = s.jx + F[0].h1, hy = XO ? s.jy : s.jy + F[1].h1, hz = XO ? s.jz : s.jz + F[2].h1;
     const i64 rho = s.rho + s.rho;
     const i64 j[3] = {hx + hx, hy + hy, hz + hz};
-    i64 U[3];
-    fx_velocity<3>(rho, j, U, bad);
+    const double ri = fx_reciprocal(rho, bad);
+    const i64 U[3] = {fx_ratio(j[0], rho, ri, bad), fx_ratio(j[1], rho, ri, bad), fx_ratio(j[2], rho, ri, bad)};
     const i64 cxx = s.xx + s.xx - fx_mul(j[0], U[0]), cyy = s.yy + s.yy - fx_mul(j[1], U[1]);
     const i64 czz = s.zz + s.zz - fx_mul(j[2], U[2]);
     const i64 cxy = s.xy + s.xy - fx_mul(j[0], U[1]), cxz = s.xz + s.xz - fx_mul(j[0], U[2]);
@@ -476,10 +481,9 @@ FX_HD void fx_collide9(const FxSums9<i64> &s, const FxForce (&F)[2], const FxRat
 {
     const i64 hx = s.jx + F[0].h1, hy = XO ? s.jy : s.jy + F[1].h1;
     const i64 rho = s.rho + s.rho;
-    const i64 j[3] = {hx + hx, hy + hy, 0};
-    i64 U[3];
-    fx_velocity<2>(rho, j, U, bad);
-    const i64 ux = U[0], uy = U[1], uhx = ux >> 1, uhy = uy >> 1;
+    const i64 j[2] = {hx + hx, hy + hy};
+    const double ri = fx_reciprocal(rho, bad);
+    const i64 ux = fx_ratio(j[0], rho, ri, bad), uy = fx_ratio(j[1], rho, ri, bad), uhx = ux >> 1, uhy = uy >> 1;
     const i64 cxx = s.xx + s.xx - fx_mul(j[0], ux), cyy = s.yy + s.yy - fx_mul(j[1], uy);
     const i64 cxy = s.xy + s.xy - fx_mul(j[0], uy);
     // (T + omega_3 (2 rho / 3 - T)) / 4, (1 - omega_4) D / 4, (1 - omega_5) c_xy / 4

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_device.cuh"
+#include "lbm_fixed.cuh"
 
 namespace lbmk {
 
@@ -86,6 +87,7 @@ struct BatchItem {
                       // D2Q5: [16] holds P3 + (2/3) S3 of the uniform-velocity form
     float frho_ref;
     int variant;      // collision variant of this member (batch_variant)
+    FxRates fx;       // its fixed-point relaxation factors (FP64 storage, unit higher rates)
     float fref[5];    // D2Q5 reduced precision, uniform velocity: M g_ref - g_ref, added after the collision
     double mat[25];   // D2Q5 with a uniform advecting velocity, FP64: step matrix M (row-major)
 };
