@@ -141,10 +141,58 @@ __device__ __forceinline__ void collide_w1(double (&f)[9], double Fx, double Fy,
     f[7] = P2m - P1m;
 }
 
+// One node's step in fixed point (unit higher rates): shape(d) gives the force
+// shape's component d, q1 = a_pre / 4 and q2 = (a_pre + a_post) / 4, put(a, f)
+// takes a result.  Returns false for a node that needs the FP64 form (its
+// results are then void).
+template <bool FORCED, bool XO, class Shape, class Put>
+__device__ __forceinline__ bool fixed_step9(const double (&f)[9], const FxRates &w, double q1, double q2, Shape shape,
+                                            Put put)
+{
+    const int em = fx_emax(f);
+    const int k = FxGrid<9>::S + 1023 - em;
+    int bad = fx_in_range(em) ? 0 : -1;
+    FxForce F[2] = {{0, 0}, {0, 0}};
+    if (FORCED) {
+        const unsigned dither = (unsigned)fx_bits(f[0]);
+#pragma unroll
+        for (int d = 0; d < (XO ? 1 : 2); d++)
+            if (!fx_force(shape(d), q1, q2, k, em, dither >> (8 * d), F[d])) bad = -1;
+    }
+    i64 X[9];
+    fx_load(f, k, X);
+    FxSums9<i64> s;
+    fx_sums9(X, s);
+    fx_collide9<XO>(s, F, w, X, bad);
+#pragma unroll
+    for (int a = 0; a < 9; a++) put(a, fx_value_pos(X[a], k + 1, bad));
+    return bad >= 0;
+}
+
+// The FP64 form of a node's step; gsum = (a_pre + a_post) / 12.
+template <bool W1, bool XO, class Shape>
+__device__ __forceinline__ void double_step9(double (&f)[9], const Rates9 &w, bool forced, double apre, double gsum,
+                                             Shape shape)
+{
+    double Fx = 0.0, Fy = 0.0, Gx = 0.0, Gy = 0.0;
+    if (forced) {
+        const double Px = shape(0);
+        Fx = apre * Px;
+        Gx = gsum * Px;
+        if (!XO) {
+            const double Py = shape(1);
+            Fy = apre * Py;
+            Gy = gsum * Py;
+        }
+    }
+    if (W1) collide_w1<XO>(f, Fx, Fy, Gx, Gy, w);
+    else collide(f, Fx, Fy, Gx, Gy, w);
+}
+
 // XO (unit higher rates only): the force has no y component (checked on the host).
 template <int FK, bool W1, bool XO>
 __global__ void __launch_bounds__(kBlock)
-k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double apre, double gsum, Rates9 w)
+k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double apre, double gsum, Rates9 w, FxRates fx)
 {
     int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
@@ -152,19 +200,14 @@ k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double a
     node_xy(g, i, x, y);
     double f[9];
     load_pulled<LD2Q9>(P, g, x, y, 0, i, f);
-    double Fx = 0.0, Fy = 0.0, Gx = 0.0, Gy = 0.0;
-    if (FK != FK_NONE) {
-        const double Px = field_value(F, FK, 0, x, y, 0, i);
-        Fx = apre * Px;
-        Gx = gsum * Px;
-        if (!XO) {
-            const double Py = field_value(F, FK, 1, x, y, 0, i);
-            Fy = apre * Py;
-            Gy = gsum * Py;
-        }
+    auto shape = [&](int d) { return field_value(F, FK, d, x, y, 0, i); };
+    if (W1) {
+        if (fixed_step9<FK != FK_NONE, XO>(f, fx, 0.25 * apre, 3.0 * gsum, shape,
+                                           [&](int a, double v) { P.out[a][i] = v; }))
+            return;
+        load_pulled<LD2Q9>(P, g, x, y, 0, i, f);
     }
-    if (W1) collide_w1<XO>(f, Fx, Fy, Gx, Gy, w);
-    else collide(f, Fx, Fy, Gx, Gy, w);
+    double_step9<W1, XO>(f, w, FK != FK_NONE, apre, gsum, shape);
 #pragma unroll
     for (int a = 0; a < 9; a++) P.out[a][i] = f[a];
 }
@@ -186,7 +229,7 @@ constexpr int kClusterThreads = 384;  // >= 32-rounded 341, the largest block (4
 template <int FK, bool W1>
 __global__ void __launch_bounds__(kClusterThreads)
 k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom g, FieldDev F, double apre,
-                double gsum, Rates9 w, int P, int nsteps)
+                double gsum, Rates9 w, FxRates fx, int P, int nsteps)
 {
     extern __shared__ double sm[];  // [2][9][P]
     cg::cluster_group cl = cg::this_cluster();
@@ -198,14 +241,13 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
 #pragma unroll
         for (int a = 0; a < 9; a++) sm[a * P + l] = fin[a * g.Np + i];
     const int x = own ? i % g.nx : 0, y = own ? i / g.nx : 0;
-    double Fx = 0.0, Fy = 0.0, Gx = 0.0, Gy = 0.0;
+    double Px = 0.0, Py = 0.0;
     if (FK != FK_NONE && own) {
-        const double Px = field_value(F, FK, 0, x, y, 0, i), Py = field_value(F, FK, 1, x, y, 0, i);
-        Fx = apre * Px;
-        Fy = apre * Py;
-        Gx = gsum * Px;
-        Gy = gsum * Py;
+        Px = field_value(F, FK, 0, x, y, 0, i);
+        Py = field_value(F, FK, 1, x, y, 0, i);
     }
+    auto shape = [&](int d) { return d == 0 ? Px : Py; };
+    const double q1 = 0.25 * apre, q2 = 3.0 * gsum;
     // pull sources of this node: owner block, offset inside its buffer
     int src_blk[9], src_off[9];
     if (own) {
@@ -223,16 +265,22 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
     for (int k = 0; k < nsteps; k++) {
         if (own) {
             double f[9];
+            auto pull = [&]() {
 #pragma unroll
-            for (int a = 0; a < 9; a++) {
-                const double *base = cl.map_shared_rank(sm + cur * 9 * P, src_blk[a]);
-                f[a] = base[src_off[a]];
-            }
-            if (W1) collide_w1(f, Fx, Fy, Gx, Gy, w);
-            else collide(f, Fx, Fy, Gx, Gy, w);
+                for (int a = 0; a < 9; a++) {
+                    const double *base = cl.map_shared_rank(sm + cur * 9 * P, src_blk[a]);
+                    f[a] = base[src_off[a]];
+                }
+            };
             double *nxt = sm + (cur ^ 1) * 9 * P;
+            auto put = [&](int a, double v) { nxt[a * P + l] = v; };
+            pull();
+            if (!W1 || !fixed_step9<FK != FK_NONE, false>(f, fx, q1, q2, shape, put)) {
+                if (W1) pull();
+                double_step9<W1, false>(f, w, FK != FK_NONE, apre, gsum, shape);
 #pragma unroll
-            for (int a = 0; a < 9; a++) nxt[a * P + l] = f[a];
+                for (int a = 0; a < 9; a++) put(a, f[a]);
+            }
         }
         cur ^= 1;
         cl.sync();
@@ -257,21 +305,23 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     double f[9];
     load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
     if (L.mrho) fused_fields<LD2Q9>(B, L, it, i, x, y, 0, f, ap.x);  // fused readback of f(t)'s fields
-    double Fx = 0.0, Fy = 0.0, Gx = 0.0, Gy = 0.0;
-    const int fk = B.fkind;
-    if (fk != FK_NONE) {
-        const double Px = field_value(B.F, fk, 0, x, y, 0, i), Py = field_value(B.F, fk, 1, x, y, 0, i);
-        Fx = ap.x * Px;
-        Fy = ap.x * Py;
-        Gx = ap.y * Px;
-        Gy = ap.y * Py;
-    }
+    const bool forced = B.fkind != FK_NONE;
+    auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, 0, i) : 0.0; };
+    auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates9 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
-    if (B.variant == 3) collide_w1<true>(f, Fx, Fy, Gx, Gy, w);  // uniform over the member
-    else if (B.variant == 1) collide_w1<false>(f, Fx, Fy, Gx, Gy, w);
-    else collide(f, Fx, Fy, Gx, Gy, w);
+    if (B.variant == 3) {  // uniform over the member
+        if (fixed_step9<true, true>(f, B.fx, 0.25 * ap.x, 3.0 * ap.y, shape, put)) return;
+        load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
+        double_step9<true, true>(f, w, forced, ap.x, ap.y, shape);
+    } else if (B.variant == 1) {
+        if (fixed_step9<true, false>(f, B.fx, 0.25 * ap.x, 3.0 * ap.y, shape, put)) return;
+        load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
+        double_step9<true, false>(f, w, forced, ap.x, ap.y, shape);
+    } else {
+        double_step9<false, false>(f, w, forced, ap.x, ap.y, shape);
+    }
 #pragma unroll
-    for (int a = 0; a < 9; a++) fout[a * g.Np + i] = f[a];
+    for (int a = 0; a < 9; a++) put(a, f[a]);
 }
 
 template <int TB, int MODE>
@@ -285,20 +335,21 @@ template <bool W1>
 cudaError_t cluster_launch(cudaLaunchConfig_t &cfg, int C, const LaunchArgs &a, double gsum, const Rates9 &w, int P,
                            int nsteps)
 {
+    const FxRates fx = fx_rates9(a.omega[3], a.omega[4], a.omega[5]);
     switch (a.fkind) {
     case FK_NONE:
         if (C > 8) cudaFuncSetAttribute(k_cluster_steps<FK_NONE, W1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_NONE, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, P,
+        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_NONE, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, fx, P,
                                   nsteps);
     case FK_CONST:
         if (C > 8) cudaFuncSetAttribute(k_cluster_steps<FK_CONST, W1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_CONST, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, P,
+        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_CONST, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, fx, P,
                                   nsteps);
     default:
         if (C > 8)
             cudaFuncSetAttribute(k_cluster_steps<FK_GENERAL, W1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_GENERAL, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w,
-                                  P, nsteps);
+                                  fx, P, nsteps);
     }
 }
 
@@ -307,15 +358,16 @@ void step_launch(const LaunchArgs &a, int grid, double gsum, const Rates9 &w)
 {
     const Planes<double, 9> P = make_planes<double, 9>(a.fin, a.fout, a.g.Np);
     const bool xo = W1 && force_x_only(a.fkind, a.F, 2);
+    const FxRates fx = fx_rates9(a.omega[3], a.omega[4], a.omega[5]);
     switch (a.fkind) {
-    case FK_NONE: k_step<FK_NONE, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w); break;
+    case FK_NONE: k_step<FK_NONE, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx); break;
     case FK_CONST:
-        if (xo) k_step<FK_CONST, W1, W1><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w);
-        else k_step<FK_CONST, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w);
+        if (xo) k_step<FK_CONST, W1, W1><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
+        else k_step<FK_CONST, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
         break;
     default:
-        if (xo) k_step<FK_GENERAL, W1, W1><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w);
-        else k_step<FK_GENERAL, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w);
+        if (xo) k_step<FK_GENERAL, W1, W1><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
+        else k_step<FK_GENERAL, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
         break;
     }
 }
@@ -333,6 +385,7 @@ void d2q9_batch_coef(const double omega[9], BatchItem &item)
     const double c[6] = {omega[3] / 12.0, omega[4] / 4.0, omega[5] / 4.0,
                          omega[6] / 4.0, omega[7] / 4.0, omega[8] / 4.0};
     for (int k = 0; k < 6; k++) item.coef[k] = c[k];
+    item.fx = fx_rates9(omega[3], omega[4], omega[5]);
 }
 
 cudaError_t d2q9_batch_step(const BatchLaunch &L, int nblocks, int tile, cudaStream_t s)
