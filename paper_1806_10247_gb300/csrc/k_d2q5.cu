@@ -141,9 +141,30 @@ __device__ __forceinline__ void collide_mat(double (&g)[5], double P, double aha
     g[0] = total - ((g[1] + g[2]) + (g[3] + g[4]));
 }
 
+// One node's step at a uniform velocity in fixed point: P the source shape at
+// the node, q1 = a_pre / 2, q2 = (a_pre + a_post) / 2.  Returns false for a node
+// that needs the FP64 form.
+template <bool SRC, class Put>
+__device__ __forceinline__ bool fixed_step5(const double (&f)[5], const FxCoef5 &c, double P, double q1, double q2,
+                                            Put put)
+{
+    const int em = fx_emax(f);
+    const int k = FxGrid<5>::S + 1023 - em;
+    int bad = fx_in_range(em) ? 0 : -1;
+    FxForce S{0, 0};
+    if (SRC && !fx_force(P, q1, q2, k - 1, em, (unsigned)fx_bits(f[0]), S)) bad = -1;
+    i64 X[5];
+    fx_load(f, k, X);
+    fx_collide5(X, S.h1, S.h2, c);
+#pragma unroll
+    for (int a = 0; a < 5; a++) put(a, fx_value_signed(X[a], k, bad));
+    return bad >= 0;
+}
+
 template <int SK>
 __global__ void __launch_bounds__(kBlock)
-k_step_mat(const __grid_constant__ Planes<double, 5> P, Geom g, FieldDev S, double ahalf, double hsum, Mat5 M)
+k_step_mat(const __grid_constant__ Planes<double, 5> P, Geom g, FieldDev S, double ahalf, double hsum, Mat5 M,
+           const __grid_constant__ FxCoef5 fx)
 {
     int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
@@ -151,12 +172,15 @@ k_step_mat(const __grid_constant__ Planes<double, 5> P, Geom g, FieldDev S, doub
     node_xy(g, i, x, y);
     double f[5];
     load_pulled<LD2Q5>(P, g, x, y, 0, i, f);
-    if (SK != FK_NONE) collide_mat<true>(f, field_value(S, SK, 0, x, y, 0, i), ahalf, hsum, M.m);
-    else collide_mat<false>(f, 0.0, ahalf, hsum, M.m);
+    const double Ps = SK != FK_NONE ? field_value(S, SK, 0, x, y, 0, i) : 0.0;
+    if (fx.ok) {
+        if (fixed_step5<SK != FK_NONE>(f, fx, Ps, ahalf, 5.0 * hsum, [&](int a, double v) { P.out[a][i] = v; })) return;
+        load_pulled<LD2Q5>(P, g, x, y, 0, i, f);
+    }
+    collide_mat<SK != FK_NONE>(f, Ps, ahalf, hsum, M.m);
 #pragma unroll
     for (int a = 0; a < 5; a++) P.out[a][i] = f[a];
 }
-
 
 template <int SK, int VK>
 __global__ void __launch_bounds__(kBlock)
@@ -192,7 +216,8 @@ void launch_v(const LaunchArgs &a, int grid, double hsum, const Rates5 &w)
         const double ux = a.vkind == FK_CONST ? a.V.cval[0] : 0.0;
         const double uy = a.vkind == FK_CONST ? a.V.cval[1] : 0.0;
         k_step_mat<SK><<<grid, kBlock, 0, a.stream>>>(make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
-                                                       0.5 * a.apre, hsum, make_mat(make_coef(w, ux, uy)));
+                                                       0.5 * a.apre, hsum, make_mat(make_coef(w, ux, uy)),
+                                                       fx_coef5(w.c1, w.c2, w.c3, w.c4, ux, uy));
         return;
     }
     k_step<SK, FK_GENERAL><<<grid, kBlock, 0, a.stream>>>(make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
@@ -219,6 +244,10 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     if (B.vkind != FK_GENERAL) {
         const bool src = B.fkind != FK_NONE;
         const double P = src ? field_value(B.F, B.fkind, 0, x, y, 0, i) : 0.0;
+        if (B.fx5.ok) {
+            if (fixed_step5<true>(f, B.fx5, P, ap.x, 5.0 * ap.y, [&](int a, double v) { fout[a * g.Np + i] = v; })) return;
+            load_pulled<LD2Q5>(fin, g, x, y, 0, i, f);
+        }
         if (src) collide_mat<true>(f, P, ap.x, ap.y, B.mat);
         else collide_mat<false>(f, 0.0, 0.0, 0.0, B.mat);
     } else {
@@ -257,6 +286,7 @@ void d2q5_batch_coef(const double omega[9], BatchItem &item)
     for (int k = 0; k < 16; k++) item.coef[k] = v[k];
     const Mat5 M = make_mat(c);
     for (int k = 0; k < 25; k++) item.mat[k] = M.m[k];
+    item.fx5 = fx_coef5(w.c1, w.c2, w.c3, w.c4, ux, uy);
 }
 
 cudaError_t d2q5_batch_step(const BatchLaunch &L, int nblocks, int tile, cudaStream_t s)

@@ -525,4 +525,59 @@ FX_HD void fx_collide9(const FxSums9<i64> &s, const FxForce (&F)[2], const FxRat
     f[7] = a0;
 }
 
+// ---- D2Q5 ---------------------------------------------------------------------
+// Step coefficients of a uniform advecting velocity (k_d2q5.cu Coef5) as
+// fractions of 2^63: h1 = A1 phi - c1 kx, h2 = A2 phi - c2 ky, h3 = P3 phi + X3
+// kx + Y3 ky + S3 (kxx + kyy), h4 = P4 phi + X4 kx + Y4 ky + D4 (kxx - kyy).  ok
+// = 0 when one of them is not below 1 (advecting velocities near 1 and above).
+struct FxCoef5 {
+    i64 A1, c1, A2, c2, P3, X3, Y3, S3, P4, X4, Y4, D4;
+    int ok;
+};
+inline FxCoef5 fx_coef5(double c1, double c2, double c3, double c4, double ux, double uy)
+{
+    FxCoef5 k{};
+    k.ok = ux > -0.9 && ux < 0.9 && uy > -0.9 && uy < 0.9;  // with rates below 2 every coefficient is below 1
+    if (!k.ok) return k;
+    // products of fractions, in integers: 2^-62 instead of FP64's 2^-53
+    auto mul = [](i64 a, i64 b) { return 2 * fx_mul(a, b); };
+    const i64 C1 = fx_fraction(c1, 63), C2 = fx_fraction(c2, 63), C3 = fx_fraction(c3, 63), C4 = fx_fraction(c4, 63);
+    const i64 X = fx_fraction(ux, 63), Y = fx_fraction(uy, 63), X2 = mul(X, X), Y2 = mul(Y, Y);
+    k.A1 = mul(C1, X);
+    k.c1 = C1;
+    k.A2 = mul(C2, Y);
+    k.c2 = C2;
+    const i64 q1 = mul(C1, X2), q2 = mul(C2, Y2), r3 = mul(C3, X2) + mul(C3, Y2), r4 = mul(C4, X2) - mul(C4, Y2);
+    k.P3 = mul(C3, kFx3) - r3 + q1 + q2;  // c3 (2/3 - ux^2 - uy^2) + c1 ux^2 + c2 uy^2
+    k.X3 = 2 * mul(C3, X) - mul(C1, X);
+    k.Y3 = 2 * mul(C3, Y) - mul(C2, Y);
+    k.S3 = -C3;
+    k.P4 = q1 - q2 - r4;
+    k.X4 = 2 * mul(C4, X) - mul(C1, X);
+    k.Y4 = mul(C2, Y) - 2 * mul(C4, Y);
+    k.D4 = -C4;
+    return k;
+}
+
+constexpr i64 kFx5 = 0x3333333333333333ll;  // 1/5
+
+// The scalar step at a uniform velocity: h = S_pre / 2, t = (S_pre + S_post) / 2
+// (what the zeroth moment gains).  The rest population is what the others leave
+// of the exact total.
+FX_HD void fx_collide5(i64 (&g)[5], i64 h, i64 t, const FxCoef5 &c)
+{
+    const i64 kx = g[1] - g[3], ky = g[2] - g[4], sx = g[1] + g[3], sy = g[2] + g[4];
+    const i64 phi0 = g[0] + (sx + sy), phi = phi0 + h;
+    const i64 p2 = phi + phi, x2 = kx + kx, y2 = ky + ky, s2 = 2 * (sx + sy), d2 = 2 * (sx - sy);
+    const i64 h1 = fx_mul(p2, c.A1) - fx_mul(x2, c.c1), h2 = fx_mul(p2, c.A2) - fx_mul(y2, c.c2);
+    const i64 h3 = fx_mul(t, kFx5) + fx_mul(p2, c.P3) + fx_mul(x2, c.X3) + fx_mul(y2, c.Y3) + fx_mul(s2, c.S3);
+    const i64 h4 = fx_mul(p2, c.P4) + fx_mul(x2, c.X4) + fx_mul(y2, c.Y4) + fx_mul(d2, c.D4);
+    const i64 e1 = h3 + h4, e2 = h3 - h4;
+    g[1] += e1 + h1;
+    g[2] += e2 + h2;
+    g[3] += e1 - h1;
+    g[4] += e2 - h2;
+    g[0] = phi0 + t - ((g[1] + g[2]) + (g[3] + g[4]));
+}
+
 }  // namespace lbmk

@@ -89,6 +89,7 @@ struct BatchItem {
     int variant;      // collision variant of this member (batch_variant)
     FxRates fx;       // its fixed-point relaxation factors (FP64 storage, unit higher rates)
     float fref[5];    // D2Q5 reduced precision, uniform velocity: M g_ref - g_ref, added after the collision
+    FxCoef5 fx5;      // D2Q5 with a uniform advecting velocity, FP64: fixed-point coefficients
     double mat[25];   // D2Q5 with a uniform advecting velocity, FP64: step matrix M (row-major)
 };
 
