@@ -116,26 +116,70 @@ __device__ __forceinline__ void collide(double (&f)[15], const double (&F)[3], c
     f[14] += d0 - dx;
 }
 
-template <int FK>
-__global__ void __launch_bounds__(kBlock)
-k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double apre, double apost, Rates15 w)
+// One node's step in fixed point (omega_10 .. omega_14 = 1): shape(d) gives the
+// force shape's component d, q1 = a_pre / 4 and q2 = (a_pre + a_post) / 4, put(a,
+// f) takes a result.  Returns false for a node that needs the FP64 form.
+template <bool FORCED, bool XO, class Shape, class Put>
+__device__ __forceinline__ bool fixed_step15(const double (&f)[15], const FxRates &w, double q1, double q2, Shape shape,
+                                             Put put)
 {
-    int i = blockIdx.x * kBlock + threadIdx.x;
-    if (i >= g.N) return;
-    int x, y, z;
-    node_xyz(g, i, x, y, z);
-    double f[15];
-    load_pulled<LD3Q15>(P, g, x, y, z, i, f);
+    const int em = fx_emax(f);
+    const int k = FxGrid<15>::S + 1023 - em;
+    int bad = fx_in_range(em) ? 0 : -1;
+    FxForce F[3] = {{0, 0}, {0, 0}, {0, 0}};
+    if (FORCED) {
+        const unsigned dither = (unsigned)fx_bits(f[0]);
+#pragma unroll
+        for (int d = 0; d < (XO ? 1 : 3); d++)
+            if (!fx_force(shape(d), q1, q2, k, em, dither >> (8 * d), F[d])) bad = -1;
+    }
+    i64 X[15];
+    fx_load(f, k, X);
+    FxSums15<i64> s;
+    fx_sums15(X, s);
+    fx_collide15<XO>(s, F, w, X, bad);
+#pragma unroll
+    for (int a = 0; a < 15; a++) put(a, fx_value_pos(X[a], k + 1, bad));
+    return bad >= 0;
+}
+
+template <class Shape>
+__device__ __forceinline__ void double_step15(double (&f)[15], const Rates15 &w, bool forced, double apre, double apost,
+                                              Shape shape)
+{
     double F[3] = {0.0, 0.0, 0.0}, Fq[3] = {0.0, 0.0, 0.0};
-    if (FK != FK_NONE) {
+    if (forced) {
 #pragma unroll
         for (int d = 0; d < 3; d++) {
-            const double P = field_value(Fd, FK, d, x, y, z, i);
+            const double P = shape(d);
             F[d] = apre * P;
             Fq[d] = apost * P;
         }
     }
     collide(f, F, Fq, w);
+}
+
+// FIX: the fixed-point form (omega_10 .. omega_14 = 1).  XO: the force acts
+// along x only.  Both checked on the host.
+template <int FK, bool FIX, bool XO>
+__global__ void __launch_bounds__(kBlock)
+k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double apre, double apost, Rates15 w,
+       FxRates fx)
+{
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.N) return;
+    int x, y, z;
+    node_xyz(g, i, x, y, z);
+    double f[15];
+    load_pulled<LD3Q15>(P, g, x, y, z, i, f);
+    auto shape = [&](int d) { return field_value(Fd, FK, d, x, y, z, i); };
+    if (FIX) {
+        if (fixed_step15<FK != FK_NONE, XO>(f, fx, 0.25 * apre, 0.25 * (apre + apost), shape,
+                                            [&](int a, double v) { P.out[a][i] = v; }))
+            return;
+        load_pulled<LD3Q15>(P, g, x, y, z, i, f);
+    }
+    double_step15(f, w, FK != FK_NONE, apre, apost, shape);
 #pragma unroll
     for (int a = 0; a < 15; a++) P.out[a][i] = f[a];
 }
@@ -154,17 +198,16 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     double f[15];
     load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
     if (L.mrho) fused_fields<LD3Q15>(B, L, it, i, x, y, z, f, ap.x);  // fused readback of f(t)'s fields
-    double F[3] = {0.0, 0.0, 0.0}, Fq[3] = {0.0, 0.0, 0.0};
-    if (B.fkind != FK_NONE) {
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            const double P = field_value(B.F, B.fkind, d, x, y, z, i);
-            F[d] = ap.x * P;
-            Fq[d] = ap.y * P;
-        }
-    }
+    const bool forced = B.fkind != FK_NONE;
+    auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     const Rates15 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3]};
-    collide(f, F, Fq, w);
+    if (w.t == 1.0 && w.q == 1.0) {  // uniform over the member
+        if (fixed_step15<true, false>(f, B.fx, 0.25 * ap.x, 0.25 * (ap.x + ap.y), shape,
+                                      [&](int a, double v) { fout[a * g.Np + i] = v; }))
+            return;
+        load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
+    }
+    double_step15(f, w, forced, ap.x, ap.y, shape);
 #pragma unroll
     for (int a = 0; a < 15; a++) fout[a * g.Np + i] = f[a];
 }
@@ -184,6 +227,7 @@ void d3q15_batch_coef(const double omega[9], BatchItem &item)
     item.coef[1] = omega[1];
     item.coef[2] = omega[3];
     item.coef[3] = omega[4];
+    item.fx = fx_rates27(omega[1], omega[2]);
 }
 
 cudaError_t d3q15_batch_step(const BatchLaunch &L, int nblocks, int tile, cudaStream_t s)
@@ -199,13 +243,28 @@ int d3q15_batch_resident(int tile)
 cudaError_t d3q15_step(const LaunchArgs &a)
 {
     const Rates15 w{a.omega[2], a.omega[1], a.omega[3], a.omega[4]};
-    const int grid = (a.g.N + kBlock - 1) / kBlock;
+    const FxRates fx = fx_rates27(a.omega[1], a.omega[2]);
     const Planes<double, 15> P = make_planes<double, 15>(a.fin, a.fout, a.g.Np);
+    const bool fix = w.t == 1.0 && w.q == 1.0, xo = force_x_only(a.fkind, a.F, 3);
+    const int block = spread_block(a.g.N, kBlock), grid = (a.g.N + block - 1) / block;
+#define STEP15(FK, FIX, XO) k_step<FK, FIX, XO><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx)
     switch (a.fkind) {
-    case FK_NONE: k_step<FK_NONE><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w); break;
-    case FK_CONST: k_step<FK_CONST><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w); break;
-    default: k_step<FK_GENERAL><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w); break;
+    case FK_NONE:
+        if (fix) STEP15(FK_NONE, true, false);
+        else STEP15(FK_NONE, false, false);
+        break;
+    case FK_CONST:
+        if (fix && xo) STEP15(FK_CONST, true, true);
+        else if (fix) STEP15(FK_CONST, true, false);
+        else STEP15(FK_CONST, false, false);
+        break;
+    default:
+        if (fix && xo) STEP15(FK_GENERAL, true, true);
+        else if (fix) STEP15(FK_GENERAL, true, false);
+        else STEP15(FK_GENERAL, false, false);
+        break;
     }
+#undef STEP15
     return cudaGetLastError();
 }
 

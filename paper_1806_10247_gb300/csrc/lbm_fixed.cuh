@@ -580,4 +580,114 @@ FX_HD void fx_collide5(i64 (&g)[5], i64 h, i64 t, const FxCoef5 &c)
     g[0] = phi0 + t - ((g[1] + g[2]) + (g[3] + g[4]));
 }
 
+// ---- D3Q15 --------------------------------------------------------------------
+// Axis pairs and the corner sign transform of a node's populations (k_d3q15.cu).
+template <class V>
+struct FxSums15 {
+    V rho, jx, jy, jz, xx, yy, zz, xy, xz, yz;
+};
+template <class V>
+FX_HD void fx_sums15(const V (&f)[15], FxSums15<V> &s)
+{
+    const V A1 = f[7] + f[8], B1 = f[7] - f[8];      // y+, z+
+    const V A2 = f[9] + f[10], B2 = f[9] - f[10];    // y-, z+
+    const V A3 = f[11] + f[12], B3 = f[11] - f[12];  // y+, z-
+    const V A4 = f[13] + f[14], B4 = f[13] - f[14];  // y-, z-
+    const V P1 = A1 + A2, Q1 = A1 - A2, P2 = A3 + A4, Q2 = A3 - A4;
+    const V R1 = B1 + B2, T1 = B1 - B2, R2 = B3 + B4, T2 = B3 - B4;
+    const V S = P1 + P2, axs = f[1] + f[2], ays = f[3] + f[4], azs = f[5] + f[6];
+    s.xx = axs + S;
+    s.yy = ays + S;
+    s.zz = azs + S;
+    s.rho = f[0] + axs + ays + s.zz;
+    s.jx = f[1] - f[2] + (R1 + R2);
+    s.jy = f[3] - f[4] + (Q1 + Q2);
+    s.jz = f[5] - f[6] + (P1 - P2);
+    s.xy = T1 + T2;
+    s.xz = R1 - R2;
+    s.yz = Q1 - Q2;
+}
+
+// The D3Q15 collision with omega_10 .. omega_14 = 1 (w.a, w.b as on D3Q27): the
+// relaxed second-order central moments, third-order ones 0 and the fourth-order
+// one kappa_xx kappa_yy / rho give the raw moments of the fifteen monomials,
+//   m_xyy = ux m_yy + 2 uy k_xy, m_xxy = uy m_xx + 2 ux k_xy, m_xxz = uz m_xx + 2 ux k_xz,
+//   m_xyz = ux m_yz + uy k_xz + uz k_xy, m_xxyy = k_xxyy + ux m_xyy + uy (uy k_xx + 2 ux k_xy),
+// and those the populations: the corners by the sign transform (/ 8), the axis
+// pairs from what the corners leave of the second and first moments, the rest
+// population from what all of them leave of rho, so that mass and momentum are
+// carried exactly.  f: populations on the grid k + 1.
+template <bool XO>
+FX_HD void fx_collide15(const FxSums15<i64> &s, const FxForce (&F)[3], const FxRates &w, i64 (&f)[15], int &bad)
+{
+    const i64 hx = s.jx + F[0].h1, hy = XO ? s.jy : s.jy + F[1].h1, hz = XO ? s.jz : s.jz + F[2].h1;
+    const i64 rho = s.rho + s.rho;
+    const i64 j[3] = {hx + hx, hy + hy, hz + hz};
+    const double ri = fx_reciprocal(rho, bad);
+    const i64 ux = fx_ratio(j[0], rho, ri, bad), uy = fx_ratio(j[1], rho, ri, bad), uz = fx_ratio(j[2], rho, ri, bad);
+    const i64 pxx = fx_mul(j[0], ux), pyy = fx_mul(j[1], uy), pzz = fx_mul(j[2], uz);
+    const i64 pxy = fx_mul(j[0], uy), pxz = fx_mul(j[0], uz), pyz = fx_mul(j[1], uz);
+    const i64 cxx = s.xx + s.xx - pxx, cyy = s.yy + s.yy - pyy, czz = s.zz + s.zz - pzz;
+    i64 Ts = rho;
+    if (w.b != 0) {
+        const i64 d = fx_mul(rho - (cxx + cyy + czz), w.b);
+        Ts += d + d;
+    }
+    // relaxed central moments: trace Ts, deviatoric and off-diagonal parts by 1 - omega
+    const i64 D1 = 2 * fx_mul(cxx - cyy, w.a), D2 = 2 * fx_mul(cxx - czz, w.a);
+    const i64 kxx = fx_mul(Ts + D1 + D2, kFx3), kyy = kxx - D1, kzz = kxx - D2;
+    const i64 kxy = 2 * fx_mul(s.xy + s.xy - pxy, w.a), kxz = 2 * fx_mul(s.xz + s.xz - pxz, w.a);
+    const i64 kyz = 2 * fx_mul(s.yz + s.yz - pyz, w.a);
+    // kappa_xx / rho as a fraction of 2^64 (below 1/2: the trace is about rho)
+    const i64 V = fx_ratio(kxx, rho, ri, bad);
+    const i64 mxx = kxx + pxx, myy = kyy + pyy, mzz = kzz + pzz;
+    const i64 mxy = kxy + pxy, mxz = kxz + pxz, myz = kyz + pyz;
+    i64 mxyy = fx_mul(myy, ux) + 2 * fx_mul(kxy, uy);
+    const i64 xk = 2 * fx_mul(kxy, ux);
+    i64 mxxy = fx_mul(mxx, uy) + xk;
+    i64 mxxz = fx_mul(mxx, uz) + 2 * fx_mul(kxz, ux);
+    const i64 mxyz = fx_mul(myz, ux) + fx_mul(kxz, uy) + fx_mul(kxy, uz);
+    const i64 mxxyy = fx_mul(kyy, V) + fx_mul(mxyy, ux) + fx_mul(fx_mul(kxx, uy) + xk, uy);
+    // force: the first moments gain (F_pre + F_post) / 2 in all, the cubic ones 2 / 5 (F_pre + F_post)
+    const i64 f2x = F[0].h2 + F[0].h2;
+    mxyy += f2x - fx_mul(f2x, kFx5);  // 8 / 5 h2
+    i64 tx = s.jx + F[0].h2, ty = s.jy, tz = s.jz;         // halves of the new first moments
+    if (!XO) {
+        const i64 f2y = F[1].h2 + F[1].h2, f2z = F[2].h2 + F[2].h2;
+        mxxy += f2y - fx_mul(f2y, kFx5);
+        mxxz += f2z - fx_mul(f2z, kFx5);
+        ty += F[1].h2;
+        tz += F[2].h2;
+    }
+    // corners: (S + sx Sx + sy Sy + sz Sz + sx sy Sxy + sx sz Sxz + sy sz Syz + sx sy sz Sxyz) / 8
+    {
+        const i64 U0 = mxxyy + mxxz, Ux = mxyy + mxz, Uy = mxxy + myz, Uxy = mxy + mxyz;  // z = +1
+        const i64 V0 = mxxyy - mxxz, Vx = mxyy - mxz, Vy = mxxy - myz, Vxy = mxy - mxyz;  // z = -1
+        const i64 a0 = U0 + Uy, ax = Ux + Uxy, b0 = U0 - Uy, bx = Ux - Uxy;
+        const i64 c0 = V0 + Vy, cx = Vx + Vxy, d0 = V0 - Vy, dx = Vx - Vxy;
+        f[7] = (a0 + ax) >> 3;
+        f[8] = (a0 - ax) >> 3;
+        f[9] = (b0 + bx) >> 3;
+        f[10] = (b0 - bx) >> 3;
+        f[11] = (c0 + cx) >> 3;
+        f[12] = (c0 - cx) >> 3;
+        f[13] = (d0 + dx) >> 3;
+        f[14] = (d0 - dx) >> 3;
+    }
+    // what the corners hold of the zeroth and first moments
+    const i64 A1 = f[7] + f[8], A2 = f[9] + f[10], A3 = f[11] + f[12], A4 = f[13] + f[14];
+    const i64 S = (A1 + A2) + (A3 + A4);
+    const i64 Cx = (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
+    const i64 Cy = (A1 - A2) + (A3 - A4), Cz = (A1 + A2) - (A3 + A4);
+    const i64 ex = mxx - S, ey = myy - S, ez = mzz - S;
+    const i64 ox = tx + tx - Cx, oy = ty + ty - Cy, oz = tz + tz - Cz;
+    f[1] = (ex + ox) >> 1;
+    f[2] = f[1] - ox;
+    f[3] = (ey + oy) >> 1;
+    f[4] = f[3] - oy;
+    f[5] = (ez + oz) >> 1;
+    f[6] = f[5] - oz;
+    f[0] = rho - S - (f[1] + f[2]) - (f[3] + f[4]) - (f[5] + f[6]);
+}
+
 }  // namespace lbmk

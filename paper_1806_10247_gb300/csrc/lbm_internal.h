@@ -22,6 +22,15 @@ inline bool force_x_only(int fkind, const FieldDev &F, int dim)
     return zero;
 }
 
+// Host: threads per block of a one-node-per-thread launch over N nodes: `most`,
+// or fewer (down to one warp) while the blocks would not reach every SM.
+inline int spread_block(int N, int most)
+{
+    int block = most;
+    while (block > 32 && (N + block - 1) / block < 152) block /= 2;
+    return block;
+}
+
 // Everything one launch of a step / moments / reduction kernel needs.
 struct LaunchArgs {
     Geom g;

@@ -57,8 +57,9 @@ def test_readback_sums(lattice, kind):
         err = q * 2.0 ** -53 * np.abs(f).sum(axis=0)
     else:
         err = 0.5 * q * 2.0 ** -GRID[lattice] * top + 2.0 ** -53 * np.abs(f.sum(axis=0))
+    off = np.array([math.fsum([*f[:, k], -rho[k]]) for k in range(L.N)])  # the exact difference
+    assert (np.abs(off) <= err).all()
     exact = np.array([math.fsum(f[:, k]) for k in range(L.N)])
-    assert (np.abs(rho - exact) <= err).all()
     if u is None:
         return
     for d in range(L.dim):
@@ -100,3 +101,98 @@ def test_readback_sums_of_deviations(lattice, storage, amp):
         e = np.array([_velocity(lattice, a) for a in range(q)])
         for d in range(L.dim):
             assert np.abs(u[d] - (f * e[:, d, None]).sum(axis=0) / rho).max() <= 2 * q * 2.0 ** -53
+
+
+def _oracle(lattice, shape, wall, omega, f, tables=None, uadv=None):
+    from oracle import oracle as O
+    R = O.OracleContext(lattice, shape, omega=omega, wall=wall)
+    assert R.set_populations(f, 0) == 0
+    if tables is not None:
+        P = O.expand_separable(tables, shape)
+        assert (R.set_source(P[0]) if lattice == lbm.D2Q5_CDE else R.set_force(P)) == 0
+    if uadv is not None:
+        n = int(np.prod(shape))
+        assert R.set_velocity(np.repeat(np.asarray(uadv)[:, None], n, axis=1)) == 0
+    return R
+
+
+@pytest.mark.parametrize("kind", ["plain", "mixed", "negative", "fast", "tiny", "huge", "forced"])
+@pytest.mark.parametrize("lattice", [lbm.D2Q9, lbm.D2Q5_CDE, lbm.D3Q27, lbm.D3Q15])
+def test_step_in_and_out_of_range(lattice, kind):
+    """One step of every single-lattice and batched launch from states on both
+    sides of what the fixed-point form takes (scale, sign, speed, size of the
+    force), walls on one axis, against the oracle to the parity bar: 1e-12 of the
+    largest population."""
+    rng = np.random.default_rng(11)
+    q, shape = lbm.Q[lattice], SHAPE[lattice]
+    n = int(np.prod(shape))
+    e = np.array([_velocity(lattice, a) for a in range(q)], dtype=np.float64)
+    w = np.array([_weight(lattice, a) for a in range(q)])
+    speed = 0.35 if kind == "fast" else 0.02
+    u = speed * rng.standard_normal((e.shape[1], n))
+    f = w[:, None] * (1.0 + 3.0 * (e @ u)) * (1.0 + 0.01 * rng.standard_normal((q, n)))
+    if kind == "mixed":  # one node in three far outside the others' scale
+        f[:, ::3] *= 2.0 ** rng.integers(-700, 1, (1, len(range(0, n, 3))))
+    elif kind == "negative":
+        f[1, ::4] *= -0.3
+    elif kind == "tiny":
+        f *= 2.0 ** -600
+    elif kind == "huge":
+        f *= 2.0 ** 55
+    f = np.ascontiguousarray(f)
+    scale = np.abs(f).max()
+    x = np.arange(shape[0])
+    amp = (0.4 if kind == "forced" else 1e-4) * scale
+    one = np.array([1.0])
+    comp = [(amp * np.sin(1.0 + x), one, one), (amp * np.cos(x), one, one), (amp * np.sin(2.0 * x), one, one)]
+    scalar = lattice == lbm.D2Q5_CDE
+    wall = (0, 0, 0) if scalar else (0, 1, 0)
+    for ncomp in (1,) if scalar else (1, 3 if q > 9 else 2):
+        dims = 1 if scalar else (2 if q == 9 else 3)
+        tables = [comp[d] if d < ncomp else (np.zeros(shape[0]), one, one) for d in range(dims)]
+        R = _oracle(lattice, shape, wall, OMEGA[lattice], f, tables, (0.05, -0.02) if scalar else None)
+        assert R.step(1) == 0
+        ref = R.populations()[1]
+        for members in (0, 2):
+            lats = []
+            for _ in range(max(1, members)):
+                L = lbm.Lattice(lattice, shape, OMEGA[lattice], wall=wall)
+                if scalar:
+                    L.set_velocity(tables=[(np.array([0.05]), one, one), (np.array([-0.02]), one, one)])
+                    L.set_source(tables=tables)
+                else:
+                    L.set_force(tables=tables)
+                L.set_populations(f)
+                lats.append(L)
+            if members:
+                B = lbm.Batch(lats)
+                B.step(1)
+            else:
+                lats[0].step(1)
+            for L in lats:
+                assert np.abs(L.get_populations() - ref).max() <= 1e-12 * scale
+
+
+def _weight(lattice, a):
+    e = np.abs(_velocity(lattice, a)).sum()
+    if lattice == lbm.D3Q27:
+        return (2 / 3) ** (3 - e) * (1 / 6) ** e
+    if lattice == lbm.D3Q15:
+        return (2 / 9, 1 / 9, 0, 1 / 72)[e]
+    if lattice == lbm.D2Q5_CDE:
+        return (1 / 3, 1 / 6)[e]
+    return (4 / 9, 1 / 9, 1 / 36)[e]
+
+
+def test_step_passes_nan_on():
+    """A NaN population is passed on by the step (and reported by lbm_reduce)."""
+    for lattice in (lbm.D2Q9, lbm.D2Q5_CDE, lbm.D3Q27, lbm.D3Q15):
+        L = lbm.Lattice(lattice, SHAPE[lattice], OMEGA[lattice])
+        L.init_equilibrium(1.0)
+        f = L.get_populations()
+        f[2, 3] = np.nan
+        L.set_populations(f)
+        L.step(1)
+        assert np.isnan(L.get_populations()).any()
+        with pytest.raises(lbm.LBMError):
+            L.reduce()
