@@ -7,9 +7,11 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstring>
 #include <mutex>
 #include <string>
 
@@ -176,35 +178,62 @@ k_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float *_
     }
 }
 
-__global__ void __launch_bounds__(kT) k_tanh_bwd(float *__restrict__ g, const float *__restrict__ y, long long count)
+// g *= 1 - y^2, four values per thread where both arrays are 16-byte aligned.
+__global__ void __launch_bounds__(kT)
+k_tanh_bwd(float *__restrict__ g, const float *__restrict__ y, long long count, int vec)
 {
     const long long i = (long long)blockIdx.x * kT + threadIdx.x;
-    if (i < count) g[i] *= 1.0f - y[i] * y[i];
+    if (vec && 4 * i + 4 <= count) {
+        float4 a = reinterpret_cast<float4 *>(g)[i];
+        const float4 b = __ldg(reinterpret_cast<const float4 *>(y) + i);
+        a.x *= 1.0f - b.x * b.x;
+        a.y *= 1.0f - b.y * b.y;
+        a.z *= 1.0f - b.z * b.z;
+        a.w *= 1.0f - b.w * b.w;
+        reinterpret_cast<float4 *>(g)[i] = a;
+        return;
+    }
+    for (long long k = 4 * i; k < 4 * i + 4 && k < count; k++) g[k] *= 1.0f - y[k] * y[k];
 }
 
-// g = 2 (y - t) / count and loss = mean((y - t)^2), one block (fixed order).
-__global__ void __launch_bounds__(1024)
-k_mse(const float *__restrict__ y, const float *__restrict__ t, float *__restrict__ g, long long count,
-      double *__restrict__ loss)
+// g = 2 (y - t) / count and the partial sums of (y - t)^2 of kMseBlocks blocks
+// at most (one block took 0.3 ms for 524,288 values, the memory's time is 1 us);
+// k_mse_final adds them in order: loss = mean((y - t)^2).
+constexpr int kMseBlocks = 304;
+__device__ __forceinline__ double block_sum_f64(double acc)
 {
-    __shared__ double sh[32];
-    double acc = 0.0;
-    const float scale = 2.0f / (float)count;
-    for (long long i = threadIdx.x; i < count; i += 1024) {
-        const float d = y[i] - t[i];
-        g[i] = scale * d;
-        acc += (double)d * (double)d;
-    }
+    __shared__ double sh[kT / 32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        acc = sh[threadIdx.x];
+    acc = threadIdx.x < kT / 32 ? sh[threadIdx.x] : 0.0;
+    if (threadIdx.x < 32)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (threadIdx.x == 0) *loss = acc / (double)count;
+    return acc;  // valid in thread 0
+}
+__global__ void __launch_bounds__(kT)
+k_mse(const float *__restrict__ y, const float *__restrict__ t, float *__restrict__ g, long long count,
+      double *__restrict__ part)
+{
+    double acc = 0.0;
+    const float scale = 2.0f / (float)count;
+    for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < count; i += (long long)gridDim.x * kT) {
+        const float d = y[i] - t[i];
+        g[i] = scale * d;
+        acc += (double)d * (double)d;
     }
+    acc = block_sum_f64(acc);
+    if (threadIdx.x == 0) part[blockIdx.x] = acc;
+}
+__global__ void __launch_bounds__(kT) k_mse_final(const double *__restrict__ part, int n, long long count,
+                                                  double *__restrict__ loss)
+{
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += kT) acc += part[i];
+    acc = block_sum_f64(acc);
+    if (threadIdx.x == 0) *loss = acc / (double)count;
 }
 
 // Adam (bias-corrected) on FP32 master weights; also refreshes the BF16 copy.
@@ -252,15 +281,226 @@ __device__ int g_tc_status;
 
 int round16(int v) { return (v + 15) / 16 * 16; }
 
+int round8(int v) { return (v + 7) / 8 * 8; }
+
 enum TcMode { TC_FWD = 0, TC_BWD_IN = 1 };
 
-// TC_FWD:    y[n,o,p] = act(b[o] + sum_{i,tap} w[o,i,tap] x[n,i,p + shift(tap)])
-//            rows: pixels of y; K = (i, tap); N = o.
-// TC_BWD_IN: gx[n,i,p] = sum_{o,tap} w[o,i,tap] gy[n,o,p - shift(tap)]
-//            rows: pixels of x; K = (o, tap); N = i.
-template <int MODE>
+// Pixel coordinates of pixel q of a batch (32-bit: the launchers check the sizes).
+struct Pixel {
+    int n, p;        // sample, position inside it
+    int d, h, w;
+};
+__device__ __forceinline__ Pixel pixel_at(const Shape &s, unsigned q)
+{
+    const unsigned sp = (unsigned)(s.d * s.h * s.w);
+    Pixel x;
+    x.n = (int)(q / sp);
+    x.p = (int)(q - (unsigned)x.n * sp);
+    const unsigned r = (unsigned)x.p / (unsigned)s.w;
+    x.w = x.p - (int)(r * (unsigned)s.w);
+    x.d = (int)(r / (unsigned)s.h);
+    x.h = (int)(r - (unsigned)x.d * (unsigned)s.h);
+    return x;
+}
+// Position of the source pixel of tap (a, f, e), shifted by sgn * dilation; -1 outside.
+__device__ __forceinline__ int tap_source(const Shape &s, const Pixel &x, int a, int f, int e, int sgn)
+{
+    const int zd = x.d + sgn * s.dd * (a - (s.kd - 1) / 2);
+    const int zh = x.h + sgn * s.dh * (f - (s.kh - 1) / 2);
+    const int zw = x.w + sgn * s.dw * (e - (s.kw - 1) / 2);
+    const bool in = (unsigned)zd < (unsigned)s.d && (unsigned)zh < (unsigned)s.h && (unsigned)zw < (unsigned)s.w;
+    return in ? (zd * s.h + zh) * s.w + zw : -1;
+}
+__device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
+{
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    unsigned u;
+    memcpy(&u, &v, sizeof u);
+    return u;
+}
+
+// The images as one line of positions: every row of w pixels is followed by hw
+// empty ones (hw: the taps' reach along w), so that position + shift is the
+// shifted pixel of the same row, or an empty one, for every |shift| <= hw.
+struct Line {
+    int hw, wp;       // reach, positions per row
+    unsigned total;   // positions of the batch
+    int sp;
+};
+__host__ __device__ inline Line line_of(const Shape &s)
+{
+    Line l;
+    l.hw = s.dw * ((s.kw - 1) / 2);
+    l.wp = s.w + l.hw;
+    l.sp = s.d * s.h * s.w;
+    l.total = (unsigned)s.n * (unsigned)(s.d * s.h) * (unsigned)l.wp;
+    return l;
+}
+// Sample, plane, row and column of a position; w < 0 outside the batch and on empty positions.
+__device__ __forceinline__ Pixel position_at(const Shape &s, const Line &l, int q)
+{
+    Pixel x;
+    x.n = x.d = x.h = x.p = 0;
+    x.w = -1;
+    if (q < 0 || (unsigned)q >= l.total) return x;
+    const unsigned r = (unsigned)q / (unsigned)l.wp;
+    const int w = q - (int)(r * (unsigned)l.wp);
+    const unsigned z = r / (unsigned)s.h;
+    x.h = (int)(r - z * (unsigned)s.h);
+    x.n = (int)(z / (unsigned)s.d);
+    x.d = (int)(z - (unsigned)x.n * (unsigned)s.d);
+    x.w = w < s.w ? w : -1;
+    return x;
+}
+
+// Forward pass and input gradient (see k_tc_conv_gather below for the sums), by
+// shifted views of one staged tile: a block stages, for each of the kd x kh rows
+// of taps, the 128 positions of its tile and the hw positions on either side, as
+// rows of 8 channels (16 bytes per position).  The A operand of the tap at
+// distance t along w is that tile read from position hw + t on: the matrix
+// descriptor's start address moves by 16 t bytes.  A value is loaded kd kh times
+// instead of once per tap, and nothing is copied per tap.
+// C16: channels padded to 16, in units of 16 (0: any).
+template <int MODE, int C16>
 __global__ void __launch_bounds__(nntc::kM)
 k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
+          float *__restrict__ out, Shape s, int act, int c16, int Np)
+{
+    using namespace nntc;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) unsigned long long mbar;
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x;
+    const int cin = MODE == TC_FWD ? s.ci : s.co;    // channels of the gathered operand
+    const int cout = MODE == TC_FWD ? s.co : s.ci;   // channels of the result
+    const int sgn = MODE == TC_FWD ? 1 : -1;
+    const Line l = line_of(s);
+    const int G8 = 2 * (C16 ? C16 : c16);             // channel groups of eight
+    const int R = (kM + 2 * l.hw + 7) / 8 * 8;        // staged positions
+    const int segs = s.kd * s.kh, taps = segs * s.kw;
+    unsigned char *As = smem;
+    unsigned char *Bs = smem + segs * G8 * R * 16;
+    const unsigned ntiles = (l.total + kM - 1) / kM;
+    const uint32_t ncols = tmem_cols(Np);
+    const uint32_t lboA = (uint32_t)R * 16, lboB = (uint32_t)(Np / 8) * 128;
+    if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
+    if (tid == 0) mbar_init(smem_u32(&mbar));
+    // weights: K = (tap, channel), one 16-byte row of eight channels at a time
+    for (int idx = tid; idx < Np * taps * G8; idx += kM) {
+        const int k8 = idx / Np, r = idx - k8 * Np, tap = k8 / G8, c0 = (k8 - tap * G8) * 8;
+        __nv_bfloat16 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const int c = c0 + j;
+            v[j] = __float2bfloat16_rn(0.f);
+            if (r < cout && c < cin)
+                v[j] = MODE == TC_FWD ? w[((long long)r * s.ci + c) * taps + tap]
+                                      : w[((long long)c * s.ci + r) * taps + tap];
+        }
+        uint4 u;
+        memcpy(&u, v, sizeof u);
+        *reinterpret_cast<uint4 *>(Bs + core_off(r, 8 * k8, Np)) = u;
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem = tmem_base, a0 = smem_u32(As), b0 = smem_u32(Bs);
+    bool ok = true;
+    uint32_t phase = 0;
+    for (unsigned tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        const int q0 = (int)(tile * kM);
+        for (int j = tid; j < kM + 2 * l.hw; j += kM) {
+            const Pixel x = position_at(s, l, q0 + j - l.hw);
+            const float *base = in + (long long)x.n * cin * l.sp + x.w;
+            for (int seg = 0; seg < segs; seg++) {
+                const int a = seg / s.kh, f = seg - a * s.kh;
+                const int zd = x.d + sgn * s.dd * (a - (s.kd - 1) / 2), zh = x.h + sgn * s.dh * (f - (s.kh - 1) / 2);
+                const bool have = x.w >= 0 && (unsigned)zd < (unsigned)s.d && (unsigned)zh < (unsigned)s.h;
+                const float *src = base + (have ? (zd * s.h + zh) * s.w : 0);
+                unsigned char *dst = As + ((seg * G8) * R + j) * 16;
+#pragma unroll
+                for (int g = 0; g < G8; g++) {
+                    float v[8];
+#pragma unroll
+                    for (int i = 0; i < 8; i++) {
+                        const int c = 8 * g + i;
+                        v[i] = have && c < cin ? __ldg(src + (long long)c * l.sp) : 0.f;
+                    }
+                    *reinterpret_cast<uint4 *>(dst + g * R * 16) = make_uint4(
+                        pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+                }
+            }
+        }
+        fence_smem_to_async();
+        fence_before_sync();
+        __syncthreads();
+        fence_after_sync();
+        if (tid == 0) {
+            const uint32_t id = idesc_bf16(kM, Np);
+            uint32_t more = 0;
+            for (int seg = 0; seg < segs; seg++)
+                for (int e = 0; e < s.kw; e++) {
+                    const int shift = l.hw + sgn * s.dw * (e - (s.kw - 1) / 2);
+                    for (int g = 0; g < G8; g += 2) {
+                        const uint64_t ad = smem_desc(a0 + (uint32_t)((seg * G8 + g) * R + shift) * 16, lboA, 128);
+                        const uint64_t bd = smem_desc(b0 + (uint32_t)((seg * s.kw + e) * G8 + g) * lboB, lboB, 128);
+                        mma_bf16(tmem, ad, bd, id, more);
+                        more = 1;
+                    }
+                }
+            mma_commit(smem_u32(&mbar));
+        }
+        ok = __syncthreads_and(mbar_wait_bounded(smem_u32(&mbar), phase));
+        fence_after_sync();
+        phase ^= 1u;
+        if (!ok) break;
+        const Pixel x = position_at(s, l, q0 + tid);
+        float *dst = out + (long long)x.n * cout * l.sp + (x.d * s.h + x.h) * s.w + x.w;
+        for (int c0 = 0; c0 < Np; c0 += 16) {
+            float v[16];
+            tmem_load16(tmem + ((uint32_t)(32 * (tid >> 5)) << 16) + (uint32_t)c0, v);
+            if (x.w >= 0) {
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const int o = c0 + j;
+                    if (o < cout) {
+                        float r = v[j];
+                        if (MODE == TC_FWD) {
+                            r += b[o];
+                            if (act == 1) r = tanhf(r);
+                        }
+                        dst[(long long)o * l.sp] = r;
+                    }
+                }
+            }
+        }
+        // the next tile's MMAs overwrite the accumulators every warp has just read
+        fence_before_sync();
+    }
+    if (!ok) {
+        if (tid == 0) atomicOr(&g_tc_status, 1);
+        mbar_wait_bounded(smem_u32(&mbar), phase ^ 1u);  // the MMAs end before their accumulators are freed
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    if (tid < 32) tmem_dealloc(tmem, ncols);
+}
+
+// The same products with the A operand gathered tap by tap, for shapes whose
+// staged tile (kd kh (128 + 2 hw) positions) does not fit in shared memory.
+// TC_FWD:    y[n,o,p] = act(b[o] + sum_{i,tap} w[o,i,tap] x[n,i,p + shift(tap)])
+//            rows: pixels of y; K = (tap, i); N = o.
+// TC_BWD_IN: gx[n,i,p] = sum_{o,tap} w[o,i,tap] gy[n,o,p - shift(tap)]
+//            rows: pixels of x; K = (tap, o); N = i.
+// K runs over the taps, then over the gathered channels in groups of eight (the
+// channel count padded to C8): a thread finds a tap's source pixel once, loads
+// eight channels there (adjacent threads, adjacent pixels) and stores them as
+// one 16-byte row of a core matrix.  A block keeps the weights in shared memory
+// and walks over the 128-pixel tiles blockIdx.x, blockIdx.x + gridDim.x, ...
+template <int MODE>
+__global__ void __launch_bounds__(nntc::kM)
+k_tc_conv_gather(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
           float *__restrict__ out, Shape s, int act, int Kp, int Np)
 {
     using namespace nntc;
@@ -273,57 +513,78 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
     const int taps = s.kd * s.kh * s.kw;
     const int cin = MODE == TC_FWD ? s.ci : s.co;    // channels of the gathered operand
     const int cout = MODE == TC_FWD ? s.co : s.ci;   // channels of the result
-    const int K = cin * taps;
+    const int C8 = (cin + 7) >> 3, groups = taps * C8;
     const int sgn = MODE == TC_FWD ? 1 : -1;
-    const long long sp = (long long)s.d * s.h * s.w, npix = (long long)s.n * sp;
-    const long long m = (long long)blockIdx.x * kM + tid;
+    const int sp = s.d * s.h * s.w;
+    const unsigned npix = (unsigned)s.n * (unsigned)sp, ntiles = (npix + kM - 1) / kM;
     const uint32_t ncols = tmem_cols(Np);
+    const uint32_t lboA = (kM / 8) * 128, lboB = (uint32_t)(Np / 8) * 128;
     if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
     if (tid == 0) mbar_init(smem_u32(&mbar));
-    const bool valid = m < npix;
-    int n_ = 0, pd = 0, ph = 0, pw = 0;
-    long long p = 0;
-    if (valid) {
-        n_ = (int)(m / sp);
-        p = m % sp;
-        pw = (int)(p % s.w);
-        ph = (int)((p / s.w) % s.h);
-        pd = (int)(p / ((long long)s.w * s.h));
-    }
-    for (int k = 0; k < Kp; k++) {
-        float v = 0.f;
-        if (valid && k < K) {
-            const int c = k / taps, tap = k - c * taps;
-            const int e = tap % s.kw, f = (tap / s.kw) % s.kh, a = tap / (s.kw * s.kh);
-            const int zd = pd + sgn * s.dd * (a - (s.kd - 1) / 2);
-            const int zh = ph + sgn * s.dh * (f - (s.kh - 1) / 2);
-            const int zw = pw + sgn * s.dw * (e - (s.kw - 1) / 2);
-            if (zd >= 0 && zd < s.d && zh >= 0 && zh < s.h && zw >= 0 && zw < s.w)
-                v = in[((long long)n_ * cin + c) * sp + ((long long)zd * s.h + zh) * s.w + zw];
+    for (int idx = tid; idx < Np * (Kp >> 3); idx += kM) {
+        const int k8 = idx / Np, r = idx - k8 * Np;  // r: output channel; k8: (tap, channel group)
+        const int tap = k8 / C8, c0 = (k8 - tap * C8) * 8;
+        __nv_bfloat16 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const int c = c0 + j;
+            v[j] = __float2bfloat16_rn(0.f);
+            if (k8 < groups && r < cout && c < cin)
+                v[j] = MODE == TC_FWD ? w[((long long)r * s.ci + c) * taps + tap]
+                                      : w[((long long)c * s.ci + r) * taps + tap];
         }
-        *reinterpret_cast<__nv_bfloat16 *>(As + core_off(tid, k, kM)) = __float2bfloat16_rn(v);
+        uint4 u;
+        memcpy(&u, v, sizeof u);
+        *reinterpret_cast<uint4 *>(Bs + core_off(r, 8 * k8, Np)) = u;
     }
-    for (int idx = tid; idx < Np * Kp; idx += kM) {
-        const int r = idx / Kp, k = idx - r * Kp;  // r: output channel, k: (input channel, tap)
-        __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-        if (r < cout && k < K) {
-            const int c = k / taps, tap = k - c * taps;
-            v = MODE == TC_FWD ? w[((long long)r * s.ci + c) * taps + tap] : w[((long long)c * s.ci + r) * taps + tap];
-        }
-        *reinterpret_cast<__nv_bfloat16 *>(Bs + core_off(r, k, Np)) = v;
-    }
-    fence_smem_to_async();
+    // the K padding of this thread's row
+    for (int k8 = groups; k8 < (Kp >> 3); k8++)
+        *reinterpret_cast<uint4 *>(As + core_off(tid, 8 * k8, kM)) = make_uint4(0, 0, 0, 0);
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = tmem_base;
-    if (tid == 0) {
-        issue_tile(tmem, smem_u32(As), smem_u32(Bs), Kp, Np, false);
-        mma_commit(smem_u32(&mbar));
-    }
-    const bool ok = __syncthreads_and(mbar_wait_bounded(smem_u32(&mbar), 0));
-    fence_after_sync();
-    if (ok) {
+    bool ok = true;
+    uint32_t phase = 0;
+    for (unsigned tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        const unsigned q = tile * kM + tid;
+        const bool valid = q < npix;
+        const Pixel x = pixel_at(s, valid ? q : 0);
+        const float *base = in + (long long)x.n * cin * sp;
+        int a = 0, f = 0, e = 0;
+        for (int tap = 0; tap < taps; tap++) {
+            const int at = valid ? tap_source(s, x, a, f, e, sgn) : -1;
+            const float *src = base + (at < 0 ? 0 : at);
+            for (int g = 0; g < C8; g++) {
+                float v[8];
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const int c = 8 * g + j;
+                    v[j] = at >= 0 && c < cin ? __ldg(src + (long long)c * sp) : 0.f;
+                }
+                *reinterpret_cast<uint4 *>(As + core_off(tid, 8 * (tap * C8 + g), kM)) =
+                    make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+            }
+            if (++e == s.kw) {
+                e = 0;
+                if (++f == s.kh) {
+                    f = 0;
+                    a++;
+                }
+            }
+        }
+        fence_smem_to_async();
+        fence_before_sync();
+        __syncthreads();
+        fence_after_sync();
+        if (tid == 0) {
+            issue_tile(tmem, smem_u32(As), lboA, smem_u32(Bs), lboB, Kp, Np);
+            mma_commit(smem_u32(&mbar));
+        }
+        ok = __syncthreads_and(mbar_wait_bounded(smem_u32(&mbar), phase));
+        fence_after_sync();
+        phase ^= 1u;
+        if (!ok) break;
         for (int c0 = 0; c0 < Np; c0 += 16) {
             float v[16];
             tmem_load16(tmem + ((uint32_t)(32 * (tid >> 5)) << 16) + (uint32_t)c0, v);
@@ -337,14 +598,17 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
                             r += b[o];
                             if (act == 1) r = tanhf(r);
                         }
-                        out[((long long)n_ * cout + o) * sp + p] = r;
+                        out[((long long)x.n * cout + o) * sp + x.p] = r;
                     }
                 }
             }
         }
-    } else {
+        // the next tile's MMAs overwrite the accumulators every warp has just read
+        fence_before_sync();
+    }
+    if (!ok) {
         if (tid == 0) atomicOr(&g_tc_status, 1);
-        mbar_wait_bounded(smem_u32(&mbar), 0);  // the MMAs end before their accumulators are freed
+        mbar_wait_bounded(smem_u32(&mbar), phase ^ 1u);  // the MMAs end before their accumulators are freed
     }
     fence_before_sync();
     __syncthreads();
@@ -352,72 +616,97 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
     if (tid < 32) tmem_dealloc(tmem, ncols);
 }
 
-// Weight gradient, partial sums: block (g, t) accumulates, over the 128-pixel
-// chunks c = g, g + G, ..., the rows r = 128 t .. 128 t + 127 of
-// part[g][r][o] = sum_p x[n,i,p + shift(tap)] gy[n,o,p], r = i * taps + tap
-// (rows: weight entries; K: pixels; N: o).  k_tc_reduce_w adds the G partial
-// sums in a fixed order.
+// Weight gradient, partial sums: block g accumulates, over the 128-position
+// chunks c = g, g + G, ... of the line of positions, the rows r = tap * ci + i of
+// part[g][r][o] = sum_p x[n,i,p + shift(tap)] gy[n,o,p]
+// (rows: weight entries, `tiles` tiles of 128; K: positions; N: o), and in FP32
+// the sums of gy, bpart[g][o].  k_tc_reduce_w adds the G partial sums in a fixed
+// order.  A thread loads the value of one position (and the first 2 hw threads
+// one of the halo) once per row of taps and channel, rounds it once and stores
+// it in the kw columns that its taps along w put it in.  Columns are stored two
+// bytes at a time; the core matrices lie kPad bytes further apart along K than
+// they are long, so that the 32 columns of a warp fall on 16 different banks (two
+// columns share a word).
+constexpr int kPad = 16;
+template <int N16>
 __global__ void __launch_bounds__(nntc::kM)
-k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float *__restrict__ part, Shape s, int G,
-                int Mp, int Np)
+k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float *__restrict__ part,
+                float *__restrict__ bpart, Shape s, int G, int tiles)
 {
     using namespace nntc;
+    constexpr int Np = 16 * N16;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long mbar;
     __shared__ uint32_t tmem_base;
-    unsigned char *As = smem;
-    unsigned char *Bs = smem + kM * kM * 2;
+    __shared__ float bsum[kM / 32][Np];
     const int tid = threadIdx.x;
-    const int taps = s.kd * s.kh * s.kw, Kw = s.ci * taps;
-    const long long sp = (long long)s.d * s.h * s.w, npix = (long long)s.n * sp;
-    const long long nchunks = (npix + kM - 1) / kM;
-    const int g = blockIdx.x, row0 = blockIdx.y * kM;
-    const uint32_t ncols = tmem_cols(Np);
+    const Line l = line_of(s);
+    const int segs = s.kd * s.kh, Kw = s.ci * segs * s.kw, rows = (Kw + 7) / 8 * 8;
+    const uint32_t lboA = (uint32_t)rows * 16 + kPad, lboB = (uint32_t)Np * 16 + kPad;
+    unsigned char *Bs = smem;
+    unsigned char *As = smem + (kM / 8) * lboB;  // last: the rows past `rows` of the last tile read what follows
+    const unsigned nchunks = (l.total + kM - 1) / kM;
+    const int g = blockIdx.x;
+    const uint32_t ncols = tmem_cols(tiles * Np);
     if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
     if (tid == 0) mbar_init(smem_u32(&mbar));
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = tmem_base;
+    float bacc[Np];
+#pragma unroll
+    for (int o = 0; o < Np; o++) bacc[o] = 0.f;
     bool ok = true;
     int round = 0;
-    for (long long c = g; c < nchunks && ok; c += G, round++) {
-        // this thread stages pixel j = tid of the chunk: column j of A and of B
-        const long long q = c * kM + tid;
-        const bool valid = q < npix;
-        int n_ = 0, pd = 0, ph = 0, pw = 0;
-        long long p = 0;
-        if (valid) {
-            n_ = (int)(q / sp);
-            p = q % sp;
-            pw = (int)(p % s.w);
-            ph = (int)((p / s.w) % s.h);
-            pd = (int)(p / ((long long)s.w * s.h));
-        }
-        for (int rr = 0; rr < kM; rr++) {
-            const int r = row0 + rr;
-            float v = 0.f;
-            if (valid && r < Kw) {
-                const int i = r / taps, tap = r - i * taps;
-                const int e = tap % s.kw, f = (tap / s.kw) % s.kh, a = tap / (s.kw * s.kh);
-                const int zd = pd + s.dd * (a - (s.kd - 1) / 2);
-                const int zh = ph + s.dh * (f - (s.kh - 1) / 2);
-                const int zw = pw + s.dw * (e - (s.kw - 1) / 2);
-                if (zd >= 0 && zd < s.d && zh >= 0 && zh < s.h && zw >= 0 && zw < s.w)
-                    v = x[((long long)n_ * s.ci + i) * sp + ((long long)zd * s.h + zh) * s.w + zw];
+    for (unsigned c = g; c < nchunks && ok; c += G, round++) {
+        const int q0 = (int)(c * kM);
+        {
+            const Pixel px = position_at(s, l, q0 + tid);
+            const bool valid = px.w >= 0;
+            const float *src = gy + (long long)px.n * s.co * l.sp + (valid ? (px.d * s.h + px.h) * s.w + px.w : 0);
+            unsigned char *col = Bs + (tid >> 3) * lboB + (tid & 7) * 2;
+#pragma unroll
+            for (int o = 0; o < Np; o++) {
+                const float v = valid && o < s.co ? __ldg(src + (long long)o * l.sp) : 0.f;
+                bacc[o] += v;
+                *reinterpret_cast<__nv_bfloat16 *>(col + o * 16) = __float2bfloat16_rn(v);
             }
-            *reinterpret_cast<__nv_bfloat16 *>(As + core_off(rr, tid, kM)) = __float2bfloat16_rn(v);
         }
-        for (int o = 0; o < Np; o++) {
-            const float v = (valid && o < s.co) ? gy[((long long)n_ * s.co + o) * sp + p] : 0.f;
-            *reinterpret_cast<__nv_bfloat16 *>(Bs + core_off(o, tid, Np)) = __float2bfloat16_rn(v);
+        for (int j = tid - l.hw; j < kM + l.hw; j += kM) {
+            const Pixel px = position_at(s, l, q0 + j);
+            const float *base = x + (long long)px.n * s.ci * l.sp + px.w;
+            for (int seg = 0; seg < segs; seg++) {
+                const int a = seg / s.kh, f = seg - a * s.kh;
+                const int zd = px.d + s.dd * (a - (s.kd - 1) / 2), zh = px.h + s.dh * (f - (s.kh - 1) / 2);
+                const bool have = px.w >= 0 && (unsigned)zd < (unsigned)s.d && (unsigned)zh < (unsigned)s.h;
+                const float *src = base + (have ? (zd * s.h + zh) * s.w : 0);
+                for (int i0 = 0; i0 < s.ci; i0 += 8) {
+                    __nv_bfloat16 v[8];
+#pragma unroll
+                    for (int i = 0; i < 8; i++)
+                        v[i] = __float2bfloat16_rn(have && i0 + i < s.ci ? __ldg(src + (long long)(i0 + i) * l.sp) : 0.f);
+                    for (int e = 0; e < s.kw; e++) {
+                        const int k = j - s.dw * (e - (s.kw - 1) / 2);
+                        if ((unsigned)k >= (unsigned)kM) continue;
+                        unsigned char *dst = As + (k >> 3) * lboA + (k & 7) * 2 + ((seg * s.kw + e) * s.ci + i0) * 16;
+#pragma unroll
+                        for (int i = 0; i < 8; i++)
+                            if (i0 + i < s.ci) *reinterpret_cast<__nv_bfloat16 *>(dst + i * 16) = v[i];
+                    }
+                }
+            }
         }
         fence_smem_to_async();
         fence_before_sync();
         __syncthreads();
         fence_after_sync();
         if (tid == 0) {
-            issue_tile(tmem, smem_u32(As), smem_u32(Bs), kM, Np, round > 0);
+            const uint32_t id = idesc_bf16(kM, Np), a0 = smem_u32(As), b0 = smem_u32(Bs);
+            for (int t = 0; t < tiles; t++)
+                for (int k = 0; k < kM / 16; k++)
+                    mma_bf16(tmem + (uint32_t)(t * Np), smem_desc(a0 + (uint32_t)t * kM * 16 + 2u * k * lboA, lboA, 128),
+                             smem_desc(b0 + 2u * k * lboB, lboB, 128), id, (round > 0 || k > 0) ? 1u : 0u);
             mma_commit(smem_u32(&mbar));
         }
         // the next chunk overwrites the operands: wait for this chunk's MMAs
@@ -425,108 +714,204 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
         fence_after_sync();
     }
     if (ok) {
-        const int r = row0 + tid;
-        for (int c0 = 0; c0 < Np; c0 += 16) {
-            float v[16];
-            tmem_load16(tmem + ((uint32_t)(32 * (tid >> 5)) << 16) + (uint32_t)c0, v);
+        for (int t = 0; t < tiles; t++)
 #pragma unroll
-            for (int j = 0; j < 16; j++) part[((long long)g * Mp + r) * Np + c0 + j] = round > 0 ? v[j] : 0.f;
-        }
+            for (int c0 = 0; c0 < Np; c0 += 16) {
+                float v[16];
+                tmem_load16(tmem + ((uint32_t)(32 * (tid >> 5)) << 16) + (uint32_t)(t * Np + c0), v);
+                const long long r = (long long)g * tiles * kM + t * kM + tid;
+#pragma unroll
+                for (int j = 0; j < 16; j++) part[r * Np + c0 + j] = round > 0 ? v[j] : 0.f;
+            }
     } else {
         if (tid == 0) atomicOr(&g_tc_status, 1);
         mbar_wait_bounded(smem_u32(&mbar), (uint32_t)((round - 1) & 1));
     }
+#pragma unroll
+    for (int o = 0; o < Np; o++) {
+        float v = bacc[o];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+        if ((tid & 31) == 0) bsum[tid >> 5][o] = v;
+    }
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
+    if (tid < Np) bpart[g * Np + tid] = (bsum[0][tid] + bsum[1][tid]) + (bsum[2][tid] + bsum[3][tid]);
     if (tid < 32) tmem_dealloc(tmem, ncols);
 }
 
-// gw[o][i][tap] = sum_{g = 0..G-1} part[g][i * taps + tap][o], in order of g.
+// gw[o][i][tap] = sum_g part[g][tap * ci + i][o], and after the Kw rows gb[o] =
+// sum_g bpart[g][o].  One block per row: thread t adds the partial sums g = t / 16,
+// t / 16 + 16, ... of channel o0 + t % 16, then the sixteen are added in order (a
+// fixed order: deterministic).
 __global__ void __launch_bounds__(kT)
-k_tc_reduce_w(const float *__restrict__ part, float *__restrict__ gw, int co, int Kw, int G, int Mp, int Np)
+k_tc_reduce_w(const float *__restrict__ part, const float *__restrict__ bpart, float *__restrict__ gw,
+              float *__restrict__ gb, int ci, int co, int taps, int G, int Mp, int Np)
 {
-    const int idx = blockIdx.x * kT + threadIdx.x;
-    if (idx >= co * Kw) return;
-    const int o = idx / Kw, r = idx - o * Kw;
-    float acc = 0.f;
-    for (int g = 0; g < G; g++) acc += part[((long long)g * Mp + r) * Np + o];
-    gw[idx] = acc;
-}
-
-// gb[o] = sum_{n,p} gy[n,o,p] (one block per channel, fixed order).
-__global__ void __launch_bounds__(kT) k_bias_grad(const float *__restrict__ gy, float *__restrict__ gb, Shape s)
-{
-    const long long sp = (long long)s.d * s.h * s.w;
-    const int o = blockIdx.x;
-    float acc = 0.0f;
-    for (long long q = threadIdx.x; q < (long long)s.n * sp; q += kT) {
-        const int n = (int)(q / sp);
-        acc += gy[((long long)n * s.co + o) * sp + q % sp];
+    __shared__ float sh[16][17];
+    const int r = blockIdx.x, Kw = ci * taps, lane = threadIdx.x & 15, row = threadIdx.x >> 4;
+    const int tap = r / ci, i = r - tap * ci;
+    const float *src = r < Kw ? part + (long long)r * Np : bpart;
+    const long long stride = r < Kw ? (long long)Mp * Np : Np;
+    for (int o0 = 0; o0 < co; o0 += 16) {
+        float acc = 0.f;
+#pragma unroll 4
+        for (int g = row; g < G; g += 16) acc += src[g * stride + o0 + lane];
+        sh[row][lane] = acc;
+        __syncthreads();
+        if (row == 0 && o0 + lane < co) {
+            float t = 0.f;
+#pragma unroll
+            for (int k = 0; k < 16; k++) t += sh[k][lane];
+            if (r < Kw) gw[((long long)(o0 + lane) * ci + i) * taps + tap] = t;
+            else gb[o0 + lane] = t;
+        }
+        __syncthreads();
     }
-    acc = block_sum(acc);
-    if (threadIdx.x == 0) gb[o] = acc;
 }
 
-// Partial-sum workspace of the weight gradient, one per device, grown on
-// demand (cudaMalloc only when a larger one is needed).
-std::mutex g_ws_mu;
-float *g_ws[64] = {};
-size_t g_ws_cap[64] = {};
+// Scratch of one call, allocated and freed in stream order from a pool of the
+// library's own (one per device; it keeps at most kPoolKeep bytes between uses),
+// so that calls on different streams and threads never share it.
+constexpr size_t kPoolKeep = 64u << 20;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[64] = {};
 
-float *tc_workspace(size_t floats)
+cudaMemPool_t scratch_pool()
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    std::lock_guard<std::mutex> lock(g_ws_mu);
-    if (g_ws_cap[dev] < floats) {
-        if (g_ws[dev]) cudaFree(g_ws[dev]);
-        g_ws[dev] = nullptr;
-        g_ws_cap[dev] = 0;
-        if (cudaMalloc(&g_ws[dev], floats * sizeof(float)) != cudaSuccess) {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps p{};
+        p.allocType = cudaMemAllocationTypePinned;
+        p.handleTypes = cudaMemHandleTypeNone;
+        p.location.type = cudaMemLocationTypeDevice;
+        p.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &p) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
-        g_ws_cap[dev] = floats;
+        unsigned long long keep = kPoolKeep;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        g_pool[dev] = pool;
     }
-    return g_ws[dev];
+    return g_pool[dev];
 }
 
-bool tc_fits(int kdim, int ndim) { return round16(kdim) <= nntc::kMaxKp && round16(ndim) <= nntc::kMaxNp; }
+void *scratch_alloc(size_t bytes, cudaStream_t st)
+{
+    cudaMemPool_t pool = scratch_pool();
+    void *p = nullptr;
+    if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, st) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
+// Padded K of the gathering convolution: the channels of a tap in groups of eight.
+int tc_kp(int cin, int taps) { return round16(taps * round8(cin)); }
+// Positions of the batch in 32 bits (the kernels' index type), with room for a
+// tile and its halo past the last one.
+bool tc_sizes(const Shape &s)
+{
+    const long long hw = (long long)s.dw * ((s.kw - 1) / 2);
+    return hw < (1LL << 20) && (long long)s.d * s.h * s.w < (1LL << 30) &&
+           (long long)s.n * s.d * s.h * (s.w + hw) < (1LL << 31) - (1LL << 21);
+}
+constexpr size_t kSmemMost = 220u * 1024u;
+size_t gather_smem(const Shape &s, int cin, int cout)
+{
+    return (size_t)(nntc::kM + round16(cout)) * tc_kp(cin, s.kd * s.kh * s.kw) * 2;
+}
+size_t staged_smem(const Shape &s, int cin, int cout)
+{
+    const size_t R = (nntc::kM + 2 * (size_t)s.dw * ((s.kw - 1) / 2) + 7) / 8 * 8, segs = (size_t)s.kd * s.kh;
+    return segs * (round16(cin) / 8) * R * 16 + segs * s.kw * round16(cin) * round16(cout) * 2;
+}
+// The shapes the tensor-core kernels take: what a tile holds (include/lbm.h) and
+// fits in shared memory one way or the other.
+bool tc_fits(const Shape &s, int cin, int cout)
+{
+    return round16(cin * s.kd * s.kh * s.kw) <= nntc::kMaxKp && round16(cout) <= nntc::kMaxNp && tc_sizes(s) &&
+           (staged_smem(s, cin, cout) <= kSmemMost || gather_smem(s, cin, cout) <= kSmemMost);
+}
+
+// Blocks of a kernel that an SM holds at once, times the SMs, by registers, shared
+// memory, tensor memory columns and threads.  (The occupancy query answers 1 for
+// kernels that allocate tensor memory.)
+template <class K>
+unsigned resident_grid(K kernel, size_t smem, int ncols)
+{
+    int dev = 0, sms = 152, per_sm = 512 / ncols;
+    cudaFuncAttributes a{};
+    if (cudaFuncGetAttributes(&a, kernel) == cudaSuccess) {
+        const int regs = (a.numRegs + 7) / 8 * 8 * nntc::kM;
+        per_sm = std::min(per_sm, 65536 / regs);
+        per_sm = std::min(per_sm, (int)(227 * 1024 / (smem + a.sharedSizeBytes + 1024)));
+    } else {
+        cudaGetLastError();
+    }
+    per_sm = std::max(1, std::min(per_sm, 2048 / nntc::kM));
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return (unsigned)(per_sm * sms);
+}
+
+template <class K, class... A>
+int tc_launch(K kernel, unsigned tiles, size_t smem, int Np, cudaStream_t st, const char *what, A... args)
+{
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return nn_fail(LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e));
+    const unsigned most = resident_grid(kernel, smem, nntc::tmem_cols(Np));
+    kernel<<<tiles < most ? tiles : most, nntc::kM, smem, st>>>(args...);
+    return launched(what);
+}
 
 template <int MODE>
 int tc_conv_launch(const float *in, const void *w, const float *b, float *out, const Shape &s, int act,
                    cudaStream_t st, const char *what)
 {
-    const int taps = s.kd * s.kh * s.kw;
-    const int K = (MODE == TC_FWD ? s.ci : s.co) * taps, Np = round16(MODE == TC_FWD ? s.co : s.ci);
-    const int Kp = round16(K);
-    const size_t smem = (size_t)(nntc::kM + Np) * Kp * 2 + nntc::kSlack;
-    cudaError_t e = cudaFuncSetAttribute(k_tc_conv<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return nn_fail(LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e));
-    const long long npix = (long long)s.n * s.d * s.h * s.w;
-    k_tc_conv<MODE><<<(unsigned)((npix + nntc::kM - 1) / nntc::kM), nntc::kM, smem, st>>>(
-        in, reinterpret_cast<const __nv_bfloat16 *>(w), b, out, s, act, Kp, Np);
-    return launched(what);
+    const int cin = MODE == TC_FWD ? s.ci : s.co, cout = MODE == TC_FWD ? s.co : s.ci, Np = round16(cout);
+    const __nv_bfloat16 *wb = reinterpret_cast<const __nv_bfloat16 *>(w);
+    // the staged form where it fits (every shape the network uses).  16 -> 16 channels,
+    // 1 x 3 x 3 taps, dilation 8, 32 x 128^2 pixels, forward: 45 us (the memory's time
+    // is 10); gathering every tap's value by value, with a division per index, took
+    // about 900.  Now bound by instruction issue (62 %): tanh and the staging.
+    const size_t staged = staged_smem(s, cin, cout);
+    if (staged <= kSmemMost) {
+        const unsigned tiles = (line_of(s).total + nntc::kM - 1) / nntc::kM;
+        const int c16 = round16(cin) / 16;
+        if (c16 == 1) return tc_launch(k_tc_conv<MODE, 1>, tiles, staged, Np, st, what, in, wb, b, out, s, act, c16, Np);
+        return tc_launch(k_tc_conv<MODE, 0>, tiles, staged, Np, st, what, in, wb, b, out, s, act, c16, Np);
+    }
+    const unsigned npix = (unsigned)((long long)s.n * s.d * s.h * s.w);
+    return tc_launch(k_tc_conv_gather<MODE>, (npix + nntc::kM - 1) / nntc::kM, gather_smem(s, cin, cout), Np, st, what, in,
+                     wb, b, out, s, act, tc_kp(cin, s.kd * s.kh * s.kw), Np);
 }
 
-int tc_conv_bwd_w_launch(const float *x, const float *gy, float *gw, const Shape &s, cudaStream_t st)
+template <int N16>
+int tc_conv_bwd_w_launch(const float *x, const float *gy, float *gw, float *gb, const Shape &s, cudaStream_t st)
 {
-    const int taps = s.kd * s.kh * s.kw, Kw = s.ci * taps;
-    const int Mp = (Kw + nntc::kM - 1) / nntc::kM * nntc::kM, Np = round16(s.co);
-    const long long npix = (long long)s.n * s.d * s.h * s.w;
-    const long long nchunks = (npix + nntc::kM - 1) / nntc::kM;
-    const int G = (int)(nchunks < 128 ? nchunks : 128);
-    float *part = tc_workspace((size_t)G * Mp * Np);
-    if (!part) return nn_fail(LBM_ENOMEM, "conv3d_backward: tensor-core workspace");
-    const size_t smem = (size_t)(nntc::kM + Np) * nntc::kM * 2 + nntc::kSlack;
-    cudaError_t e = cudaFuncSetAttribute(k_tc_conv_bwd_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr int Np = 16 * N16;
+    const int taps = s.kd * s.kh * s.kw, Kw = s.ci * taps, rows = (Kw + 7) / 8 * 8;
+    const int tiles = (Kw + nntc::kM - 1) / nntc::kM, Mp = tiles * nntc::kM;
+    const unsigned nchunks = (line_of(s).total + nntc::kM - 1) / nntc::kM;
+    const size_t smem = (size_t)(nntc::kM / 8) * (rows * 16 + kPad + Np * 16 + kPad) + (size_t)(Mp - rows) * 16;
+    cudaError_t e = cudaFuncSetAttribute(k_tc_conv_bwd_w<N16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return nn_fail(LBM_ECUDA, "conv3d_backward(weights): %s", cudaGetErrorString(e));
-    k_tc_conv_bwd_w<<<dim3((unsigned)G, (unsigned)(Mp / nntc::kM)), nntc::kM, smem, st>>>(x, gy, part, s, G, Mp, Np);
-    int rc = launched("conv3d_backward(weights)");
-    if (rc != LBM_OK) return rc;
-    k_tc_reduce_w<<<grid_of((long long)s.co * Kw, kT), kT, 0, st>>>(part, gw, s.co, Kw, G, Mp, Np);
-    return launched("conv3d_backward(weight reduction)");
+    unsigned G = resident_grid(k_tc_conv_bwd_w<N16>, smem, nntc::tmem_cols(tiles * Np));
+    if (G > nchunks) G = nchunks;
+    float *part = static_cast<float *>(scratch_alloc((size_t)G * (Mp + 1) * Np * sizeof(float), st));
+    if (!part) return nn_fail(LBM_ENOMEM, "conv3d_backward: tensor-core workspace");
+    float *bpart = part + (size_t)G * Mp * Np;
+    k_tc_conv_bwd_w<N16><<<G, nntc::kM, smem, st>>>(x, gy, part, bpart, s, (int)G, tiles);
+    k_tc_reduce_w<<<Kw + 1, kT, 0, st>>>(part, bpart, gw, gb, s.ci, s.co, taps, (int)G, Mp, Np);
+    const int rc = launched("conv3d_backward(weights)");
+    cudaFreeAsync(part, st);
+    return rc;
 }
 
 int check_shape(const int *sp, const int *k, const int *dil, int n, int ci, int co, Shape &s)
@@ -568,7 +953,7 @@ int lbm_nn_conv3d_forward(const float *x, const void *w, int w_bf16, const float
     if (rc != LBM_OK) return rc;
     if (!x || !w || !b || !y) return nn_fail(LBM_EINVAL, "conv3d_forward: NULL pointer");
     if (act != 0 && act != 1) return nn_fail(LBM_EINVAL, "conv3d_forward: act must be 0 or 1");
-    if (w_bf16 && tc_fits(ci * s.kd * s.kh * s.kw, co))
+    if (w_bf16 && tc_fits(s, ci, co))
         return tc_conv_launch<TC_FWD>(x, w, b, y, s, act, (cudaStream_t)stream, "conv3d_forward");
     k_conv_fwd<<<grid_of(s.out_count(), kT), kT, 0, (cudaStream_t)stream>>>(x, w, w_bf16, b, y, s, act);
     return launched("conv3d_forward");
@@ -584,7 +969,7 @@ int lbm_nn_conv3d_backward(const float *x, const void *w, int w_bf16, const floa
     cudaStream_t st = (cudaStream_t)stream;
     const int taps = s.kd * s.kh * s.kw;
     if (gx) {
-        if (w_bf16 && tc_fits(co * taps, ci)) {
+        if (w_bf16 && tc_fits(s, co, ci)) {
             rc = tc_conv_launch<TC_BWD_IN>(gy, w, nullptr, gx, s, 0, st, "conv3d_backward(input)");
         } else {
             k_conv_bwd_in<<<grid_of(s.in_count(), kT), kT, 0, st>>>(gy, w, w_bf16, gx, s);
@@ -592,12 +977,13 @@ int lbm_nn_conv3d_backward(const float *x, const void *w, int w_bf16, const floa
         }
         if (rc != LBM_OK) return rc;
     }
-    if (w_bf16 && ci * taps <= nntc::kMaxKp && round16(co) <= nntc::kMaxNp) {
-        rc = tc_conv_bwd_w_launch(x, gy, gw, s, st);
-        if (rc != LBM_OK) return rc;
-        k_bias_grad<<<(unsigned)co, kT, 0, st>>>(gy, gb, s);
-        return launched("conv3d_backward(bias)");
-    }
+    if (w_bf16 && ci * taps <= nntc::kMaxKp && round16(co) <= nntc::kMaxNp && tc_sizes(s))
+        switch (round16(co) / 16) {
+        case 1: return tc_conv_bwd_w_launch<1>(x, gy, gw, gb, s, st);
+        case 2: return tc_conv_bwd_w_launch<2>(x, gy, gw, gb, s, st);
+        case 3: return tc_conv_bwd_w_launch<3>(x, gy, gw, gb, s, st);
+        default: return tc_conv_bwd_w_launch<4>(x, gy, gw, gb, s, st);
+        }
     const long long blocks = (long long)co * ci * taps + co;
     k_conv_bwd_w<<<(unsigned)blocks, kT, 0, st>>>(x, gy, gw, gb, s);
     return launched("conv3d_backward(weights)");
@@ -607,15 +993,24 @@ int lbm_nn_tanh_backward(float *g, const float *y, long long count, void *stream
 {
     if (!g || !y || count < 0) return nn_fail(LBM_EINVAL, "tanh_backward: bad arguments");
     if (count == 0) return LBM_OK;
-    k_tanh_bwd<<<grid_of(count, kT), kT, 0, (cudaStream_t)stream>>>(g, y, count);
+    const int vec = (reinterpret_cast<uintptr_t>(g) | reinterpret_cast<uintptr_t>(y)) % 16 == 0;
+    k_tanh_bwd<<<grid_of((count + 3) / 4, kT), kT, 0, (cudaStream_t)stream>>>(g, y, count, vec);
     return launched("tanh_backward");
 }
 
 int lbm_nn_mse(const float *y, const float *t, float *g, long long count, double *loss, void *stream)
 {
     if (!y || !t || !g || !loss || count < 1) return nn_fail(LBM_EINVAL, "mse: bad arguments");
-    k_mse<<<1, 1024, 0, (cudaStream_t)stream>>>(y, t, g, count, loss);
-    return launched("mse");
+    cudaStream_t st = (cudaStream_t)stream;
+    const long long want = (count + 4 * kT - 1) / (4 * kT);
+    const int blocks = (int)(want < kMseBlocks ? want : kMseBlocks);
+    double *part = static_cast<double *>(scratch_alloc(blocks * sizeof(double), st));
+    if (!part) return nn_fail(LBM_ENOMEM, "mse: workspace");
+    k_mse<<<blocks, kT, 0, st>>>(y, t, g, count, part);
+    k_mse_final<<<1, kT, 0, st>>>(part, blocks, count, loss);
+    const int rc = launched("mse");
+    cudaFreeAsync(part, st);
+    return rc;
 }
 
 int lbm_nn_adam(float *p, const float *g, float *m, float *v, void *p_bf16, long long count, double lr, double b1,

@@ -20,11 +20,7 @@ namespace nntc {
 constexpr int kM = 128;          // rows of one MMA tile (pixels or weight rows)
 constexpr int kMaxKp = 512;      // padded K of one tile
 constexpr int kMaxNp = 64;       // padded N (output channels) of one tile
-// Slack after the operand tiles: even a descriptor read with its two strides
-// exchanged (at most 15 * 2048 + 255 bytes past a tile's start) stays inside
-// the block's own shared memory.
-constexpr int kSlack = 32768;
-constexpr unsigned long long kWaitNs = 2000000000ull;  // bound of every wait: 2 s
+constexpr long long kWaitClocks = 4000000000ll;  // bound of every wait: about 2 s
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -82,18 +78,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t addr, uint32_t parity)
         : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-// Wait for phase `parity` of the barrier, giving up after kWaitNs.
+// Wait for phase `parity` of the barrier, giving up after kWaitClocks.  (Timed by
+// the SM's own clock: reading the global timer in every thread of every wait took
+// most of these kernels' time.)
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t addr, uint32_t parity)
 {
-    const unsigned long long t0 = global_ns();
+    if (mbar_try_wait(addr, parity)) return true;
+    const long long t0 = clock64();
     while (!mbar_try_wait(addr, parity))
-        if (global_ns() - t0 > kWaitNs) return false;
+        if (clock64() - t0 > kWaitClocks) return false;
     return true;
 }
 
@@ -115,15 +108,16 @@ __device__ __forceinline__ void mma_commit(uint32_t mbar)
 }
 
 // Issue the MMAs of one tile: kM rows of A (Kp values each, at a0) times Np
-// rows of B (at b0), into the FP32 accumulators at tmem.
-__device__ __forceinline__ void issue_tile(uint32_t tmem, uint32_t a0, uint32_t b0, int Kp, int Np, bool accumulate)
+// rows of B (at b0), into the FP32 accumulators at tmem; lboA and lboB are the
+// byte distances between core matrices along K.
+__device__ __forceinline__ void issue_tile(uint32_t tmem, uint32_t a0, uint32_t lboA, uint32_t b0, uint32_t lboB, int Kp,
+                                           int Np)
 {
     const uint32_t id = idesc_bf16(kM, Np);
-    const uint32_t lboA = (kM / 8) * 128, lboB = (uint32_t)(Np / 8) * 128;
     for (int s = 0; s < Kp / 16; s++) {
         const uint64_t ad = smem_desc(a0 + (uint32_t)s * 2u * lboA, lboA, 128);
         const uint64_t bd = smem_desc(b0 + (uint32_t)s * 2u * lboB, lboB, 128);
-        mma_bf16(tmem, ad, bd, id, (accumulate || s > 0) ? 1u : 0u);
+        mma_bf16(tmem, ad, bd, id, s > 0 ? 1u : 0u);
     }
 }
 
@@ -142,6 +136,6 @@ __device__ __forceinline__ void tmem_load16(uint32_t taddr, float (&v)[16])
     for (int j = 0; j < 16; j++) v[j] = __uint_as_float(r[j]);
 }
 
-__host__ __device__ constexpr int tmem_cols(int Np) { return Np <= 32 ? 32 : (Np <= 64 ? 64 : 128); }
+__host__ __device__ constexpr int tmem_cols(int Np) { return Np <= 32 ? 32 : (Np <= 64 ? 64 : (Np <= 128 ? 128 : 256)); }
 
 }  // namespace nntc
