@@ -164,9 +164,9 @@ __device__ __forceinline__ bool fixed_step5(const double (&f)[5], const FxCoef5 
 template <int SK>
 __global__ void __launch_bounds__(kBlock)
 k_step_mat(const __grid_constant__ Planes<double, 5> P, Geom g, FieldDev S, double ahalf, double hsum, Mat5 M,
-           const __grid_constant__ FxCoef5 fx)
+           const __grid_constant__ FxCoef5 fx, double q2)
 {
-    int i = blockIdx.x * kBlock + threadIdx.x;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
     node_xy(g, i, x, y);
@@ -174,7 +174,7 @@ k_step_mat(const __grid_constant__ Planes<double, 5> P, Geom g, FieldDev S, doub
     load_pulled<LD2Q5>(P, g, x, y, 0, i, f);
     const double Ps = SK != FK_NONE ? field_value(S, SK, 0, x, y, 0, i) : 0.0;
     if (fx.ok) {
-        if (fixed_step5<SK != FK_NONE>(f, fx, Ps, ahalf, 5.0 * hsum, [&](int a, double v) { P.out[a][i] = v; })) return;
+        if (fixed_step5<SK != FK_NONE>(f, fx, Ps, ahalf, q2, [&](int a, double v) { P.out[a][i] = v; })) return;
         load_pulled<LD2Q5>(P, g, x, y, 0, i, f);
     }
     collide_mat<SK != FK_NONE>(f, Ps, ahalf, hsum, M.m);
@@ -215,16 +215,18 @@ void launch_v(const LaunchArgs &a, int grid, double hsum, const Rates5 &w)
     if (a.vkind != FK_GENERAL) {
         const double ux = a.vkind == FK_CONST ? a.V.cval[0] : 0.0;
         const double uy = a.vkind == FK_CONST ? a.V.cval[1] : 0.0;
-        k_step_mat<SK><<<grid, kBlock, 0, a.stream>>>(make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
+        const int block = spread_block(a.g.N, kBlock);
+        k_step_mat<SK><<<(a.g.N + block - 1) / block, block, 0, a.stream>>>(make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
                                                        0.5 * a.apre, hsum, make_mat(make_coef(w, ux, uy)),
-                                                       fx_coef5(w.c1, w.c2, w.c3, w.c4, ux, uy));
+                                                       fx_coef5(w.c1, w.c2, w.c3, w.c4, ux, uy),
+                                                       0.5 * (a.apre + a.apost));
         return;
     }
     k_step<SK, FK_GENERAL><<<grid, kBlock, 0, a.stream>>>(make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
                                                           a.V, a.apre, hsum, w);
 }
 
-// Batched form; FP64 pairs hold (a_pre/2, (a_pre + a_post)/10) per step and
+// Batched form; FP64 pairs hold (a_pre/2, (a_pre + a_post)/2) per step and
 // item (a_pre is halved on the host: one multiply fewer per node).
 // coef[0..11] = Coef5 of a uniform advecting velocity, coef[12..15] = Rates5,
 // mat = the step matrix of a uniform advecting velocity.
@@ -245,17 +247,17 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
         const bool src = B.fkind != FK_NONE;
         const double P = src ? field_value(B.F, B.fkind, 0, x, y, 0, i) : 0.0;
         if (B.fx5.ok) {
-            if (fixed_step5<true>(f, B.fx5, P, ap.x, 5.0 * ap.y, [&](int a, double v) { fout[a * g.Np + i] = v; })) return;
+            if (fixed_step5<true>(f, B.fx5, P, ap.x, ap.y, [&](int a, double v) { fout[a * g.Np + i] = v; })) return;
             load_pulled<LD2Q5>(fin, g, x, y, 0, i, f);
         }
-        if (src) collide_mat<true>(f, P, ap.x, ap.y, B.mat);
+        if (src) collide_mat<true>(f, P, ap.x, ap.y / 5.0, B.mat);
         else collide_mat<false>(f, 0.0, 0.0, 0.0, B.mat);
     } else {
         double Spre = 0.0, H0 = 0.0;
         if (B.fkind != FK_NONE) {
             const double P = field_value(B.F, B.fkind, 0, x, y, 0, i);
             Spre = (2.0 * ap.x) * P;
-            H0 = ap.y * P;
+            H0 = (ap.y / 5.0) * P;
         }
         const Rates5 w{B.coef[12], B.coef[13], B.coef[14], B.coef[15]};
         const double ux = field_value(B.V, FK_GENERAL, 0, x, y, 0, i);

@@ -192,9 +192,10 @@ __device__ __forceinline__ void double_step9(double (&f)[9], const Rates9 &w, bo
 // XO (unit higher rates only): the force has no y component (checked on the host).
 template <int FK, bool W1, bool XO>
 __global__ void __launch_bounds__(kBlock)
-k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double apre, double gsum, Rates9 w, FxRates fx)
+k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double apre, double gsum, Rates9 w, FxRates fx,
+       double q1, double q2)
 {
-    int i = blockIdx.x * kBlock + threadIdx.x;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
     node_xy(g, i, x, y);
@@ -202,7 +203,7 @@ k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double a
     load_pulled<LD2Q9>(P, g, x, y, 0, i, f);
     auto shape = [&](int d) { return field_value(F, FK, d, x, y, 0, i); };
     if (W1) {
-        if (fixed_step9<FK != FK_NONE, XO>(f, fx, 0.25 * apre, 3.0 * gsum, shape,
+        if (fixed_step9<FK != FK_NONE, XO>(f, fx, q1, q2, shape,
                                            [&](int a, double v) { P.out[a][i] = v; }))
             return;
         load_pulled<LD2Q9>(P, g, x, y, 0, i, f);
@@ -219,9 +220,17 @@ k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double a
 // their post-collision populations twice (current and next step) in its
 // shared memory; a pull from a node of another block reads that block's
 // shared memory directly.  One cluster barrier per step separates the
-// writes of a step from the reads of the next.  The per-node arithmetic is
-// `collide` above, so the result equals n single-step launches up to the
-// compiler's multiply-add contraction.
+// writes of a step from the reads of the next.
+//
+// A step of ~100 nodes is one warp per SM: its time is the latency of one node's
+// chain of operations.  With unit higher rates the state is therefore kept in
+// fixed point from the first step to the last (fx_collide9_run: one scale for the
+// lattice, no conversions inside a step, mass and momentum exact), and rounded to
+// FP64 once at the end.  A lattice whose nodes differ by more than 2^3 in scale,
+// or whose values leave the range on the way, runs the FP64 steps from the start
+// state instead (every block learns of it at the barrier after the last step).
+// 3 x 33, 100 steps: FP64 steps 3.05 us each, FP64 state with a fixed-point
+// collision 1.84, fixed-point state 1.40.
 namespace cg = cooperative_groups;
 
 constexpr int kClusterThreads = 384;  // >= 32-rounded 341, the largest block (48 KB of shared memory)
@@ -232,22 +241,18 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
                 double gsum, Rates9 w, FxRates fx, int P, int nsteps)
 {
     extern __shared__ double sm[];  // [2][9][P]
+    __shared__ int range[3];        // smallest and largest exponent of this block's nodes; a value left the range
     cg::cluster_group cl = cg::this_cluster();
-    const int b = (int)cl.block_rank();
+    const int b = (int)cl.block_rank(), nblk = (int)cl.num_blocks();
     const int l = threadIdx.x;
     const int i = b * P + l;
     const bool own = l < P && i < g.N;
-    if (own)
-#pragma unroll
-        for (int a = 0; a < 9; a++) sm[a * P + l] = fin[a * g.Np + i];
     const int x = own ? i % g.nx : 0, y = own ? i / g.nx : 0;
     double Px = 0.0, Py = 0.0;
     if (FK != FK_NONE && own) {
         Px = field_value(F, FK, 0, x, y, 0, i);
         Py = field_value(F, FK, 1, x, y, 0, i);
     }
-    auto shape = [&](int d) { return d == 0 ? Px : Py; };
-    const double q1 = 0.25 * apre, q2 = 3.0 * gsum;
     // pull sources of this node: owner block, offset inside its buffer
     int src_blk[9], src_off[9];
     if (own) {
@@ -260,38 +265,112 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
             src_off[a] = aa * P + (j - (j / P) * P);
         }
     }
-    cl.sync();
-    int cur = 0;
-    for (int k = 0; k < nsteps; k++) {
+    bool fixed = false;
+    if (W1) {
+        // the lattice's scale
+        if (l < 3) range[l] = l == 0 ? 0x7fffffff : 0;
+        __syncthreads();
+        double f[9];
         if (own) {
-            double f[9];
-            auto pull = [&]() {
 #pragma unroll
-                for (int a = 0; a < 9; a++) {
-                    const double *base = cl.map_shared_rank(sm + cur * 9 * P, src_blk[a]);
-                    f[a] = base[src_off[a]];
-                }
-            };
-            double *nxt = sm + (cur ^ 1) * 9 * P;
-            auto put = [&](int a, double v) { nxt[a * P + l] = v; };
-            pull();
-            if (!W1 || !fixed_step9<FK != FK_NONE, false>(f, fx, q1, q2, shape, put)) {
-                if (W1) pull();
-                double_step9<W1, false>(f, w, FK != FK_NONE, apre, gsum, shape);
+            for (int a = 0; a < 9; a++) f[a] = fin[a * g.Np + i];
+            const int em = fx_emax(f);
+            atomicMin(&range[0], em);
+            atomicMax(&range[1], em);
+        }
+        cl.sync();
+        int lo = 0x7fffffff, hi = 0;
+        for (int r = 0; r < nblk; r++) {
+            const int *other = cl.map_shared_rank(range, r);
+            lo = min(lo, other[0]);
+            hi = max(hi, other[1]);
+        }
+        const int k = FxGrid<9>::S + 1023 - hi;
+        int bad = fx_in_range(hi) && hi - lo <= 3 ? 0 : -1;
+        // F_pre / 2 (rounded once), and (F_pre + F_post) / 2 with 16 more bits,
+        // whose rounding error is carried from step to step
+        i64 h[2] = {0, 0}, t[2] = {0, 0}, rest[2] = {0x8000, 0x8000};
+        if (FK != FK_NONE) {
+            const double Pd[2] = {Px, Py};
 #pragma unroll
-                for (int a = 0; a < 9; a++) put(a, f[a]);
+            for (int d = 0; d < 2; d++) {
+                const double f1 = 0.5 * apre * Pd[d], f2 = 6.0 * gsum * Pd[d];
+                const unsigned m1 = fx_hi(fx_bits(f1)) & 0x7fffffffu, m2 = fx_hi(fx_bits(f2)) & 0x7fffffffu;
+                if ((int)(max(m1, m2) >> 20) > hi - 13) bad = -1;
+                h[d] = fx_round(fx_ldexp(f1, k));
+                t[d] = fx_round(fx_ldexp(f2, k + 16));
             }
         }
-        cur ^= 1;
-        cl.sync();
-    }
-    if (own)
+        i64 *fs = reinterpret_cast<i64 *>(sm);
+        if (own) {
+            i64 X[9];
+            fx_load(f, k, X);
 #pragma unroll
-        for (int a = 0; a < 9; a++) fout[a * g.Np + i] = sm[cur * 9 * P + a * P + l];
+            for (int a = 0; a < 9; a++) fs[a * P + l] = X[a];
+        }
+        cl.sync();
+        int cur = 0;
+        for (int n = 0; n < nsteps; n++) {
+            if (own) {
+                i64 X[9];
+#pragma unroll
+                for (int a = 0; a < 9; a++) X[a] = cl.map_shared_rank(fs + cur * 9 * P, src_blk[a])[src_off[a]];
+                i64 add[2] = {0, 0};
+                if (FK != FK_NONE) {
+#pragma unroll
+                    for (int d = 0; d < 2; d++) {
+                        rest[d] += t[d];
+                        add[d] = rest[d] >> 16;
+                        rest[d] &= 0xffff;
+                    }
+                }
+                fx_collide9_run(X, h, add, fx, bad);
+                i64 *nxt = fs + (cur ^ 1) * 9 * P;
+#pragma unroll
+                for (int a = 0; a < 9; a++) nxt[a * P + l] = X[a];
+            }
+            cur ^= 1;
+            cl.sync();
+        }
+        if (own && bad < 0) range[2] = 1;
+        cl.sync();
+        int failed = 0;
+        for (int r = 0; r < nblk; r++) failed |= cl.map_shared_rank(range, r)[2];
+        fixed = !failed;
+        if (fixed && own)
+#pragma unroll
+            for (int a = 0; a < 9; a++) fout[a * g.Np + i] = fx_value(fs[cur * 9 * P + a * P + l], k);
+    }
+    if (!fixed) {
+        if (W1) cl.sync();  // every block has read its neighbours' last results
+        auto shape = [&](int d) { return d == 0 ? Px : Py; };
+        if (own)
+#pragma unroll
+            for (int a = 0; a < 9; a++) sm[a * P + l] = fin[a * g.Np + i];
+        cl.sync();
+        int cur = 0;
+        for (int n = 0; n < nsteps; n++) {
+            if (own) {
+                double f[9];
+#pragma unroll
+                for (int a = 0; a < 9; a++) f[a] = cl.map_shared_rank(sm + cur * 9 * P, src_blk[a])[src_off[a]];
+                double_step9<W1, false>(f, w, FK != FK_NONE, apre, gsum, shape);
+                double *nxt = sm + (cur ^ 1) * 9 * P;
+#pragma unroll
+                for (int a = 0; a < 9; a++) nxt[a * P + l] = f[a];
+            }
+            cur ^= 1;
+            cl.sync();
+        }
+        if (own)
+#pragma unroll
+            for (int a = 0; a < 9; a++) fout[a * g.Np + i] = sm[cur * 9 * P + a * P + l];
+    }
+    cl.sync();  // no block leaves while another may still read its shared memory
 }
 
 // Batched form: one launch for every lattice of a batch; pairs hold
-// (a_pre, (a_pre + a_post)/12) per step and item.
+// (a_pre / 4, (a_pre + a_post) / 4) per step and item.
 // One node of a batched launch (member `it`, node i; B staged in shared memory).
 __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch &L, int it, int i)
 {
@@ -304,21 +383,21 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     node_xy(g, i, x, y);
     double f[9];
     load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-    if (L.mrho) fused_fields<LD2Q9>(B, L, it, i, x, y, 0, f, ap.x);  // fused readback of f(t)'s fields
+    if (L.mrho) fused_fields<LD2Q9>(B, L, it, i, x, y, 0, f, 4.0 * ap.x);  // fused readback of f(t)'s fields
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, 0, i) : 0.0; };
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates9 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
     if (B.variant == 3) {  // uniform over the member
-        if (fixed_step9<true, true>(f, B.fx, 0.25 * ap.x, 3.0 * ap.y, shape, put)) return;
+        if (fixed_step9<true, true>(f, B.fx, ap.x, ap.y, shape, put)) return;
         load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-        double_step9<true, true>(f, w, forced, ap.x, ap.y, shape);
+        double_step9<true, true>(f, w, forced, 4.0 * ap.x, ap.y / 3.0, shape);
     } else if (B.variant == 1) {
-        if (fixed_step9<true, false>(f, B.fx, 0.25 * ap.x, 3.0 * ap.y, shape, put)) return;
+        if (fixed_step9<true, false>(f, B.fx, ap.x, ap.y, shape, put)) return;
         load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-        double_step9<true, false>(f, w, forced, ap.x, ap.y, shape);
+        double_step9<true, false>(f, w, forced, 4.0 * ap.x, ap.y / 3.0, shape);
     } else {
-        double_step9<false, false>(f, w, forced, ap.x, ap.y, shape);
+        double_step9<false, false>(f, w, forced, 4.0 * ap.x, ap.y / 3.0, shape);
     }
 #pragma unroll
     for (int a = 0; a < 9; a++) put(a, f[a]);
@@ -354,20 +433,22 @@ cudaError_t cluster_launch(cudaLaunchConfig_t &cfg, int C, const LaunchArgs &a, 
 }
 
 template <bool W1>
-void step_launch(const LaunchArgs &a, int grid, double gsum, const Rates9 &w)
+void step_launch(const LaunchArgs &a, double gsum, const Rates9 &w)
 {
+    const int block = spread_block(a.g.N, kBlock), grid = (a.g.N + block - 1) / block;
+    const double q1 = 0.25 * a.apre, q2 = 0.25 * (a.apre + a.apost);
     const Planes<double, 9> P = make_planes<double, 9>(a.fin, a.fout, a.g.Np);
     const bool xo = W1 && force_x_only(a.fkind, a.F, 2);
     const FxRates fx = fx_rates9(a.omega[3], a.omega[4], a.omega[5]);
     switch (a.fkind) {
-    case FK_NONE: k_step<FK_NONE, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx); break;
+    case FK_NONE: k_step<FK_NONE, W1, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2); break;
     case FK_CONST:
-        if (xo) k_step<FK_CONST, W1, W1><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
-        else k_step<FK_CONST, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
+        if (xo) k_step<FK_CONST, W1, W1><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
+        else k_step<FK_CONST, W1, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
         break;
     default:
-        if (xo) k_step<FK_GENERAL, W1, W1><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
-        else k_step<FK_GENERAL, W1, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx);
+        if (xo) k_step<FK_GENERAL, W1, W1><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
+        else k_step<FK_GENERAL, W1, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
         break;
     }
 }
@@ -433,9 +514,8 @@ cudaError_t d2q9_step(const LaunchArgs &a)
     Rates9 w{a.omega[3] / 12.0, a.omega[4] / 4.0, a.omega[5] / 4.0,
              a.omega[6] / 4.0, a.omega[7] / 4.0, a.omega[8] / 4.0};
     const double gsum = (a.apre + a.apost) / 12.0;
-    const int grid = (a.g.N + kBlock - 1) / kBlock;
-    if (d2q9_high_rates_one(a.omega)) step_launch<true>(a, grid, gsum, w);
-    else step_launch<false>(a, grid, gsum, w);
+    if (d2q9_high_rates_one(a.omega)) step_launch<true>(a, gsum, w);
+    else step_launch<false>(a, gsum, w);
     return cudaGetLastError();
 }
 

@@ -164,7 +164,7 @@ __device__ __forceinline__ void double_step15(double (&f)[15], const Rates15 &w,
 template <int FK, bool FIX, bool XO>
 __global__ void __launch_bounds__(kBlock)
 k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double apre, double apost, Rates15 w,
-       FxRates fx)
+       FxRates fx, double q1, double q2)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
@@ -174,7 +174,7 @@ k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double
     load_pulled<LD3Q15>(P, g, x, y, z, i, f);
     auto shape = [&](int d) { return field_value(Fd, FK, d, x, y, z, i); };
     if (FIX) {
-        if (fixed_step15<FK != FK_NONE, XO>(f, fx, 0.25 * apre, 0.25 * (apre + apost), shape,
+        if (fixed_step15<FK != FK_NONE, XO>(f, fx, q1, q2, shape,
                                             [&](int a, double v) { P.out[a][i] = v; }))
             return;
         load_pulled<LD3Q15>(P, g, x, y, z, i, f);
@@ -184,7 +184,7 @@ k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double
     for (int a = 0; a < 15; a++) P.out[a][i] = f[a];
 }
 
-// Batched form; pairs hold (a_pre, a_post) per step and item.
+// Batched form; pairs hold (a_pre / 4, (a_pre + a_post) / 4) per step and item.
 // One node of a batched launch (member `it`, node i; B staged in shared memory).
 __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch &L, int it, int i)
 {
@@ -197,17 +197,17 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     node_xyz(g, i, x, y, z);
     double f[15];
     load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
-    if (L.mrho) fused_fields<LD3Q15>(B, L, it, i, x, y, z, f, ap.x);  // fused readback of f(t)'s fields
+    if (L.mrho) fused_fields<LD3Q15>(B, L, it, i, x, y, z, f, 4.0 * ap.x);  // fused readback of f(t)'s fields
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     const Rates15 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3]};
     if (w.t == 1.0 && w.q == 1.0) {  // uniform over the member
-        if (fixed_step15<true, false>(f, B.fx, 0.25 * ap.x, 0.25 * (ap.x + ap.y), shape,
+        if (fixed_step15<true, false>(f, B.fx, ap.x, ap.y, shape,
                                       [&](int a, double v) { fout[a * g.Np + i] = v; }))
             return;
         load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
     }
-    double_step15(f, w, forced, ap.x, ap.y, shape);
+    double_step15(f, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
 #pragma unroll
     for (int a = 0; a < 15; a++) fout[a * g.Np + i] = f[a];
 }
@@ -244,10 +244,11 @@ cudaError_t d3q15_step(const LaunchArgs &a)
 {
     const Rates15 w{a.omega[2], a.omega[1], a.omega[3], a.omega[4]};
     const FxRates fx = fx_rates27(a.omega[1], a.omega[2]);
+    const double q1 = 0.25 * a.apre, q2 = 0.25 * (a.apre + a.apost);
     const Planes<double, 15> P = make_planes<double, 15>(a.fin, a.fout, a.g.Np);
     const bool fix = w.t == 1.0 && w.q == 1.0, xo = force_x_only(a.fkind, a.F, 3);
     const int block = spread_block(a.g.N, kBlock), grid = (a.g.N + block - 1) / block;
-#define STEP15(FK, FIX, XO) k_step<FK, FIX, XO><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx)
+#define STEP15(FK, FIX, XO) k_step<FK, FIX, XO><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2)
     switch (a.fkind) {
     case FK_NONE:
         if (fix) STEP15(FK_NONE, true, false);

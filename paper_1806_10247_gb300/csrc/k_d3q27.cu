@@ -26,8 +26,6 @@
 namespace lbmk {
 namespace {
 
-constexpr int kBlock = 256;
-
 struct Rates27 {
     double wb, ws, w3, w4, w5, w6;
 };
@@ -357,13 +355,20 @@ __device__ __forceinline__ void double_step27(double (&m)[27], const Rates27 &w,
     else collide<XO>(m, F, Fq, w);
 }
 
+// 6 resident blocks of 128 threads (80 registers, 40 bytes spilled): the step
+// waits for the conversions' results and for integer chains more than for
+// memory, so warps in flight matter.  Kolmogorov 256^3 FP64, 4 steps and the
+// fields: 2 blocks of 256 threads 9.63 ms, 4 of 128 8.41, 5 of 128 8.37, 6 of 128
+// 8.16; 8 or 10 of 64 8.38 / 8.36.
+constexpr int kStepBlock = 128, kStepMinBlocks = 6;
+
 // XO: the force has no y and z components (checked on the host).
 template <int FK, bool W1, bool XO>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kStepBlock, W1 ? kStepMinBlocks : 1)
 k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double apre, double apost, Rates27 w,
-       FxRates fx)
+       FxRates fx, double q1, double q2)
 {
-    int i = blockIdx.x * kBlock + threadIdx.x;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y, z;
     node_xyz(g, i, x, y, z);
@@ -371,7 +376,7 @@ k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double
     load_pulled<LD3Q27>(P, g, x, y, z, i, m);
     auto shape = [&](int d) { return field_value(Fd, FK, d, x, y, z, i); };
     if (W1) {
-        if (fixed_step27<FK != FK_NONE, XO>(m, fx, 0.25 * apre, 0.25 * (apre + apost), shape,
+        if (fixed_step27<FK != FK_NONE, XO>(m, fx, q1, q2, shape,
                                             [&](int a, double v) { P.out[a][i] = v; }))
             return;
         load_pulled<LD3Q27>(P, g, x, y, z, i, m);
@@ -381,7 +386,7 @@ k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double
     for (int a = 0; a < 27; a++) P.out[a][i] = m[a];
 }
 
-// Batched form; pairs hold (a_pre, a_post) per step and item.
+// Batched form; pairs hold (a_pre / 4, (a_pre + a_post) / 4) per step and item.
 // One node of a batched launch (member `it`, node i; B staged in shared memory).
 __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch &L, int it, int i)
 {
@@ -395,28 +400,29 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     double m[27];
     load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
     // fused readback of f(t)'s fields
-    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, ap.x);
+    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, 4.0 * ap.x);
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates27 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
     if (B.variant == 3) {  // uniform over the member
-        if (fixed_step27<true, true>(m, B.fx, 0.25 * ap.x, 0.25 * (ap.x + ap.y), shape, put)) return;
+        if (fixed_step27<true, true>(m, B.fx, ap.x, ap.y, shape, put)) return;
         load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
-        double_step27<true, true>(m, w, forced, ap.x, ap.y, shape);
+        double_step27<true, true>(m, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
     } else if (B.variant == 1) {
-        if (fixed_step27<true, false>(m, B.fx, 0.25 * ap.x, 0.25 * (ap.x + ap.y), shape, put)) return;
+        if (fixed_step27<true, false>(m, B.fx, ap.x, ap.y, shape, put)) return;
         load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
-        double_step27<true, false>(m, w, forced, ap.x, ap.y, shape);
+        double_step27<true, false>(m, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
     } else {
-        double_step27<false, false>(m, w, forced, ap.x, ap.y, shape);
+        double_step27<false, false>(m, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
     }
 #pragma unroll
     for (int a = 0; a < 27; a++) put(a, m[a]);
 }
 
+// At most 128 registers: 16 warps per SM at every tile size.
 template <int TB, int MODE>
-__global__ void __launch_bounds__(TB) k_batch(const __grid_constant__ BatchLaunch L)
+__global__ void __launch_bounds__(TB, 512 / TB) k_batch(const __grid_constant__ BatchLaunch L)
 {
     batch_tiles<TB, MODE>(L, [](const BatchItem &B, const BatchLaunch &L2, int it, int i) { batch_node(B, L2, it, i); });
 }
@@ -447,25 +453,26 @@ bool d3q27_high_rates_one(const double omega[9]) { return high_rates_one(omega);
 cudaError_t d3q27_step(const LaunchArgs &a)
 {
     Rates27 w{a.omega[1], a.omega[2], a.omega[3], a.omega[4], a.omega[5], a.omega[6]};
-    const int grid = (a.g.N + kBlock - 1) / kBlock;
+    const int block = spread_block(a.g.N, kStepBlock), grid = (a.g.N + block - 1) / block;
+    const double q1 = 0.25 * a.apre, q2 = 0.25 * (a.apre + a.apost);
     const bool w1 = high_rates_one(a.omega);
     const Planes<double, 27> P = make_planes<double, 27>(a.fin, a.fout, a.g.Np);
     const bool xo = force_x_only(a.fkind, a.F, 3);
     const FxRates fx = fx_rates27(a.omega[1], a.omega[2]);
     switch (a.fkind) {
     case FK_NONE:
-        if (w1) k_step<FK_NONE, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
-        else k_step<FK_NONE, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        if (w1) k_step<FK_NONE, true, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
+        else k_step<FK_NONE, false, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
         break;
     case FK_CONST:
-        if (w1 && xo) k_step<FK_CONST, true, true><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
-        else if (w1) k_step<FK_CONST, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
-        else k_step<FK_CONST, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        if (w1 && xo) k_step<FK_CONST, true, true><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
+        else if (w1) k_step<FK_CONST, true, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
+        else k_step<FK_CONST, false, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
         break;
     default:
-        if (w1 && xo) k_step<FK_GENERAL, true, true><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
-        else if (w1) k_step<FK_GENERAL, true, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
-        else k_step<FK_GENERAL, false, false><<<grid, kBlock, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx);
+        if (w1 && xo) k_step<FK_GENERAL, true, true><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
+        else if (w1) k_step<FK_GENERAL, true, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
+        else k_step<FK_GENERAL, false, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
         break;
     }
     return cudaGetLastError();

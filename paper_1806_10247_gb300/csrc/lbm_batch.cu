@@ -117,20 +117,21 @@ int bfail(lbm_batch *b, int code, const char *fmt, ...)
         if (e_ != cudaSuccess) return bfail(b, LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e_)); \
     } while (0)
 
-// Second value of a step's envelope pair as the batched kernels expect it:
-// D2Q9 (a_pre + a_post)/12, D2Q5 (a_pre + a_post)/10, D3Q27 and D3Q15 a_post --
-// the same expressions as the single-lattice launchers.
-double pair_second(int lattice, double apre, double apost)
+// A step's envelope pair as the FP64 batched kernels take it: quarters of a_pre
+// and of a_pre + a_post for the flow lattices (halved moments), halves for D2Q5.
+double2 pair64(int lattice, double apre, double apost)
 {
-    if (lattice == LBM_D2Q9) return (apre + apost) / 12.0;
-    if (lattice == LBM_D2Q5_CDE) return (apre + apost) / 10.0;
-    return apost;
+    const double c = lattice == LBM_D2Q5_CDE ? 0.5 : 0.25;
+    return make_double2(c * apre, c * (apre + apost));
 }
-
-// First value of an FP64 pair: a_pre, halved for D2Q5 (its step takes
-// g_0 + (a_pre/2) S; halving is exact, so a kernel that needs a_pre itself
-// doubles it back exactly).  Reduced-precision pairs carry a_pre.
-double pair_first(int lattice, double apre) { return lattice == LBM_D2Q5_CDE ? 0.5 * apre : apre; }
+// The pair of the reduced-precision kernels: a_pre and D2Q9 (a_pre + a_post)/12,
+// D2Q5 (a_pre + a_post)/10, D3Q27 a_post -- the same expressions as the
+// single-lattice launchers.
+float2 pair32(int lattice, double apre, double apost)
+{
+    const double second = lattice == LBM_D2Q9 ? (apre + apost) / 12.0 : (lattice == LBM_D2Q5_CDE ? (apre + apost) / 10.0 : apost);
+    return make_float2((float)apre, (float)second);
+}
 
 int grow_pairs(lbm_batch *b, int s, size_t need)
 {
@@ -429,10 +430,9 @@ void fill_pairs(const lbm_batch *b, void *dst, long k)
         for (long s = 0; s < k; s++) {
             double apre, apost;
             lbmc::envelope_pair(c, c->t + s, apre, apost);
-            const double second = pair_second(b->lattice, apre, apost);
             const size_t at = (size_t)s * b->count + i;
-            if (fp32) reinterpret_cast<float2 *>(dst)[at] = make_float2((float)apre, (float)second);
-            else reinterpret_cast<double2 *>(dst)[at] = make_double2(pair_first(b->lattice, apre), second);
+            if (fp32) reinterpret_cast<float2 *>(dst)[at] = pair32(b->lattice, apre, apost);
+            else reinterpret_cast<double2 *>(dst)[at] = pair64(b->lattice, apre, apost);
         }
     }
 }
@@ -465,9 +465,8 @@ void inline_pairs_of_step(const lbm_batch *b, BatchLaunch &L, long k)
     for (int i = 0; i < b->count; i++) {
         double apre, apost;
         lbmc::envelope_pair(b->ctx[i], b->ctx[i]->t + k, apre, apost);
-        const double second = pair_second(b->lattice, apre, apost);
-        L.inl[i] = make_double2(pair_first(b->lattice, apre), second);
-        L.inlf[i] = make_float2((float)apre, (float)second);
+        L.inl[i] = pair64(b->lattice, apre, apost);
+        L.inlf[i] = pair32(b->lattice, apre, apost);
     }
 }
 
