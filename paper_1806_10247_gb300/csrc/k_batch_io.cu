@@ -33,8 +33,8 @@ __device__ __forceinline__ void member_moments(const BatchItem &B, const BatchMo
         m0 += B.rho_ref;  // the rest state carries no momentum
     }
     const bool forced = M.half && B.fkind != FK_NONE;
-    const double apre = M.apre ? __ldg(M.apre + it) : M.apre_inl[it];
-    store_fields<L>(m0, j, forced, apre, B.F, B.fkind, x, y, z, i, g.N, __ldg(M.off + it), M.rho, M.u);
+    const double ahalf = M.ahalf ? __ldg(M.ahalf + it) : M.ahalf_inl[it];
+    store_fields<L>(m0, j, forced, ahalf, B.F, B.fkind, x, y, z, i, g.N, __ldg(M.off + it), M.rho, M.u);
 }
 
 template <class L, class T>

@@ -100,7 +100,7 @@ k_gather(Geom g, const double *__restrict__ stored, double *__restrict__ plain)
 // h * Eq. 43 (scalar).  Outputs are dense [N] / [dim][N] arrays.
 template <class L>
 __global__ void __launch_bounds__(kBlock)
-k_moments(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, double apre, int half,
+k_moments(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, double ahalf, int half,
           double *__restrict__ rho, double *__restrict__ u)
 {
     int i = blockIdx.x * kBlock + threadIdx.x;
@@ -111,7 +111,7 @@ k_moments(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, double 
     load_pulled<L>(fin, g, x, y, z, i, f);
     double m0, j[3];
     zeroth_first<L>(f, m0, j);
-    store_fields<L>(m0, j, half && fkind != FK_NONE, apre, F, fkind, x, y, z, i, g.N, 0, rho, u);
+    store_fields<L>(m0, j, half && fkind != FK_NONE, ahalf, F, fkind, x, y, z, i, g.N, 0, rho, u);
 }
 
 // Reduction slots.
@@ -159,7 +159,7 @@ __device__ void block_reduce_store(double (&v)[R_SLOTS], double *out)
 // then overwritten), and a flag for non-finite or non-positive densities.
 template <class L>
 __global__ void __launch_bounds__(kBlock)
-k_reduce_partial(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, double apre,
+k_reduce_partial(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, double ahalf,
                  double *__restrict__ snap, int have_snap, double *__restrict__ partials)
 {
     double v[R_SLOTS] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -174,15 +174,16 @@ k_reduce_partial(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, 
         v[R_MASS] += m0;
         bool bad = !isfinite(m0) || (L::Q != 5 && !(m0 > 0.0));
         if (L::Q == 5) {
-            double phi = fkind != FK_NONE ? m0 + 0.5 * (apre * field_value(F, fkind, 0, x, y, z, i)) : m0;
+            double phi = fkind != FK_NONE ? m0 + ahalf * field_value(F, fkind, 0, x, y, z, i) : m0;
             if (have_snap) v[R_DU] = fmax(v[R_DU], fabs(phi - snap[i]));
             snap[i] = phi;
         } else {
+            const double rinv = recip_density(m0);
 #pragma unroll
             for (int d = 0; d < L::DIM; d++) {
                 v[R_JX + d] += j[d];
-                double jd = fkind != FK_NONE ? j[d] + 0.5 * (apre * field_value(F, fkind, d, x, y, z, i)) : j[d];
-                double ud = jd / m0;
+                double jd = field_zero(F, fkind, d) ? j[d] : j[d] + ahalf * field_value(F, fkind, d, x, y, z, i);
+                double ud = jd * rinv;
                 bad = bad || !isfinite(ud);
                 if (have_snap) v[R_DU] = fmax(v[R_DU], fabs(ud - snap[(long long)d * g.N + i]));
                 snap[(long long)d * g.N + i] = ud;
@@ -220,7 +221,7 @@ k_reduce_partial_sums(Geom g, const double *__restrict__ fin, double *__restrict
 
 template <class L, class T>
 __global__ void __launch_bounds__(kBlock)
-k_reduce_partial_rp(Geom g, const T *__restrict__ fin, double rho_ref, int fkind, FieldDev F, double apre,
+k_reduce_partial_rp(Geom g, const T *__restrict__ fin, double rho_ref, int fkind, FieldDev F, double ahalf,
                     double *__restrict__ snap, int have_snap, int with_snap, double *__restrict__ partials)
 {
     double v[R_SLOTS] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -235,17 +236,18 @@ k_reduce_partial_rp(Geom g, const T *__restrict__ fin, double rho_ref, int fkind
         bool bad = !isfinite(m0) || (L::Q != 5 && !(m0 > 0.0));
         if (L::Q == 5) {
             if (with_snap) {
-                double phi = fkind != FK_NONE ? m0 + 0.5 * (apre * field_value(F, fkind, 0, x, y, z, i)) : m0;
+                double phi = fkind != FK_NONE ? m0 + ahalf * field_value(F, fkind, 0, x, y, z, i) : m0;
                 if (have_snap) v[R_DU] = fmax(v[R_DU], fabs(phi - snap[i]));
                 snap[i] = phi;
             }
         } else {
+            const double rinv = with_snap ? recip_density(m0) : 0.0;
 #pragma unroll
             for (int d = 0; d < L::DIM; d++) {
                 v[R_JX + d] += j[d];
                 if (with_snap) {
-                    double jd = fkind != FK_NONE ? j[d] + 0.5 * (apre * field_value(F, fkind, d, x, y, z, i)) : j[d];
-                    double ud = jd / m0;
+                    double jd = field_zero(F, fkind, d) ? j[d] : j[d] + ahalf * field_value(F, fkind, d, x, y, z, i);
+                    double ud = jd * rinv;
                     bad = bad || !isfinite(ud);
                     if (have_snap) v[R_DU] = fmax(v[R_DU], fabs(ud - snap[(long long)d * g.N + i]));
                     snap[(long long)d * g.N + i] = ud;
@@ -365,7 +367,7 @@ k_gather_rp(Geom g, double rho_ref, Ref5 R, const T *__restrict__ stored, double
 
 template <class L, class T>
 __global__ void __launch_bounds__(kBlock)
-k_moments_rp(Geom g, const T *__restrict__ fin, double rho_ref, int fkind, FieldDev F, double apre, int half,
+k_moments_rp(Geom g, const T *__restrict__ fin, double rho_ref, int fkind, FieldDev F, double ahalf, int half,
              double *__restrict__ rho, double *__restrict__ u)
 {
     int i = blockIdx.x * kBlock + threadIdx.x;
@@ -375,7 +377,7 @@ k_moments_rp(Geom g, const T *__restrict__ fin, double rho_ref, int fkind, Field
     double dm0, j[3];
     dev_moments<L, T>(fin, g, x, y, z, i, dm0, j);
     const double m0 = rho_ref + dm0;
-    store_fields<L>(m0, j, half && fkind != FK_NONE, apre, F, fkind, x, y, z, i, g.N, 0, rho, u);
+    store_fields<L>(m0, j, half && fkind != FK_NONE, ahalf, F, fkind, x, y, z, i, g.N, 0, rho, u);
 }
 
 // Strain rate from the non-equilibrium second moments (Sec. 6.6): with
@@ -560,13 +562,13 @@ cudaError_t moments(int lattice, const LaunchArgs &a, double *rho, double *u, in
             return by_storage(a.storage, [&](auto T) {
                 using TT = decltype(T);
                 k_moments_rp<LT, TT><<<grid_for(a.g.N), kBlock, 0, a.stream>>>(
-                    a.g, reinterpret_cast<const TT *>(a.fin), a.rho_ref, a.fkind, a.F, a.apre, half, rho, u);
+                    a.g, reinterpret_cast<const TT *>(a.fin), a.rho_ref, a.fkind, a.F, 0.5 * a.apre, half, rho, u);
                 return cudaGetLastError();
             });
         });
     return by_lattice64(lattice, [&](auto L) {
         using LT = decltype(L);
-        k_moments<LT><<<grid_for(a.g.N), kBlock, 0, a.stream>>>(a.g, a.fin, a.fkind, a.F, a.apre, half,
+        k_moments<LT><<<grid_for(a.g.N), kBlock, 0, a.stream>>>(a.g, a.fin, a.fkind, a.F, 0.5 * a.apre, half,
                                                                 rho, u);
         return cudaGetLastError();
     });
@@ -641,20 +643,20 @@ cudaError_t reduce(int lattice, const LaunchArgs &a, double *snap, int have_snap
             return by_storage(a.storage, [&](auto T) {
                 using TT = decltype(T);
                 k_reduce_partial_rp<LT, TT><<<nblocks, kBlock, 0, a.stream>>>(
-                    a.g, reinterpret_cast<const TT *>(a.fin), a.rho_ref, a.fkind, a.F, a.apre, snap, have_snap, 1,
-                    partials);
+                    a.g, reinterpret_cast<const TT *>(a.fin), a.rho_ref, a.fkind, a.F, 0.5 * a.apre, snap, have_snap, 1,
+                    nblocks == 1 ? out : partials);
                 cudaError_t e = cudaGetLastError();
-                if (e != cudaSuccess) return e;
+                if (e != cudaSuccess || nblocks == 1) return e;  // one block's sums are the sums
                 k_reduce_final<<<1, kBlock, 0, a.stream>>>(partials, nblocks, out);
                 return cudaGetLastError();
             });
         });
     return by_lattice64(lattice, [&](auto L) {
         using LT = decltype(L);
-        k_reduce_partial<LT><<<nblocks, kBlock, 0, a.stream>>>(a.g, a.fin, a.fkind, a.F, a.apre, snap,
-                                                              have_snap, partials);
+        k_reduce_partial<LT><<<nblocks, kBlock, 0, a.stream>>>(a.g, a.fin, a.fkind, a.F, 0.5 * a.apre, snap,
+                                                              have_snap, nblocks == 1 ? out : partials);
         cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || nblocks == 1) return e;
         k_reduce_final<<<1, kBlock, 0, a.stream>>>(partials, nblocks, out);
         return cudaGetLastError();
     });
@@ -764,7 +766,7 @@ cudaError_t reduce_sums(int lattice, const LaunchArgs &a, double *partials, int 
             return by_storage(a.storage, [&](auto T) {
                 using TT = decltype(T);
                 k_reduce_partial_rp<LT, TT><<<nblocks, kBlock, 0, a.stream>>>(
-                    a.g, reinterpret_cast<const TT *>(a.fin), a.rho_ref, a.fkind, a.F, a.apre, nullptr, 0, 0,
+                    a.g, reinterpret_cast<const TT *>(a.fin), a.rho_ref, a.fkind, a.F, 0.5 * a.apre, nullptr, 0, 0,
                     partials);
                 cudaError_t e = cudaGetLastError();
                 if (e != cudaSuccess) return e;

@@ -242,7 +242,7 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     node_xy(g, i, x, y);
     double f[5];
     load_pulled<LD2Q5>(fin, g, x, y, 0, i, f);
-    if (L.mrho) fused_fields<LD2Q5>(B, L, it, i, x, y, 0, f, 2.0 * ap.x);  // fused readback of f(t)'s scalar
+    if (L.mrho) fused_fields<LD2Q5>(B, L, it, i, x, y, 0, f, ap.x);  // fused readback of f(t)'s scalar
     if (B.vkind != FK_GENERAL) {
         const bool src = B.fkind != FK_NONE;
         const double P = src ? field_value(B.F, B.fkind, 0, x, y, 0, i) : 0.0;

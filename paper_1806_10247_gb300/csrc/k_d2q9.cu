@@ -383,7 +383,7 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     node_xy(g, i, x, y);
     double f[9];
     load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-    if (L.mrho) fused_fields<LD2Q9>(B, L, it, i, x, y, 0, f, 4.0 * ap.x);  // fused readback of f(t)'s fields
+    if (L.mrho) fused_fields<LD2Q9>(B, L, it, i, x, y, 0, f, 2.0 * ap.x);  // fused readback of f(t)'s fields
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, 0, i) : 0.0; };
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };

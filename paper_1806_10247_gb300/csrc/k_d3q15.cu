@@ -197,7 +197,7 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     node_xyz(g, i, x, y, z);
     double f[15];
     load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
-    if (L.mrho) fused_fields<LD3Q15>(B, L, it, i, x, y, z, f, 4.0 * ap.x);  // fused readback of f(t)'s fields
+    if (L.mrho) fused_fields<LD3Q15>(B, L, it, i, x, y, z, f, 2.0 * ap.x);  // fused readback of f(t)'s fields
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     const Rates15 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3]};

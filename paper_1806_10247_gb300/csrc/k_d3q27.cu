@@ -400,7 +400,7 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     double m[27];
     load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
     // fused readback of f(t)'s fields
-    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, 4.0 * ap.x);
+    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, 2.0 * ap.x);
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };

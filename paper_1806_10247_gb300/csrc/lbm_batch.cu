@@ -68,7 +68,7 @@ struct lbm_batch {
     // packed moments (lbm_batch_moments_packed)
     long long total_nodes = 0;
     long long *d_off = nullptr;        // first node of each member in the packed output
-    double *h_apre = nullptr;          // pinned a_pre of each member, and its device copy
+    double *h_apre = nullptr;          // pinned a_pre / 2 of each member, and its device copy
     double *d_apre = nullptr;
     cudaEvent_t ev_apre = nullptr;     // recorded after the a_pre copy
     double *d_mom = nullptr;           // device staging of the packed output (host destinations)
@@ -86,7 +86,7 @@ struct lbm_batch {
     cudaEvent_t ev_read[kReadbackSlots] = {};
     bool read_recorded[kReadbackSlots] = {};
     cudaEvent_t ev_state = nullptr;
-    double *h_apreq[kReadbackSlots] = {};  // pinned a_pre of each member, per slot
+    double *h_apreq[kReadbackSlots] = {};  // pinned a_pre / 2 of each member, per slot
     double *d_apreq[kReadbackSlots] = {};
     int qslot = 0;   // slot of the next readback (the slots are used in turn)
     bool copies_pending = false;
@@ -603,8 +603,8 @@ int packed_readback_async(lbm_batch *b, double *rho, double *u, int where, int h
     for (int i = 0; i < b->count; i++) {
         double apre, apost;
         lbmc::envelope_pair(b->ctx[i], b->ctx[i]->t, apre, apost);
-        if (inl) M.apre_inl[i] = apre;
-        else b->h_apreq[slot][i] = apre;
+        if (inl) M.ahalf_inl[i] = 0.5 * apre;
+        else b->h_apreq[slot][i] = 0.5 * apre;
     }
     // order after the state on the batch stream; a member buffer already read
     // by another batch's pending readback keeps that reader too (this copy
@@ -627,7 +627,7 @@ int packed_readback_async(lbm_batch *b, double *rho, double *u, int where, int h
     M.count = b->count;
     M.parity = parity;
     M.half = half;
-    M.apre = inl ? nullptr : b->d_apreq[slot];
+    M.ahalf = inl ? nullptr : b->d_apreq[slot];
     M.off = b->d_off;
     M.rho = drho;
     M.u = du;
@@ -930,8 +930,8 @@ int lbm_batch_moments_packed(lbm_batch *b, double *rho, double *u, int where, in
     for (int i = 0; i < b->count; i++) {
         double apre, apost;
         lbmc::envelope_pair(b->ctx[i], b->ctx[i]->t, apre, apost);
-        if (inl) M.apre_inl[i] = apre;
-        else b->h_apre[i] = apre;
+        if (inl) M.ahalf_inl[i] = 0.5 * apre;
+        else b->h_apre[i] = 0.5 * apre;
     }
     if (!inl) {
         BCK(cudaMemcpyAsync(b->d_apre, b->h_apre, b->count * sizeof(double), cudaMemcpyHostToDevice, b->stream),
@@ -943,7 +943,7 @@ int lbm_batch_moments_packed(lbm_batch *b, double *rho, double *u, int where, in
     M.count = b->count;
     M.parity = parity;
     M.half = half_forced ? 1 : 0;
-    M.apre = inl ? nullptr : b->d_apre;
+    M.ahalf = inl ? nullptr : b->d_apre;
     M.off = b->d_off;
     M.rho = drho;
     M.u = du;

@@ -963,7 +963,7 @@ int lbm_reduce(lbm_ctx *c, double out[5])
     LaunchArgs a = launch_args(c, c->A, nullptr, apre, apost);
     const int nb = reduce_blocks(c->g);
     CK(reduce(c->lattice, a, c->snap, c->have_snap ? 1 : 0, c->partials, nb, c->red_out), "reduce kernels");
-    c->launches += 2;
+    c->launches += nb == 1 ? 1 : 2;
     double r[8];
     CK(cudaMemcpyAsync(r, c->red_out, sizeof r, cudaMemcpyDeviceToHost, c->stream), "copy reduction");
     CK(cudaStreamSynchronize(c->stream), "lbm_reduce");

@@ -105,6 +105,45 @@ FX_HD float fx_rcp_approx(float x)
     return 1.0f / x;
 #endif
 }
+FX_HD unsigned fx_float_bits(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(x);
+#else
+    unsigned b;
+    memcpy(&b, &x, 4);
+    return b;
+#endif
+}
+FX_HD float fx_float(unsigned b)
+{
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float x;
+    memcpy(&x, &b, 4);
+    return x;
+#endif
+}
+// A positive normal float as a double: the exponent field re-biased, the mantissa
+// moved up (no FP64 conversion).
+FX_HD double fx_widen(float x)
+{
+    return fx_double(((u64)fx_float_bits(x) << 29) + ((u64)(1023 - 127) << 52));
+}
+// 1/x for a positive normal x, within 0.51 units of the last place: a 22-bit
+// reciprocal of the mantissa r with one third-order correction, r (1 + e + e^2),
+// e = 1 - x r; three FP64 operations (the correctly rounded division and
+// reciprocal of the maths library take about seven).
+FX_HD double fx_recip(double x)
+{
+    const u64 b = fx_bits(x);
+    const u64 m = (b & 0x000fffffffffffffull) | 0x3ff0000000000000ull;      // mantissa in [1, 2)
+    const double r = fx_widen(fx_rcp_approx(fx_float(0x3f800000u | ((unsigned)(m >> 29) & 0x7fffffu))));
+    const double e = fma(-fx_double(m), r, 1.0);
+    const double p = fma(e, e, e);
+    return fx_ldexp(fma(r, p, r), 1023 - (int)(b >> 52));
+}
 
 // ---- scale --------------------------------------------------------------------
 constexpr int kEmaxLo = 500, kEmaxHi = 1073;  // biased exponents the fixed-point forms take (2^-523 .. 2^50)
@@ -156,6 +195,27 @@ FX_HD void fx_load(const double (&f)[Q], int k, i64 (&X)[Q])
 #pragma unroll
 #endif
     for (int a = 0; a < Q; a++) X[a] = fx_round(fx_ldexp(f[a], k));
+}
+
+// The same in integers alone (a conversion costs half a clock of the FP64 unit,
+// this about a tenth of the integer units'), to nearest with halves away from
+// zero: exact for values within S - 52 binary orders of the largest.  SIGNED =
+// false takes |f|.
+template <int Q, bool SIGNED>
+FX_HD void fx_load_int(const double (&f)[Q], int emax, i64 (&X)[Q])
+{
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < Q; a++) {
+        const u64 b = fx_bits(f[a]);
+        const int e = (int)(fx_hi(b) >> 20) & 0x7ff;
+        const int sh = emax - e < 63 ? emax - e : 63;
+        const u64 m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+        const i64 v = (i64)(((m << (FxGrid<Q>::S - 51)) >> sh) + 1) >> 1;
+        const i64 s = (i64)b >> 63;
+        X[a] = SIGNED ? (v ^ s) - s : v;
+    }
 }
 
 // X 2^-k, rounded to nearest even; 0 gives 0.
@@ -229,7 +289,7 @@ FX_HD double fx_reciprocal(i64 rho, int &bad)
     const int rh = (int)(rho >> 32);
     bad |= rh - (1 << 20);
     const double r = fx_ldexp(fx_to_double(rho), -32);
-    const double x = (double)fx_rcp_approx((float)rh);
+    const double x = fx_widen(fx_rcp_approx((float)rh));
     // x (1 + e + e^2) with e = 1 - r x, |e| < 2^-19
     const double e = fma(-r, x, 1.0);
     const double p = fma(e, e, e);

@@ -223,9 +223,8 @@ __device__ __forceinline__ void sum_moments(const V (&f)[L::Q], V &m0, V (&j)[3]
 // Zeroth and first moments of a node as every FP64 readback and reduction
 // forms them: summed in fixed point (lbm_fixed.cuh), where the sums are exact,
 // and rounded once; a node outside the fixed-point range is summed in FP64.  The
-// FP64 sums of D3Q27 took 40 clocks of an SM's FP64 unit per node, the 27 + 4
-// conversions take 15.5.  D2Q5's four FP64 adds cost less than six conversions
-// and stay.
+// FP64 sums of D3Q27 took 40 clocks of an SM's FP64 unit per node, the four
+// conversions back take 2.  D2Q5's four FP64 adds stay.
 template <class L>
 __device__ __forceinline__ void zeroth_first(const double (&f)[L::Q], double &m0, double (&j)[3])
 {
@@ -233,7 +232,7 @@ __device__ __forceinline__ void zeroth_first(const double (&f)[L::Q], double &m0
     if (L::Q != 5 && fx_in_range(em)) {
         const int k = FxGrid<L::Q>::S + 1023 - em;
         i64 X[L::Q], M, J[3];
-        fx_load(f, k, X);
+        fx_load_int<L::Q, true>(f, em, X);
         sum_moments<L>(X, M, J);
         m0 = fx_value(M, k);
 #pragma unroll
@@ -284,27 +283,42 @@ __device__ __forceinline__ void zeroth_first(const float (&d)[L::Q], double &m0,
     sum_moments<L>(dd, m0, j);
 }
 
+// 1/rho of the readbacks: fx_recip for a positive normal rho, the correctly rounded
+// reciprocal for any other.
+__device__ __forceinline__ double recip_density(double rho)
+{
+    const unsigned e = fx_hi(fx_bits(rho)) >> 20;
+    return e - 1u < 2045u && e > 2u && e < 2044u ? fx_recip(rho) : __drcp_rn(rho);
+}
+
+// Whether component c of a shape is known to vanish everywhere.
+__device__ __forceinline__ bool field_zero(const FieldDev &F, int kind, int c)
+{
+    return kind == FK_NONE || (kind == FK_CONST ? F.cval[c] == 0.0 : ((F.zmask >> c) & 1) != 0);
+}
+
 // The packed fields of a node from its zeroth and first moments, as every
 // readback writes them: rho (phi for the scalar lattice) at rho[off + i],
-// velocity component d at u[dim * off + d * N + i] = j_d (1/rho), with 1/rho
-// correctly rounded; with `forced` the pre-collision half force / source
-// a_pre P / 2 is included (Eq. 25 / 43).  Rounded operation by operation (no
-// contraction), so that every kernel that forms them gives the same bits.
+// velocity component d at u[dim * off + d * N + i] = j_d (1/rho); with `forced`
+// the pre-collision half force / source (a_pre / 2) P is included (Eq. 25 / 43;
+// ahalf = a_pre / 2, components that vanish everywhere are left out).  Rounded
+// operation by operation (no contraction), so that every kernel that forms them
+// gives the same bits.
 template <class L>
-__device__ __forceinline__ void store_fields(double m0, const double (&j)[3], bool forced, double apre, const FieldDev &F,
+__device__ __forceinline__ void store_fields(double m0, const double (&j)[3], bool forced, double ahalf, const FieldDev &F,
                                              int fkind, int x, int y, int z, int i, int N, long long off, double *rho,
                                              double *u)
 {
     if (L::Q == 5) {
-        rho[off + i] = forced ? __dadd_rn(m0, __dmul_rn(0.5, __dmul_rn(apre, field_value(F, fkind, 0, x, y, z, i)))) : m0;
+        rho[off + i] = forced ? __dadd_rn(m0, __dmul_rn(ahalf, field_value(F, fkind, 0, x, y, z, i))) : m0;
         return;
     }
     rho[off + i] = m0;
-    const double rinv = __drcp_rn(m0);
+    const double rinv = recip_density(m0);
 #pragma unroll
     for (int d = 0; d < L::DIM; d++) {
-        const double jd =
-            forced ? __dadd_rn(j[d], __dmul_rn(0.5, __dmul_rn(apre, field_value(F, fkind, d, x, y, z, i)))) : j[d];
+        double jd = j[d];
+        if (forced && !field_zero(F, fkind, d)) jd = __dadd_rn(jd, __dmul_rn(ahalf, field_value(F, fkind, d, x, y, z, i)));
         u[L::DIM * off + (long long)d * N + i] = __dmul_rn(jd, rinv);
     }
 }

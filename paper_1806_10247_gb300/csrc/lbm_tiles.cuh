@@ -83,11 +83,11 @@ __device__ __forceinline__ void batch_tiles(const BatchLaunch &L, Node node)
 // the packed readback kernel forms them.
 template <class L>
 __device__ __forceinline__ void fused_fields(const BatchItem &B, const BatchLaunch &Ln, int it, int i, int x, int y, int z,
-                                             const double (&f)[L::Q], double apre)
+                                             const double (&f)[L::Q], double ahalf)
 {
     double m0, j[3];
     zeroth_first<L>(f, m0, j);
-    store_fields<L>(m0, j, Ln.mhalf && B.fkind != FK_NONE, apre, B.F, B.fkind, x, y, z, i, B.g.N, __ldg(Ln.moff + it),
+    store_fields<L>(m0, j, Ln.mhalf && B.fkind != FK_NONE, ahalf, B.F, B.fkind, x, y, z, i, B.g.N, __ldg(Ln.moff + it),
                     Ln.mrho, Ln.mu);
 }
 
