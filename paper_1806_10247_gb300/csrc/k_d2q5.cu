@@ -154,7 +154,7 @@ __device__ __forceinline__ bool fixed_step5(const double (&f)[5], const FxCoef5 
     FxForce S{0, 0};
     if (SRC && !fx_force(P, q1, q2, k - 1, em, (unsigned)fx_bits(f[0]), S)) bad = -1;
     i64 X[5];
-    fx_load(f, k, X);
+    fx_load_int<5, true>(f, em, X);
     fx_collide5(X, S.h1, S.h2, c);
 #pragma unroll
     for (int a = 0; a < 5; a++) put(a, fx_value_signed(X[a], k, bad));

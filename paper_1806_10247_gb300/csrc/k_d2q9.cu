@@ -159,8 +159,12 @@ __device__ __forceinline__ bool fixed_step9(const double (&f)[9], const FxRates 
         for (int d = 0; d < (XO ? 1 : 2); d++)
             if (!fx_force(shape(d), q1, q2, k, em, dither >> (8 * d), F[d])) bad = -1;
     }
+    // D2Q9's populations at rest lie within the five binary orders that convert
+    // exactly; a negative one takes the FP64 form
     i64 X[9];
-    fx_load(f, k, X);
+    fx_load_int<9, false>(f, em, X);
+#pragma unroll
+    for (int a = 0; a < 9; a++) bad |= (int)fx_hi(fx_bits(f[a]));
     FxSums9<i64> s;
     fx_sums9(X, s);
     fx_collide9<XO>(s, F, w, X, bad);

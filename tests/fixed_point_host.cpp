@@ -15,7 +15,14 @@ static void run(long n, double *f, int *ok, Collide collide)
         int bad = fx_in_range(em) ? 0 : -1;
         if (bad == 0) {
             i64 X[Q];
-            fx_load(v, k, X);
+            if constexpr (Q == 9) {  // the kernels' own way in: see fixed_step9 and fixed_step5
+                fx_load_int<9, false>(v, em, X);
+                for (int a = 0; a < 9; a++) bad |= (int)fx_hi(fx_bits(v[a]));
+            } else if constexpr (Q == 5) {
+                fx_load_int<5, true>(v, em, X);
+            } else {
+                fx_load(v, k, X);
+            }
             collide(i, v, X, k, em, bad);
             for (int a = 0; a < Q; a++)
                 v[a] = Q == 5 ? fx_value_signed(X[a], k, bad) : fx_value_pos(X[a], k + 1, bad);
