@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step_mat(const __grid_constant__ Planes<double, 5> P, Geom g, FieldDev S, double ahalf, double hsum, Mat5 M,
            const __grid_constant__ FxCoef5 fx, double q2)
 {
+    step_begin();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
@@ -187,6 +188,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step(const __grid_constant__ Planes<double, 5> P, Geom g, FieldDev S, FieldDev V, double apre, double hsum,
        Rates5 w)
 {
+    step_begin();
     int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
@@ -216,13 +218,13 @@ void launch_v(const LaunchArgs &a, int grid, double hsum, const Rates5 &w)
         const double ux = a.vkind == FK_CONST ? a.V.cval[0] : 0.0;
         const double uy = a.vkind == FK_CONST ? a.V.cval[1] : 0.0;
         const int block = spread_block(a.g.N, kBlock);
-        k_step_mat<SK><<<(a.g.N + block - 1) / block, block, 0, a.stream>>>(make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
+        launch_step(a.overlap, k_step_mat<SK>, (a.g.N + block - 1) / block, block, a.stream, make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
                                                        0.5 * a.apre, hsum, make_mat(make_coef(w, ux, uy)),
                                                        fx_coef5(w.c1, w.c2, w.c3, w.c4, ux, uy),
                                                        0.5 * (a.apre + a.apost));
         return;
     }
-    k_step<SK, FK_GENERAL><<<grid, kBlock, 0, a.stream>>>(make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
+    launch_step(a.overlap, k_step<SK, FK_GENERAL>, grid, kBlock, a.stream, make_planes<double, 5>(a.fin, a.fout, a.g.Np), a.g, a.F,
                                                           a.V, a.apre, hsum, w);
 }
 

@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double apre, double gsum, Rates9 w, FxRates fx,
        double q1, double q2)
 {
+    step_begin();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
@@ -445,14 +446,14 @@ void step_launch(const LaunchArgs &a, double gsum, const Rates9 &w)
     const bool xo = W1 && force_x_only(a.fkind, a.F, 2);
     const FxRates fx = fx_rates9(a.omega[3], a.omega[4], a.omega[5]);
     switch (a.fkind) {
-    case FK_NONE: k_step<FK_NONE, W1, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2); break;
+    case FK_NONE: launch_step(a.overlap, k_step<FK_NONE, W1, false>, grid, block, a.stream, P, a.g, a.F, a.apre, gsum, w, fx, q1, q2); break;
     case FK_CONST:
-        if (xo) k_step<FK_CONST, W1, W1><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
-        else k_step<FK_CONST, W1, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
+        if (xo) launch_step(a.overlap, k_step<FK_CONST, W1, W1>, grid, block, a.stream, P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
+        else launch_step(a.overlap, k_step<FK_CONST, W1, false>, grid, block, a.stream, P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
         break;
     default:
-        if (xo) k_step<FK_GENERAL, W1, W1><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
-        else k_step<FK_GENERAL, W1, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
+        if (xo) launch_step(a.overlap, k_step<FK_GENERAL, W1, W1>, grid, block, a.stream, P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
+        else launch_step(a.overlap, k_step<FK_GENERAL, W1, false>, grid, block, a.stream, P, a.g, a.F, a.apre, gsum, w, fx, q1, q2);
         break;
     }
 }

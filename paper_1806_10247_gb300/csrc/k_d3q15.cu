@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double apre, double apost, Rates15 w,
        FxRates fx, double q1, double q2)
 {
+    step_begin();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y, z;
@@ -248,7 +249,7 @@ cudaError_t d3q15_step(const LaunchArgs &a)
     const Planes<double, 15> P = make_planes<double, 15>(a.fin, a.fout, a.g.Np);
     const bool fix = w.t == 1.0 && w.q == 1.0, xo = force_x_only(a.fkind, a.F, 3);
     const int block = spread_block(a.g.N, kBlock), grid = (a.g.N + block - 1) / block;
-#define STEP15(FK, FIX, XO) k_step<FK, FIX, XO><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2)
+#define STEP15(FK, FIX, XO) launch_step(a.overlap, k_step<FK, FIX, XO>, grid, block, a.stream, P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2)
     switch (a.fkind) {
     case FK_NONE:
         if (fix) STEP15(FK_NONE, true, false);

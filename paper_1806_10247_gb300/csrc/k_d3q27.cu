@@ -362,24 +362,36 @@ __device__ __forceinline__ void double_step27(double (&m)[27], const Rates27 &w,
 // 8.16; 8 or 10 of 64 8.38 / 8.36.
 constexpr int kStepBlock = 128, kStepMinBlocks = 6;
 
-// XO: the force has no y and z components (checked on the host).
-template <int FK, bool W1, bool XO>
+// The step loads its populations over the read-only path; overlapped steps (see
+// step_wait) may not, and the plain loads cost this kernel 2.5 % (160^3, 8 steps
+// and the fields: 3.59 / 3.65 ms).  The launches that overlap hides are 8 % of 64^3
+// (0.637 -> 0.584 ms for 16 steps and the fields), 1.5 % of 96^3 and nothing from 102^3 on:
+// the line lies between the two.  No step_next: a grid of 152 to 912 blocks
+// leaves room on every SM, and blocks placed while those of the step before still
+// run come to lie unevenly (40^3: 0.270 ms apart, 0.293 so, 0.233 with the
+// blocks placed as the earlier ones end).
+constexpr int kOverlapNodes = 1 << 20;
+
+// XO: the force has no y and z components (checked on the host).  OV: an
+// overlapped step.
+template <int FK, bool W1, bool XO, bool OV>
 __global__ void __launch_bounds__(kStepBlock, W1 ? kStepMinBlocks : 1)
 k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double apre, double apost, Rates27 w,
        FxRates fx, double q1, double q2)
 {
+    if (OV) step_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y, z;
     node_xyz(g, i, x, y, z);
     double m[27];
-    load_pulled<LD3Q27>(P, g, x, y, z, i, m);
+    load_pulled<LD3Q27, !OV>(P, g, x, y, z, i, m);
     auto shape = [&](int d) { return field_value(Fd, FK, d, x, y, z, i); };
     if (W1) {
         if (fixed_step27<FK != FK_NONE, XO>(m, fx, q1, q2, shape,
                                             [&](int a, double v) { P.out[a][i] = v; }))
             return;
-        load_pulled<LD3Q27>(P, g, x, y, z, i, m);
+        load_pulled<LD3Q27, !OV>(P, g, x, y, z, i, m);
     }
     double_step27<W1, XO>(m, w, FK != FK_NONE, apre, apost, shape);
 #pragma unroll
@@ -459,23 +471,20 @@ cudaError_t d3q27_step(const LaunchArgs &a)
     const Planes<double, 27> P = make_planes<double, 27>(a.fin, a.fout, a.g.Np);
     const bool xo = force_x_only(a.fkind, a.F, 3);
     const FxRates fx = fx_rates27(a.omega[1], a.omega[2]);
+    const bool ov = w1 && a.g.N <= kOverlapNodes;
+#define STEP27(FK, W1, XO, OV) \
+    launch_step(OV && a.overlap, k_step<FK, W1, XO, OV>, grid, block, a.stream, P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2)
+#define STEP27_W1(FK, XO) (ov ? STEP27(FK, true, XO, true) : STEP27(FK, true, XO, false))
     switch (a.fkind) {
-    case FK_NONE:
-        if (w1) k_step<FK_NONE, true, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        else k_step<FK_NONE, false, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        break;
+    case FK_NONE: return w1 ? STEP27_W1(FK_NONE, false) : STEP27(FK_NONE, false, false, false);
     case FK_CONST:
-        if (w1 && xo) k_step<FK_CONST, true, true><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        else if (w1) k_step<FK_CONST, true, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        else k_step<FK_CONST, false, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        break;
+        return !w1 ? STEP27(FK_CONST, false, false, false) : xo ? STEP27_W1(FK_CONST, true) : STEP27_W1(FK_CONST, false);
     default:
-        if (w1 && xo) k_step<FK_GENERAL, true, true><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        else if (w1) k_step<FK_GENERAL, true, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        else k_step<FK_GENERAL, false, false><<<grid, block, 0, a.stream>>>(P, a.g, a.F, a.apre, a.apost, w, fx, q1, q2);
-        break;
+        return !w1 ? STEP27(FK_GENERAL, false, false, false)
+                   : xo ? STEP27_W1(FK_GENERAL, true) : STEP27_W1(FK_GENERAL, false);
     }
-    return cudaGetLastError();
+#undef STEP27_W1
+#undef STEP27
 }
 
 }  // namespace lbmk

@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step9(const __grid_constant__ Planes<T, 9> P, Geom g, FieldDev F, float apre, float gsum, Rates9f w, float rref,
         unsigned long long srkey)
 {
+    step_begin();
     int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
@@ -475,6 +476,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step5(const __grid_constant__ Planes<T, 5> P, Geom g, FieldDev S, FieldDev V, float apre, float hsum, Rates5f w,
         Coef5f k, float rref, Ref5f cref, unsigned long long srkey)
 {
+    step_begin();
     int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
@@ -767,6 +769,7 @@ __global__ void __launch_bounds__(kBlock, 4)
 k_step27(const __grid_constant__ Planes<T, 27> P, Geom g, FieldDev Fd, float apre, float apost, Rates27f w,
          float rref, unsigned long long srkey)
 {
+    step_begin();
     int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
     int x, y, z;
@@ -817,7 +820,7 @@ template <> struct Pair16<__half> {
     {
         return (unsigned)__half_as_ushort(a) | ((unsigned)__half_as_ushort(b) << 16);
     }
-    __device__ static f2 get2(const __half *p) { return from_bits(__ldg(reinterpret_cast<const unsigned *>(p))); }
+    __device__ static f2 get2(const __half *p) { return from_bits(*reinterpret_cast<const unsigned *>(p)); }
     __device__ static void put2(__half *p, const f2 &v) { *reinterpret_cast<unsigned *>(p) = to_bits(v); }
     __device__ static void put2raw(__half *p, __half a, __half b) { *reinterpret_cast<unsigned *>(p) = raw_bits(a, b); }
 };
@@ -841,7 +844,7 @@ template <> struct Pair16<__nv_bfloat16> {
     }
     __device__ static f2 get2(const __nv_bfloat16 *p)
     {
-        return from_bits(__ldg(reinterpret_cast<const unsigned *>(p)));
+        return from_bits(*reinterpret_cast<const unsigned *>(p));
     }
     __device__ static void put2(__nv_bfloat16 *p, const f2 &v) { *reinterpret_cast<unsigned *>(p) = to_bits(v); }
     __device__ static void put2raw(__nv_bfloat16 *p, __nv_bfloat16 a, __nv_bfloat16 b)
@@ -854,7 +857,7 @@ template <> struct Pair16<__nv_bfloat16> {
 template <class T>
 __device__ __forceinline__ void get4(const T *p, float (&w)[4])
 {
-    const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p));
+    const uint2 u = *reinterpret_cast<const uint2 *>(p);
     const f2 lo = Pair16<T>::from_bits(u.x), hi = Pair16<T>::from_bits(u.y);
     w[0] = lo.v.x;
     w[1] = lo.v.y;
@@ -965,6 +968,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step9x2(const __grid_constant__ Planes<T, 9> P, Geom g, FieldDev F, float apre, float gsum, Rates9f w, float rref,
           unsigned long long srkey)
 {
+    step_begin();
     const int t = blockIdx.x * kBlock + threadIdx.x;
     if (t >= (g.N >> 1)) return;
     const int i0 = 2 * t;
@@ -995,6 +999,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step5x2(const __grid_constant__ Planes<T, 5> P, Geom g, FieldDev S, float apre, float hsum, Coef5f k, Ref5f cref,
           unsigned long long srkey)
 {
+    step_begin();
     const int t = blockIdx.x * kBlock + threadIdx.x;
     if (t >= (g.N >> 1)) return;
     const int i0 = 2 * t;
@@ -1092,6 +1097,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step9x4(const __grid_constant__ Planes<T, 9> P, Geom g, FieldDev F, float apre, float gsum, Rates9f w, float rref,
           unsigned long long srkey)
 {
+    step_begin();
     const int t = blockIdx.x * kBlock + threadIdx.x;
     if (t >= (g.N >> 2)) return;
     const int i0 = 4 * t;
@@ -1124,6 +1130,7 @@ __global__ void __launch_bounds__(kBlock)
 k_step5x4(const __grid_constant__ Planes<T, 5> P, Geom g, FieldDev S, float apre, float hsum, Coef5f k, Ref5f cref,
           unsigned long long srkey)
 {
+    step_begin();
     const int t = blockIdx.x * kBlock + threadIdx.x;
     if (t >= (g.N >> 2)) return;
     const int i0 = 4 * t;
@@ -1202,6 +1209,7 @@ __global__ void __launch_bounds__(kBlockPair, LBM_PAIR_MIN_BLOCKS)
 k_step27x2(const __grid_constant__ Planes<T, 27> P, Geom g, FieldDev Fd, float apre, float apost, Rates27f w,
            float rref, unsigned long long srkey)
 {
+    step_begin();
     const int t = blockIdx.x * kBlockPair + threadIdx.x;
     if (t >= (g.N >> 1)) return;
     const int i0 = 2 * t;
@@ -1406,27 +1414,27 @@ void step9_launch(const Planes<T, 9> &fin, const LaunchArgs &a, int grid, float 
             // four consecutive nodes of a row per thread
             const int qgrid = (a.g.N / 4 + kBlock - 1) / kBlock;
             if (a.fkind == FK_NONE)
-                k_step9x4<T, FK_NONE, SR><<<qgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
+                launch_step(a.overlap, k_step9x4<T, FK_NONE, SR>, qgrid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
             else if (a.fkind == FK_CONST)
-                k_step9x4<T, FK_CONST, SR><<<qgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
-            else k_step9x4<T, FK_GENERAL, SR><<<qgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
+                launch_step(a.overlap, k_step9x4<T, FK_CONST, SR>, qgrid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
+            else launch_step(a.overlap, k_step9x4<T, FK_GENERAL, SR>, qgrid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
             return;
         }
         if (a.g.nx % 2 == 0) {
             // two x-neighbouring nodes per thread, packed FP32x2 arithmetic
             const int pgrid = (a.g.N / 2 + kBlock - 1) / kBlock;
             if (a.fkind == FK_NONE)
-                k_step9x2<T, FK_NONE, SR><<<pgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
+                launch_step(a.overlap, k_step9x2<T, FK_NONE, SR>, pgrid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
             else if (a.fkind == FK_CONST)
-                k_step9x2<T, FK_CONST, SR><<<pgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
-            else k_step9x2<T, FK_GENERAL, SR><<<pgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
+                launch_step(a.overlap, k_step9x2<T, FK_CONST, SR>, pgrid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
+            else launch_step(a.overlap, k_step9x2<T, FK_GENERAL, SR>, pgrid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
             return;
         }
     }
-    if (a.fkind == FK_NONE) k_step9<T, FK_NONE, W1, SR><<<grid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
+    if (a.fkind == FK_NONE) launch_step(a.overlap, k_step9<T, FK_NONE, W1, SR>, grid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
     else if (a.fkind == FK_CONST)
-        k_step9<T, FK_CONST, W1, SR><<<grid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
-    else k_step9<T, FK_GENERAL, W1, SR><<<grid, kBlock, 0, s>>>(fin, a.g, a.F, apre, gsum, w, rref, k);
+        launch_step(a.overlap, k_step9<T, FK_CONST, W1, SR>, grid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
+    else launch_step(a.overlap, k_step9<T, FK_GENERAL, W1, SR>, grid, kBlock, s, fin, a.g, a.F, apre, gsum, w, rref, k);
 }
 
 template <class T, int SK, bool SR>
@@ -1437,20 +1445,20 @@ void step5_launch(const Planes<T, 5> &fin, const LaunchArgs &a, int grid, float 
         if (uni && a.g.nx % 4 == 0) {
             // four consecutive nodes of a row per thread
             const int qgrid = (a.g.N / 4 + kBlock - 1) / kBlock;
-            k_step5x4<T, SK, SR><<<qgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, hsum, k, cref, a.srkey);
+            launch_step(a.overlap, k_step5x4<T, SK, SR>, qgrid, kBlock, s, fin, a.g, a.F, apre, hsum, k, cref, a.srkey);
             return;
         }
         if (uni && a.g.nx % 2 == 0) {
             // two x-neighbouring nodes per thread, packed FP32x2 arithmetic
             const int pgrid = (a.g.N / 2 + kBlock - 1) / kBlock;
-            k_step5x2<T, SK, SR><<<pgrid, kBlock, 0, s>>>(fin, a.g, a.F, apre, hsum, k, cref, a.srkey);
+            launch_step(a.overlap, k_step5x2<T, SK, SR>, pgrid, kBlock, s, fin, a.g, a.F, apre, hsum, k, cref, a.srkey);
             return;
         }
     }
     if (uni)
-        k_step5<T, SK, true, SR><<<grid, kBlock, 0, s>>>(fin, a.g, a.F, a.V, apre, hsum, w, k, rref, cref, a.srkey);
+        launch_step(a.overlap, k_step5<T, SK, true, SR>, grid, kBlock, s, fin, a.g, a.F, a.V, apre, hsum, w, k, rref, cref, a.srkey);
     else
-        k_step5<T, SK, false, SR><<<grid, kBlock, 0, s>>>(fin, a.g, a.F, a.V, apre, hsum, w, k, rref, cref, a.srkey);
+        launch_step(a.overlap, k_step5<T, SK, false, SR>, grid, kBlock, s, fin, a.g, a.F, a.V, apre, hsum, w, k, rref, cref, a.srkey);
 }
 
 template <class T, int FK, bool SR>
@@ -1462,15 +1470,15 @@ void step27_launch(const Planes<T, 27> &fin, const LaunchArgs &a, float ap, floa
             // two x-neighbouring nodes per thread, packed FP32x2 arithmetic
             const int pgrid = (a.g.N / 2 + kBlockPair - 1) / kBlockPair;
             if (FK != FK_NONE && force_x_only(FK, a.F, 3))
-                k_step27x2<T, FK, SR, true><<<pgrid, kBlockPair, 0, s>>>(fin, a.g, a.F, ap, aq, w, rref, a.srkey);
+                launch_step(a.overlap, k_step27x2<T, FK, SR, true>, pgrid, kBlockPair, s, fin, a.g, a.F, ap, aq, w, rref, a.srkey);
             else
-                k_step27x2<T, FK, SR, false><<<pgrid, kBlockPair, 0, s>>>(fin, a.g, a.F, ap, aq, w, rref, a.srkey);
+                launch_step(a.overlap, k_step27x2<T, FK, SR, false>, pgrid, kBlockPair, s, fin, a.g, a.F, ap, aq, w, rref, a.srkey);
             return;
         }
     }
     const int grid = (a.g.N + kBlock - 1) / kBlock;
-    if (w1) k_step27<T, FK, true, SR><<<grid, kBlock, 0, s>>>(fin, a.g, a.F, ap, aq, w, rref, a.srkey);
-    else k_step27<T, FK, false, SR><<<grid, kBlock, 0, s>>>(fin, a.g, a.F, ap, aq, w, rref, a.srkey);
+    if (w1) launch_step(a.overlap, k_step27<T, FK, true, SR>, grid, kBlock, s, fin, a.g, a.F, ap, aq, w, rref, a.srkey);
+    else launch_step(a.overlap, k_step27<T, FK, false, SR>, grid, kBlock, s, fin, a.g, a.F, ap, aq, w, rref, a.srkey);
 }
 
 template <class T, bool SR>
@@ -1532,9 +1540,9 @@ cudaError_t step_t(int lattice, const LaunchArgs &a)
 template <class T, int TB, int M>
 cudaError_t batch_tbm(int lattice, const BatchLaunch &L, int nblocks, cudaStream_t s)
 {
-    if (lattice == LD2Q9::ID) k_batch9<T, TB, M><<<nblocks, TB, 0, s>>>(L);
-    else if (lattice == LD2Q5::ID) k_batch5<T, TB, M><<<nblocks, TB, 0, s>>>(L);
-    else k_batch27<T, TB, M><<<nblocks, TB, 0, s>>>(L);
+    if (lattice == LD2Q9::ID) launch_step(L.overlap, k_batch9<T, TB, M>, nblocks, TB, s, L);
+    else if (lattice == LD2Q5::ID) launch_step(L.overlap, k_batch5<T, TB, M>, nblocks, TB, s, L);
+    else launch_step(L.overlap, k_batch27<T, TB, M>, nblocks, TB, s, L);
     return cudaGetLastError();
 }
 
@@ -1647,6 +1655,7 @@ __global__ void __launch_bounds__(kBlock)
 k_lref_step9(const __grid_constant__ Planes<T, 9> P, Geom g, FieldDev F, float apre, float gsum, Rates9f w, float rref,
              LrefK R, unsigned long long srkey)
 {
+    step_begin();
     const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
@@ -1674,6 +1683,7 @@ __global__ void __launch_bounds__(kBlock)
 k_lref_step5(const __grid_constant__ Planes<T, 5> P, Geom g, FieldDev S, float apre, float hsum, Coef5f k, Ref5f cref,
              LrefK R, unsigned long long srkey)
 {
+    step_begin();
     const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= g.N) return;
     int x, y;
@@ -1865,6 +1875,7 @@ __global__ void __launch_bounds__(kBlock, LBM_LREF9X4_MIN_BLOCKS)
 k_lref_step9x4(const __grid_constant__ Planes<T, 9> P, Geom g, FieldDev F, float apre, float gsum, Rates9f w,
                float rref, LrefK R, unsigned long long srkey)
 {
+    step_begin();
     const int t = blockIdx.x * kBlock + threadIdx.x;
     if (t >= (g.N >> 2)) return;
     const int i0 = 4 * t;
@@ -1901,6 +1912,7 @@ __global__ void __launch_bounds__(kBlock)
 k_lref_step5x4(const __grid_constant__ Planes<T, 5> P, Geom g, FieldDev S, float apre, float hsum, Coef5f k,
                Ref5f cref, LrefK R, unsigned long long srkey)
 {
+    step_begin();
     const int t = blockIdx.x * kBlock + threadIdx.x;
     if (t >= (g.N >> 2)) return;
     const int i0 = 4 * t;
@@ -2112,8 +2124,8 @@ cudaError_t lref_step_ts(int lattice, const LaunchArgs &a, const LrefK &R)
                         (float)(a.omega[6] / 4.0), (float)(a.omega[7] / 4.0), (float)(a.omega[8] / 4.0)};
         const float gsum = (float)((a.apre + a.apost) / 12.0), apre = (float)a.apre;
         const bool w1 = a.omega[6] == 1.0 && a.omega[7] == 1.0 && a.omega[8] == 1.0;
-#define LREF9(FKV, W1V) k_lref_step9<T, FKV, W1V, SR><<<grid, kBlock, 0, s>>>(P, a.g, a.F, apre, gsum, w, rref, R, key)
-#define LREF9X4(FKV) k_lref_step9x4<T, FKV, SR><<<qgrid, kBlock, 0, s>>>(P, a.g, a.F, apre, gsum, w, rref, R, key)
+#define LREF9(FKV, W1V) launch_step(a.overlap, k_lref_step9<T, FKV, W1V, SR>, grid, kBlock, s, P, a.g, a.F, apre, gsum, w, rref, R, key)
+#define LREF9X4(FKV) launch_step(a.overlap, k_lref_step9x4<T, FKV, SR>, qgrid, kBlock, s, P, a.g, a.F, apre, gsum, w, rref, R, key)
         const int qgrid = (a.g.N / 4 + kBlock - 1) / kBlock;
         if (w1 && a.g.nx % 4 == 0) {
             if (a.fkind == FK_NONE) LREF9X4(FK_NONE);
@@ -2143,15 +2155,15 @@ cudaError_t lref_step_ts(int lattice, const LaunchArgs &a, const LrefK &R)
         if (a.g.nx % 4 == 0) {
             const int qgrid = (a.g.N / 4 + kBlock - 1) / kBlock;
             if (a.fkind == FK_NONE)
-                k_lref_step5x4<T, FK_NONE, SR><<<qgrid, kBlock, 0, s>>>(P, a.g, a.F, apre, hsum, k, cref, R, key);
+                launch_step(a.overlap, k_lref_step5x4<T, FK_NONE, SR>, qgrid, kBlock, s, P, a.g, a.F, apre, hsum, k, cref, R, key);
             else if (a.fkind == FK_CONST)
-                k_lref_step5x4<T, FK_CONST, SR><<<qgrid, kBlock, 0, s>>>(P, a.g, a.F, apre, hsum, k, cref, R, key);
-            else k_lref_step5x4<T, FK_GENERAL, SR><<<qgrid, kBlock, 0, s>>>(P, a.g, a.F, apre, hsum, k, cref, R, key);
+                launch_step(a.overlap, k_lref_step5x4<T, FK_CONST, SR>, qgrid, kBlock, s, P, a.g, a.F, apre, hsum, k, cref, R, key);
+            else launch_step(a.overlap, k_lref_step5x4<T, FK_GENERAL, SR>, qgrid, kBlock, s, P, a.g, a.F, apre, hsum, k, cref, R, key);
         } else if (a.fkind == FK_NONE)
-            k_lref_step5<T, FK_NONE, SR><<<grid, kBlock, 0, s>>>(P, a.g, a.F, apre, hsum, k, cref, R, key);
+            launch_step(a.overlap, k_lref_step5<T, FK_NONE, SR>, grid, kBlock, s, P, a.g, a.F, apre, hsum, k, cref, R, key);
         else if (a.fkind == FK_CONST)
-            k_lref_step5<T, FK_CONST, SR><<<grid, kBlock, 0, s>>>(P, a.g, a.F, apre, hsum, k, cref, R, key);
-        else k_lref_step5<T, FK_GENERAL, SR><<<grid, kBlock, 0, s>>>(P, a.g, a.F, apre, hsum, k, cref, R, key);
+            launch_step(a.overlap, k_lref_step5<T, FK_CONST, SR>, grid, kBlock, s, P, a.g, a.F, apre, hsum, k, cref, R, key);
+        else launch_step(a.overlap, k_lref_step5<T, FK_GENERAL, SR>, grid, kBlock, s, P, a.g, a.F, apre, hsum, k, cref, R, key);
     } else {
         return cudaErrorInvalidValue;
     }

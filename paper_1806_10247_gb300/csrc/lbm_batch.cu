@@ -515,6 +515,7 @@ int capture_graph(lbm_batch *b, int parity)
         L.count = b->count;
         L.k = k;
         L.parity = (parity + k) & 1;
+        L.overlap = k > 0;
         if (fp32) L.pairsf = reinterpret_cast<const float2 *>(b->d_gpairs);
         else L.pairs = b->d_gpairs;
         e = launch_one(b, L, b->gstream);
@@ -719,6 +720,7 @@ int lbm_batch_step(lbm_batch *b, long n)
     for (long k = 0; k < n; k++) {
         L.k = (int)k;
         L.parity = (parity + (int)k) & 1;
+        L.overlap = k > 0;
         if (inline_pairs) inline_pairs_of_step(b, L, k);
         cudaError_t e = launch_one(b, L, b->stream);
         if (e != cudaSuccess) return bfail(b, LBM_ECUDA, "lbm_batch_step: kernel: %s", cudaGetErrorString(e));

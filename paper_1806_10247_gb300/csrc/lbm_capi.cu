@@ -765,6 +765,7 @@ int lbm_step(lbm_ctx *c, long n)
         double apre, apost;
         envelope_pair(c, c->t, apre, apost);
         LaunchArgs a = launch_args(c, c->A, c->B, apre, apost);
+        a.overlap = k > 0 && !(c->lref_every && c->lref_since == 0);  // not behind a rebuild
         cudaError_t e;
         if (c->lref_every) {
             e = lref_step(c->lattice, a, lref_of(c));

@@ -48,7 +48,27 @@ struct LaunchArgs {
     int sround;          // 16-bit storage: round the stored deviations stochastically
     unsigned long long srkey;  // ... with random bits keyed by this step key
     double gref[5];      // D2Q5, reduced precision: reference populations of the deviations
+    bool overlap;        // the work before it on the stream is this context's previous step (launch_step)
 };
+
+// Launch of a step kernel (one that begins with step_wait).  overlap: the work
+// before it on the stream is the previous step of the same call, which alone it
+// depends on: its blocks may be placed before that step has ended.  On a small
+// grid a step is a few microseconds, about half of them the launch.
+template <class... P, class... A>
+inline cudaError_t launch_step(bool overlap, void (*kernel)(P...), int grid, int block, cudaStream_t s, const A &...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 // D2Q5 reduced-precision storage keeps deviations d = g - g_ref from a
 // uniform reference g_ref (sum g_ref = rho_ref): the rest state w rho_ref, or,
@@ -123,6 +143,7 @@ struct BatchLaunch {
     // single = 1: the batch has one member, whose descriptor travels here in
     // the launch arguments (read from the constant bank, nothing staged).
     int single;
+    int overlap;  // host: see launch_step
     BatchItem one;
     int k;
     int parity;

@@ -47,6 +47,7 @@ __device__ __forceinline__ void persist_run(const BatchLaunch &L, int &t0, int &
 template <int TB, int MODE, class Node>
 __device__ __forceinline__ void batch_tiles(const BatchLaunch &L, Node node)
 {
+    step_begin();
     if (MODE == TILE_SINGLE) {
         const int i = blockIdx.x * TB + (int)threadIdx.x;
         if (i < L.one.g.N) node(L.one, L, 0, i);
@@ -114,15 +115,15 @@ inline int tile_mode(const BatchLaunch &L) { return L.single ? TILE_SINGLE : (L.
     do {                                                                                           \
         const int m_ = tile_mode(L);                                                               \
         switch (tile) {                                                                            \
-        case 128: if (m_ == TILE_SINGLE) KERNEL<128, TILE_SINGLE><<<(nblocks), 128, 0, (s)>>>(L);   \
-                  else if (m_ == TILE_PERSIST) KERNEL<128, TILE_PERSIST><<<(nblocks), 128, 0, (s)>>>(L); \
-                  else KERNEL<128, TILE_ONE><<<(nblocks), 128, 0, (s)>>>(L); break;                 \
-        case 256: if (m_ == TILE_SINGLE) KERNEL<256, TILE_SINGLE><<<(nblocks), 256, 0, (s)>>>(L);   \
-                  else if (m_ == TILE_PERSIST) KERNEL<256, TILE_PERSIST><<<(nblocks), 256, 0, (s)>>>(L); \
-                  else KERNEL<256, TILE_ONE><<<(nblocks), 256, 0, (s)>>>(L); break;                 \
-        case 512: if (m_ == TILE_SINGLE) KERNEL<512, TILE_SINGLE><<<(nblocks), 512, 0, (s)>>>(L);   \
-                  else if (m_ == TILE_PERSIST) KERNEL<512, TILE_PERSIST><<<(nblocks), 512, 0, (s)>>>(L); \
-                  else KERNEL<512, TILE_ONE><<<(nblocks), 512, 0, (s)>>>(L); break;                 \
+        case 128: if (m_ == TILE_SINGLE) launch_step((L).overlap, KERNEL<128, TILE_SINGLE>, (nblocks), 128, (s), (L));   \
+                  else if (m_ == TILE_PERSIST) launch_step((L).overlap, KERNEL<128, TILE_PERSIST>, (nblocks), 128, (s), (L)); \
+                  else launch_step((L).overlap, KERNEL<128, TILE_ONE>, (nblocks), 128, (s), (L)); break;                 \
+        case 256: if (m_ == TILE_SINGLE) launch_step((L).overlap, KERNEL<256, TILE_SINGLE>, (nblocks), 256, (s), (L));   \
+                  else if (m_ == TILE_PERSIST) launch_step((L).overlap, KERNEL<256, TILE_PERSIST>, (nblocks), 256, (s), (L)); \
+                  else launch_step((L).overlap, KERNEL<256, TILE_ONE>, (nblocks), 256, (s), (L)); break;                 \
+        case 512: if (m_ == TILE_SINGLE) launch_step((L).overlap, KERNEL<512, TILE_SINGLE>, (nblocks), 512, (s), (L));   \
+                  else if (m_ == TILE_PERSIST) launch_step((L).overlap, KERNEL<512, TILE_PERSIST>, (nblocks), 512, (s), (L)); \
+                  else launch_step((L).overlap, KERNEL<512, TILE_ONE>, (nblocks), 512, (s), (L)); break;                 \
         default: return cudaErrorInvalidValue;                                                     \
         }                                                                                          \
         return cudaGetLastError();                                                                 \
