@@ -1982,6 +1982,25 @@ k_lref_decode(const T *__restrict__ st, Geom g, LrefK R, float *__restrict__ dev
     for (int a = 0; a < L::Q; a++) dev[a * g.Np + i] = lref_dec<L, T>(R, st + a * g.Np, a, i, sinv);
 }
 
+// The readback's fields straight from the stored values, each decoded as the FP32
+// copy would hold it: the copy and its passes left out (8192^2 D2Q5: 1.12 -> 0.64 ms).
+template <class L, class T>
+__global__ void __launch_bounds__(kBlock)
+k_lref_moments(const T *__restrict__ st, Geom g, LrefK R, double rho_ref, int fkind, FieldDev F, double ahalf, int half,
+               double *__restrict__ rho, double *__restrict__ u)
+{
+    const int i = blockIdx.x * kBlock + threadIdx.x;
+    if (i >= g.N) return;
+    int x, y;
+    node_xy(g, i, x, y);
+    const float sinv = __ldg(R.scale + 1);
+    float d[L::Q];
+    pull_node<L>(g, x, y, 0, i, d, [&](int p, int k) { return lref_dec<L, T>(R, st + p * g.Np, p, k, sinv); });
+    double dm0, j[3];
+    zeroth_first<L>(d, dm0, j);
+    store_fields<L>(rho_ref + dm0, j, half && fkind != FK_NONE, ahalf, F, fkind, x, y, 0, i, g.N, 0, rho, u);
+}
+
 // The block's largest m into bmax[blockIdx.x].
 __device__ __forceinline__ void block_max_to(float m, float *bmax)
 {
@@ -2291,6 +2310,24 @@ cudaError_t lref_step(int lattice, const LaunchArgs &a, const Lref &L)
     if (a.storage == 2) return a.sround ? lref_step_ts<__half, true>(lattice, a, R) : lref_step_ts<__half, false>(lattice, a, R);
     if (a.storage == 3)
         return a.sround ? lref_step_ts<__nv_bfloat16, true>(lattice, a, R) : lref_step_ts<__nv_bfloat16, false>(lattice, a, R);
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t lref_moments(int lattice, int storage, const LaunchArgs &a, const Lref &L, const void *stored, double *rho,
+                         double *u, int half)
+{
+    const LrefK R = lref_k(L, a.g);
+    const int grid = (a.g.N + kBlock - 1) / kBlock;
+    auto go = [&](auto lat, auto type) {
+        using T = decltype(type);
+        k_lref_moments<decltype(lat), T><<<grid, kBlock, 0, a.stream>>>(static_cast<const T *>(stored), a.g, R, a.rho_ref,
+                                                                      a.fkind, a.F, 0.5 * a.apre, half, rho, u);
+        return cudaGetLastError();
+    };
+    const bool q9 = lattice == LD2Q9::ID;
+    if (!q9 && lattice != LD2Q5::ID) return cudaErrorInvalidValue;
+    if (storage == 2) return q9 ? go(LD2Q9{}, __half{}) : go(LD2Q5{}, __half{});
+    if (storage == 3) return q9 ? go(LD2Q9{}, __nv_bfloat16{}) : go(LD2Q5{}, __nv_bfloat16{});
     return cudaErrorInvalidValue;
 }
 

@@ -804,7 +804,9 @@ int lbm_moments(lbm_ctx *c, double *rho, double *u, int where, int half_forced)
     if (rho == nullptr || (c->lattice != LBM_D2Q5_CDE && u == nullptr))
         return fail(c, LBM_EINVAL, "lbm_moments: NULL output");
     if (where != 0 && where != 1) return fail(c, LBM_EINVAL, "lbm_moments: where must be 0 or 1");
-    LrefView view(c, true);
+    // a local reference: read in its own form; the view still makes the FP32 copy's
+    // buffer, which lbm_reduce_sums_noalloc finds there after this call
+    LrefView view(c, false);
     if (view.rc != LBM_OK) return view.rc;
     double apre, apost;
     envelope_pair(c, c->t, apre, apost);
@@ -824,7 +826,10 @@ int lbm_moments(lbm_ctx *c, double *rho, double *u, int where, int half_forced)
         drho = st;
         du = st + N;
     }
-    CK(moments(c->lattice, a, drho, du, half_forced ? 1 : 0), "moments kernel");
+    const int half = half_forced ? 1 : 0;
+    CK(view.on ? lref_moments(c->lattice, view.st0, a, lref_of(c), view.A0, drho, du, half)
+               : moments(c->lattice, a, drho, du, half),
+       "moments kernel");
     c->launches++;
     if (where == 0) {
         CK(cudaMemcpyAsync(rho, drho, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "copy rho");

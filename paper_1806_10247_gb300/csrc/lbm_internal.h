@@ -256,6 +256,9 @@ cudaError_t lref_step(int lattice, const LaunchArgs &a, const Lref &L);
 // Stored values -> FP32 deviations (the FP32 forms' stored layout).
 cudaError_t lref_decode(int lattice, int storage, const Geom &g, const Lref &L, const void *stored, float *dev,
                         cudaStream_t s);
+// The fields that moments() forms of those deviations, without storing them (a: as for moments()).
+cudaError_t lref_moments(int lattice, int storage, const LaunchArgs &a, const Lref &L, const void *stored, double *rho,
+                         double *u, int half);
 // The plain 16-bit deviations as this encoding (reference 0, every sigma 1).
 cudaError_t lref_reset(int lattice, const Geom &g, const Lref &L, cudaStream_t s);
 // FP32 deviations -> stored values at the current reference and sigma.

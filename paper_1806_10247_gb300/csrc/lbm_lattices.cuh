@@ -323,16 +323,16 @@ __device__ __forceinline__ bool field_zero(const FieldDev &F, int kind, int c)
 // readback writes them: rho (phi for the scalar lattice) at rho[off + i],
 // velocity component d at u[dim * off + d * N + i] = j_d (1/rho); with `forced`
 // the pre-collision half force / source (a_pre / 2) P is included (Eq. 25 / 43;
-// ahalf = a_pre / 2, components that vanish everywhere are left out).  Rounded
-// operation by operation (no contraction), so that every kernel that forms them
-// gives the same bits.
+// ahalf = a_pre / 2, components that vanish everywhere are left out), in
+// one fused multiply-add: every rounding is spelt out, so that every kernel that
+// forms the fields gives the same bits.
 template <class L>
 __device__ __forceinline__ void store_fields(double m0, const double (&j)[3], bool forced, double ahalf, const FieldDev &F,
                                              int fkind, int x, int y, int z, int i, int N, long long off, double *rho,
                                              double *u)
 {
     if (L::Q == 5) {
-        rho[off + i] = forced ? __dadd_rn(m0, __dmul_rn(ahalf, field_value(F, fkind, 0, x, y, z, i))) : m0;
+        rho[off + i] = forced ? __fma_rn(ahalf, field_value(F, fkind, 0, x, y, z, i), m0) : m0;
         return;
     }
     rho[off + i] = m0;
@@ -340,7 +340,7 @@ __device__ __forceinline__ void store_fields(double m0, const double (&j)[3], bo
 #pragma unroll
     for (int d = 0; d < L::DIM; d++) {
         double jd = j[d];
-        if (forced && !field_zero(F, fkind, d)) jd = __dadd_rn(jd, __dmul_rn(ahalf, field_value(F, fkind, d, x, y, z, i)));
+        if (forced && !field_zero(F, fkind, d)) jd = __fma_rn(ahalf, field_value(F, fkind, d, x, y, z, i), jd);
         u[L::DIM * off + (long long)d * N + i] = __dmul_rn(jd, rinv);
     }
 }
