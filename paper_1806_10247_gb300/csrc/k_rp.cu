@@ -1507,6 +1507,156 @@ void step27_launch(const Planes<T, 27> &fin, const LaunchArgs &a, float ap, floa
     else launch_step(a.overlap, k_step27<T, FK, false, SR>, grid, kBlock, s, fin, a.g, a.F, ap, aq, w, rref, a.srkey);
 }
 
+// ------------------------------------------------- two steps in one pass ---
+// FP32 2D lattices larger than the L2 are bound by HBM: 8 Q bytes a node and step.
+// Here a block takes a strip of TX columns down `rows` rows and makes both steps of
+// a row before it goes on: the first step's results live in a ring of four rows in
+// shared memory (nine or five planes of TX + 2 columns), of which three feed the
+// second step of the row before.  The populations cross HBM once for two steps; the
+// strip's two border columns and the segment's two border rows are stepped twice.
+// The next row's loads are in flight during the second step.  Every operation is
+// that of two single steps, so the bits are theirs.  Bound by issue (78 % at 4096^2,
+// DRAM 5.0 of 6.8 TB/s): 16 steps and the fields of a 4096^2 channel 3.30 -> 2.44 ms,
+// of a 4096^2 scalar 1.91 -> 1.60; strips of 64 columns 2.65 / 1.76, of 256
+// 2.50 / 1.59.  (D3Q27 in 32 x 8 columns, three planes in the ring: 1.55 times slower
+// than single steps, its two blocks per SM wait at the barriers.)
+struct Col9w1 {
+    Rates9f w;
+    float rref;
+    template <int FK>
+    __device__ __forceinline__ void operator()(float (&d)[9], const FieldDev &F, int x, int y, int i, float apre,
+                                               float gsum) const
+    {
+        float Fx = 0.f, Fy = 0.f, Gx = 0.f, Gy = 0.f;
+        if (FK != FK_NONE) {
+            const float Px = field_value_f(F, FK, 0, x, y, 0, i), Py = field_value_f(F, FK, 1, x, y, 0, i);
+            Fx = apre * Px;
+            Fy = apre * Py;
+            Gx = gsum * Px;
+            Gy = gsum * Py;
+        }
+        collide9_w1(d, rref, Fx, Fy, Gx, Gy, w);
+    }
+};
+struct Col5u {
+    Coef5f k;
+    Ref5f cref;
+    template <int FK>
+    __device__ __forceinline__ void operator()(float (&d)[5], const FieldDev &S, int x, int y, int i, float apre,
+                                               float hsum) const
+    {
+        float Sp = 0.f, H0 = 0.f;
+        if (FK != FK_NONE) {
+            const float Ps = field_value_f(S, FK, 0, x, y, 0, i);
+            Sp = apre * Ps;
+            H0 = hsum * Ps;
+        }
+        collide5u(d, 0.0f, Sp, H0, k);
+#pragma unroll
+        for (int a = 0; a < 5; a++) d[a] += cref.v[a];
+    }
+};
+
+template <class L, int FK, int TX, class Col>
+__global__ void __launch_bounds__(TX + 32)
+k_two_steps(const __grid_constant__ Planes<float, L::Q> P, Geom g, FieldDev F, Col col, float pre1, float sum1,
+            float pre2, float sum2, int strips, int rows)
+{
+    constexpr int Q = L::Q;
+    __shared__ float ring[4][Q][TX + 2];  // [row & 3][plane][column x0 - 1 ..]
+    step_begin();
+    const int x0 = (blockIdx.x % strips) * TX, wout = min(TX, g.nx - x0);
+    const int y0 = (blockIdx.x / strips) * rows, hout = min(rows, g.ny - y0);
+    // a thread's column: the strip's own in order (aligned accesses), then its borders
+    const int t = threadIdx.x;
+    const bool own = t < wout;
+    const int c = t < TX ? t + 1 : (t == TX ? 0 : wout + 1);
+    bool in = own || t == TX || t == TX + 1;
+    int x = x0 - 1 + c;
+    if (x < 0 || x >= g.nx) {
+        in = in && !g.wall[0];
+        x += x < 0 ? g.nx : -g.nx;
+    }
+    // row k of the segment is lattice row y0 - 1 + k
+    auto row = [&](int k, int &y) {
+        y = y0 - 1 + k;
+        if (y < 0 || y >= g.ny) {
+            if (g.wall[1]) return false;
+            y += y < 0 ? g.ny : -g.ny;
+        }
+        return in;
+    };
+    float d[Q];
+    int y;
+    bool have = row(0, y);
+    if (have) load_pulled_dev<L, float>(P, g, x, y, 0, x + g.nx * y, d);
+    for (int k = 0; k < hout + 2; k++) {
+        if (have) {
+            col.template operator()<FK>(d, F, x, y, x + g.nx * y, pre1, sum1);
+#pragma unroll
+            for (int a = 0; a < Q; a++) ring[k & 3][a][c] = d[a];
+        }
+        have = k < hout + 1 && row(k + 1, y);
+        if (have) load_pulled_dev<L, float>(P, g, x, y, 0, x + g.nx * y, d);
+        // one barrier a row: the row written next is not among the three being read
+        __syncthreads();
+        if (k < 2 || !own) continue;
+        const int ys = y0 + k - 2, i = x + g.nx * ys;
+        float e[Q];
+        if ((g.wall[0] && (x == 0 || x == g.nx - 1)) || (g.wall[1] && (ys == 0 || ys == g.ny - 1))) {
+#pragma unroll
+            for (int a = 0; a < Q; a++) {
+                const int sx = x - L::ex(a), sy = ys - L::ey(a);
+                const bool opp = (g.wall[0] && (sx < 0 || sx >= g.nx)) || (g.wall[1] && (sy < 0 || sy >= g.ny));
+                e[a] = opp ? ring[(k - 1) & 3][L::opp(a)][c] : ring[(k - 1 - L::ey(a)) & 3][a][c - L::ex(a)];
+            }
+        } else {
+#pragma unroll
+            for (int a = 0; a < Q; a++) e[a] = ring[(k - 1 - L::ey(a)) & 3][a][c - L::ex(a)];
+        }
+        col.template operator()<FK>(e, F, x, ys, i, pre2, sum2);
+#pragma unroll
+        for (int a = 0; a < Q; a++) P.out[a][i] = e[a];
+    }
+}
+
+// Rows of a segment: 32, or 16 where 32 leave fewer than 4096 blocks, four waves (channel
+// 4096^2, 16 steps: 2.44 / 2.47 ms with 32 / 16 rows, 3072^2 1.48 / 1.45, 2048^2
+// 0.76 / 0.70).
+template <class L, class Col>
+cudaError_t two_steps_launch(const LaunchArgs &a, const Col &col, float pre1, float sum1, float pre2, float sum2)
+{
+    constexpr int TX = 128;
+    const long long strips = (a.g.nx + TX - 1) / TX;
+    const int rows = strips * ((a.g.ny + 31) / 32) >= 4096 ? 32 : 16;
+    const int grid = (int)(strips * ((a.g.ny + rows - 1) / rows));
+    const Planes<float, L::Q> P = make_planes<float, L::Q>(a.fin, a.fout, a.g.Np);
+    auto go = [&](auto kernel) {
+        return launch_step(a.overlap, kernel, grid, TX + 32, a.stream, P, a.g, a.F, col, pre1, sum1, pre2, sum2, (int)strips,
+                           rows);
+    };
+    if (a.fkind == FK_NONE) return go(k_two_steps<L, FK_NONE, TX, Col>);
+    if (a.fkind == FK_CONST) return go(k_two_steps<L, FK_CONST, TX, Col>);
+    return go(k_two_steps<L, FK_GENERAL, TX, Col>);
+}
+
+Rates9f rates9f(const double omega[9])
+{
+    return Rates9f{(float)(omega[3] / 12.0), (float)(omega[4] / 4.0), (float)(omega[5] / 4.0),
+                   (float)(omega[6] / 4.0),  (float)(omega[7] / 4.0), (float)(omega[8] / 4.0)};
+}
+Col5u col5u(const LaunchArgs &a)
+{
+    const double ux = a.vkind == FK_CONST ? a.V.cval[0] : 0.0, uy = a.vkind == FK_CONST ? a.V.cval[1] : 0.0;
+    Col5u r{make_coef5f(a.omega, ux, uy), Ref5f{}};
+    if (a.vkind != FK_GENERAL) {
+        double c[5];
+        d2q5_reference_change(a.omega, ux, uy, a.gref, c);
+        for (int q = 0; q < 5; q++) r.cref.v[q] = (float)c[q];
+    }
+    return r;
+}
+
 template <class T, bool SR>
 cudaError_t step_ts(int lattice, const LaunchArgs &a)
 {
@@ -1515,8 +1665,7 @@ cudaError_t step_ts(int lattice, const LaunchArgs &a)
     const cudaStream_t s = a.stream;
     if (lattice == LD2Q9::ID) {
         const Planes<T, 9> fin = make_planes<T, 9>(a.fin, a.fout, a.g.Np);
-        const Rates9f w{(float)(a.omega[3] / 12.0), (float)(a.omega[4] / 4.0), (float)(a.omega[5] / 4.0),
-                        (float)(a.omega[6] / 4.0), (float)(a.omega[7] / 4.0), (float)(a.omega[8] / 4.0)};
+        const Rates9f w = rates9f(a.omega);
         const float gsum = (float)((a.apre + a.apost) / 12.0), apre = (float)a.apre;
         const bool w1 = a.omega[6] == 1.0 && a.omega[7] == 1.0 && a.omega[8] == 1.0;
         if (w1) step9_launch<T, true, SR>(fin, a, grid, apre, gsum, w, rref, s);
@@ -1524,16 +1673,9 @@ cudaError_t step_ts(int lattice, const LaunchArgs &a)
     } else if (lattice == LD2Q5::ID) {
         const Rates5f w{(float)(a.omega[1] / 2.0), (float)(a.omega[2] / 2.0), (float)(a.omega[3] / 4.0),
                         (float)(a.omega[4] / 4.0)};
-        const double ux = a.vkind == FK_CONST ? a.V.cval[0] : 0.0, uy = a.vkind == FK_CONST ? a.V.cval[1] : 0.0;
-        const Coef5f k = make_coef5f(a.omega, ux, uy);
+        const auto [k, cref] = col5u(a);
         const float hsum = (float)((a.apre + a.apost) / 10.0), apre = (float)a.apre;
         const bool uni = a.vkind != FK_GENERAL;
-        Ref5f cref{};
-        if (uni) {
-            double c[5];
-            d2q5_reference_change(a.omega, ux, uy, a.gref, c);
-            for (int q = 0; q < 5; q++) cref.v[q] = (float)c[q];
-        }
         const Planes<T, 5> fin = make_planes<T, 5>(a.fin, a.fout, a.g.Np);
         if (a.fkind == FK_NONE) step5_launch<T, FK_NONE, SR>(fin, a, grid, apre, hsum, w, k, rref, cref, uni, s);
         else if (a.fkind == FK_CONST)
@@ -2272,6 +2414,30 @@ cudaError_t rp_step(int lattice, const LaunchArgs &a)
     case 3: return step_t<__nv_bfloat16>(lattice, a);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// FP32 lattices whose two buffers exceed the L2: below, the second step's reads do
+// not leave it (16 steps and the fields, single steps / two in a pass: channel 1300^2,
+// 122 MB, 365 / 384 us; 1400^2, 141 MB, 427 / 396; scalar 1800^2, 130 MB, 407 / 417;
+// 2000^2, 160 MB, 496 / 455).  16-bit storage is bound by issue, not by HBM.
+constexpr long long kTwoStepBytes = 136ll << 20;
+
+bool rp_takes_two(int lattice, const LaunchArgs &a)
+{
+    const int q = lattice == LD2Q9::ID ? LD2Q9::Q : LD2Q5::Q;
+    if (a.storage != 1 || (long long)a.g.N * q * 8 <= kTwoStepBytes) return false;
+    if (lattice == LD2Q9::ID) return a.omega[6] == 1.0 && a.omega[7] == 1.0 && a.omega[8] == 1.0;
+    return lattice == LD2Q5::ID && a.vkind != FK_GENERAL;
+}
+
+cudaError_t rp_two_steps(int lattice, const LaunchArgs &a, double apre2, double apost2)
+{
+    const float pre1 = (float)a.apre, pre2 = (float)apre2;
+    if (lattice == LD2Q9::ID)
+        return two_steps_launch<LD2Q9>(a, Col9w1{rates9f(a.omega), (float)a.rho_ref}, pre1,
+                                       (float)((a.apre + a.apost) / 12.0), pre2, (float)((apre2 + apost2) / 12.0));
+    return two_steps_launch<LD2Q5>(a, col5u(a), pre1, (float)((a.apre + a.apost) / 10.0), pre2,
+                                   (float)((apre2 + apost2) / 10.0));
 }
 
 cudaError_t rp_cluster_steps9(const LaunchArgs &a, int nsteps)

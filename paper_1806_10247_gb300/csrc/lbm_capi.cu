@@ -767,10 +767,17 @@ int lbm_step(lbm_ctx *c, long n)
         LaunchArgs a = launch_args(c, c->A, c->B, apre, apost);
         a.overlap = k > 0 && !(c->lref_every && c->lref_since == 0);  // not behind a rebuild
         cudaError_t e;
+        int made = 1;
         if (c->lref_every) {
             e = lref_step(c->lattice, a, lref_of(c));
         } else if (c->storage != LBM_FP64) {
-            e = rp_step(c->lattice, a);
+            if (n - k >= 2 && rp_takes_two(c->lattice, a)) {
+                envelope_pair(c, c->t + 1, apre, apost);
+                e = rp_two_steps(c->lattice, a, apre, apost);
+                made = 2;
+            } else {
+                e = rp_step(c->lattice, a);
+            }
         } else {
             switch (c->lattice) {
             case LBM_D2Q9: e = d2q9_step(a); break;
@@ -784,7 +791,8 @@ int lbm_step(lbm_ctx *c, long n)
         double *tmp = c->A;
         c->A = c->B;
         c->B = tmp;
-        c->t++;
+        c->t += made;
+        k += made - 1;
         if (c->lref_every && ++c->lref_since >= c->lref_every) {
             // rebuild the local reference from the state, in place
             const int rc = lref_rebuild_state(c, lref_of(c));

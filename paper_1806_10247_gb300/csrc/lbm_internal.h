@@ -208,6 +208,10 @@ cudaError_t d3q15_step(const LaunchArgs &a);
 // cudaErrorNotSupported when the lattice is too large.  fin -> fout after
 // nsteps steps (fout may equal fin).
 cudaError_t d2q9_cluster_steps(const LaunchArgs &a, int nsteps);
+// Two steps of a reduced-precision lattice in one pass (where rp_takes_two), `a` the
+// first's and a_pre / a_post of the second: the state two steps on in a.fout.
+bool rp_takes_two(int lattice, const LaunchArgs &a);
+cudaError_t rp_two_steps(int lattice, const LaunchArgs &a, double apre2, double apost2);
 // The same for reduced-precision storage (deviations kept in the storage type).
 cudaError_t rp_cluster_steps9(const LaunchArgs &a, int nsteps);
 cudaError_t d3q27_step(const LaunchArgs &a);
