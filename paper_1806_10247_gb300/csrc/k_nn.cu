@@ -281,8 +281,6 @@ __device__ int g_tc_status;
 
 int round16(int v) { return (v + 15) / 16 * 16; }
 
-int round8(int v) { return (v + 7) / 8 * 8; }
-
 enum TcMode { TC_FWD = 0, TC_BWD_IN = 1 };
 
 // Pixel coordinates of pixel q of a batch (32-bit: the launchers check the sizes).
@@ -353,154 +351,21 @@ __device__ __forceinline__ Pixel position_at(const Shape &s, const Line &l, int 
     return x;
 }
 
-// Forward pass and input gradient (see k_tc_conv_gather below for the sums), by
-// shifted views of one staged tile: a block stages, for each of the kd x kh rows
-// of taps, the 128 positions of its tile and the hw positions on either side, as
-// rows of 8 channels (16 bytes per position).  The A operand of the tap at
-// distance t along w is that tile read from position hw + t on: the matrix
-// descriptor's start address moves by 16 t bytes.  A value is loaded kd kh times
-// instead of once per tap, and nothing is copied per tap.
-// C16: channels padded to 16, in units of 16 (0: any).
-template <int MODE, int C16>
-__global__ void __launch_bounds__(nntc::kM)
-k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
-          float *__restrict__ out, Shape s, int act, int c16, int Np)
-{
-    using namespace nntc;
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long mbar;
-    __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x;
-    const int cin = MODE == TC_FWD ? s.ci : s.co;    // channels of the gathered operand
-    const int cout = MODE == TC_FWD ? s.co : s.ci;   // channels of the result
-    const int sgn = MODE == TC_FWD ? 1 : -1;
-    const Line l = line_of(s);
-    const int G8 = 2 * (C16 ? C16 : c16);             // channel groups of eight
-    const int R = (kM + 2 * l.hw + 7) / 8 * 8;        // staged positions
-    const int segs = s.kd * s.kh, taps = segs * s.kw;
-    unsigned char *As = smem;
-    unsigned char *Bs = smem + segs * G8 * R * 16;
-    const unsigned ntiles = (l.total + kM - 1) / kM;
-    const uint32_t ncols = tmem_cols(Np);
-    const uint32_t lboA = (uint32_t)R * 16, lboB = (uint32_t)(Np / 8) * 128;
-    if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
-    if (tid == 0) mbar_init(smem_u32(&mbar));
-    // weights: K = (tap, channel), one 16-byte row of eight channels at a time
-    for (int idx = tid; idx < Np * taps * G8; idx += kM) {
-        const int k8 = idx / Np, r = idx - k8 * Np, tap = k8 / G8, c0 = (k8 - tap * G8) * 8;
-        __nv_bfloat16 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-            const int c = c0 + j;
-            v[j] = __float2bfloat16_rn(0.f);
-            if (r < cout && c < cin)
-                v[j] = MODE == TC_FWD ? w[((long long)r * s.ci + c) * taps + tap]
-                                      : w[((long long)c * s.ci + r) * taps + tap];
-        }
-        uint4 u;
-        memcpy(&u, v, sizeof u);
-        *reinterpret_cast<uint4 *>(Bs + core_off(r, 8 * k8, Np)) = u;
-    }
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    const uint32_t tmem = tmem_base, a0 = smem_u32(As), b0 = smem_u32(Bs);
-    bool ok = true;
-    uint32_t phase = 0;
-    for (unsigned tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int q0 = (int)(tile * kM);
-        for (int j = tid; j < kM + 2 * l.hw; j += kM) {
-            const Pixel x = position_at(s, l, q0 + j - l.hw);
-            const float *base = in + (long long)x.n * cin * l.sp + x.w;
-            for (int seg = 0; seg < segs; seg++) {
-                const int a = seg / s.kh, f = seg - a * s.kh;
-                const int zd = x.d + sgn * s.dd * (a - (s.kd - 1) / 2), zh = x.h + sgn * s.dh * (f - (s.kh - 1) / 2);
-                const bool have = x.w >= 0 && (unsigned)zd < (unsigned)s.d && (unsigned)zh < (unsigned)s.h;
-                const float *src = base + (have ? (zd * s.h + zh) * s.w : 0);
-                unsigned char *dst = As + ((seg * G8) * R + j) * 16;
-#pragma unroll
-                for (int g = 0; g < G8; g++) {
-                    float v[8];
-#pragma unroll
-                    for (int i = 0; i < 8; i++) {
-                        const int c = 8 * g + i;
-                        v[i] = have && c < cin ? __ldg(src + (long long)c * l.sp) : 0.f;
-                    }
-                    *reinterpret_cast<uint4 *>(dst + g * R * 16) = make_uint4(
-                        pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-                }
-            }
-        }
-        fence_smem_to_async();
-        fence_before_sync();
-        __syncthreads();
-        fence_after_sync();
-        if (tid == 0) {
-            const uint32_t id = idesc_bf16(kM, Np);
-            uint32_t more = 0;
-            for (int seg = 0; seg < segs; seg++)
-                for (int e = 0; e < s.kw; e++) {
-                    const int shift = l.hw + sgn * s.dw * (e - (s.kw - 1) / 2);
-                    for (int g = 0; g < G8; g += 2) {
-                        const uint64_t ad = smem_desc(a0 + (uint32_t)((seg * G8 + g) * R + shift) * 16, lboA, 128);
-                        const uint64_t bd = smem_desc(b0 + (uint32_t)((seg * s.kw + e) * G8 + g) * lboB, lboB, 128);
-                        mma_bf16(tmem, ad, bd, id, more);
-                        more = 1;
-                    }
-                }
-            mma_commit(smem_u32(&mbar));
-        }
-        ok = __syncthreads_and(mbar_wait_bounded(smem_u32(&mbar), phase));
-        fence_after_sync();
-        phase ^= 1u;
-        if (!ok) break;
-        const Pixel x = position_at(s, l, q0 + tid);
-        float *dst = out + (long long)x.n * cout * l.sp + (x.d * s.h + x.h) * s.w + x.w;
-        for (int c0 = 0; c0 < Np; c0 += 16) {
-            float v[16];
-            tmem_load16(tmem + ((uint32_t)(32 * (tid >> 5)) << 16) + (uint32_t)c0, v);
-            if (x.w >= 0) {
-#pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const int o = c0 + j;
-                    if (o < cout) {
-                        float r = v[j];
-                        if (MODE == TC_FWD) {
-                            r += b[o];
-                            if (act == 1) r = tanhf(r);
-                        }
-                        dst[(long long)o * l.sp] = r;
-                    }
-                }
-            }
-        }
-        // the next tile's MMAs overwrite the accumulators every warp has just read
-        fence_before_sync();
-    }
-    if (!ok) {
-        if (tid == 0) atomicOr(&g_tc_status, 1);
-        mbar_wait_bounded(smem_u32(&mbar), phase ^ 1u);  // the MMAs end before their accumulators are freed
-    }
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    if (tid < 32) tmem_dealloc(tmem, ncols);
-}
-
-// The same products with the A operand gathered tap by tap, for shapes whose
-// staged tile (kd kh (128 + 2 hw) positions) does not fit in shared memory.
+// Forward pass and input gradient.
 // TC_FWD:    y[n,o,p] = act(b[o] + sum_{i,tap} w[o,i,tap] x[n,i,p + shift(tap)])
-//            rows: pixels of y; K = (tap, i); N = o.
+//            rows: pixels of y; K = (i, tap); N = o.
 // TC_BWD_IN: gx[n,i,p] = sum_{o,tap} w[o,i,tap] gy[n,o,p - shift(tap)]
-//            rows: pixels of x; K = (tap, o); N = i.
-// K runs over the taps, then over the gathered channels in groups of eight (the
-// channel count padded to C8): a thread finds a tap's source pixel once, loads
-// eight channels there (adjacent threads, adjacent pixels) and stores them as
-// one 16-byte row of a core matrix.  A block keeps the weights in shared memory
-// and walks over the 128-pixel tiles blockIdx.x, blockIdx.x + gridDim.x, ...
-template <int MODE>
-__global__ void __launch_bounds__(nntc::kM)
-k_tc_conv_gather(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
+//            rows: pixels of x; K = (o, tap); N = i.
+// K runs over the gathered channels, then over the taps: the order of the FP32 sums
+// is part of the result, since the next layer rounds it to BF16.  A thread gathers
+// its pixel's row of K, eight values to a 16-byte row of a core matrix.  A block
+// keeps the weights in shared memory and walks over the 128-pixel tiles blockIdx.x,
+// blockIdx.x + gridDim.x, ...  TAPS = 9 (1 x 3 x 3): the nine source positions are
+// found once per pixel and (channel, tap) of every value is known at compile time;
+// 0: any taps, counted along.  For the shapes that the staged form below does not take.
+template <int MODE, int TAPS>
+__global__ void __launch_bounds__(nntc::kM, TAPS ? 5 : 1)
+k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
           float *__restrict__ out, Shape s, int act, int Kp, int Np)
 {
     using namespace nntc;
@@ -513,7 +378,7 @@ k_tc_conv_gather(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
     const int taps = s.kd * s.kh * s.kw;
     const int cin = MODE == TC_FWD ? s.ci : s.co;    // channels of the gathered operand
     const int cout = MODE == TC_FWD ? s.co : s.ci;   // channels of the result
-    const int C8 = (cin + 7) >> 3, groups = taps * C8;
+    const int K = cin * taps;
     const int sgn = MODE == TC_FWD ? 1 : -1;
     const int sp = s.d * s.h * s.w;
     const unsigned npix = (unsigned)s.n * (unsigned)sp, ntiles = (npix + kM - 1) / kM;
@@ -522,14 +387,13 @@ k_tc_conv_gather(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
     if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
     if (tid == 0) mbar_init(smem_u32(&mbar));
     for (int idx = tid; idx < Np * (Kp >> 3); idx += kM) {
-        const int k8 = idx / Np, r = idx - k8 * Np;  // r: output channel; k8: (tap, channel group)
-        const int tap = k8 / C8, c0 = (k8 - tap * C8) * 8;
+        const int k8 = idx / Np, r = idx - k8 * Np;  // r: output channel
         __nv_bfloat16 v[8];
 #pragma unroll
         for (int j = 0; j < 8; j++) {
-            const int c = c0 + j;
+            const int k = 8 * k8 + j, c = k / taps, tap = k - c * taps;
             v[j] = __float2bfloat16_rn(0.f);
-            if (k8 < groups && r < cout && c < cin)
+            if (r < cout && k < K)
                 v[j] = MODE == TC_FWD ? w[((long long)r * s.ci + c) * taps + tap]
                                       : w[((long long)c * s.ci + r) * taps + tap];
         }
@@ -537,9 +401,6 @@ k_tc_conv_gather(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
         memcpy(&u, v, sizeof u);
         *reinterpret_cast<uint4 *>(Bs + core_off(r, 8 * k8, Np)) = u;
     }
-    // the K padding of this thread's row
-    for (int k8 = groups; k8 < (Kp >> 3); k8++)
-        *reinterpret_cast<uint4 *>(As + core_off(tid, 8 * k8, kM)) = make_uint4(0, 0, 0, 0);
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
@@ -551,26 +412,49 @@ k_tc_conv_gather(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
         const bool valid = q < npix;
         const Pixel x = pixel_at(s, valid ? q : 0);
         const float *base = in + (long long)x.n * cin * sp;
-        int a = 0, f = 0, e = 0;
-        for (int tap = 0; tap < taps; tap++) {
-            const int at = valid ? tap_source(s, x, a, f, e, sgn) : -1;
-            const float *src = base + (at < 0 ? 0 : at);
-            for (int g = 0; g < C8; g++) {
+        auto put8 = [&](int k8, const float (&v)[8]) {
+            *reinterpret_cast<uint4 *>(As + core_off(tid, 8 * k8, kM)) = make_uint4(
+                pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+        };
+        if constexpr (TAPS == 9) {
+            int at[9];
+#pragma unroll
+            for (int tap = 0; tap < 9; tap++) at[tap] = valid ? tap_source(s, x, 0, tap / 3, tap % 3, sgn) : -1;
+            for (int c0 = 0; c0 < cin; c0 += 8) {
+                const float *src = base + (long long)c0 * sp;
+#pragma unroll
+                for (int g = 0; g < 9; g++) {  // eight channels' taps are nine groups
+                    const int k8 = 9 * (c0 >> 3) + g;
+                    if (k8 >= (Kp >> 3)) break;
+                    float v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        const int c = (8 * g + j) / 9, tap = (8 * g + j) % 9;
+                        v[j] = at[tap] >= 0 && c0 + c < cin ? __ldg(src + c * sp + at[tap]) : 0.f;
+                    }
+                    put8(k8, v);
+                }
+            }
+        } else {
+            int c = 0, a = 0, f = 0, e = 0;
+            for (int k8 = 0; k8 < (Kp >> 3); k8++) {
                 float v[8];
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
-                    const int c = 8 * g + j;
-                    v[j] = at >= 0 && c < cin ? __ldg(src + (long long)c * sp) : 0.f;
+                    const int at = valid && c < cin ? tap_source(s, x, a, f, e, sgn) : -1;
+                    v[j] = at >= 0 ? __ldg(base + (long long)c * sp + at) : 0.f;
+                    if (++e == s.kw) {
+                        e = 0;
+                        if (++f == s.kh) {
+                            f = 0;
+                            if (++a == s.kd) {
+                                a = 0;
+                                c++;
+                            }
+                        }
+                    }
                 }
-                *reinterpret_cast<uint4 *>(As + core_off(tid, 8 * (tap * C8 + g), kM)) =
-                    make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-            }
-            if (++e == s.kw) {
-                e = 0;
-                if (++f == s.kh) {
-                    f = 0;
-                    a++;
-                }
+                put8(k8, v);
             }
         }
         fence_smem_to_async();
@@ -599,6 +483,159 @@ k_tc_conv_gather(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
                             if (act == 1) r = tanhf(r);
                         }
                         out[((long long)x.n * cout + o) * sp + x.p] = r;
+                    }
+                }
+            }
+        }
+        // the next tile's MMAs overwrite the accumulators every warp has just read
+        fence_before_sync();
+    }
+    if (!ok) {
+        if (tid == 0) atomicOr(&g_tc_status, 1);
+        mbar_wait_bounded(smem_u32(&mbar), phase ^ 1u);  // the MMAs end before their accumulators are freed
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    if (tid < 32) tmem_dealloc(tmem, ncols);
+}
+
+// The same for 1 x 3 x 3 taps and up to 16 channels (every layer of the network), with
+// each value loaded three times instead of nine: a block stages, for each of the
+// three rows of taps, the 128 positions of its tile and the hw positions on either
+// side as BF16, eight channels (16 bytes) a position; a thread then reads the sixteen
+// channels of its nine taps from there and writes its row of K.  16 -> 16 channels,
+// dilation 8, 32 x 128^2 pixels, forward: 61 us (the memory's time is 10); the gather
+// above, nine loads a value from L1 and L2, 88; a division per gathered value and a block
+// per tile about 900.  Now bound by instruction issue: tanh, the staging and the rows of K.
+constexpr int kStagedChannels = 16;
+template <int MODE>
+__global__ void __launch_bounds__(nntc::kM)
+k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
+          float *__restrict__ out, Shape s, int act, int Kp, int Np)
+{
+    using namespace nntc;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) unsigned long long mbar;
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x;
+    const int cin = MODE == TC_FWD ? s.ci : s.co;    // channels of the gathered operand
+    const int cout = MODE == TC_FWD ? s.co : s.ci;   // channels of the result
+    const int sgn = MODE == TC_FWD ? 1 : -1;
+    const Line l = line_of(s);
+    constexpr int G8 = kStagedChannels / 8;           // channel groups of eight
+    const int R = (kM + 2 * l.hw + 7) / 8 * 8;        // staged positions
+    constexpr int segs = 3, taps = 9;
+    const int K = cin * taps;
+    unsigned char *St = smem;
+    unsigned char *As = St + segs * G8 * R * 16;
+    unsigned char *Bs = As + kM * Kp * 2;
+    const unsigned ntiles = (l.total + kM - 1) / kM;
+    const uint32_t ncols = tmem_cols(Np);
+    const uint32_t lboA = (kM / 8) * 128, lboB = (uint32_t)(Np / 8) * 128;
+    if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
+    if (tid == 0) mbar_init(smem_u32(&mbar));
+    for (int idx = tid; idx < Np * (Kp >> 3); idx += kM) {
+        const int k8 = idx / Np, r = idx - k8 * Np;  // r: output channel
+        __nv_bfloat16 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const int k = 8 * k8 + j, c = k / taps, tap = k - c * taps;
+            v[j] = __float2bfloat16_rn(0.f);
+            if (r < cout && k < K)
+                v[j] = MODE == TC_FWD ? w[((long long)r * s.ci + c) * taps + tap]
+                                      : w[((long long)c * s.ci + r) * taps + tap];
+        }
+        uint4 u;
+        memcpy(&u, v, sizeof u);
+        *reinterpret_cast<uint4 *>(Bs + core_off(r, 8 * k8, Np)) = u;
+    }
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem = tmem_base;
+    bool ok = true;
+    uint32_t phase = 0;
+    for (unsigned tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        const int q0 = (int)(tile * kM);
+        for (int j = tid; j < kM + 2 * l.hw; j += kM) {
+            const Pixel x = position_at(s, l, q0 + j - l.hw);
+            const float *base = in + (long long)x.n * cin * l.sp + x.w;
+            for (int seg = 0; seg < segs; seg++) {
+                const int zh = x.h + sgn * s.dh * (seg - 1);
+                const bool have = x.w >= 0 && (unsigned)zh < (unsigned)s.h;
+                const float *src = base + (have ? (x.d * s.h + zh) * s.w : 0);
+                unsigned char *dst = St + ((seg * G8) * R + j) * 16;
+#pragma unroll
+                for (int g = 0; g < G8; g++) {
+                    float v[8];
+#pragma unroll
+                    for (int i = 0; i < 8; i++) {
+                        const int c = 8 * g + i;
+                        v[i] = have && c < cin ? __ldg(src + (long long)c * l.sp) : 0.f;
+                    }
+                    *reinterpret_cast<uint4 *>(dst + g * R * 16) = make_uint4(
+                        pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+                }
+            }
+        }
+        __syncthreads();
+        {
+            // half words of word c / 2 of tap's vector: channels c, c + 1
+            unsigned v[taps][8];
+#pragma unroll
+            for (int tap = 0; tap < taps; tap++) {
+                const int at = tid + l.hw + sgn * s.dw * (tap % 3 - 1);
+#pragma unroll
+                for (int g = 0; g < G8; g++) {
+                    const uint4 u = *reinterpret_cast<const uint4 *>(St + ((tap / 3 * G8 + g) * R + at) * 16);
+                    v[tap][4 * g] = u.x;
+                    v[tap][4 * g + 1] = u.y;
+                    v[tap][4 * g + 2] = u.z;
+                    v[tap][4 * g + 3] = u.w;
+                }
+            }
+#pragma unroll
+            for (int k8 = 0; k8 < kStagedChannels * taps / 8; k8++) {
+                if (k8 >= (Kp >> 3)) break;
+                unsigned o[4];
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const int k0 = 8 * k8 + 2 * j, k1 = k0 + 1, c0 = k0 / taps, c1 = k1 / taps;
+                    o[j] = __byte_perm(v[k0 % taps][c0 / 2], v[k1 % taps][c1 / 2],
+                                       (c0 & 1 ? 0x32 : 0x10) | (c1 & 1 ? 0x7600 : 0x5400));
+                }
+                *reinterpret_cast<uint4 *>(As + core_off(tid, 8 * k8, kM)) = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+        }
+        fence_smem_to_async();
+        fence_before_sync();
+        __syncthreads();
+        fence_after_sync();
+        if (tid == 0) {
+            issue_tile(tmem, smem_u32(As), lboA, smem_u32(Bs), lboB, Kp, Np);
+            mma_commit(smem_u32(&mbar));
+        }
+        ok = __syncthreads_and(mbar_wait_bounded(smem_u32(&mbar), phase));
+        fence_after_sync();
+        phase ^= 1u;
+        if (!ok) break;
+        const Pixel x = position_at(s, l, q0 + tid);
+        float *dst = out + (long long)x.n * cout * l.sp + (x.d * s.h + x.h) * s.w + x.w;
+        for (int c0 = 0; c0 < Np; c0 += 16) {
+            float v[16];
+            tmem_load16(tmem + ((uint32_t)(32 * (tid >> 5)) << 16) + (uint32_t)c0, v);
+            if (x.w >= 0) {
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    const int o = c0 + j;
+                    if (o < cout) {
+                        float r = v[j];
+                        if (MODE == TC_FWD) {
+                            r += b[o];
+                            if (act == 1) r = tanhf(r);
+                        }
+                        dst[(long long)o * l.sp] = r;
                     }
                 }
             }
@@ -812,8 +849,6 @@ void *scratch_alloc(size_t bytes, cudaStream_t st)
     return p;
 }
 
-// Padded K of the gathering convolution: the channels of a tap in groups of eight.
-int tc_kp(int cin, int taps) { return round16(taps * round8(cin)); }
 // Positions of the batch in 32 bits (the kernels' index type), with room for a
 // tile and its halo past the last one.
 bool tc_sizes(const Shape &s)
@@ -822,22 +857,10 @@ bool tc_sizes(const Shape &s)
     return hw < (1LL << 20) && (long long)s.d * s.h * s.w < (1LL << 30) &&
            (long long)s.n * s.d * s.h * (s.w + hw) < (1LL << 31) - (1LL << 21);
 }
-constexpr size_t kSmemMost = 220u * 1024u;
-size_t gather_smem(const Shape &s, int cin, int cout)
-{
-    return (size_t)(nntc::kM + round16(cout)) * tc_kp(cin, s.kd * s.kh * s.kw) * 2;
-}
-size_t staged_smem(const Shape &s, int cin, int cout)
-{
-    const size_t R = (nntc::kM + 2 * (size_t)s.dw * ((s.kw - 1) / 2) + 7) / 8 * 8, segs = (size_t)s.kd * s.kh;
-    return segs * (round16(cin) / 8) * R * 16 + segs * s.kw * round16(cin) * round16(cout) * 2;
-}
-// The shapes the tensor-core kernels take: what a tile holds (include/lbm.h) and
-// fits in shared memory one way or the other.
+// The shapes the tensor-core kernels take: what a tile holds (include/lbm.h).
 bool tc_fits(const Shape &s, int cin, int cout)
 {
-    return round16(cin * s.kd * s.kh * s.kw) <= nntc::kMaxKp && round16(cout) <= nntc::kMaxNp && tc_sizes(s) &&
-           (staged_smem(s, cin, cout) <= kSmemMost || gather_smem(s, cin, cout) <= kSmemMost);
+    return round16(cin * s.kd * s.kh * s.kw) <= nntc::kMaxKp && round16(cout) <= nntc::kMaxNp && tc_sizes(s);
 }
 
 // Blocks of a kernel that an SM holds at once, times the SMs, by registers, shared
@@ -876,20 +899,19 @@ int tc_conv_launch(const float *in, const void *w, const float *b, float *out, c
 {
     const int cin = MODE == TC_FWD ? s.ci : s.co, cout = MODE == TC_FWD ? s.co : s.ci, Np = round16(cout);
     const __nv_bfloat16 *wb = reinterpret_cast<const __nv_bfloat16 *>(w);
-    // the staged form where it fits (every shape the network uses).  16 -> 16 channels,
-    // 1 x 3 x 3 taps, dilation 8, 32 x 128^2 pixels, forward: 45 us (the memory's time
-    // is 10); gathering every tap's value by value, with a division per index, took
-    // about 900.  Now bound by instruction issue (62 %): tanh and the staging.
-    const size_t staged = staged_smem(s, cin, cout);
-    if (staged <= kSmemMost) {
-        const unsigned tiles = (line_of(s).total + nntc::kM - 1) / nntc::kM;
-        const int c16 = round16(cin) / 16;
-        if (c16 == 1) return tc_launch(k_tc_conv<MODE, 1>, tiles, staged, Np, st, what, in, wb, b, out, s, act, c16, Np);
-        return tc_launch(k_tc_conv<MODE, 0>, tiles, staged, Np, st, what, in, wb, b, out, s, act, c16, Np);
+    const int taps = s.kd * s.kh * s.kw, Kp = round16(cin * taps);
+    const size_t smem = (size_t)(nntc::kM + Np) * Kp * 2;
+    if (s.kd == 1 && s.kh == 3 && s.kw == 3) {
+        const Line l = line_of(s);
+        const size_t stage = (size_t)3 * (kStagedChannels / 8) * ((nntc::kM + 2 * (size_t)l.hw + 7) / 8 * 8) * 16;
+        if (cin <= kStagedChannels && smem + stage <= 220u * 1024u)  // the dilation decides
+            return tc_launch(k_tc_conv_staged<MODE>, (l.total + nntc::kM - 1) / nntc::kM, smem + stage, Np, st, what, in,
+                             wb, b, out, s, act, Kp, Np);
     }
-    const unsigned npix = (unsigned)((long long)s.n * s.d * s.h * s.w);
-    return tc_launch(k_tc_conv_gather<MODE>, (npix + nntc::kM - 1) / nntc::kM, gather_smem(s, cin, cout), Np, st, what, in,
-                     wb, b, out, s, act, tc_kp(cin, s.kd * s.kh * s.kw), Np);
+    const unsigned npix = (unsigned)((long long)s.n * s.d * s.h * s.w), tiles = (npix + nntc::kM - 1) / nntc::kM;
+    if (s.kd == 1 && s.kh == 3 && s.kw == 3)
+        return tc_launch(k_tc_conv<MODE, 9>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
+    return tc_launch(k_tc_conv<MODE, 0>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
 }
 
 template <int N16>
