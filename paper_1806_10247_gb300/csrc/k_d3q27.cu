@@ -61,14 +61,6 @@ __device__ __forceinline__ void raw_bwd_h(double &m0, double &m1, double &m2)
     m1 = f0;
     m2 = fp;
 }
-// Halved central moments about u -> halved raw moments (one axis; uh = u / 2):
-// m1 = k1 + u k0 and m2 = k2 + 2 u k1 + u^2 k0 with the halves carried along.
-__device__ __forceinline__ void shift_bwd_h(double k0, double &k1, double &k2, double u, double uh)
-{
-    const double m1 = fma(uh, k0, k1);
-    k2 = fma(u, k1 + m1, k2);
-    k1 = m1;
-}
 
 // Apply a 1D operation to the nine triples along axis `ax` (0 x, 1 y, 2 z).
 template <int AX, class Op>
@@ -83,12 +75,13 @@ __device__ __forceinline__ void along(double (&m)[27], Op op)
     }
 }
 
-// The back-shift with a compile-time zero pattern: bit k of Z set means m[k]
+// The back-shift, halved central moments about u -> halved raw moments (per line, uh =
+// u / 2: m1 = k1 + u k0 and m2 = k2 + 2 u k1 + u^2 k0 with the halves carried along),
+// with a compile-time zero pattern: bit k of Z set means m[k]
 // is exactly 0 on entry (the unit-rates collision leaves 16 of the 27 halved
 // central moments at 0).  An operation with a known-zero operand is left out
 // and its value taken as is: fma(a, 0, x) = x, fma(a, x, 0) = a x, x + 0 = x
-// (equal to the full operation up to the sign of a zero result).  Z = 0 is
-// shift_bwd_h on every line.
+// (equal to the full operation up to the sign of a zero result).
 template <int AX>
 __host__ __device__ constexpr int line_base(int t)
 {
@@ -100,7 +93,7 @@ __host__ __device__ constexpr int line_stride()
     return AX == 0 ? 1 : (AX == 1 ? 3 : 9);
 }
 
-// Zero pattern after shift_bwd_h along AX: on a line (k0, k1, k2), the new k1
+// Zero pattern after the back-shift along AX: on a line (k0, k1, k2), the new k1
 // is 0 when k0 and k1 are, the new k2 when all three are.
 template <int AX>
 __host__ __device__ constexpr unsigned shift_zeros(unsigned z)
