@@ -50,12 +50,15 @@ Q_NAME = {W.D2Q9: "d2q9", W.D2Q5: "d2q5", W.D3Q27: "d3q27", W.D3Q15: "d3q15"}
 ELEM = {"fp64": 8, "fp32": 4, "fp16": 2, "bf16": 2}
 
 # ---------------------------------------------------------------------------
-# Algorithmic FP64 work per node of each FP64 step formulation, counted from
+# Algorithmic work per node of each FP64 step formulation in FP64 operations, counted from
 # its formulas (each add, multiply or fused multiply-add one operation; the
 # correctly rounded reciprocal 1/rho one operation).  The derivation of each
 # count is written out in the design notes; the bench uses the fixed count,
 # never the instruction count of the current build.  The FMA / add / multiply
 # split weights the measured rates of the FP64 unit into the peak of that mix.
+# The steps do most of these operations in 64-bit integers at a scale of the node
+# (csrc/lbm_fixed.cuh) beside the FP64 unit, which an FP64 evaluation could not leave:
+# the fraction of its rate says how many times faster than that bound the step is.
 _C = "paper_1806_10247_gb300/csrc/"
 _H = [_C + "lbm_lattices.cuh", _C + "lbm_device.cuh"]
 ALG_FP64 = {
@@ -82,55 +85,42 @@ ALG_FP64 = {
 # kernel sources still hash to the value it was measured on.  Traffic per
 # launch scales with the node count once the state is larger than L2.
 TRAFFIC = {
-    ("d3q27", "fp64"): {"src": [_C + "k_d3q27.cu"] + _H, "sha": "4be8a09ad4918a7a",
-                        "bytes_per_node": (1529.134848 + 1477.492224) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
-                        "profile": "profiles/k_step_d3q27_kolmogorov_fp64.md"},
-    ("d3q27", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                        "bytes_per_node": (1812.015360 + 1756.774400) * 1e6 / 256 ** 3, "captured_nodes": 256 ** 3,
-                        "profile": "profiles/reduced_precision_traffic.md"},
-    ("d3q27", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                        "bytes_per_node": (382.343680 + 333.836032) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
-                        "profile": "profiles/reduced_precision_traffic.md"},
-    ("d3q27", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                        "bytes_per_node": (382.267392 + 333.867776) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
-                        "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q9", "fp64"): {"src": [_C + "k_d2q9.cu"] + _H, "sha": "018f6162beb1528d",
-                       "bytes_per_node": (151.018240 + 99.837696) * 1e6 / (2048 * 1024),
-                       "captured_nodes": 2048 * 1024, "profile": "profiles/k_step_d2q9_channel2048_fp64.md"},
-    ("d2q9", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                       "bytes_per_node": (1207.990016 + 1153.966848) * 1e6 / (8192 * 4096),
-                       "captured_nodes": 8192 * 4096, "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q9", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                       "bytes_per_node": (604.020736 + 551.098112) * 1e6 / (8192 * 4096),
-                       "captured_nodes": 8192 * 4096, "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q9", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                       "bytes_per_node": (604.019712 + 551.259904) * 1e6 / (8192 * 4096),
-                       "captured_nodes": 8192 * 4096, "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q5", "fp64"): {"src": [_C + "k_d2q5.cu"] + _H, "sha": "80d05b85abca33c6", "above_l2": True,
-                       "bytes_per_node": (2684.653056 + 2632.778752) * 1e6 / 8192 ** 2,
-                       "captured_nodes": 8192 ** 2, "profile": "profiles/k_step5_k_step_mat_cde8192.md"},
-    ("d2q5", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                       "bytes_per_node": (1342.345984 + 1290.611200) * 1e6 / 8192 ** 2,
-                       "captured_nodes": 8192 ** 2, "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q5", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                       "bytes_per_node": (671.200256 + 620.869632) * 1e6 / 8192 ** 2,
-                       "captured_nodes": 8192 ** 2, "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q5", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "93ac4523479a40ea", "above_l2": True,
-                       "bytes_per_node": (671.203840 + 621.302016) * 1e6 / 8192 ** 2,
-                       "captured_nodes": 8192 ** 2, "profile": "profiles/reduced_precision_traffic.md"},
-    # batched kernels (keys of the batched launches; the single-lattice
-    # captures above do not describe them)
-    ("d2q9_batch", "fp32"): {"src": [_C + "k_rp.cu", _C + "lbm_tiles.cuh", _C + "lbm_batch.cu"] + _H,
-                             "sha": "a4c28ce2b40de990", "above_l2": True,
-                             "bytes_per_node": (379.160576 + 335.486720) * 1e6 / 10521531, "captured_nodes": 10521531,
-                             "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q5_batch", "fp32"): {"src": [_C + "k_rp.cu", _C + "lbm_tiles.cuh", _C + "lbm_batch.cu"] + _H,
-                             "sha": "a4c28ce2b40de990", "above_l2": True,
-                             "bytes_per_node": (211.178752 + 167.969792) * 1e6 / 10521531, "captured_nodes": 10521531,
-                             "profile": "profiles/reduced_precision_traffic.md"},
-    ("d2q5_sweep", "fp64"): {"src": [_C + "k_d2q5.cu", _C + "lbm_tiles.cuh"] + _H, "sha": "47b4fe221b263702",
-                             "bytes_per_node": 14.0096e6 / 349184, "captured_nodes": 349184,
-                             "profile": "profiles/k_batch_d2q5_cde_sweep_fp64.md"},
+    ("d3q27", "fp64"): {"src": [_C + "k_d3q27.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "91b3ca51611b3206",
+                        "bytes_per_node": (1528.952320 + 1509.775872) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
+                        "profile": "profiles/step_traffic.md"},
+    ("d3q27", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                        "bytes_per_node": (1812.021504 + 1767.237376) * 1e6 / 256 ** 3, "captured_nodes": 256 ** 3,
+                        "profile": "profiles/step_traffic.md"},
+    ("d3q27", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                        "bytes_per_node": (382.267904 + 333.303040) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
+                        "profile": "profiles/step_traffic.md"},
+    ("d3q27", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                        "bytes_per_node": (382.292480 + 333.123840) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
+                        "profile": "profiles/step_traffic.md"},
+    ("d2q9", "fp64"): {"src": [_C + "k_d2q9.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "2c2f5e8bbf069d40",
+                       "bytes_per_node": (151.032832 + 103.470080) * 1e6 / (2048 * 1024), "captured_nodes": 2048 * 1024,
+                       "profile": "profiles/step_traffic.md"},
+    ("d2q9", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                       "bytes_per_node": (1208.190464 + 1157.165568) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
+                       "profile": "profiles/step_traffic.md"},
+    ("d2q9", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                       "bytes_per_node": (604.020736 + 552.885760) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
+                       "profile": "profiles/step_traffic.md"},
+    ("d2q9", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                       "bytes_per_node": (604.098048 + 553.156096) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
+                       "profile": "profiles/step_traffic.md"},
+    ("d2q5", "fp64"): {"src": [_C + "k_d2q5.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "c3366801003844ff", "above_l2": True,
+                       "bytes_per_node": (2684.602368 + 2640.131072) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+                       "profile": "profiles/step_traffic.md"},
+    ("d2q5", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                       "bytes_per_node": (1342.337792 + 1293.668096) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+                       "profile": "profiles/step_traffic.md"},
+    ("d2q5", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                       "bytes_per_node": (671.212288 + 620.969216) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+                       "profile": "profiles/step_traffic.md"},
+    ("d2q5", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
+                       "bytes_per_node": (671.193344 + 621.036032) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+                       "profile": "profiles/step_traffic.md"},
 }
 
 
@@ -615,6 +605,8 @@ def roofline_block(kind, storage, nodes, kernel_s, hbm, hbm_src, peak, traffic_k
                                      "FP64 unit weighted by this formulation's mix (SM clock during the probe "
                                      f"{peak['probe_sm_mhz']:.0f} MHz)",
                       "ops_per_node": alg["ops"], "fma_per_node": alg["fma"], "formulation": alg["form"],
+                      "note": "the step evaluates most of these operations in 64-bit fixed point on the integer "
+                              "units, so that it passes the rate of the FP64 unit, the bound of an FP64 evaluation",
                       "hbm": hbm_part})
         r["flops"] = {"achieved": tf, "peak": peak["tflops_fma"], "unit": "TFLOP/s", "frac": tf / peak["tflops_fma"],
                       "flops_per_node": 2 * alg["fma"] + alg["addmul"],

@@ -229,8 +229,8 @@ int lbm_set_stochastic_rounding(lbm_ctx *ctx, int on, unsigned long long seed);
  * reference and sigma are rebuilt from the state (the node's own moments), so
  * the 16-bit values hold only the non-equilibrium part and the change since
  * (the rebuild runs in place: two passes over the stored values).  Reads and
- * writes of the state (moments, reductions, populations, init) go through
- * FP32 deviations.
+ * writes of the state are those of the FP32 deviations (lbm_moments decodes them as it
+ * reads, the others go through an FP32 copy).
  * Memory: 2 x (1 or 3) floats per node on top of the 16-bit state (two
  * references), and q floats per node from the first read or write of the
  * state on.
@@ -255,8 +255,10 @@ int lbm_set_local_reference(lbm_ctx *ctx, int every);
  * (Eq. 32 / 48).  Exception: a small D2Q9 lattice (up to ~5000 nodes, any
  * storage) with a constant force envelope takes all n >= 2 steps in ONE launch of a
  * thread-block cluster that holds the state in its distributed shared memory
- * (same per-node arithmetic, one cluster barrier per step; counted as one
- * launch).  Asynchronous on the context's stream.
+ * (one cluster barrier per step; counted as one launch; in FP64 the state stays in
+ * fixed point between the steps where the rates allow, so that it differs from single
+ * steps in the last bits), and a large FP32 D2Q9 or D2Q5 lattice takes two steps in a
+ * launch, with the bits of single steps.  Asynchronous on the context's stream.
  * Errors: LBM_ESTATE (not initialised), LBM_EINVAL (n < 0), LBM_ECUDA. */
 int lbm_step(lbm_ctx *ctx, long n);
 
@@ -509,9 +511,9 @@ void lbm_batch_destroy(lbm_batch *b);
 
 /* ---- Device facts and the FP64 throughput probe ---------------------------
  *
- * The paper has no counterpart.  On this GPU the FP64 step kernels are bound
- * by the FP64 unit rather than by memory, so their roofline is stated
- * against the FP64 instruction rate measured on the device that runs them. */
+ * The paper has no counterpart.  On this GPU an FP64 step evaluated in
+ * FP64 instructions is bound by the FP64 unit rather than by memory, so the FP64 kernels
+ * are stated against the FP64 instruction rate measured on the device that runs them. */
 
 /* Message of the last failure of lbm_device_info / lbm_probe_fp64 (per thread). */
 const char *lbm_probe_last_error(void);
@@ -563,7 +565,7 @@ const char *lbm_nn_last_error(void);
  * take CUDA-core kernels with FP32 operands. */
 
 /* Status of the tensor-core kernels since the last call: *status = 1 if a
- * kernel's wait for its tensor-core work gave up after 2 s (its outputs are
+ * kernel's wait for its tensor-core work gave up after about 2 s (its outputs are
  * then not written), else 0; the flag is cleared.  Synchronises the device.
  * Errors: LBM_EINVAL (status NULL), LBM_ECUDA. */
 int lbm_nn_tc_status(int *status);
