@@ -1,8 +1,8 @@
 // Device facts and an FP64 throughput probe, for the roofline of the FP64
-// step kernels.  The paper has no counterpart: on this GPU the FP64 step
-// kernels are bound by the FP64 unit, not by memory, so their roofline needs
-// the FP64 instruction rate the unit actually sustains, measured on the
-// device that runs them.
+// step kernels.  The paper has no counterpart: on this GPU an FP64
+// evaluation of a step is bound by the FP64 unit, not by memory, so the FP64 kernels
+// (which do most of it in fixed point) are stated against the FP64 instruction rate
+// that the unit actually sustains, measured on the device that runs them.
 //
 // The probe kernel runs 8 or 16 independent dependency chains per thread of
 // one FP64 operation (FMA, add or multiply).  The second and third operands
