@@ -420,11 +420,14 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
             int at[9];
 #pragma unroll
             for (int tap = 0; tap < 9; tap++) at[tap] = valid ? tap_source(s, x, 0, tap / 3, tap % 3, sgn) : -1;
-            for (int c0 = 0; c0 < cin; c0 += 8) {
+            // over every group of the padded K: eight channels' taps are nine groups, and a
+            // channel count that is an odd multiple of eight leaves one of zeros beyond them
+            for (int k0 = 0; k0 < (Kp >> 3); k0 += 9) {
+                const int c0 = 8 * (k0 / 9);
                 const float *src = base + (long long)c0 * sp;
 #pragma unroll
-                for (int g = 0; g < 9; g++) {  // eight channels' taps are nine groups
-                    const int k8 = 9 * (c0 >> 3) + g;
+                for (int g = 0; g < 9; g++) {
+                    const int k8 = k0 + g;
                     if (k8 >= (Kp >> 3)) break;
                     float v[8];
 #pragma unroll
