@@ -656,7 +656,8 @@ FX_HD void fx_collide9_run(i64 (&f)[9], const i64 (&h)[2], const i64 (&t)[2], co
 // Step coefficients of a uniform advecting velocity (k_d2q5.cu Coef5) as
 // fractions of 2^63: h1 = A1 phi - c1 kx, h2 = A2 phi - c2 ky, h3 = P3 phi + X3
 // kx + Y3 ky + S3 (kxx + kyy), h4 = P4 phi + X4 kx + Y4 ky + D4 (kxx - kyy).  ok
-// = 0 when one of them is not below 1 (advecting velocities near 1 and above).
+// = 0 where that form does not apply: an advecting velocity near 1 and above, or a
+// P3 that is not below 1 (both components large, omega_1 and omega_2 near 2).
 struct FxCoef5 {
     i64 A1, c1, A2, c2, P3, X3, Y3, S3, P4, X4, Y4, D4;
     int ok;
@@ -664,7 +665,11 @@ struct FxCoef5 {
 inline FxCoef5 fx_coef5(double c1, double c2, double c3, double c4, double ux, double uy)
 {
     FxCoef5 k{};
-    k.ok = ux > -0.9 && ux < 0.9 && uy > -0.9 && uy < 0.9;  // with rates below 2 every coefficient is below 1
+    // With rates in (0, 2) (c1, c2 < 1, c3, c4 < 1/2) and |u| < 0.9 the others are below
+    // 1: X3 = ux (2 c3 - c1), P4 = (c1 - c4) ux^2 - (c2 - c4) uy^2 and so on.  P3 = c3 (2/3
+    // - ux^2 - uy^2) + c1 ux^2 + c2 uy^2 goes up to 1.6.
+    const double P3 = c3 * (2.0 / 3.0 - ux * ux - uy * uy) + c1 * ux * ux + c2 * uy * uy;
+    k.ok = ux > -0.9 && ux < 0.9 && uy > -0.9 && uy < 0.9 && P3 > -0.99 && P3 < 0.99;
     if (!k.ok) return k;
     // products of fractions, in integers: 2^-62 instead of FP64's 2^-53
     auto mul = [](i64 a, i64 b) { return 2 * fx_mul(a, b); };
