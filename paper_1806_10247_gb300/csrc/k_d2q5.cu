@@ -228,8 +228,7 @@ void launch_v(const LaunchArgs &a, int grid, double hsum, const Rates5 &w)
                                                           a.V, a.apre, hsum, w);
 }
 
-// Batched form; FP64 pairs hold (a_pre/2, (a_pre + a_post)/2) per step and
-// item (a_pre is halved on the host: one multiply fewer per node).
+// Batched form; a step's amplitudes per item in Amp64.
 // coef[0..11] = Coef5 of a uniform advecting velocity, coef[12..15] = Rates5,
 // mat = the step matrix of a uniform advecting velocity.
 // One node of a batched launch (member `it`, node i; B staged in shared memory).
@@ -239,27 +238,27 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     const int p = B.parity + L.parity;
     const double *fin = B.buf[p & 1];
     double *fout = B.buf[(p + 1) & 1];
-    const double2 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
+    const Amp64 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
     int x, y;
     node_xy(g, i, x, y);
     double f[5];
     load_pulled<LD2Q5>(fin, g, x, y, 0, i, f);
-    if (L.mrho) fused_fields<LD2Q5>(B, L, it, i, x, y, 0, f, ap.x);  // fused readback of f(t)'s scalar
+    if (L.mrho) fused_fields<LD2Q5>(B, L, it, i, x, y, 0, f, ap.q1);  // fused readback of f(t)'s scalar
     if (B.vkind != FK_GENERAL) {
         const bool src = B.fkind != FK_NONE;
         const double P = src ? field_value(B.F, B.fkind, 0, x, y, 0, i) : 0.0;
         if (B.fx5.ok) {
-            if (fixed_step5<true>(f, B.fx5, P, ap.x, ap.y, [&](int a, double v) { fout[a * g.Np + i] = v; })) return;
+            if (fixed_step5<true>(f, B.fx5, P, ap.q1, ap.q2, [&](int a, double v) { fout[a * g.Np + i] = v; })) return;
             load_pulled<LD2Q5>(fin, g, x, y, 0, i, f);
         }
-        if (src) collide_mat<true>(f, P, ap.x, ap.y / 5.0, B.mat);
+        if (src) collide_mat<true>(f, P, ap.q1, ap.g, B.mat);
         else collide_mat<false>(f, 0.0, 0.0, 0.0, B.mat);
     } else {
         double Spre = 0.0, H0 = 0.0;
         if (B.fkind != FK_NONE) {
             const double P = field_value(B.F, B.fkind, 0, x, y, 0, i);
-            Spre = (2.0 * ap.x) * P;
-            H0 = (ap.y / 5.0) * P;
+            Spre = (2.0 * ap.q1) * P;
+            H0 = ap.g * P;
         }
         const Rates5 w{B.coef[12], B.coef[13], B.coef[14], B.coef[15]};
         const double ux = field_value(B.V, FK_GENERAL, 0, x, y, 0, i);

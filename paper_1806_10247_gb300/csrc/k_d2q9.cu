@@ -374,8 +374,8 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
     cl.sync();  // no block leaves while another may still read its shared memory
 }
 
-// Batched form: one launch for every lattice of a batch; pairs hold
-// (a_pre / 4, (a_pre + a_post) / 4) per step and item.
+// Batched form: one launch for every lattice of a batch; a step's amplitudes per
+// item in Amp64.
 // One node of a batched launch (member `it`, node i; B staged in shared memory).
 __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch &L, int it, int i)
 {
@@ -383,26 +383,26 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     const int p = B.parity + L.parity;
     const double *fin = B.buf[p & 1];
     double *fout = B.buf[(p + 1) & 1];
-    const double2 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
+    const Amp64 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
     int x, y;
     node_xy(g, i, x, y);
     double f[9];
     load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-    if (L.mrho) fused_fields<LD2Q9>(B, L, it, i, x, y, 0, f, 2.0 * ap.x);  // fused readback of f(t)'s fields
+    if (L.mrho) fused_fields<LD2Q9>(B, L, it, i, x, y, 0, f, 2.0 * ap.q1);  // fused readback of f(t)'s fields
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, 0, i) : 0.0; };
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates9 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
     if (B.variant == 3) {  // uniform over the member
-        if (fixed_step9<true, true>(f, B.fx, ap.x, ap.y, shape, put)) return;
+        if (fixed_step9<true, true>(f, B.fx, ap.q1, ap.q2, shape, put)) return;
         load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-        double_step9<true, true>(f, w, forced, 4.0 * ap.x, ap.y / 3.0, shape);
+        double_step9<true, true>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else if (B.variant == 1) {
-        if (fixed_step9<true, false>(f, B.fx, ap.x, ap.y, shape, put)) return;
+        if (fixed_step9<true, false>(f, B.fx, ap.q1, ap.q2, shape, put)) return;
         load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-        double_step9<true, false>(f, w, forced, 4.0 * ap.x, ap.y / 3.0, shape);
+        double_step9<true, false>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else {
-        double_step9<false, false>(f, w, forced, 4.0 * ap.x, ap.y / 3.0, shape);
+        double_step9<false, false>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
     }
 #pragma unroll
     for (int a = 0; a < 9; a++) put(a, f[a]);

@@ -185,7 +185,7 @@ k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double
     for (int a = 0; a < 15; a++) P.out[a][i] = f[a];
 }
 
-// Batched form; pairs hold (a_pre / 4, (a_pre + a_post) / 4) per step and item.
+// Batched form; a step's amplitudes per item in Amp64.
 // One node of a batched launch (member `it`, node i; B staged in shared memory).
 __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch &L, int it, int i)
 {
@@ -193,22 +193,22 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     const int p = B.parity + L.parity;
     const double *fin = B.buf[p & 1];
     double *fout = B.buf[(p + 1) & 1];
-    const double2 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
+    const Amp64 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
     int x, y, z;
     node_xyz(g, i, x, y, z);
     double f[15];
     load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
-    if (L.mrho) fused_fields<LD3Q15>(B, L, it, i, x, y, z, f, 2.0 * ap.x);  // fused readback of f(t)'s fields
+    if (L.mrho) fused_fields<LD3Q15>(B, L, it, i, x, y, z, f, 2.0 * ap.q1);  // fused readback of f(t)'s fields
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     const Rates15 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3]};
     if (w.t == 1.0 && w.q == 1.0) {  // uniform over the member
-        if (fixed_step15<true, false>(f, B.fx, ap.x, ap.y, shape,
+        if (fixed_step15<true, false>(f, B.fx, ap.q1, ap.q2, shape,
                                       [&](int a, double v) { fout[a * g.Np + i] = v; }))
             return;
         load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
     }
-    double_step15(f, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
+    double_step15(f, w, forced, 4.0 * ap.q1, ap.g, shape);
 #pragma unroll
     for (int a = 0; a < 15; a++) fout[a * g.Np + i] = f[a];
 }

@@ -391,7 +391,7 @@ k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double
     for (int a = 0; a < 27; a++) P.out[a][i] = m[a];
 }
 
-// Batched form; pairs hold (a_pre / 4, (a_pre + a_post) / 4) per step and item.
+// Batched form; a step's amplitudes per item in Amp64.
 // One node of a batched launch (member `it`, node i; B staged in shared memory).
 __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch &L, int it, int i)
 {
@@ -399,27 +399,27 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     const int p = B.parity + L.parity;
     const double *fin = B.buf[p & 1];
     double *fout = B.buf[(p + 1) & 1];
-    const double2 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
+    const Amp64 ap = L.pairs ? L.pairs[(size_t)L.k * L.count + it] : L.inl[it];
     int x, y, z;
     node_xyz(g, i, x, y, z);
     double m[27];
     load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
     // fused readback of f(t)'s fields
-    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, 2.0 * ap.x);
+    if (L.mrho) fused_fields<LD3Q27>(B, L, it, i, x, y, z, m, 2.0 * ap.q1);
     const bool forced = B.fkind != FK_NONE;
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates27 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
     if (B.variant == 3) {  // uniform over the member
-        if (fixed_step27<true, true>(m, B.fx, ap.x, ap.y, shape, put)) return;
+        if (fixed_step27<true, true>(m, B.fx, ap.q1, ap.q2, shape, put)) return;
         load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
-        double_step27<true, true>(m, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
+        double_step27<true, true>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else if (B.variant == 1) {
-        if (fixed_step27<true, false>(m, B.fx, ap.x, ap.y, shape, put)) return;
+        if (fixed_step27<true, false>(m, B.fx, ap.q1, ap.q2, shape, put)) return;
         load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
-        double_step27<true, false>(m, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
+        double_step27<true, false>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else {
-        double_step27<false, false>(m, w, forced, 4.0 * ap.x, 4.0 * (ap.y - ap.x), shape);
+        double_step27<false, false>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
     }
 #pragma unroll
     for (int a = 0; a < 27; a++) put(a, m[a]);

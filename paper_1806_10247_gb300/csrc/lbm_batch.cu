@@ -49,9 +49,9 @@ struct lbm_batch {
     bool items_valid = false;
     std::vector<long long> item_version;
     std::vector<double *> item_buf0;   // buf[0] of each uploaded descriptor
-    double2 *d_pairs[2] = {nullptr, nullptr};
-    double2 *h_pairs[2] = {nullptr, nullptr};
-    size_t pairs_cap[2] = {0, 0};  // double2 entries per slot
+    Amp64 *d_pairs[2] = {nullptr, nullptr};
+    Amp64 *h_pairs[2] = {nullptr, nullptr};
+    size_t pairs_cap[2] = {0, 0};  // entries per slot
     cudaEvent_t ev[2] = {nullptr, nullptr};
     int slot = 0;
     long long launches = 0;
@@ -61,8 +61,8 @@ struct lbm_batch {
     cudaGraphExec_t gexec = nullptr;
     int gparity = -1;                  // descriptor parity the graph was captured for
     cudaStream_t gstream = nullptr;    // private stream used only to capture
-    double2 *h_gpairs = nullptr;       // pinned envelope pairs of one replay (double2 or float2)
-    double2 *d_gpairs = nullptr;
+    Amp64 *h_gpairs = nullptr;         // pinned envelope pairs of one replay (Amp64 or float2)
+    Amp64 *d_gpairs = nullptr;
     bool gpairs_filled = false;        // constant envelopes: pairs written once
     cudaEvent_t ev_graph = nullptr;    // recorded after each replay
     // packed moments (lbm_batch_moments_packed)
@@ -117,20 +117,17 @@ int bfail(lbm_batch *b, int code, const char *fmt, ...)
         if (e_ != cudaSuccess) return bfail(b, LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e_)); \
     } while (0)
 
-// A step's envelope pair as the FP64 batched kernels take it: quarters of a_pre
-// and of a_pre + a_post for the flow lattices (halved moments), halves for D2Q5.
-double2 pair64(int lattice, double apre, double apost)
+// A step's amplitudes as the FP64 batched kernels take them (Amp64).
+Amp64 pair64(int lattice, double apre, double apost)
 {
     const double c = lattice == LBM_D2Q5_CDE ? 0.5 : 0.25;
-    return make_double2(c * apre, c * (apre + apost));
+    const double g = lattice == LBM_D2Q9 ? (apre + apost) / 12.0 : (lattice == LBM_D2Q5_CDE ? (apre + apost) / 10.0 : apost);
+    return Amp64{c * apre, c * (apre + apost), g};
 }
-// The pair of the reduced-precision kernels: a_pre and D2Q9 (a_pre + a_post)/12,
-// D2Q5 (a_pre + a_post)/10, D3Q27 a_post -- the same expressions as the
-// single-lattice launchers.
+// The pair of the reduced-precision kernels.
 float2 pair32(int lattice, double apre, double apost)
 {
-    const double second = lattice == LBM_D2Q9 ? (apre + apost) / 12.0 : (lattice == LBM_D2Q5_CDE ? (apre + apost) / 10.0 : apost);
-    return make_float2((float)apre, (float)second);
+    return make_float2((float)apre, (float)pair64(lattice, apre, apost).g);
 }
 
 int grow_pairs(lbm_batch *b, int s, size_t need)
@@ -143,8 +140,8 @@ int grow_pairs(lbm_batch *b, int s, size_t need)
     b->h_pairs[s] = nullptr;
     b->d_pairs[s] = nullptr;
     b->pairs_cap[s] = 0;
-    BCK(cudaMallocHost(&b->h_pairs[s], cap * sizeof(double2)), "cudaMallocHost(pairs)");
-    BCK(cudaMalloc(&b->d_pairs[s], cap * sizeof(double2)), "cudaMalloc(pairs)");
+    BCK(cudaMallocHost(&b->h_pairs[s], cap * sizeof(Amp64)), "cudaMallocHost(pairs)");
+    BCK(cudaMalloc(&b->d_pairs[s], cap * sizeof(Amp64)), "cudaMalloc(pairs)");
     b->pairs_cap[s] = cap;
     return LBM_OK;
 }
@@ -420,7 +417,7 @@ cudaError_t launch_one(lbm_batch *b, const BatchLaunch &L, cudaStream_t s)
     return launch_tiled(b, L, b->tile_idx, b->persistent, s);
 }
 
-// Envelope pairs of steps t_i .. t_i + k - 1 of every member into dst (double2
+// Envelope pairs of steps t_i .. t_i + k - 1 of every member into dst (Amp64
 // for FP64 batches, float2 otherwise), [k][count].
 void fill_pairs(const lbm_batch *b, void *dst, long k)
 {
@@ -432,7 +429,7 @@ void fill_pairs(const lbm_batch *b, void *dst, long k)
             lbmc::envelope_pair(c, c->t + s, apre, apost);
             const size_t at = (size_t)s * b->count + i;
             if (fp32) reinterpret_cast<float2 *>(dst)[at] = pair32(b->lattice, apre, apost);
-            else reinterpret_cast<double2 *>(dst)[at] = pair64(b->lattice, apre, apost);
+            else reinterpret_cast<Amp64 *>(dst)[at] = pair64(b->lattice, apre, apost);
         }
     }
 }
@@ -449,7 +446,7 @@ int stage_pairs(lbm_batch *b, BatchLaunch &L, long n)
     if (rc != LBM_OK) return rc;
     fill_pairs(b, b->h_pairs[s], n);
     const bool fp32 = reduced_precision(b);
-    const size_t esz = fp32 ? sizeof(float2) : sizeof(double2);
+    const size_t esz = fp32 ? sizeof(float2) : sizeof(Amp64);
     BCK(cudaMemcpyAsync(b->d_pairs[s], b->h_pairs[s], (size_t)n * b->count * esz, cudaMemcpyHostToDevice,
                         b->stream),
         "lbm_batch_step: copy envelope pairs");
@@ -498,7 +495,7 @@ int capture_graph(lbm_batch *b, int parity)
         cudaGraphExecDestroy(b->gexec);
         b->gexec = nullptr;
     }
-    const size_t bytes = (size_t)b->graph_steps * b->count * sizeof(double2);
+    const size_t bytes = (size_t)b->graph_steps * b->count * sizeof(Amp64);
     if (!b->gstream) BCK(cudaStreamCreateWithFlags(&b->gstream, cudaStreamNonBlocking), "graph stream");
     if (!b->ev_graph) BCK(cudaEventCreateWithFlags(&b->ev_graph, cudaEventDisableTiming), "graph event");
     if (!b->h_gpairs) {

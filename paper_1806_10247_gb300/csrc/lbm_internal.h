@@ -131,6 +131,14 @@ void batch_coef(int lattice, const double omega[9], BatchItem &item);
 // as input and its envelope pair pairs[k * count + i], or inl[i] when pairs is
 // NULL (batches of at most kInlinePairs lattices: no per-step copy).
 constexpr int kInlinePairs = 32;
+// Envelope amplitudes of one step of an FP64 member: of the fixed-point form q1, q2
+// (flow: a_pre / 4, (a_pre + a_post) / 4; D2Q5: a_pre / 2, (a_pre + a_post) / 2), and
+// what the FP64 form takes besides a_pre: D2Q9 (a_pre + a_post) / 12, D2Q5 (a_pre +
+// a_post) / 10, D3Q27 and D3Q15 a_post (each formed on the host as a single lattice's
+// launch forms it, so that a member of a batch has its bits).
+struct Amp64 {
+    double q1, q2, g;
+};
 struct BatchLaunch {
     const BatchItem *items;
     const int *first;  // first tile of each item (ascending, first[0] = 0)
@@ -147,9 +155,9 @@ struct BatchLaunch {
     BatchItem one;
     int k;
     int parity;
-    const double2 *pairs;
-    double2 inl[kInlinePairs];
-    // reduced-precision kernels read the same pairs in FP32
+    const Amp64 *pairs;
+    Amp64 inl[kInlinePairs];
+    // reduced-precision kernels: (a_pre, g) in FP32
     const float2 *pairsf;
     float2 inlf[kInlinePairs];
     // Fused readback (FP64 kernels, lbm_batch_step_read): when mrho is not
