@@ -255,9 +255,8 @@ int lbm_set_local_reference(lbm_ctx *ctx, int every);
  * (Eq. 32 / 48).  Exception: a small D2Q9 lattice (up to ~5000 nodes, any
  * storage) with a constant force envelope takes all n >= 2 steps in ONE launch of a
  * thread-block cluster that holds the state in its distributed shared memory
- * (one cluster barrier per step; counted as one launch; in FP64 the state stays in
- * fixed point between the steps where the rates allow, so that it differs from single
- * steps in the last bits), and a large FP32 D2Q9 or D2Q5 lattice takes two steps in a
+ * (same per-node arithmetic, one cluster barrier per step; counted as one
+ * launch), and a large FP32 D2Q9 or D2Q5 lattice takes two steps in a
  * launch, with the bits of single steps.  Asynchronous on the context's stream.
  * Errors: LBM_ESTATE (not initialised), LBM_EINVAL (n < 0), LBM_ECUDA. */
 int lbm_step(lbm_ctx *ctx, long n);

@@ -227,15 +227,14 @@ k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double a
 // shared memory directly.  One cluster barrier per step separates the
 // writes of a step from the reads of the next.
 //
+// The per-node arithmetic is that of the single-step launches (the fixed-point
+// step with unit higher rates, node by node the FP64 form where that does not apply) and
+// the state is FP64 between the steps, so the result is theirs, however the steps
+// are cut into calls (up to the compiler's multiply-add contraction in the FP64 form).
 // A step of ~100 nodes is one warp per SM: its time is the latency of one node's
-// chain of operations.  With unit higher rates the state is therefore kept in
-// fixed point from the first step to the last (fx_collide9_run: one scale for the
-// lattice, no conversions inside a step, mass and momentum exact), and rounded to
-// FP64 once at the end.  A lattice whose nodes differ by more than 2^3 in scale,
-// or whose values leave the range on the way, runs the FP64 steps from the start
-// state instead (every block learns of it at the barrier after the last step).
-// 3 x 33, 100 steps: FP64 steps 3.05 us each, FP64 state with a fixed-point
-// collision 1.84, fixed-point state 1.40.
+// chain of operations (3 x 33, 100 steps: 1.63 us a step in fixed point, 3.06 in FP64;
+// 48 x 96 3.06 and 7.2).  Keeping the fixed-point state from step to step at one scale
+// for the lattice takes 1.38, but then the result depends on how the steps are cut.
 namespace cg = cooperative_groups;
 
 constexpr int kClusterThreads = 384;  // >= 32-rounded 341, the largest block (48 KB of shared memory)
@@ -243,21 +242,24 @@ constexpr int kClusterThreads = 384;  // >= 32-rounded 341, the largest block (4
 template <int FK, bool W1>
 __global__ void __launch_bounds__(kClusterThreads)
 k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom g, FieldDev F, double apre,
-                double gsum, Rates9 w, FxRates fx, int P, int nsteps)
+                double gsum, Rates9 w, FxRates fx, double q1, double q2, int P, int nsteps)
 {
     extern __shared__ double sm[];  // [2][9][P]
-    __shared__ int range[3];        // smallest and largest exponent of this block's nodes; a value left the range
     cg::cluster_group cl = cg::this_cluster();
-    const int b = (int)cl.block_rank(), nblk = (int)cl.num_blocks();
+    const int b = (int)cl.block_rank();
     const int l = threadIdx.x;
     const int i = b * P + l;
     const bool own = l < P && i < g.N;
+    if (own)
+#pragma unroll
+        for (int a = 0; a < 9; a++) sm[a * P + l] = fin[a * g.Np + i];
     const int x = own ? i % g.nx : 0, y = own ? i / g.nx : 0;
     double Px = 0.0, Py = 0.0;
     if (FK != FK_NONE && own) {
         Px = field_value(F, FK, 0, x, y, 0, i);
         Py = field_value(F, FK, 1, x, y, 0, i);
     }
+    auto shape = [&](int d) { return d == 0 ? Px : Py; };
     // pull sources of this node: owner block, offset inside its buffer
     int src_blk[9], src_off[9];
     if (own) {
@@ -270,108 +272,34 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
             src_off[a] = aa * P + (j - (j / P) * P);
         }
     }
-    bool fixed = false;
-    if (W1) {
-        // the lattice's scale
-        if (l < 3) range[l] = l == 0 ? 0x7fffffff : 0;
-        __syncthreads();
-        double f[9];
+    cl.sync();
+    int cur = 0;
+    for (int n = 0; n < nsteps; n++) {
         if (own) {
-#pragma unroll
-            for (int a = 0; a < 9; a++) f[a] = fin[a * g.Np + i];
-            const int em = fx_emax(f);
-            atomicMin(&range[0], em);
-            atomicMax(&range[1], em);
-        }
-        cl.sync();
-        int lo = 0x7fffffff, hi = 0;
-        for (int r = 0; r < nblk; r++) {
-            const int *other = cl.map_shared_rank(range, r);
-            lo = min(lo, other[0]);
-            hi = max(hi, other[1]);
-        }
-        const int k = FxGrid<9>::S + 1023 - hi;
-        int bad = fx_in_range(hi) && hi - lo <= 3 ? 0 : -1;
-        // F_pre / 2 (rounded once), and (F_pre + F_post) / 2 with 16 more bits,
-        // whose rounding error is carried from step to step
-        i64 h[2] = {0, 0}, t[2] = {0, 0}, rest[2] = {0x8000, 0x8000};
-        if (FK != FK_NONE) {
-            const double Pd[2] = {Px, Py};
-#pragma unroll
-            for (int d = 0; d < 2; d++) {
-                const double f1 = 0.5 * apre * Pd[d], f2 = 6.0 * gsum * Pd[d];
-                const unsigned m1 = fx_hi(fx_bits(f1)) & 0x7fffffffu, m2 = fx_hi(fx_bits(f2)) & 0x7fffffffu;
-                if ((int)(max(m1, m2) >> 20) > hi - 13) bad = -1;
-                h[d] = fx_round(fx_ldexp(f1, k));
-                t[d] = fx_round(fx_ldexp(f2, k + 16));
-            }
-        }
-        i64 *fs = reinterpret_cast<i64 *>(sm);
-        if (own) {
-            i64 X[9];
-            fx_load(f, k, X);
-#pragma unroll
-            for (int a = 0; a < 9; a++) fs[a * P + l] = X[a];
-        }
-        cl.sync();
-        int cur = 0;
-        for (int n = 0; n < nsteps; n++) {
-            if (own) {
-                i64 X[9];
-#pragma unroll
-                for (int a = 0; a < 9; a++) X[a] = cl.map_shared_rank(fs + cur * 9 * P, src_blk[a])[src_off[a]];
-                i64 add[2] = {0, 0};
-                if (FK != FK_NONE) {
-#pragma unroll
-                    for (int d = 0; d < 2; d++) {
-                        rest[d] += t[d];
-                        add[d] = rest[d] >> 16;
-                        rest[d] &= 0xffff;
-                    }
-                }
-                fx_collide9_run(X, h, add, fx, bad);
-                i64 *nxt = fs + (cur ^ 1) * 9 * P;
-#pragma unroll
-                for (int a = 0; a < 9; a++) nxt[a * P + l] = X[a];
-            }
-            cur ^= 1;
-            cl.sync();
-        }
-        if (own && bad < 0) range[2] = 1;
-        cl.sync();
-        int failed = 0;
-        for (int r = 0; r < nblk; r++) failed |= cl.map_shared_rank(range, r)[2];
-        fixed = !failed;
-        if (fixed && own)
-#pragma unroll
-            for (int a = 0; a < 9; a++) fout[a * g.Np + i] = fx_value(fs[cur * 9 * P + a * P + l], k);
-    }
-    if (!fixed) {
-        if (W1) cl.sync();  // every block has read its neighbours' last results
-        auto shape = [&](int d) { return d == 0 ? Px : Py; };
-        if (own)
-#pragma unroll
-            for (int a = 0; a < 9; a++) sm[a * P + l] = fin[a * g.Np + i];
-        cl.sync();
-        int cur = 0;
-        for (int n = 0; n < nsteps; n++) {
-            if (own) {
-                double f[9];
+            double f[9];
+            double *nxt = sm + (cur ^ 1) * 9 * P;
+            auto pull = [&]() {
 #pragma unroll
                 for (int a = 0; a < 9; a++) f[a] = cl.map_shared_rank(sm + cur * 9 * P, src_blk[a])[src_off[a]];
+            };
+            pull();
+            bool done = false;
+            if (W1) {
+                done = fixed_step9<FK != FK_NONE, false>(f, fx, q1, q2, shape, [&](int a, double v) { nxt[a * P + l] = v; });
+                if (!done) pull();
+            }
+            if (!done) {
                 double_step9<W1, false>(f, w, FK != FK_NONE, apre, gsum, shape);
-                double *nxt = sm + (cur ^ 1) * 9 * P;
 #pragma unroll
                 for (int a = 0; a < 9; a++) nxt[a * P + l] = f[a];
             }
-            cur ^= 1;
-            cl.sync();
         }
-        if (own)
-#pragma unroll
-            for (int a = 0; a < 9; a++) fout[a * g.Np + i] = sm[cur * 9 * P + a * P + l];
+        cur ^= 1;
+        cl.sync();
     }
-    cl.sync();  // no block leaves while another may still read its shared memory
+    if (own)
+#pragma unroll
+        for (int a = 0; a < 9; a++) fout[a * g.Np + i] = sm[cur * 9 * P + a * P + l];
 }
 
 // Batched form: one launch for every lattice of a batch; a step's amplitudes per
@@ -420,20 +348,21 @@ cudaError_t cluster_launch(cudaLaunchConfig_t &cfg, int C, const LaunchArgs &a, 
                            int nsteps)
 {
     const FxRates fx = fx_rates9(a.omega[3], a.omega[4], a.omega[5]);
+    const double q1 = 0.25 * a.apre, q2 = 0.25 * (a.apre + a.apost);
     switch (a.fkind) {
     case FK_NONE:
         if (C > 8) cudaFuncSetAttribute(k_cluster_steps<FK_NONE, W1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_NONE, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, fx, P,
-                                  nsteps);
+        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_NONE, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, fx, q1,
+                                  q2, P, nsteps);
     case FK_CONST:
         if (C > 8) cudaFuncSetAttribute(k_cluster_steps<FK_CONST, W1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_CONST, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, fx, P,
-                                  nsteps);
+        return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_CONST, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w, fx, q1,
+                                  q2, P, nsteps);
     default:
         if (C > 8)
             cudaFuncSetAttribute(k_cluster_steps<FK_GENERAL, W1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         return cudaLaunchKernelEx(&cfg, k_cluster_steps<FK_GENERAL, W1>, a.fin, a.fout, a.g, a.F, a.apre, gsum, w,
-                                  fx, P, nsteps);
+                                  fx, q1, q2, P, nsteps);
     }
 }
 

@@ -585,73 +585,6 @@ FX_HD void fx_collide9(const FxSums9<i64> &s, const FxForce (&F)[2], const FxRat
     f[7] = a0;
 }
 
-// The same collision on one grid for a whole run of steps (the cluster form of a
-// small lattice, which keeps its state in fixed point): moments are not halved and
-// the grid is not refined; a line's two outer populations share its second
-// moment, the odd unit included, so that mass and momentum stay exact.  h: F_pre
-// / 2 and t: (F_pre + F_post) / 2 per axis; bad < 0 also when a result leaves
-// |f| < 2^59 (FxGrid<9>::S + 2, what the next step's sums leave room for).
-FX_HD void fx_back_exact(i64 &m0, i64 &m1, i64 &m2)
-{
-    const i64 p = (m2 + m1) >> 1, m = p - m1;
-    m1 = m0 - p - m;
-    m0 = m;
-    m2 = p;
-}
-FX_HD void fx_collide9_run(i64 (&f)[9], const i64 (&h)[2], const i64 (&t)[2], const FxRates &w, int &bad)
-{
-    FxSums9<i64> s;
-    fx_sums9(f, s);
-    const i64 jx = s.jx + h[0], jy = s.jy + h[1], rho = s.rho;
-    const double ri = fx_reciprocal(rho, bad);
-    const i64 ux = fx_ratio(jx, rho, ri, bad), uy = fx_ratio(jy, rho, ri, bad);
-    const i64 cxx = s.xx - fx_mul(jx, ux), cyy = s.yy - fx_mul(jy, uy), cxy = s.xy - fx_mul(jx, uy);
-    const i64 r6 = fx_mul(rho, kFx6);
-    i64 Tq = r6;
-    if (w.c != 0) Tq += fx_mul(4 * r6 - (cxx + cyy), w.c);
-    const i64 Dq = fx_mul(cxx - cyy, w.a);
-    i64 m20 = 2 * (Tq + Dq), m02 = 2 * (Tq - Dq), m11 = 4 * fx_mul(cxy, w.b), m22 = fx_mul(rho, kFx9);
-    // back-shift along x, then along y
-    m20 += fx_mul(jx, ux);
-    i64 m21 = fx_mul(m11 + m11, ux), m12 = fx_mul(m02, ux);
-    m22 += fx_mul(m12, ux);
-    m02 += fx_mul(jy, uy);
-    const i64 y11 = m11 + fx_mul(jx, uy);
-    m12 += fx_mul(m11 + y11, uy);
-    m11 = y11;
-    const i64 y21 = m21 + fx_mul(m20, uy);
-    m22 += fx_mul(m21 + y21, uy);
-    m21 = y21;
-    // post-collision force: m_10 gains F_post / 2 (j: t in all), m_12 2 / 3 t
-    i64 a0 = rho, a1 = s.jx + t[0], a2 = m20, b0 = s.jy + t[1], b1 = m11, b2 = m21 + fx_mul(t[1] + t[1], kFx3), c0 = m02,
-        c1 = m12 + fx_mul(t[0] + t[0], kFx3), c2 = m22;
-    fx_back_exact(a0, b0, c0);  // x-order 0; e_y = -1, 0, +1
-    fx_back_exact(a1, b1, c1);
-    fx_back_exact(a2, b2, c2);
-    fx_back_exact(a0, a1, a2);  // e_y = -1: e_x = -1, 0, +1
-    fx_back_exact(b0, b1, b2);
-    fx_back_exact(c0, c1, c2);
-    f[0] = b1;
-    f[1] = b2;
-    f[3] = b0;
-    f[2] = c1;
-    f[5] = c2;
-    f[6] = c0;
-    f[4] = a1;
-    f[8] = a2;
-    f[7] = a0;
-    // |f| < 2^59: the top five bits of every result agree
-    unsigned top = 0;
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-    for (int a = 0; a < 9; a++) {
-        const unsigned hi = (unsigned)((u64)f[a] >> 32);
-        top |= hi ^ (hi << 1);
-    }
-    if (top & 0xf0000000u) bad = -1;
-}
-
 // ---- D2Q5 ---------------------------------------------------------------------
 // Step coefficients of a uniform advecting velocity (k_d2q5.cu Coef5) as
 // fractions of 2^63: h1 = A1 phi - c1 kx, h2 = A2 phi - c2 ky, h3 = P3 phi + X3
