@@ -143,15 +143,15 @@ __device__ __forceinline__ void collide_w1(double (&f)[9], double Fx, double Fy,
 
 // One node's step in fixed point (unit higher rates): shape(d) gives the force
 // shape's component d, q1 = a_pre / 4 and q2 = (a_pre + a_post) / 4, put(a, f)
-// takes a result.  Returns false for a node that needs the FP64 form (its
-// results are then void).
+// takes a result.
 template <bool FORCED, bool XO, class Shape, class Put>
-__device__ __forceinline__ bool fixed_step9(const double (&f)[9], const FxRates &w, double q1, double q2, Shape shape,
+__device__ __forceinline__ FxStep fixed_step9(const double (&f)[9], const FxRates &w, double q1, double q2, Shape shape,
                                             Put put)
 {
     const int em = fx_emax(f);
     const int k = FxGrid<9>::S + 1023 - em;
-    int bad = fx_in_range(em) ? 0 : -1;
+    if (!fx_in_range(em)) return FX_NOT;
+    int bad = 0;
     FxForce F[2] = {{0, 0}, {0, 0}};
     if (FORCED) {
         const unsigned dither = (unsigned)fx_bits(f[0]);
@@ -161,16 +161,17 @@ __device__ __forceinline__ bool fixed_step9(const double (&f)[9], const FxRates 
     }
     // D2Q9's populations at rest lie within the five binary orders that convert
     // exactly; a negative one takes the FP64 form
-    i64 X[9];
-    fx_load_int<9, false>(f, em, X);
 #pragma unroll
     for (int a = 0; a < 9; a++) bad |= (int)fx_hi(fx_bits(f[a]));
+    if (bad < 0) return FX_NOT;
+    i64 X[9];
+    fx_load_int<9, false>(f, em, X);
     FxSums9<i64> s;
     fx_sums9(X, s);
     fx_collide9<XO>(s, F, w, X, bad);
 #pragma unroll
     for (int a = 0; a < 9; a++) put(a, fx_value_pos(X[a], k + 1, bad));
-    return bad >= 0;
+    return bad >= 0 ? FX_DONE : FX_GIVEN_UP;
 }
 
 // The FP64 form of a node's step; gsum = (a_pre + a_post) / 12.
@@ -208,10 +209,9 @@ k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double a
     load_pulled<LD2Q9>(P, g, x, y, 0, i, f);
     auto shape = [&](int d) { return field_value(F, FK, d, x, y, 0, i); };
     if (W1) {
-        if (fixed_step9<FK != FK_NONE, XO>(f, fx, q1, q2, shape,
-                                           [&](int a, double v) { P.out[a][i] = v; }))
-            return;
-        load_pulled<LD2Q9>(P, g, x, y, 0, i, f);
+        const FxStep r = fixed_step9<FK != FK_NONE, XO>(f, fx, q1, q2, shape, [&](int a, double v) { P.out[a][i] = v; });
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD2Q9>(P, g, x, y, 0, i, f);
     }
     double_step9<W1, XO>(f, w, FK != FK_NONE, apre, gsum, shape);
 #pragma unroll
@@ -283,12 +283,10 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
                 for (int a = 0; a < 9; a++) f[a] = cl.map_shared_rank(sm + cur * 9 * P, src_blk[a])[src_off[a]];
             };
             pull();
-            bool done = false;
-            if (W1) {
-                done = fixed_step9<FK != FK_NONE, false>(f, fx, q1, q2, shape, [&](int a, double v) { nxt[a * P + l] = v; });
-                if (!done) pull();
-            }
-            if (!done) {
+            FxStep r = FX_NOT;
+            if (W1) r = fixed_step9<FK != FK_NONE, false>(f, fx, q1, q2, shape, [&](int a, double v) { nxt[a * P + l] = v; });
+            if (r == FX_GIVEN_UP) pull();
+            if (r != FX_DONE) {
                 double_step9<W1, false>(f, w, FK != FK_NONE, apre, gsum, shape);
 #pragma unroll
                 for (int a = 0; a < 9; a++) nxt[a * P + l] = f[a];
@@ -322,12 +320,14 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates9 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
     if (B.variant == 3) {  // uniform over the member
-        if (fixed_step9<true, true>(f, B.fx, ap.q1, ap.q2, shape, put)) return;
-        load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
+        const FxStep r = fixed_step9<true, true>(f, B.fx, ap.q1, ap.q2, shape, put);
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
         double_step9<true, true>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else if (B.variant == 1) {
-        if (fixed_step9<true, false>(f, B.fx, ap.q1, ap.q2, shape, put)) return;
-        load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
+        const FxStep r = fixed_step9<true, false>(f, B.fx, ap.q1, ap.q2, shape, put);
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
         double_step9<true, false>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else {
         double_step9<false, false>(f, w, forced, 4.0 * ap.q1, ap.g, shape);

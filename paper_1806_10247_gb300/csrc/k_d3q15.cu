@@ -118,20 +118,22 @@ __device__ __forceinline__ void collide(double (&f)[15], const double (&F)[3], c
 
 // One node's step in fixed point (omega_10 .. omega_14 = 1): shape(d) gives the
 // force shape's component d, q1 = a_pre / 4 and q2 = (a_pre + a_post) / 4, put(a,
-// f) takes a result.  Returns false for a node that needs the FP64 form.
+// f) takes a result.
 template <bool FORCED, bool XO, class Shape, class Put>
-__device__ __forceinline__ bool fixed_step15(const double (&f)[15], const FxRates &w, double q1, double q2, Shape shape,
+__device__ __forceinline__ FxStep fixed_step15(const double (&f)[15], const FxRates &w, double q1, double q2, Shape shape,
                                              Put put)
 {
     const int em = fx_emax(f);
     const int k = FxGrid<15>::S + 1023 - em;
-    int bad = fx_in_range(em) ? 0 : -1;
+    if (!fx_in_range(em)) return FX_NOT;
+    int bad = 0;
     FxForce F[3] = {{0, 0}, {0, 0}, {0, 0}};
     if (FORCED) {
         const unsigned dither = (unsigned)fx_bits(f[0]);
 #pragma unroll
         for (int d = 0; d < (XO ? 1 : 3); d++)
             if (!fx_force(shape(d), q1, q2, k, em, dither >> (8 * d), F[d])) bad = -1;
+        if (bad < 0) return FX_NOT;
     }
     i64 X[15];
     fx_load(f, k, X);
@@ -140,7 +142,7 @@ __device__ __forceinline__ bool fixed_step15(const double (&f)[15], const FxRate
     fx_collide15<XO>(s, F, w, X, bad);
 #pragma unroll
     for (int a = 0; a < 15; a++) put(a, fx_value_pos(X[a], k + 1, bad));
-    return bad >= 0;
+    return bad >= 0 ? FX_DONE : FX_GIVEN_UP;
 }
 
 template <class Shape>
@@ -175,10 +177,9 @@ k_step(const __grid_constant__ Planes<double, 15> P, Geom g, FieldDev Fd, double
     load_pulled<LD3Q15>(P, g, x, y, z, i, f);
     auto shape = [&](int d) { return field_value(Fd, FK, d, x, y, z, i); };
     if (FIX) {
-        if (fixed_step15<FK != FK_NONE, XO>(f, fx, q1, q2, shape,
-                                            [&](int a, double v) { P.out[a][i] = v; }))
-            return;
-        load_pulled<LD3Q15>(P, g, x, y, z, i, f);
+        const FxStep r = fixed_step15<FK != FK_NONE, XO>(f, fx, q1, q2, shape, [&](int a, double v) { P.out[a][i] = v; });
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD3Q15>(P, g, x, y, z, i, f);
     }
     double_step15(f, w, FK != FK_NONE, apre, apost, shape);
 #pragma unroll
@@ -203,10 +204,10 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     auto shape = [&](int d) { return forced ? field_value(B.F, B.fkind, d, x, y, z, i) : 0.0; };
     const Rates15 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3]};
     if (w.t == 1.0 && w.q == 1.0) {  // uniform over the member
-        if (fixed_step15<true, false>(f, B.fx, ap.q1, ap.q2, shape,
-                                      [&](int a, double v) { fout[a * g.Np + i] = v; }))
-            return;
-        load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
+        const FxStep r =
+            fixed_step15<true, false>(f, B.fx, ap.q1, ap.q2, shape, [&](int a, double v) { fout[a * g.Np + i] = v; });
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
     }
     double_step15(f, w, forced, 4.0 * ap.q1, ap.g, shape);
 #pragma unroll

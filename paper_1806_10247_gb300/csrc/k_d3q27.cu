@@ -304,21 +304,22 @@ __device__ __forceinline__ void collide_w1(double (&m)[27], const double (&F)[3]
 
 // One node's step in fixed point (unit higher rates): get() pulls the
 // populations, shape(d) gives the force shape's component d, q1 = a_pre / 4 and
-// q2 = (a_pre + a_post) / 4, put(a, f) stores a result.  Returns false for a
-// node that needs the FP64 form (what it has stored is then overwritten).
+// q2 = (a_pre + a_post) / 4, put(a, f) stores a result.
 template <bool FORCED, bool XO, class Shape, class Put>
-__device__ __forceinline__ bool fixed_step27(const double (&f)[27], const FxRates &w, double q1, double q2, Shape shape,
+__device__ __forceinline__ FxStep fixed_step27(const double (&f)[27], const FxRates &w, double q1, double q2, Shape shape,
                                              Put put)
 {
     const int em = fx_emax(f);
     const int k = FxGrid<27>::S + 1023 - em;
-    int bad = fx_in_range(em) ? 0 : -1;
+    if (!fx_in_range(em)) return FX_NOT;
+    int bad = 0;
     FxForce F[3] = {{0, 0}, {0, 0}, {0, 0}};
     if (FORCED) {
         const unsigned dither = (unsigned)fx_bits(f[13]);
 #pragma unroll
         for (int d = 0; d < (XO ? 1 : 3); d++)
             if (!fx_force(shape(d), q1, q2, k, em, dither >> (8 * d), F[d])) bad = -1;
+        if (bad < 0) return FX_NOT;
     }
     i64 X[27];
     fx_load(f, k, X);
@@ -327,7 +328,7 @@ __device__ __forceinline__ bool fixed_step27(const double (&f)[27], const FxRate
     fx_collide27<XO>(s, F, w, X, bad);
 #pragma unroll
     for (int a = 0; a < 27; a++) put(a, fx_value_pos(X[a], k + 1, bad));
-    return bad >= 0;
+    return bad >= 0 ? FX_DONE : FX_GIVEN_UP;
 }
 
 // The FP64 form of a node's step.
@@ -381,10 +382,9 @@ k_step(const __grid_constant__ Planes<double, 27> P, Geom g, FieldDev Fd, double
     load_pulled<LD3Q27, !OV>(P, g, x, y, z, i, m);
     auto shape = [&](int d) { return field_value(Fd, FK, d, x, y, z, i); };
     if (W1) {
-        if (fixed_step27<FK != FK_NONE, XO>(m, fx, q1, q2, shape,
-                                            [&](int a, double v) { P.out[a][i] = v; }))
-            return;
-        load_pulled<LD3Q27, !OV>(P, g, x, y, z, i, m);
+        const FxStep r = fixed_step27<FK != FK_NONE, XO>(m, fx, q1, q2, shape, [&](int a, double v) { P.out[a][i] = v; });
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD3Q27, !OV>(P, g, x, y, z, i, m);
     }
     double_step27<W1, XO>(m, w, FK != FK_NONE, apre, apost, shape);
 #pragma unroll
@@ -411,12 +411,14 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
     auto put = [&](int a, double v) { fout[a * g.Np + i] = v; };
     const Rates27 w{B.coef[0], B.coef[1], B.coef[2], B.coef[3], B.coef[4], B.coef[5]};
     if (B.variant == 3) {  // uniform over the member
-        if (fixed_step27<true, true>(m, B.fx, ap.q1, ap.q2, shape, put)) return;
-        load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
+        const FxStep r = fixed_step27<true, true>(m, B.fx, ap.q1, ap.q2, shape, put);
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
         double_step27<true, true>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else if (B.variant == 1) {
-        if (fixed_step27<true, false>(m, B.fx, ap.q1, ap.q2, shape, put)) return;
-        load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
+        const FxStep r = fixed_step27<true, false>(m, B.fx, ap.q1, ap.q2, shape, put);
+        if (r == FX_DONE) return;
+        if (r == FX_GIVEN_UP) load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
         double_step27<true, false>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
     } else {
         double_step27<false, false>(m, w, forced, 4.0 * ap.q1, ap.g, shape);

@@ -17,11 +17,11 @@
 // between the two conversions.  The result is rounded to FP64 once, to nearest
 // even.
 //
-// What the fixed-point form does not take (a population that is not finite, an
-// exponent outside [kEmaxLo, kEmaxHi], |u| >= 1/2, a density far below the
-// largest population, a force as large as the populations, a result that is
-// negative or below 2^-25 of the largest population) is left to the FP64 form:
-// the functions return false and the caller takes that node's FP64 path.
+// What the fixed-point form does not take is left to the FP64 form of that node: known
+// before any of its work, a population that is not finite, an exponent outside
+// [kEmaxLo, kEmaxHi] (a scalar on a background of 0) or a force as large as the
+// populations; found on the way, |u| >= 1/2, a density far below the largest population, a
+// result that is negative or below 2^-25 of the largest population (FxStep).
 //
 // Everything here compiles for the host too (tests run it against 64-bit and
 // wider arithmetic on the CPU).
@@ -38,6 +38,11 @@
 #endif
 
 namespace lbmk {
+
+// What a node's step in fixed point did: FX_DONE, FX_NOT (nothing: the populations are as
+// they were) or FX_GIVEN_UP (its results are void, the populations to be pulled again:
+// keeping them beside the fixed-point values would cost registers at every node).
+enum FxStep { FX_DONE, FX_NOT, FX_GIVEN_UP };
 
 typedef long long i64;
 typedef unsigned long long u64;
