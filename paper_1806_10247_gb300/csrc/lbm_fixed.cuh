@@ -223,6 +223,38 @@ FX_HD void fx_load_int(const double (&f)[Q], int emax, i64 (&X)[Q])
     }
 }
 
+// FP32 deviations as integers X = d 2^(182 - em), em the biased exponent of the largest:
+// 24-bit values, 32 bits below the largest one's last, rounded towards zero.  Not taken:
+// em below 56, where the leading bit that a zero or a subnormal value does not have
+// (added to every value) would not yet be shifted out, and a value that is not finite.
+enum FxDev { FXD_ZERO, FXD_TAKEN, FXD_NOT };
+template <int Q>
+FX_HD FxDev fx_load_dev(const float (&d)[Q], int &em, i64 (&X)[Q])
+{
+    unsigned m = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < Q; a++) {
+        const unsigned b = fx_float_bits(d[a]) & 0x7fffffffu;
+        m = b > m ? b : m;
+    }
+    em = (int)(m >> 23);
+    if (m == 0) return FXD_ZERO;
+    if (em < 56 || em >= 255) return FXD_NOT;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < Q; a++) {
+        const unsigned b = fx_float_bits(d[a]);
+        const int sh = em - (int)((b >> 23) & 0xffu);
+        const u64 v = (u64)((b & 0x7fffffu) | 0x800000u) << 32 >> (sh < 63 ? sh : 63);
+        const i64 s = (i64)((int)b >> 31);
+        X[a] = ((i64)v ^ s) - s;
+    }
+    return FXD_TAKEN;
+}
+
 // X 2^-k, rounded to nearest even; 0 gives 0.
 FX_HD double fx_value(i64 X, int k)
 {

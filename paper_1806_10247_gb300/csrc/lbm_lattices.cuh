@@ -273,25 +273,15 @@ __device__ __forceinline__ void zeroth_first(const double (&f)[L::Q], double &m0
 template <class L>
 __device__ __forceinline__ void zeroth_first(const float (&d)[L::Q], double &m0, double (&j)[3])
 {
-    unsigned m = 0;
-#pragma unroll
-    for (int a = 0; a < L::Q; a++) m = max(m, __float_as_uint(d[a]) & 0x7fffffffu);
-    const int em = (int)(m >> 23);
-    if (m == 0) {  // a node at the reference state
+    int em;
+    i64 X[L::Q];
+    const FxDev r = fx_load_dev(d, em, X);
+    if (r == FXD_ZERO) {  // a node at the reference state
         m0 = j[0] = j[1] = j[2] = 0.0;
         return;
     }
-    if (em >= 40 && em < 255) {
-        i64 X[L::Q], M, J[3];
-#pragma unroll
-        for (int a = 0; a < L::Q; a++) {
-            const unsigned b = __float_as_uint(d[a]);
-            const int e = (int)((b >> 23) & 0xffu);
-            // a zero or subnormal value lies more than 2^39 below the largest: nothing is left of it
-            const u64 v = (u64)((b & 0x7fffffu) | 0x800000u) << 32 >> min(em - e, 63);
-            const i64 s = (i64)((int)b >> 31);
-            X[a] = ((i64)v ^ s) - s;
-        }
+    if (r == FXD_TAKEN) {
+        i64 M, J[3];
         sum_moments<L>(X, M, J);
         const int k = 23 + 32 + 127 - em;  // X = d 2^k
         m0 = fx_value(M, k);
