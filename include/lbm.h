@@ -268,7 +268,7 @@ int lbm_step(lbm_ctx *ctx, long n);
  * formed in fixed point at the scale of the node's largest population (exactly,
  * up to 3 to 5 bits below that population's last one) and rounded once, on D2Q5
  * and outside 2^-523 .. 2^50 in FP64; j + a_pre P/2 rounded once; u = that times
- * 1/rho (within 0.51 units of its last place), the product rounded.  Every FP64 readback
+ * the correctly rounded 1/rho, the product rounded.  Every FP64 readback
  * (lbm_batch_moments, lbm_batch_moments_packed, lbm_batch_step_read) returns
  * these same bits.  where = 0: host pointers (the call synchronises);
  * where = 1: device pointers (asynchronous).

@@ -136,18 +136,27 @@ FX_HD double fx_widen(float x)
 {
     return fx_double(((u64)fx_float_bits(x) << 29) + ((u64)(1023 - 127) << 52));
 }
-// 1/x for a positive normal x, within 0.51 units of the last place: a 22-bit
-// reciprocal of the mantissa r with one third-order correction, r (1 + e + e^2),
-// e = 1 - x r; three FP64 operations (the correctly rounded division and
-// reciprocal of the maths library take about seven).
+// 1/x for a positive normal x (biased exponent 3 .. 2043), correctly rounded: a 22-bit
+// reciprocal of the mantissa r with one third-order correction, r (1 + e + e^2), e = 1 -
+// x r, is within 0.51 units of the last place; with X and Y the mantissas of x and of that
+// result as integers, 2^105 - X Y (known from its low 64 bits, as it is below X in
+// magnitude) tells whether a neighbour is nearer.  Three FP64 operations and about
+// fifteen of the integer unit, where the maths library's reciprocal takes about seven of
+// the FP64 unit, which bounds the readbacks.
 FX_HD double fx_recip(double x)
 {
+    constexpr u64 kMant = 0x000fffffffffffffull, kLead = 0x0010000000000000ull;
     const u64 b = fx_bits(x);
-    const u64 m = (b & 0x000fffffffffffffull) | 0x3ff0000000000000ull;      // mantissa in [1, 2)
+    const u64 m = (b & kMant) | 0x3ff0000000000000ull;      // mantissa in [1, 2)
     const double r = fx_widen(fx_rcp_approx(fx_float(0x3f800000u | ((unsigned)(m >> 29) & 0x7fffffu))));
     const double e = fma(-fx_double(m), r, 1.0);
     const double p = fma(e, e, e);
-    return fx_ldexp(fma(r, p, r), 1023 - (int)(b >> 52));
+    u64 y = fx_bits(fma(r, p, r));
+    const i64 X = (i64)((b & kMant) | kLead);
+    const i64 R2 = (i64)(0ull - 2ull * (u64)X * ((y & kMant) | kLead));
+    if (R2 > X) y++;
+    if (R2 < -X) y--;
+    return fx_ldexp(fx_double(y), 1023 - (int)(b >> 52));
 }
 
 // ---- scale --------------------------------------------------------------------

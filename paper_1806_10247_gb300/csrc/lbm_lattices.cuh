@@ -295,12 +295,11 @@ __device__ __forceinline__ void zeroth_first(const float (&d)[L::Q], double &m0,
     sum_moments<L>(dd, m0, j);
 }
 
-// 1/rho of the readbacks: fx_recip for a positive normal rho, the correctly rounded
-// reciprocal for any other.
+// The correctly rounded 1/rho of the readbacks.
 __device__ __forceinline__ double recip_density(double rho)
 {
-    const unsigned e = fx_hi(fx_bits(rho)) >> 20;
-    return e - 1u < 2045u && e > 2u && e < 2044u ? fx_recip(rho) : __drcp_rn(rho);
+    const unsigned e = fx_hi(fx_bits(rho)) >> 20;  // (a negative rho: above 2047)
+    return e > 2u && e < 2044u ? fx_recip(rho) : __drcp_rn(rho);
 }
 
 // Whether component c of a shape is known to vanish everywhere.

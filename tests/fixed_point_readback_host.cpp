@@ -21,3 +21,9 @@ extern "C" void deviation_sums(long n, const float *d, double *m0, double *jx, i
         jx[i] = fx_value(s.jx, 182 - em);
     }
 }
+
+// 1/x as the readbacks form it.
+extern "C" void reciprocals(long n, const double *x, double *r)
+{
+    for (long i = 0; i < n; i++) r[i] = fx_recip(x[i]);
+}

@@ -59,3 +59,13 @@ def test_non_finite_deviations_are_left_to_fp64(host):
     m0, jx, taken = np.zeros(2), np.zeros(2), np.zeros(2, np.int32)
     host.deviation_sums(ctypes.c_long(2), _p(d), _p(m0), _p(jx), _p(taken))
     assert not taken.any()
+
+
+def test_reciprocals_are_correctly_rounded(host):
+    rng = np.random.default_rng(6)
+    x = np.concatenate([1.0 + rng.uniform(size=1000000), 1.0 + 2.0 ** -52 * np.arange(1000), 2.0 - 2.0 ** -52 * np.arange(1, 1000),
+                        1.0 / (1.0 - 2.0 ** -53 * np.arange(1, 100000)), 2.0 ** np.arange(-1019, 1020.0),
+                        rng.uniform(1, 2, 10000) * 2.0 ** rng.integers(-1019, 1019, 10000)])
+    r = np.empty_like(x)
+    host.reciprocals(ctypes.c_long(len(x)), _p(x), _p(r))
+    assert np.array_equal(r, 1.0 / x)
