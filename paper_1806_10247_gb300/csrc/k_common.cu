@@ -157,8 +157,18 @@ __device__ void block_reduce_store(double (&v)[R_SLOTS], double *out)
 // Per-block partial sums of rho (or phi^o) and momentum, the largest change
 // of the half-forced velocity (or scalar) since the snapshot (the snapshot is
 // then overwritten), and a flag for non-finite or non-positive densities.
+// Blocks of a reduction kernel that an SM holds: left to the compiler, the sums in fixed
+// point take registers for fewer (D2Q9 2, D3Q27 1), and the loads' latency is not hidden
+// (lbm_reduce, 2048 x 1024 D2Q9: 267 us with 2, 264 with 3, 240 with 4; 160^3 D3Q27 897
+// with 1, 720 with 2; 128^3 D3Q15 385 with 2, 362 with 3).
 template <class L>
-__global__ void __launch_bounds__(kBlock)
+constexpr int reduce_min_blocks()
+{
+    return L::Q <= 9 ? 4 : (L::Q == 15 ? 3 : 2);
+}
+
+template <class L>
+__global__ void __launch_bounds__(kBlock, reduce_min_blocks<L>())
 k_reduce_partial(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, double ahalf,
                  double *__restrict__ snap, int have_snap, double *__restrict__ partials)
 {
@@ -197,7 +207,7 @@ k_reduce_partial(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, 
 // Same partial sums without the velocity snapshot (mass, momentum and the
 // instability flag only); writes nothing but its partials slot.
 template <class L>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, reduce_min_blocks<L>())
 k_reduce_partial_sums(Geom g, const double *__restrict__ fin, double *__restrict__ partials)
 {
     double v[R_SLOTS] = {0, 0, 0, 0, 0, 0, 0, 0};
