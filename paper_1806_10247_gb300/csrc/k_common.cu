@@ -159,8 +159,9 @@ __device__ void block_reduce_store(double (&v)[R_SLOTS], double *out)
 // then overwritten), and a flag for non-finite or non-positive densities.
 // Blocks of a reduction kernel that an SM holds: left to the compiler, the sums in fixed
 // point take registers for fewer (D2Q9 2, D3Q27 1), and the loads' latency is not hidden
-// (lbm_reduce, 2048 x 1024 D2Q9: 267 us with 2, 264 with 3, 240 with 4; 160^3 D3Q27 897
-// with 1, 720 with 2; 128^3 D3Q15 385 with 2, 362 with 3).
+// (lbm_reduce, with the maths library's reciprocal: 2048 x 1024 D2Q9 267 us with 2, 264
+// with 3, 240 with 4; 160^3 D3Q27 897 with 1, 720 with 2; 128^3 D3Q15 385 with 2, 362
+// with 3; now 162, 644 and 300).
 template <class L>
 constexpr int reduce_min_blocks()
 {
@@ -188,12 +189,13 @@ k_reduce_partial(Geom g, const double *__restrict__ fin, int fkind, FieldDev F, 
             if (have_snap) v[R_DU] = fmax(v[R_DU], fabs(phi - snap[i]));
             snap[i] = phi;
         } else {
-            const double rinv = recip_density(m0);
+            int sh;
+            const double rinv = density_recip(m0, sh);
 #pragma unroll
             for (int d = 0; d < L::DIM; d++) {
                 v[R_JX + d] += j[d];
                 double jd = field_zero(F, fkind, d) ? j[d] : j[d] + ahalf * field_value(F, fkind, d, x, y, z, i);
-                double ud = jd * rinv;
+                double ud = over_density(jd, sh) * rinv;
                 bad = bad || !isfinite(ud);
                 if (have_snap) v[R_DU] = fmax(v[R_DU], fabs(ud - snap[(long long)d * g.N + i]));
                 snap[(long long)d * g.N + i] = ud;
@@ -251,13 +253,14 @@ k_reduce_partial_rp(Geom g, const T *__restrict__ fin, double rho_ref, int fkind
                 snap[i] = phi;
             }
         } else {
-            const double rinv = with_snap ? recip_density(m0) : 0.0;
+            int sh = 0;
+            const double rinv = with_snap ? density_recip(m0, sh) : 0.0;
 #pragma unroll
             for (int d = 0; d < L::DIM; d++) {
                 v[R_JX + d] += j[d];
                 if (with_snap) {
                     double jd = field_zero(F, fkind, d) ? j[d] : j[d] + ahalf * field_value(F, fkind, d, x, y, z, i);
-                    double ud = jd * rinv;
+                    double ud = over_density(jd, sh) * rinv;
                     bad = bad || !isfinite(ud);
                     if (have_snap) v[R_DU] = fmax(v[R_DU], fabs(ud - snap[(long long)d * g.N + i]));
                     snap[(long long)d * g.N + i] = ud;

@@ -295,11 +295,31 @@ __device__ __forceinline__ void zeroth_first(const float (&d)[L::Q], double &m0,
     sum_moments<L>(dd, m0, j);
 }
 
-// The correctly rounded 1/rho of the readbacks.
-__device__ __forceinline__ double recip_density(double rho)
+// Whether fx_recip takes a density (a negative one's exponent is above 2047).
+__device__ __forceinline__ bool recip_takes(double rho)
 {
-    const unsigned e = fx_hi(fx_bits(rho)) >> 20;  // (a negative rho: above 2047)
-    return e > 2u && e < 2044u ? fx_recip(rho) : __drcp_rn(rho);
+    const unsigned e = fx_hi(fx_bits(rho)) >> 20;
+    return e > 2u && e < 2044u;
+}
+// The correctly rounded 1/rho of the readbacks.
+__device__ __forceinline__ double recip_density(double rho) { return recip_takes(rho) ? fx_recip(rho) : __drcp_rn(rho); }
+// j / rho of the reductions is over_density(j, sh) * density_recip(rho, sh): where rho lies
+// near an end of the FP64 range (its reciprocal need not be an FP64 number) both are
+// scaled by 2^700 or 2^-700 first (sh > 0, < 0).  NaN for a density that is not positive and finite.
+__device__ __forceinline__ double over_density(double j, int sh)
+{
+    return sh == 0 ? j : j * (sh > 0 ? 0x1p700 : 0x1p-700);
+}
+__device__ __forceinline__ double density_recip(double rho, int &sh)
+{
+    sh = 0;
+    if (!recip_takes(rho)) {
+        const u64 b = fx_bits(rho);
+        if (b - 1u >= 0x7fefffffffffffffull) return fx_double(0x7ff8000000000000ull);
+        sh = b >> 52 < 3u ? 1 : -1;
+        rho = over_density(rho, sh);
+    }
+    return fx_recip(rho);
 }
 
 // Whether component c of a shape is known to vanish everywhere.
