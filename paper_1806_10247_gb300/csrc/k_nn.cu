@@ -16,9 +16,12 @@
 #include <string>
 
 #include "../../include/lbm.h"
+#include "k_nn_index.cuh"
 #include "k_nn_tc.cuh"
 
 namespace {
+
+using namespace nnix;
 
 constexpr int kT = 256;
 thread_local std::string g_nn_error;
@@ -33,14 +36,6 @@ int nn_fail(int code, const char *fmt, ...)
     g_nn_error = buf;
     return code;
 }
-
-struct Shape {
-    int n, ci, co, d, h, w;  // batch, channels in/out, spatial extents
-    int kd, kh, kw;          // kernel extents (odd)
-    int dd, dh, dw;          // dilations
-    __host__ __device__ long long in_count() const { return (long long)n * ci * d * h * w; }
-    __host__ __device__ long long out_count() const { return (long long)n * co * d * h * w; }
-};
 
 __device__ __forceinline__ float wload(const void *w, int bf16, long long i)
 {
@@ -283,72 +278,12 @@ int round16(int v) { return (v + 15) / 16 * 16; }
 
 enum TcMode { TC_FWD = 0, TC_BWD_IN = 1 };
 
-// Pixel coordinates of pixel q of a batch (32-bit: the launchers check the sizes).
-struct Pixel {
-    int n, p;        // sample, position inside it
-    int d, h, w;
-};
-__device__ __forceinline__ Pixel pixel_at(const Shape &s, unsigned q)
-{
-    const unsigned sp = (unsigned)(s.d * s.h * s.w);
-    Pixel x;
-    x.n = (int)(q / sp);
-    x.p = (int)(q - (unsigned)x.n * sp);
-    const unsigned r = (unsigned)x.p / (unsigned)s.w;
-    x.w = x.p - (int)(r * (unsigned)s.w);
-    x.d = (int)(r / (unsigned)s.h);
-    x.h = (int)(r - (unsigned)x.d * (unsigned)s.h);
-    return x;
-}
-// Position of the source pixel of tap (a, f, e), shifted by sgn * dilation; -1 outside.
-__device__ __forceinline__ int tap_source(const Shape &s, const Pixel &x, int a, int f, int e, int sgn)
-{
-    const int zd = x.d + sgn * s.dd * (a - (s.kd - 1) / 2);
-    const int zh = x.h + sgn * s.dh * (f - (s.kh - 1) / 2);
-    const int zw = x.w + sgn * s.dw * (e - (s.kw - 1) / 2);
-    const bool in = (unsigned)zd < (unsigned)s.d && (unsigned)zh < (unsigned)s.h && (unsigned)zw < (unsigned)s.w;
-    return in ? (zd * s.h + zh) * s.w + zw : -1;
-}
 __device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
 {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     unsigned u;
     memcpy(&u, &v, sizeof u);
     return u;
-}
-
-// The images as one line of positions: every row of w pixels is followed by hw
-// empty ones (hw: the taps' reach along w), so that position + shift is the
-// shifted pixel of the same row, or an empty one, for every |shift| <= hw.
-struct Line {
-    int hw, wp;       // reach, positions per row
-    unsigned total;   // positions of the batch
-    int sp;
-};
-__host__ __device__ inline Line line_of(const Shape &s)
-{
-    Line l;
-    l.hw = s.dw * ((s.kw - 1) / 2);
-    l.wp = s.w + l.hw;
-    l.sp = s.d * s.h * s.w;
-    l.total = (unsigned)s.n * (unsigned)(s.d * s.h) * (unsigned)l.wp;
-    return l;
-}
-// Sample, plane, row and column of a position; w < 0 outside the batch and on empty positions.
-__device__ __forceinline__ Pixel position_at(const Shape &s, const Line &l, int q)
-{
-    Pixel x;
-    x.n = x.d = x.h = x.p = 0;
-    x.w = -1;
-    if (q < 0 || (unsigned)q >= l.total) return x;
-    const unsigned r = (unsigned)q / (unsigned)l.wp;
-    const int w = q - (int)(r * (unsigned)l.wp);
-    const unsigned z = r / (unsigned)s.h;
-    x.h = (int)(r - z * (unsigned)s.h);
-    x.n = (int)(z / (unsigned)s.d);
-    x.d = (int)(z - (unsigned)x.n * (unsigned)s.d);
-    x.w = w < s.w ? w : -1;
-    return x;
 }
 
 // Forward pass and input gradient.
@@ -433,7 +368,7 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
 #pragma unroll
                     for (int j = 0; j < 8; j++) {
                         const int c = (8 * g + j) / 9, tap = (8 * g + j) % 9;
-                        v[j] = at[tap] >= 0 && c0 + c < cin ? __ldg(src + c * sp + at[tap]) : 0.f;
+                        v[j] = at[tap] >= 0 && c0 + c < cin ? __ldg(src + plane_offset(c, sp, at[tap])) : 0.f;
                     }
                     put8(k8, v);
                 }
@@ -445,7 +380,7 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
                     const int at = valid && c < cin ? tap_source(s, x, a, f, e, sgn) : -1;
-                    v[j] = at >= 0 ? __ldg(base + (long long)c * sp + at) : 0.f;
+                    v[j] = at >= 0 ? __ldg(base + plane_offset(c, sp, at)) : 0.f;
                     if (++e == s.kw) {
                         e = 0;
                         if (++f == s.kh) {
