@@ -446,7 +446,10 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
 // dilation 8, 32 x 128^2 pixels, forward: 61 us (the memory's time is 10); the gather
 // above, nine loads a value from L1 and L2, 88; a division per gathered value and a block
 // per tile about 900.  Now bound by instruction issue: tanh, the staging and the rows of K.
-constexpr int kStagedChannels = 16;
+// The staged positions on either side of a tile grow with the dilation: 32 x 128^2, 16 -> 16
+// channels, dilation 8, 16, 24, 63, 127: 57, 70, 73, 88, 166 us, gathered 74, 72, 72, 71, 67; 2
+// x 256 x 2048, 8, 16, 24, 127, 868: 112, 143, 143, 246, 1615, gathered 157, 157, 157, 152, 153.
+constexpr int kStagedChannels = 16, kStagedReach = 16;
 template <int MODE>
 __global__ void __launch_bounds__(nntc::kM)
 k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
@@ -598,12 +601,14 @@ k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
 // the sums of gy, bpart[g][o].  k_tc_reduce_w adds the G partial sums in a fixed
 // order.  A thread loads the value of one position (and the first 2 hw threads
 // one of the halo) once per row of taps and channel, rounds it once and stores
-// it in the kw columns that its taps along w put it in.  Columns are stored two
-// bytes at a time; the core matrices lie kPad bytes further apart along K than
+// it in the kw columns that its taps along w put it in.  FAR: tap by tap, for dilations of
+// a chunk and more, where the taps' positions lie apart, and for taps out of reach (2 x 256 x 2048 positions, 16
+// channels, dilation 868: 228 us, with the whole halo 1214; dilation 127: 260 with it).
+// Columns are stored two bytes at a time; the core matrices lie kPad bytes further apart along K than
 // they are long, so that the 32 columns of a warp fall on 16 different banks (two
 // columns share a word).
 constexpr int kPad = 16;
-template <int N16>
+template <int N16, bool FAR>
 __global__ void __launch_bounds__(nntc::kM)
 k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float *__restrict__ part,
                 float *__restrict__ bpart, Shape s, int G, int tiles)
@@ -620,6 +625,10 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
     const uint32_t lboA = (uint32_t)rows * 16 + kPad, lboB = (uint32_t)Np * 16 + kPad;
     unsigned char *Bs = smem;
     unsigned char *As = smem + (kM / 8) * lboB;  // last: the rows past `rows` of the last tile read what follows
+    const int mid = (s.kw - 1) / 2, reach = FAR ? taps_in_reach(s) : mid;
+    if (FAR && reach < mid) {  // the columns of the taps without a source stay 0
+        for (uint32_t k = tid; k < kM / 8 * lboA / 16; k += kM) reinterpret_cast<uint4 *>(As)[k] = make_uint4(0, 0, 0, 0);
+    }
     const unsigned nchunks = (l.total + kM - 1) / kM;
     const int g = blockIdx.x;
     const uint32_t ncols = tmem_cols(tiles * Np);
@@ -648,7 +657,9 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
                 *reinterpret_cast<__nv_bfloat16 *>(col + o * 16) = __float2bfloat16_rn(v);
             }
         }
-        for (int j = tid - l.hw; j < kM + l.hw; j += kM) {
+        // j: a position less q0, its value into the columns of the taps first .. last
+        int first = mid - reach, last = FAR ? first : s.kw - 1;
+        for (int j = tid - l.hw; FAR ? first <= mid + reach : j < kM + l.hw; j += FAR ? s.dw : kM) {
             const Pixel px = position_at(s, l, q0 + j);
             const float *base = x + (long long)px.n * s.ci * l.sp + px.w;
             for (int seg = 0; seg < segs; seg++) {
@@ -661,8 +672,8 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
 #pragma unroll
                     for (int i = 0; i < 8; i++)
                         v[i] = __float2bfloat16_rn(have && i0 + i < s.ci ? __ldg(src + (long long)(i0 + i) * l.sp) : 0.f);
-                    for (int e = 0; e < s.kw; e++) {
-                        const int k = j - s.dw * (e - (s.kw - 1) / 2);
+                    for (int e = FAR ? first : 0; e <= last; e++) {
+                        const int k = j - s.dw * (e - mid);
                         if ((unsigned)k >= (unsigned)kM) continue;
                         unsigned char *dst = As + (k >> 3) * lboA + (k & 7) * 2 + ((seg * s.kw + e) * s.ci + i0) * 16;
 #pragma unroll
@@ -671,6 +682,7 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
                     }
                 }
             }
+            if (FAR) last = ++first;
         }
         fence_smem_to_async();
         fence_before_sync();
@@ -842,7 +854,7 @@ int tc_conv_launch(const float *in, const void *w, const float *b, float *out, c
     if (s.kd == 1 && s.kh == 3 && s.kw == 3) {
         const Line l = line_of(s);
         const size_t stage = (size_t)3 * (kStagedChannels / 8) * ((nntc::kM + 2 * (size_t)l.hw + 7) / 8 * 8) * 16;
-        if (cin <= kStagedChannels && smem + stage <= 220u * 1024u)  // the dilation decides
+        if (cin <= kStagedChannels && l.hw <= kStagedReach && l.hw == s.dw)
             return tc_launch(k_tc_conv_staged<MODE>, (l.total + nntc::kM - 1) / nntc::kM, smem + stage, Np, st, what, in,
                              wb, b, out, s, act, Kp, Np);
     }
@@ -852,7 +864,7 @@ int tc_conv_launch(const float *in, const void *w, const float *b, float *out, c
     return tc_launch(k_tc_conv<MODE, 0>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
 }
 
-template <int N16>
+template <int N16, bool FAR>
 int tc_conv_bwd_w_launch(const float *x, const float *gy, float *gw, float *gb, const Shape &s, cudaStream_t st)
 {
     constexpr int Np = 16 * N16;
@@ -860,18 +872,25 @@ int tc_conv_bwd_w_launch(const float *x, const float *gy, float *gw, float *gb, 
     const int tiles = (Kw + nntc::kM - 1) / nntc::kM, Mp = tiles * nntc::kM;
     const unsigned nchunks = (line_of(s).total + nntc::kM - 1) / nntc::kM;
     const size_t smem = (size_t)(nntc::kM / 8) * (rows * 16 + kPad + Np * 16 + kPad) + (size_t)(Mp - rows) * 16;
-    cudaError_t e = cudaFuncSetAttribute(k_tc_conv_bwd_w<N16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_tc_conv_bwd_w<N16, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return nn_fail(LBM_ECUDA, "conv3d_backward(weights): %s", cudaGetErrorString(e));
-    unsigned G = resident_grid(k_tc_conv_bwd_w<N16>, smem, nntc::tmem_cols(tiles * Np));
+    unsigned G = resident_grid(k_tc_conv_bwd_w<N16, FAR>, smem, nntc::tmem_cols(tiles * Np));
     if (G > nchunks) G = nchunks;
     float *part = static_cast<float *>(scratch_alloc((size_t)G * (Mp + 1) * Np * sizeof(float), st));
     if (!part) return nn_fail(LBM_ENOMEM, "conv3d_backward: tensor-core workspace");
     float *bpart = part + (size_t)G * Mp * Np;
-    k_tc_conv_bwd_w<N16><<<G, nntc::kM, smem, st>>>(x, gy, part, bpart, s, (int)G, tiles);
+    k_tc_conv_bwd_w<N16, FAR><<<G, nntc::kM, smem, st>>>(x, gy, part, bpart, s, (int)G, tiles);
     k_tc_reduce_w<<<Kw + 1, kT, 0, st>>>(part, bpart, gw, gb, s.ci, s.co, taps, (int)G, Mp, Np);
     const int rc = launched("conv3d_backward(weights)");
     cudaFreeAsync(part, st);
     return rc;
+}
+
+template <int N16>
+int tc_conv_bwd_w(const float *x, const float *gy, float *gw, float *gb, const Shape &s, cudaStream_t st)
+{
+    return s.dw >= nntc::kM || taps_in_reach(s) < (s.kw - 1) / 2 ? tc_conv_bwd_w_launch<N16, true>(x, gy, gw, gb, s, st)
+                            : tc_conv_bwd_w_launch<N16, false>(x, gy, gw, gb, s, st);
 }
 
 int check_shape(const int *sp, const int *k, const int *dil, int n, int ci, int co, Shape &s)
@@ -939,10 +958,10 @@ int lbm_nn_conv3d_backward(const float *x, const void *w, int w_bf16, const floa
     }
     if (w_bf16 && ci * taps <= nntc::kMaxKp && round16(co) <= nntc::kMaxNp && tc_sizes(s))
         switch (round16(co) / 16) {
-        case 1: return tc_conv_bwd_w_launch<1>(x, gy, gw, gb, s, st);
-        case 2: return tc_conv_bwd_w_launch<2>(x, gy, gw, gb, s, st);
-        case 3: return tc_conv_bwd_w_launch<3>(x, gy, gw, gb, s, st);
-        default: return tc_conv_bwd_w_launch<4>(x, gy, gw, gb, s, st);
+        case 1: return tc_conv_bwd_w<1>(x, gy, gw, gb, s, st);
+        case 2: return tc_conv_bwd_w<2>(x, gy, gw, gb, s, st);
+        case 3: return tc_conv_bwd_w<3>(x, gy, gw, gb, s, st);
+        default: return tc_conv_bwd_w<4>(x, gy, gw, gb, s, st);
         }
     const long long blocks = (long long)co * ci * taps + co;
     k_conv_bwd_w<<<(unsigned)blocks, kT, 0, st>>>(x, gy, gw, gb, s);

@@ -49,17 +49,24 @@ NN_HD int tap_source(const Shape &s, const Pixel &x, int a, int f, int e, int sg
     return in ? (zd * s.h + zh) * s.w + zw : -1;
 }
 // The images as one line of positions: every row of w pixels is followed by hw
-// empty ones (hw: the taps' reach along w), so that position + shift is the
-// shifted pixel of the same row, or an empty one, for every |shift| <= hw.
+// empty ones, hw the largest shift along w of a tap that can meet a pixel at all (one below
+// w), so that position + shift is the shifted pixel of the same row, or an empty one, for
+// every |shift| <= hw.  Taps further out have no source anywhere.
 struct Line {
     int hw, wp;       // reach, positions per row
     unsigned total;   // positions of the batch
     int sp;
 };
+// Taps on either side of the middle one that can meet a pixel along w.
+NN_HD int taps_in_reach(const Shape &s)
+{
+    const int all = (s.kw - 1) / 2, some = (s.w - 1) / s.dw;
+    return all < some ? all : some;
+}
 NN_HD Line line_of(const Shape &s)
 {
     Line l;
-    l.hw = s.dw * ((s.kw - 1) / 2);
+    l.hw = s.dw * taps_in_reach(s);
     l.wp = s.w + l.hw;
     l.sp = s.d * s.h * s.w;
     l.total = (unsigned)s.n * (unsigned)(s.d * s.h) * (unsigned)l.wp;
