@@ -14,6 +14,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "../../include/lbm.h"
 #include "k_nn_index.cuh"
@@ -298,7 +299,7 @@ __device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
 // blockIdx.x + gridDim.x, ...  TAPS = 9 (1 x 3 x 3): the nine source positions are
 // found once per pixel and (channel, tap) of every value is known at compile time;
 // 0: any taps, counted along.  For the shapes that the staged form below does not take.
-template <int MODE, int TAPS>
+template <int MODE, int TAPS, class I>
 __global__ void __launch_bounds__(nntc::kM, TAPS ? 5 : 1)
 k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
           float *__restrict__ out, Shape s, int act, int Kp, int Np)
@@ -315,8 +316,8 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
     const int cout = MODE == TC_FWD ? s.co : s.ci;   // channels of the result
     const int K = cin * taps;
     const int sgn = MODE == TC_FWD ? 1 : -1;
-    const int sp = s.d * s.h * s.w;
-    const unsigned npix = (unsigned)s.n * (unsigned)sp, ntiles = (npix + kM - 1) / kM;
+    const I sp = (I)s.d * s.h * s.w;
+    const I npix = s.n * sp, ntiles = (npix + kM - 1) / kM;
     const uint32_t ncols = tmem_cols(Np);
     const uint32_t lboA = (kM / 8) * 128, lboB = (uint32_t)(Np / 8) * 128;
     if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
@@ -342,19 +343,19 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
     const uint32_t tmem = tmem_base;
     bool ok = true;
     uint32_t phase = 0;
-    for (unsigned tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const unsigned q = tile * kM + tid;
+    for (I tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        const I q = tile * kM + tid;
         const bool valid = q < npix;
-        const Pixel x = pixel_at(s, valid ? q : 0);
+        const Pixel<I> x = pixel_at<I>(s, valid ? q : 0);
         const float *base = in + (long long)x.n * cin * sp;
         auto put8 = [&](int k8, const float (&v)[8]) {
             *reinterpret_cast<uint4 *>(As + core_off(tid, 8 * k8, kM)) = make_uint4(
                 pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
         };
         if constexpr (TAPS == 9) {
-            int at[9];
+            I at[9];
 #pragma unroll
-            for (int tap = 0; tap < 9; tap++) at[tap] = valid ? tap_source(s, x, 0, tap / 3, tap % 3, sgn) : -1;
+            for (int tap = 0; tap < 9; tap++) at[tap] = valid ? tap_source(s, x, 0, tap / 3, tap % 3, sgn) : (I)-1;
             // over every group of the padded K: eight channels' taps are nine groups, and a
             // channel count that is an odd multiple of eight leaves one of zeros beyond them
             for (int k0 = 0; k0 < (Kp >> 3); k0 += 9) {
@@ -379,7 +380,7 @@ k_tc_conv(const float *__restrict__ in, const __nv_bfloat16 *__restrict__ w, con
                 float v[8];
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
-                    const int at = valid && c < cin ? tap_source(s, x, a, f, e, sgn) : -1;
+                    const I at = valid && c < cin ? tap_source(s, x, a, f, e, sgn) : (I)-1;
                     v[j] = at >= 0 ? __ldg(base + plane_offset(c, sp, at)) : 0.f;
                     if (++e == s.kw) {
                         e = 0;
@@ -463,7 +464,7 @@ k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
     const int cin = MODE == TC_FWD ? s.ci : s.co;    // channels of the gathered operand
     const int cout = MODE == TC_FWD ? s.co : s.ci;   // channels of the result
     const int sgn = MODE == TC_FWD ? 1 : -1;
-    const Line l = line_of(s);
+    const Line<int> l = line_of<int>(s);
     constexpr int G8 = kStagedChannels / 8;           // channel groups of eight
     const int R = (kM + 2 * l.hw + 7) / 8 * 8;        // staged positions
     constexpr int segs = 3, taps = 9;
@@ -471,7 +472,7 @@ k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
     unsigned char *St = smem;
     unsigned char *As = St + segs * G8 * R * 16;
     unsigned char *Bs = As + kM * Kp * 2;
-    const unsigned ntiles = (l.total + kM - 1) / kM;
+    const int ntiles = (l.total + kM - 1) / kM;
     const uint32_t ncols = tmem_cols(Np);
     const uint32_t lboA = (kM / 8) * 128, lboB = (uint32_t)(Np / 8) * 128;
     if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
@@ -497,10 +498,10 @@ k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
     const uint32_t tmem = tmem_base;
     bool ok = true;
     uint32_t phase = 0;
-    for (unsigned tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int q0 = (int)(tile * kM);
+    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        const int q0 = tile * kM;
         for (int j = tid; j < kM + 2 * l.hw; j += kM) {
-            const Pixel x = position_at(s, l, q0 + j - l.hw);
+            const Pixel<int> x = position_at(s, l, q0 + j - l.hw);
             const float *base = in + (long long)x.n * cin * l.sp + x.w;
             for (int seg = 0; seg < segs; seg++) {
                 const int zh = x.h + sgn * s.dh * (seg - 1);
@@ -561,7 +562,7 @@ k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
         fence_after_sync();
         phase ^= 1u;
         if (!ok) break;
-        const Pixel x = position_at(s, l, q0 + tid);
+        const Pixel<int> x = position_at(s, l, q0 + tid);
         float *dst = out + (long long)x.n * cout * l.sp + (x.d * s.h + x.h) * s.w + x.w;
         for (int c0 = 0; c0 < Np; c0 += 16) {
             float v[16];
@@ -602,8 +603,8 @@ k_tc_conv_staged(const float *__restrict__ in, const __nv_bfloat16 *__restrict__
 // order.  A thread loads the value of one position (and the first 2 hw threads
 // one of the halo) once per row of taps and channel, rounds it once and stores
 // it in the kw columns that its taps along w put it in.  FAR: tap by tap, for dilations of
-// a chunk and more, where the taps' positions lie apart, and for taps out of reach (2 x 256 x 2048 positions, 16
-// channels, dilation 868: 228 us, with the whole halo 1214; dilation 127: 260 with it).
+// a chunk and more, where the taps' positions lie apart, for taps out of reach and for 64-bit positions (2 x 256 x 2048 positions, 16
+// channels, dilation 868: 243 us, with the whole halo 1214; dilation 127: 260 with it).
 // Columns are stored two bytes at a time; the core matrices lie kPad bytes further apart along K than
 // they are long, so that the 32 columns of a warp fall on 16 different banks (two
 // columns share a word).
@@ -614,13 +615,14 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
                 float *__restrict__ bpart, Shape s, int G, int tiles)
 {
     using namespace nntc;
+    using I = typename std::conditional<FAR, long long, int>::type;
     constexpr int Np = 16 * N16;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long mbar;
     __shared__ uint32_t tmem_base;
     __shared__ float bsum[kM / 32][Np];
     const int tid = threadIdx.x;
-    const Line l = line_of(s);
+    const Line<I> l = line_of<I>(s);
     const int segs = s.kd * s.kh, Kw = s.ci * segs * s.kw, rows = (Kw + 7) / 8 * 8;
     const uint32_t lboA = (uint32_t)rows * 16 + kPad, lboB = (uint32_t)Np * 16 + kPad;
     unsigned char *Bs = smem;
@@ -629,7 +631,7 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
     if (FAR && reach < mid) {  // the columns of the taps without a source stay 0
         for (uint32_t k = tid; k < kM / 8 * lboA / 16; k += kM) reinterpret_cast<uint4 *>(As)[k] = make_uint4(0, 0, 0, 0);
     }
-    const unsigned nchunks = (l.total + kM - 1) / kM;
+    const I nchunks = (l.total + kM - 1) / kM;
     const int g = blockIdx.x;
     const uint32_t ncols = tmem_cols(tiles * Np);
     if (tid < 32) tmem_alloc(smem_u32(&tmem_base), ncols);
@@ -643,12 +645,12 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
     for (int o = 0; o < Np; o++) bacc[o] = 0.f;
     bool ok = true;
     int round = 0;
-    for (unsigned c = g; c < nchunks && ok; c += G, round++) {
-        const int q0 = (int)(c * kM);
+    for (I c = g; c < nchunks && ok; c += G, round++) {
+        const I q0 = c * kM;
         {
-            const Pixel px = position_at(s, l, q0 + tid);
+            const Pixel<I> px = position_at<I>(s, l, q0 + tid);
             const bool valid = px.w >= 0;
-            const float *src = gy + (long long)px.n * s.co * l.sp + (valid ? (px.d * s.h + px.h) * s.w + px.w : 0);
+            const float *src = gy + (long long)px.n * s.co * l.sp + (valid ? ((I)px.d * s.h + px.h) * s.w + px.w : 0);
             unsigned char *col = Bs + (tid >> 3) * lboB + (tid & 7) * 2;
 #pragma unroll
             for (int o = 0; o < Np; o++) {
@@ -659,21 +661,21 @@ k_tc_conv_bwd_w(const float *__restrict__ x, const float *__restrict__ gy, float
         }
         // j: a position less q0, its value into the columns of the taps first .. last
         int first = mid - reach, last = FAR ? first : s.kw - 1;
-        for (int j = tid - l.hw; FAR ? first <= mid + reach : j < kM + l.hw; j += FAR ? s.dw : kM) {
-            const Pixel px = position_at(s, l, q0 + j);
+        for (I j = tid - l.hw; FAR ? first <= mid + reach : j < kM + l.hw; j += FAR ? s.dw : kM) {
+            const Pixel<I> px = position_at<I>(s, l, q0 + j);
             const float *base = x + (long long)px.n * s.ci * l.sp + px.w;
             for (int seg = 0; seg < segs; seg++) {
                 const int a = seg / s.kh, f = seg - a * s.kh;
                 const int zd = px.d + s.dd * (a - (s.kd - 1) / 2), zh = px.h + s.dh * (f - (s.kh - 1) / 2);
                 const bool have = px.w >= 0 && (unsigned)zd < (unsigned)s.d && (unsigned)zh < (unsigned)s.h;
-                const float *src = base + (have ? (zd * s.h + zh) * s.w : 0);
+                const float *src = base + (have ? ((I)zd * s.h + zh) * s.w : 0);
                 for (int i0 = 0; i0 < s.ci; i0 += 8) {
                     __nv_bfloat16 v[8];
 #pragma unroll
                     for (int i = 0; i < 8; i++)
                         v[i] = __float2bfloat16_rn(have && i0 + i < s.ci ? __ldg(src + (long long)(i0 + i) * l.sp) : 0.f);
                     for (int e = FAR ? first : 0; e <= last; e++) {
-                        const int k = j - s.dw * (e - mid);
+                        const int k = (int)(j - (I)s.dw * (e - mid));
                         if ((unsigned)k >= (unsigned)kM) continue;
                         unsigned char *dst = As + (k >> 3) * lboA + (k & 7) * 2 + ((seg * s.kw + e) * s.ci + i0) * 16;
 #pragma unroll
@@ -799,18 +801,10 @@ void *scratch_alloc(size_t bytes, cudaStream_t st)
     return p;
 }
 
-// Positions of the batch in 32 bits (the kernels' index type), with room for a
-// tile and its halo past the last one.
-bool tc_sizes(const Shape &s)
-{
-    const long long hw = (long long)s.dw * ((s.kw - 1) / 2);
-    return hw < (1LL << 20) && (long long)s.d * s.h * s.w < (1LL << 30) &&
-           (long long)s.n * s.d * s.h * (s.w + hw) < (1LL << 31) - (1LL << 21);
-}
 // The shapes the tensor-core kernels take: what a tile holds (include/lbm.h).
 bool tc_fits(const Shape &s, int cin, int cout)
 {
-    return round16(cin * s.kd * s.kh * s.kw) <= nntc::kMaxKp && round16(cout) <= nntc::kMaxNp && tc_sizes(s);
+    return round16(cin * s.kd * s.kh * s.kw) <= nntc::kMaxKp && round16(cout) <= nntc::kMaxNp;
 }
 
 // Blocks of a kernel that an SM holds at once, times the SMs, by registers, shared
@@ -834,12 +828,12 @@ unsigned resident_grid(K kernel, size_t smem, int ncols)
 }
 
 template <class K, class... A>
-int tc_launch(K kernel, unsigned tiles, size_t smem, int Np, cudaStream_t st, const char *what, A... args)
+int tc_launch(K kernel, long long tiles, size_t smem, int Np, cudaStream_t st, const char *what, A... args)
 {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return nn_fail(LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e));
     const unsigned most = resident_grid(kernel, smem, nntc::tmem_cols(Np));
-    kernel<<<tiles < most ? tiles : most, nntc::kM, smem, st>>>(args...);
+    kernel<<<tiles < most ? (unsigned)tiles : most, nntc::kM, smem, st>>>(args...);
     return launched(what);
 }
 
@@ -851,17 +845,18 @@ int tc_conv_launch(const float *in, const void *w, const float *b, float *out, c
     const __nv_bfloat16 *wb = reinterpret_cast<const __nv_bfloat16 *>(w);
     const int taps = s.kd * s.kh * s.kw, Kp = round16(cin * taps);
     const size_t smem = (size_t)(nntc::kM + Np) * Kp * 2;
-    if (s.kd == 1 && s.kh == 3 && s.kw == 3) {
-        const Line l = line_of(s);
+    const bool small = narrow(s);
+    const long long npix = (long long)s.n * s.d * s.h * s.w, tiles = (npix + nntc::kM - 1) / nntc::kM;
+    if (small && s.kd == 1 && s.kh == 3 && s.kw == 3) {
+        const Line<int> l = line_of<int>(s);
         const size_t stage = (size_t)3 * (kStagedChannels / 8) * ((nntc::kM + 2 * (size_t)l.hw + 7) / 8 * 8) * 16;
         if (cin <= kStagedChannels && l.hw <= kStagedReach && l.hw == s.dw)
             return tc_launch(k_tc_conv_staged<MODE>, (l.total + nntc::kM - 1) / nntc::kM, smem + stage, Np, st, what, in,
                              wb, b, out, s, act, Kp, Np);
+        return tc_launch(k_tc_conv<MODE, 9, int>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
     }
-    const unsigned npix = (unsigned)((long long)s.n * s.d * s.h * s.w), tiles = (npix + nntc::kM - 1) / nntc::kM;
-    if (s.kd == 1 && s.kh == 3 && s.kw == 3)
-        return tc_launch(k_tc_conv<MODE, 9>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
-    return tc_launch(k_tc_conv<MODE, 0>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
+    if (small) return tc_launch(k_tc_conv<MODE, 0, int>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
+    return tc_launch(k_tc_conv<MODE, 0, long long>, tiles, smem, Np, st, what, in, wb, b, out, s, act, Kp, Np);
 }
 
 template <int N16, bool FAR>
@@ -870,12 +865,12 @@ int tc_conv_bwd_w_launch(const float *x, const float *gy, float *gw, float *gb, 
     constexpr int Np = 16 * N16;
     const int taps = s.kd * s.kh * s.kw, Kw = s.ci * taps, rows = (Kw + 7) / 8 * 8;
     const int tiles = (Kw + nntc::kM - 1) / nntc::kM, Mp = tiles * nntc::kM;
-    const unsigned nchunks = (line_of(s).total + nntc::kM - 1) / nntc::kM;
+    const long long nchunks = (line_of<long long>(s).total + nntc::kM - 1) / nntc::kM;
     const size_t smem = (size_t)(nntc::kM / 8) * (rows * 16 + kPad + Np * 16 + kPad) + (size_t)(Mp - rows) * 16;
     cudaError_t e = cudaFuncSetAttribute(k_tc_conv_bwd_w<N16, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return nn_fail(LBM_ECUDA, "conv3d_backward(weights): %s", cudaGetErrorString(e));
     unsigned G = resident_grid(k_tc_conv_bwd_w<N16, FAR>, smem, nntc::tmem_cols(tiles * Np));
-    if (G > nchunks) G = nchunks;
+    if (G > nchunks) G = (unsigned)nchunks;
     float *part = static_cast<float *>(scratch_alloc((size_t)G * (Mp + 1) * Np * sizeof(float), st));
     if (!part) return nn_fail(LBM_ENOMEM, "conv3d_backward: tensor-core workspace");
     float *bpart = part + (size_t)G * Mp * Np;
@@ -889,7 +884,7 @@ int tc_conv_bwd_w_launch(const float *x, const float *gy, float *gw, float *gb, 
 template <int N16>
 int tc_conv_bwd_w(const float *x, const float *gy, float *gw, float *gb, const Shape &s, cudaStream_t st)
 {
-    return s.dw >= nntc::kM || taps_in_reach(s) < (s.kw - 1) / 2 ? tc_conv_bwd_w_launch<N16, true>(x, gy, gw, gb, s, st)
+    return s.dw >= nntc::kM || taps_in_reach(s) < (s.kw - 1) / 2 || !narrow(s) ? tc_conv_bwd_w_launch<N16, true>(x, gy, gw, gb, s, st)
                             : tc_conv_bwd_w_launch<N16, false>(x, gy, gw, gb, s, st);
 }
 
@@ -956,7 +951,7 @@ int lbm_nn_conv3d_backward(const float *x, const void *w, int w_bf16, const floa
         }
         if (rc != LBM_OK) return rc;
     }
-    if (w_bf16 && ci * taps <= nntc::kMaxKp && round16(co) <= nntc::kMaxNp && tc_sizes(s))
+    if (w_bf16 && ci * taps <= nntc::kMaxKp && round16(co) <= nntc::kMaxNp)
         switch (round16(co) / 16) {
         case 1: return tc_conv_bwd_w<1>(x, gy, gw, gb, s, st);
         case 2: return tc_conv_bwd_w<2>(x, gy, gw, gb, s, st);
