@@ -1176,6 +1176,47 @@ def extras(lbm, stream, hbm, hbm_src, peak):
     return out
 
 
+def rounded(v, digits=5):
+    """`v` with every float in it rounded to `digits` significant digits."""
+    if isinstance(v, float):
+        return float(f"{v:.{digits}g}") if math.isfinite(v) else v
+    if isinstance(v, dict):
+        return {k: rounded(x, digits) for k, x in v.items()}
+    return [rounded(x, digits) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def brief(ext):
+    """The sub-results as the printed line holds them (a few kilobytes in all, so that
+    whatever collects the line gets it whole): of each the rates, the fraction of its
+    bound, steps, times and errors.  All else goes to stderr."""
+    def one(r):
+        out = {k: r[k] for k in ("error", "mlups", "ms_per_step", "seconds", "steps", "reached", "l2_u_vs_fp64",
+                                 "l2_vs_parabola", "l2_vs_fp64_steady", "orders") if k in r}
+        if isinstance(out.get("steps"), list):
+            del out["steps"]
+        roof = r.get("roofline") or r.get("step_kernel", {}).get("roofline")
+        if roof:
+            out["frac"] = {roof["bound"]: roof["frac"]}
+            if "hbm" in roof:
+                out["frac"]["hbm"] = roof["hbm"]["frac"]
+        if "run" in r:
+            out["run_mlups"] = r["run"]["mlups"]
+        return out
+
+    out = {}
+    for key in ("storages", "workloads", "time_to_solution"):
+        if key in ext:
+            out[key] = {k: one(v) if isinstance(v, dict) else v for k, v in ext[key].items()
+                        if k != "batched_sweep_subset"}
+    sub = ext.get("time_to_solution", {}).get("batched_sweep_subset")
+    if isinstance(sub, dict):
+        out["time_to_solution"]["batched_sweep_subset"] = \
+            {k: one(v) for k, v in sub.items() if isinstance(v, dict) and "reached" in v} or one(sub)
+    if "extras_seconds" in ext:
+        out["extras_seconds"] = ext["extras_seconds"]
+    return rounded(out)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1380,8 +1421,15 @@ def main():
             line["config"]["graph_steps"] = args.graph
         if modes is not None:
             line["launch_modes"] = modes
+        details = {"fp64_peak": peak, "e2e": e2e}
+        if e2e and "other_forms" in e2e:
+            line["e2e"] = dict(e2e, other_forms={k: v.get("value") for k, v in e2e["other_forms"].items()})
+        if peak is not None:
+            line["fp64_peak"] = {k: v for k, v in peak.items() if k != "all_configurations_ginst_per_s"}
         if ext:
-            line.update(ext)
+            line.update(brief(ext))
+            details.update(ext)
+        print(json.dumps({"details": details}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if dist:
         dist.destroy_process_group()
