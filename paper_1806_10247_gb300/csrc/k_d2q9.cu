@@ -21,6 +21,16 @@ struct Rates9 {
 // Post-collision populations of one node, in place.
 //   Fx, Fy : pre-collision force a_pre P (Eq. 25)
 //   Gx, Gy : first-moment coefficients g_1, g_2 = (F_pre + F_post)/12 (Eqs. 27-31)
+//   CHAIN  : a kernel that waits for one node's chain of operations takes the maths
+//            library's 1/rho, the shorter chain (general rates, 3 x 33, 100 steps: 453 us,
+//            467 with recip_density); the others, which the FP64 unit bounds, the one with
+//            fewer FP64 operations (2048 x 1024, 10 steps: 5106, 5175).  The bits are the same.
+template <bool CHAIN>
+__device__ __forceinline__ double one_over(double rho)
+{
+    return CHAIN ? __drcp_rn(rho) : recip_density(rho);
+}
+template <bool CHAIN>
 __device__ __forceinline__ void collide(double (&f)[9], double Fx, double Fy, double Gx, double Gy,
                                         const Rates9 &w)
 {
@@ -35,7 +45,7 @@ __device__ __forceinline__ void collide(double (&f)[9], double Fx, double Fy, do
     const double mxx = s0 + (s1 + s2), mxxy = s1 - s2, mxxyy = s1 + s2;
 
     // Eq. 25: velocity after the pre-collision half force step.
-    const double rinv = __drcp_rn(rho);
+    const double rinv = one_over<CHAIN>(rho);
     const double jfx = fma(0.5, Fx, jx), jfy = fma(0.5, Fy, jy);
     const double ux = jfx * rinv;
     const double uy = jfy * rinv;
@@ -85,7 +95,7 @@ __device__ __forceinline__ void collide(double (&f)[9], double Fx, double Fy, do
 // itself (not rebuilt as rho (j / rho)), so the step transports momentum
 // without a rounding of its own.  About 80 FP64 operations instead of 132.
 // XO: the force has no y component (its terms, additions of 0, are left out).
-template <bool XO = false>
+template <bool XO, bool CHAIN>
 __device__ __forceinline__ void collide_w1(double (&f)[9], double Fx, double Fy, double Gx, double Gy,
                                            const Rates9 &w)
 {
@@ -98,7 +108,7 @@ __device__ __forceinline__ void collide_w1(double (&f)[9], double Fx, double Fy,
     const double jy0 = B0 - C0;
     const double jx = fma(0.5, Fx, d0 + (d1 + d2)), jy = XO ? jy0 : fma(0.5, Fy, jy0);  // Eq. 25
     const double mxx = s0 + (s1 + s2), myy = B0 + C0, mxy = d1 - d2;
-    const double rinv = __drcp_rn(rho);
+    const double rinv = one_over<CHAIN>(rho);
     const double ux = jx * rinv, uy = jy * rinv;
 
     // second-order central moments, relaxed and halved (xx, yy by 1/2 ... of
@@ -175,7 +185,7 @@ __device__ __forceinline__ FxStep fixed_step9(const double (&f)[9], const FxRate
 }
 
 // The FP64 form of a node's step; gsum = (a_pre + a_post) / 12.
-template <bool W1, bool XO, class Shape>
+template <bool W1, bool XO, bool CHAIN = false, class Shape>
 __device__ __forceinline__ void double_step9(double (&f)[9], const Rates9 &w, bool forced, double apre, double gsum,
                                              Shape shape)
 {
@@ -190,8 +200,8 @@ __device__ __forceinline__ void double_step9(double (&f)[9], const Rates9 &w, bo
             Gy = gsum * Py;
         }
     }
-    if (W1) collide_w1<XO>(f, Fx, Fy, Gx, Gy, w);
-    else collide(f, Fx, Fy, Gx, Gy, w);
+    if (W1) collide_w1<XO, CHAIN>(f, Fx, Fy, Gx, Gy, w);
+    else collide<CHAIN>(f, Fx, Fy, Gx, Gy, w);
 }
 
 // XO (unit higher rates only): the force has no y component (checked on the host).
@@ -232,8 +242,8 @@ k_step(const __grid_constant__ Planes<double, 9> P, Geom g, FieldDev F, double a
 // the state is FP64 between the steps, so the result is theirs, however the steps
 // are cut into calls (up to the compiler's multiply-add contraction in the FP64 form).
 // A step of ~100 nodes is one warp per SM: its time is the latency of one node's
-// chain of operations (3 x 33, 100 steps: 1.63 us a step in fixed point, 3.06 in FP64;
-// 48 x 96 3.06 and 7.2).  Keeping the fixed-point state from step to step at one scale
+// chain of operations (3 x 33, 100 steps: 1.67 us a step in fixed point, 3.06 in FP64;
+// 48 x 96 2.93 and 7.2).  Keeping the fixed-point state from step to step at one scale
 // for the lattice takes 1.38, but then the result depends on how the steps are cut.
 namespace cg = cooperative_groups;
 
@@ -287,7 +297,7 @@ k_cluster_steps(const double *__restrict__ fin, double *__restrict__ fout, Geom 
             if (W1) r = fixed_step9<FK != FK_NONE, false>(f, fx, q1, q2, shape, [&](int a, double v) { nxt[a * P + l] = v; });
             if (r == FX_GIVEN_UP) pull();
             if (r != FX_DONE) {
-                double_step9<W1, false>(f, w, FK != FK_NONE, apre, gsum, shape);
+                double_step9<W1, false, true>(f, w, FK != FK_NONE, apre, gsum, shape);
 #pragma unroll
                 for (int a = 0; a < 9; a++) nxt[a * P + l] = f[a];
             }
@@ -323,14 +333,14 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
         const FxStep r = fixed_step9<true, true>(f, B.fx, ap.q1, ap.q2, shape, put);
         if (r == FX_DONE) return;
         if (r == FX_GIVEN_UP) load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-        double_step9<true, true>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
+        double_step9<true, true>(f, w, forced, ap.pre, ap.g, shape);
     } else if (B.variant == 1) {
         const FxStep r = fixed_step9<true, false>(f, B.fx, ap.q1, ap.q2, shape, put);
         if (r == FX_DONE) return;
         if (r == FX_GIVEN_UP) load_pulled<LD2Q9>(fin, g, x, y, 0, i, f);
-        double_step9<true, false>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
+        double_step9<true, false>(f, w, forced, ap.pre, ap.g, shape);
     } else {
-        double_step9<false, false>(f, w, forced, 4.0 * ap.q1, ap.g, shape);
+        double_step9<false, false>(f, w, forced, ap.pre, ap.g, shape);
     }
 #pragma unroll
     for (int a = 0; a < 9; a++) put(a, f[a]);

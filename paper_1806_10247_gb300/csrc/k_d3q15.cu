@@ -209,7 +209,7 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
         if (r == FX_DONE) return;
         if (r == FX_GIVEN_UP) load_pulled<LD3Q15>(fin, g, x, y, z, i, f);
     }
-    double_step15(f, w, forced, 4.0 * ap.q1, ap.g, shape);
+    double_step15(f, w, forced, ap.pre, ap.g, shape);
 #pragma unroll
     for (int a = 0; a < 15; a++) fout[a * g.Np + i] = f[a];
 }

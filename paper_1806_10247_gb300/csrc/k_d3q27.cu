@@ -187,7 +187,7 @@ __device__ __forceinline__ void collide(double (&m)[27], const double (&F)[3], c
         m[9] = fma(0.5, F[2], m[9]);
     }
     const double rho = m[0];
-    const double rinv = __drcp_rn(rho);
+    const double rinv = recip_density(rho);
     const double ux = m[1] * rinv, uy = m[3] * rinv, uz = m[9] * rinv;
 
     along<0>(m, [ux](double &a, double &b, double &c) { shift_fwd(a, b, c, ux); });
@@ -272,7 +272,7 @@ __device__ __forceinline__ void collide_w1(double (&m)[27], const double (&F)[3]
         jy = fma(0.5, F[1], jy);
         jz = fma(0.5, F[2], jz);
     }
-    const double rinv = __drcp_rn(rho);
+    const double rinv = recip_density(rho);
     const double ux = jx * rinv, uy = jy * rinv, uz = jz * rinv;
 
     // Second-order central moments (the first ones vanish) and their relaxation.
@@ -414,14 +414,14 @@ __device__ __forceinline__ void batch_node(const BatchItem &B, const BatchLaunch
         const FxStep r = fixed_step27<true, true>(m, B.fx, ap.q1, ap.q2, shape, put);
         if (r == FX_DONE) return;
         if (r == FX_GIVEN_UP) load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
-        double_step27<true, true>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
+        double_step27<true, true>(m, w, forced, ap.pre, ap.g, shape);
     } else if (B.variant == 1) {
         const FxStep r = fixed_step27<true, false>(m, B.fx, ap.q1, ap.q2, shape, put);
         if (r == FX_DONE) return;
         if (r == FX_GIVEN_UP) load_pulled<LD3Q27>(fin, g, x, y, z, i, m);
-        double_step27<true, false>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
+        double_step27<true, false>(m, w, forced, ap.pre, ap.g, shape);
     } else {
-        double_step27<false, false>(m, w, forced, 4.0 * ap.q1, ap.g, shape);
+        double_step27<false, false>(m, w, forced, ap.pre, ap.g, shape);
     }
 #pragma unroll
     for (int a = 0; a < 27; a++) put(a, m[a]);

@@ -122,7 +122,7 @@ Amp64 pair64(int lattice, double apre, double apost)
 {
     const double c = lattice == LBM_D2Q5_CDE ? 0.5 : 0.25;
     const double g = lattice == LBM_D2Q9 ? (apre + apost) / 12.0 : (lattice == LBM_D2Q5_CDE ? (apre + apost) / 10.0 : apost);
-    return Amp64{c * apre, c * (apre + apost), g};
+    return Amp64{c * apre, c * (apre + apost), g, apre};
 }
 // The pair of the reduced-precision kernels.
 float2 pair32(int lattice, double apre, double apost)

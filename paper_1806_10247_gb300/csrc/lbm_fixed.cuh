@@ -300,6 +300,14 @@ FX_HD double fx_value_signed(i64 X, int k, int &bad)
     return fx_double(fx_bits(fx_value_pos((X ^ s) - s, k, bad)) | ((u64)X & 0x8000000000000000ull));
 }
 
+// fx_value with its FP64 conversion left to |X| < 2^32, for kernels that the FP64 unit bounds.
+FX_HD double fx_value_int(i64 X, int k)
+{
+    int bad = 0;
+    const double v = fx_value_signed(X, k, bad);
+    return bad >= 0 ? v : fx_value(X, k);
+}
+
 // ---- force --------------------------------------------------------------------
 // Fixed-point form of a force along one axis at a node, on the refined grid
 // (scale 2^(k + 1)): h1 = F_pre / 4 (half of the pre-collision half force),

@@ -133,11 +133,11 @@ void batch_coef(int lattice, const double omega[9], BatchItem &item);
 constexpr int kInlinePairs = 32;
 // Envelope amplitudes of one step of an FP64 member: of the fixed-point form q1, q2
 // (flow: a_pre / 4, (a_pre + a_post) / 4; D2Q5: a_pre / 2, (a_pre + a_post) / 2), and
-// what the FP64 form takes besides a_pre: D2Q9 (a_pre + a_post) / 12, D2Q5 (a_pre +
+// what the FP64 form takes besides a_pre (pre): D2Q9 (a_pre + a_post) / 12, D2Q5 (a_pre +
 // a_post) / 10, D3Q27 and D3Q15 a_post (each formed on the host as a single lattice's
 // launch forms it, so that a member of a batch has its bits).
 struct Amp64 {
-    double q1, q2, g;
+    double q1, q2, g, pre;
 };
 struct BatchLaunch {
     const BatchItem *items;

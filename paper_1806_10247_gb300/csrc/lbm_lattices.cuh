@@ -246,8 +246,9 @@ __device__ __forceinline__ void sum_moments(const V (&f)[L::Q], V &m0, V (&j)[3]
 // forms them: summed in fixed point (lbm_fixed.cuh), where the sums are exact,
 // and rounded once; a node outside the fixed-point range is summed in FP64.  The
 // FP64 sums of D3Q27 took 40 clocks of an SM's FP64 unit per node, the four
-// conversions back take 2.  D2Q5's four FP64 adds stay.
-template <class L>
+// conversions back take 2 (INT: none, for a readback inside a step, which the FP64 unit
+// bounds more tightly).  D2Q5's four FP64 adds stay.
+template <class L, bool INT = false>
 __device__ __forceinline__ void zeroth_first(const double (&f)[L::Q], double &m0, double (&j)[3])
 {
     const int em = fx_emax(f);
@@ -256,9 +257,9 @@ __device__ __forceinline__ void zeroth_first(const double (&f)[L::Q], double &m0
         i64 X[L::Q], M, J[3];
         fx_load_int<L::Q, true>(f, em, X);
         sum_moments<L>(X, M, J);
-        m0 = fx_value(M, k);
+        m0 = INT ? fx_value_int(M, k) : fx_value(M, k);
 #pragma unroll
-        for (int d = 0; d < 3; d++) j[d] = d < L::DIM ? fx_value(J[d], k) : 0.0;
+        for (int d = 0; d < 3; d++) j[d] = d < L::DIM ? (INT ? fx_value_int(J[d], k) : fx_value(J[d], k)) : 0.0;
         return;
     }
     sum_moments<L>(f, m0, j);

@@ -87,7 +87,7 @@ __device__ __forceinline__ void fused_fields(const BatchItem &B, const BatchLaun
                                              const double (&f)[L::Q], double ahalf)
 {
     double m0, j[3];
-    zeroth_first<L>(f, m0, j);
+    zeroth_first<L, true>(f, m0, j);
     store_fields<L>(m0, j, Ln.mhalf && B.fkind != FK_NONE, ahalf, B.F, B.fkind, x, y, z, i, B.g.N, __ldg(Ln.moff + it),
                     Ln.mrho, Ln.mu);
 }
