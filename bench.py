@@ -85,41 +85,41 @@ ALG_FP64 = {
 # kernel sources still hash to the value it was measured on.  Traffic per
 # launch scales with the node count once the state is larger than L2.
 TRAFFIC = {
-    ("d3q27", "fp64"): {"src": [_C + "k_d3q27.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "91b3ca51611b3206",
-                        "bytes_per_node": (1528.952320 + 1509.775872) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
+    ("d3q27", "fp64"): {"src": [_C + "k_d3q27.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "277eaff326019fb2",
+                        "bytes_per_node": (1528.931840 + 1498.999808) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
                         "profile": "profiles/step_traffic.md"},
-    ("d3q27", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                        "bytes_per_node": (1812.021504 + 1767.237376) * 1e6 / 256 ** 3, "captured_nodes": 256 ** 3,
+    ("d3q27", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                        "bytes_per_node": (1812.077312 + 1767.237632) * 1e6 / 256 ** 3, "captured_nodes": 256 ** 3,
                         "profile": "profiles/step_traffic.md"},
-    ("d3q27", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                        "bytes_per_node": (382.267904 + 333.303040) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
+    ("d3q27", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                        "bytes_per_node": (382.268160 + 333.299200) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
                         "profile": "profiles/step_traffic.md"},
-    ("d3q27", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                        "bytes_per_node": (382.292480 + 333.123840) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
+    ("d3q27", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                        "bytes_per_node": (382.365696 + 332.693248) * 1e6 / 192 ** 3, "captured_nodes": 192 ** 3,
                         "profile": "profiles/step_traffic.md"},
-    ("d2q9", "fp64"): {"src": [_C + "k_d2q9.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "2c2f5e8bbf069d40",
-                       "bytes_per_node": (151.032832 + 103.470080) * 1e6 / (2048 * 1024), "captured_nodes": 2048 * 1024,
+    ("d2q9", "fp64"): {"src": [_C + "k_d2q9.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "6ee964a3aeea8f93",
+                       "bytes_per_node": (151.032832 + 102.737664) * 1e6 / (2048 * 1024), "captured_nodes": 2048 * 1024,
                        "profile": "profiles/step_traffic.md"},
-    ("d2q9", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                       "bytes_per_node": (1208.190464 + 1157.165568) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
+    ("d2q9", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                       "bytes_per_node": (1208.181504 + 1157.228288) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
                        "profile": "profiles/step_traffic.md"},
-    ("d2q9", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                       "bytes_per_node": (604.020736 + 552.885760) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
+    ("d2q9", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                       "bytes_per_node": (604.020480 + 553.233664) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
                        "profile": "profiles/step_traffic.md"},
-    ("d2q9", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                       "bytes_per_node": (604.098048 + 553.156096) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
+    ("d2q9", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                       "bytes_per_node": (604.019712 + 552.982272) * 1e6 / (8192 * 4096), "captured_nodes": 8192 * 4096,
                        "profile": "profiles/step_traffic.md"},
-    ("d2q5", "fp64"): {"src": [_C + "k_d2q5.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "c3366801003844ff", "above_l2": True,
-                       "bytes_per_node": (2684.602368 + 2640.131072) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+    ("d2q5", "fp64"): {"src": [_C + "k_d2q5.cu", _C + "lbm_fixed.cuh"] + _H, "sha": "2fd0178c118f4b2b", "above_l2": True,
+                       "bytes_per_node": (2684.562432 + 2640.157440) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
                        "profile": "profiles/step_traffic.md"},
-    ("d2q5", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                       "bytes_per_node": (1342.337792 + 1293.668096) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+    ("d2q5", "fp32"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                       "bytes_per_node": (1342.272512 + 1293.643776) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
                        "profile": "profiles/step_traffic.md"},
-    ("d2q5", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                       "bytes_per_node": (671.212288 + 620.969216) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+    ("d2q5", "fp16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                       "bytes_per_node": (671.183104 + 621.047296) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
                        "profile": "profiles/step_traffic.md"},
-    ("d2q5", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "09c4872d6dfa3214", "above_l2": True,
-                       "bytes_per_node": (671.193344 + 621.036032) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
+    ("d2q5", "bf16"): {"src": [_C + "k_rp.cu"] + _H, "sha": "0d2be90f17359e66", "above_l2": True,
+                       "bytes_per_node": (671.182592 + 620.990208) * 1e6 / 8192 ** 2, "captured_nodes": 8192 ** 2,
                        "profile": "profiles/step_traffic.md"},
 }
 
