@@ -808,10 +808,10 @@ bool tc_fits(const Shape &s, int cin, int cout)
 }
 
 // Blocks of a kernel that an SM holds at once, times the SMs, by registers, shared
-// memory, tensor memory columns and threads.  (The occupancy query answers 1 for
+// memory, tensor memory columns and threads, at most `most`.  (The occupancy query answers 1 for
 // kernels that allocate tensor memory.)
 template <class K>
-unsigned resident_grid(K kernel, size_t smem, int ncols)
+unsigned resident_grid(K kernel, size_t smem, int ncols, int most = 2048 / nntc::kM)
 {
     int dev = 0, sms = 152, per_sm = 512 / ncols;
     cudaFuncAttributes a{};
@@ -822,7 +822,7 @@ unsigned resident_grid(K kernel, size_t smem, int ncols)
     } else {
         cudaGetLastError();
     }
-    per_sm = std::max(1, std::min(per_sm, 2048 / nntc::kM));
+    per_sm = std::max(1, std::min(per_sm, most));
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return (unsigned)(per_sm * sms);
 }
@@ -869,7 +869,9 @@ int tc_conv_bwd_w_launch(const float *x, const float *gy, float *gw, float *gb, 
     const size_t smem = (size_t)(nntc::kM / 8) * (rows * 16 + kPad + Np * 16 + kPad) + (size_t)(Mp - rows) * 16;
     cudaError_t e = cudaFuncSetAttribute(k_tc_conv_bwd_w<N16, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return nn_fail(LBM_ECUDA, "conv3d_backward(weights): %s", cudaGetErrorString(e));
-    unsigned G = resident_grid(k_tc_conv_bwd_w<N16, FAR>, smem, nntc::tmem_cols(tiles * Np));
+    // The number of partial sums is part of the result (its last bits), so it does not follow
+    // the registers that the compiler takes: 7, 6, 5 and 4 blocks per SM fit for 16 to 64 channels.
+    unsigned G = resident_grid(k_tc_conv_bwd_w<N16, FAR>, smem, nntc::tmem_cols(tiles * Np), 8 - N16);
     if (G > nchunks) G = (unsigned)nchunks;
     float *part = static_cast<float *>(scratch_alloc((size_t)G * (Mp + 1) * Np * sizeof(float), st));
     if (!part) return nn_fail(LBM_ENOMEM, "conv3d_backward: tensor-core workspace");
